@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "expand.cuh"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -676,15 +677,12 @@ int expand_sort_launch(const Key128* keys, const uint8_t* lens, const uint32_t* 
   // the expansion: one chain, or paired receptors (no bin selection); it
   // also clears the record sort's status area
   const bool zeroed = true;
+  ExpandSource src{keys, lens, eqprev};
+  if (paired) src = ExpandSource{paired->keys, paired->lens, paired->eqprev,
+                                 paired->keys_b, paired->lens_b, paired->eq_b};
   auto expand = [&](int hist_lo, int hist_hi) {
-    if (paired)
-      launch_expand_paired(paired->keys, paired->lens, paired->eqprev, paired->keys_b,
-                           paired->lens_b, paired->eq_b, rec_off, n, d, id_bits, A, rec_cap, hist,
-                           hist_lo, hist_hi, sms, err, s, status,
-                           radix_status_bytes((int64_t)rec_cap, cfg));
-    else
-      launch_expand(keys, lens, eqprev, rec_off, n, d, seq_rep, id_bits, A, rec_cap, hist, hist_lo,
-                    hist_hi, sms, err, s, sel, status, radix_status_bytes((int64_t)rec_cap, cfg));
+    launch_expand(src, rec_off, n, d, seq_rep, id_bits, A, rec_cap, hist, hist_lo, hist_hi, sms,
+                  err, s, sel, status, radix_status_bytes((int64_t)rec_cap, cfg));
   };
   if (mode == 1) {
     const bool in_passes = hist_mode == 1;
@@ -1015,8 +1013,8 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   sel.shift = id_bits;
   sel.mask = NB - 1u;
   sel.bin_count = bins;
-  launch_expand(e.keys, e.lens, e.eqprev, e.rec_off, n, d, salt_rep, id_bits, nullptr, e.n_rec,
-                nullptr, 0, 8, sms, err, s, &sel);
+  launch_expand(ExpandSource{e.keys, e.lens, e.eqprev}, e.rec_off, n, d, salt_rep, id_bits,
+                nullptr, e.n_rec, nullptr, 0, 8, sms, err, s, &sel);
   XTN_CK(cudaGetLastError());
   std::vector<uint32_t> hb(NB);
   uint32_t herr = 0;

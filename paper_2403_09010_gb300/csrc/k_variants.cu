@@ -6,11 +6,8 @@
 //              (Appendix "Compression of TCR sequences"), its length, the
 //              mask of positions equal to their left neighbour, and its
 //              number of canonical deletion subsets (see is_canonical).
-//   k_expand : one warp per sequence (metadata of 32 sequences fetched at
-//              once); lane v takes canonical variant v (see variants.cuh),
-//              fingerprints it from the prefix sums and writes the 64-bit
-//              record  fingerprint[63:b] | id[b-1:0]  at rec_off[s] + v, so
-//              every warp store is one contiguous run.  The kernel also
+//   k_expand : the records  fingerprint[63:b] | id[b-1:0]  of every canonical
+//              deletion variant, at rec_off (see expand.cuh).  The kernel also
 //              accumulates the digit histograms of the radix passes that will
 //              sort the records (all of them, or only the first when each
 //              sort pass counts the next).
@@ -18,8 +15,10 @@
 //              positions holding c (the match vectors of the bit-parallel
 //              edit distance used in verification).
 #include <algorithm>
+#include <mutex>
+#include <type_traits>
 
-#include "variants.cuh"
+#include "expand.cuh"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -96,14 +95,7 @@ __global__ void __launch_bounds__(ENCODE_WARPS * 32)
     keys[i] = key;
     lens[i] = (uint8_t)L;
     eqprev_out[i] = eqprev;
-    if (d <= 2) {  // closed form of canonical_count, the one k_expand checks against
-      const uint32_t all = L ? (0xffffffffu >> (32 - L)) : 0u;
-      const uint32_t runs = ~eqprev & all;
-      vcount[i] = canonical_total_d2(
-          SeqShape{L, (uint32_t)__popc(runs), (uint32_t)__popc(runs & (eqprev >> 1))}, d);
-    } else {
-      vcount[i] = canonical_count(eqprev, L, (uint32_t)d);
-    }
+    vcount[i] = canonical_total(eqprev, L, d);
   }
 }
 
@@ -212,243 +204,97 @@ __device__ __forceinline__ void zero_fill(uint4* __restrict__ p, uint64_t n) {
     p[k] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-template <int SEL>
-__global__ void __launch_bounds__(EXPAND_THREADS)
-    k_expand(const Key128* __restrict__ keys, const uint8_t* __restrict__ lens,
-             const uint32_t* __restrict__ eqprev, const uint64_t* __restrict__ rec_off, int64_t n,
-             int d, const uint32_t* __restrict__ seq_rep, uint32_t id_bits,
-             uint64_t* __restrict__ out, uint64_t n_rec, uint32_t* __restrict__ hist, int hist_lo,
-             int hist_passes, int hist_hi, BinSel sel, uint32_t* __restrict__ err,
-             uint4* __restrict__ zero, uint64_t n_zero) {
-  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  __shared__ VariantTables s_tab;
-  __shared__ WarpVariants s_warp[EXPAND_THREADS / 32];
-  zero_fill(zero, n_zero);
-  constexpr int STAGE_WARPS = SEL == SEL_APPEND ? EXPAND_THREADS / 32 : 1;
-  __shared__ uint64_t s_stage[STAGE_WARPS][SEL == SEL_APPEND ? STAGE_CAP : 1];
-  WarpStage st{s_stage[SEL == SEL_APPEND ? threadIdx.x >> 5 : 0], 0u};
-  const int n_hist = SEL == SEL_COUNT ? (int)sel.mask + 1 : hist_passes * RADIX;
-  for (int k = threadIdx.x; k < n_hist; k += blockDim.x) s_hist[k] = 0;
-  init_variant_tables(&s_tab);
-  __syncthreads();
-  WarpVariants* w = &s_warp[threadIdx.x >> 5];
-  const uint32_t lane = lane_id();
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const uint64_t idmask = (id_bits >= 64) ? ~0ull : ((1ull << id_bits) - 1ull);
-  const int last_bits = hist_hi - hist_lo - 8 * (hist_passes - 1);
-  const uint32_t last_mask = (1u << last_bits) - 1u;
-  // each warp takes 32 consecutive sequences per round: their metadata is
-  // read with one coalesced load per field and handed out by shuffles
-  for (int64_t s0 = warp0 * 32; s0 < n; s0 += n_warps * 32) {
-    const int64_t my = s0 + lane;
-    Key128 mk{0ull, 0ull};
-    uint32_t mL = 0, mEq = 0, mRep = 0;
-    uint64_t mBase = 0, mEnd = 0;
-    if (my < n) {
-      mk = keys[my];
-      mL = lens[my];
-      mEq = eqprev[my];
-      mBase = rec_off[my];
-      mEnd = rec_off[my + 1];
-      if (seq_rep) mRep = seq_rep[my];
-    }
-    const int m = (n - s0 < 32) ? (int)(n - s0) : 32;
-    for (int j = 0; j < m; ++j) {
-      const int64_t s = s0 + j;
-      const Key128 k{__shfl_sync(FULL_MASK, mk.lo, j), __shfl_sync(FULL_MASK, mk.hi, j)};
-      const uint32_t L = __shfl_sync(FULL_MASK, mL, j);
-      const uint32_t eq = __shfl_sync(FULL_MASK, mEq, j);
-      const uint64_t base = __shfl_sync(FULL_MASK, mBase, j);
-      uint32_t cnt = (uint32_t)(__shfl_sync(FULL_MASK, mEnd, j) - base);
-      if (SEL == SEL_ALL && base + cnt > n_rec) {
-        if (lane == 0) atomicOr(err, DERR_RANGE);
-        cnt = 0;
-      }
-      const uint64_t salt = seq_rep ? rep_salt(__shfl_sync(FULL_MASK, mRep, j)) : 0ull;
-      const SeqShape sh = warp_prepare(w, &s_tab, k, L, eq, lane);
-      if (d <= 2) {
-        uint32_t total = canonical_total_d2(sh, d);
-        if (total != cnt) {
-          if (lane == 0) atomicOr(err, DERR_RANGE);
-          total = 0;
-        }
-        for (uint32_t v0 = 0; v0 < total; v0 += 32) {
-          const uint32_t v = v0 + lane;
-          uint64_t rec = 0;
-          if (v < total)
-            rec = (canonical_fingerprint_d2(w, &s_tab, sh, v, salt) & ~idmask) | (uint64_t)s;
-          place_record<SEL>(rec, v < total, base + v, out, n_rec, s_hist, hist_lo, hist_passes,
-                            last_mask, sel, lane, st, err);
-        }
-      } else {
-        // every subset with <= d deletions, canonical ones kept (ballot compaction)
-        const uint32_t total = cnt ? variant_count(L, (uint32_t)d) : 0u;
-        uint32_t written = 0;
-        for (uint32_t v0 = 0; v0 < total; v0 += 32) {
-          const uint32_t v = v0 + lane;
-          bool keep = false;
-          Subset ss{0u, 0u, 0u, 0u};
-          if (v < total) {
-            ss = unrank_subset(L, v);
-            keep = is_canonical(subset_mask(ss), eq);
-          }
-          const uint32_t bal = __ballot_sync(FULL_MASK, keep);
-          const uint32_t slot = written + __popc(bal & lt_mask);
-          const bool ok = keep && slot < cnt;
-          uint64_t rec = 0;
-          if (ok) rec = (subset_fingerprint(w, L, ss, salt) & ~idmask) | (uint64_t)s;
-          place_record<SEL>(rec, ok, base + slot, out, n_rec, s_hist, hist_lo, hist_passes,
-                            last_mask, sel, lane, st, err);
-          written += __popc(bal);
-        }
-        if (written != cnt && lane == 0) atomicOr(err, DERR_RANGE);
-      }
-    }
-  }
-  if constexpr (SEL == SEL_APPEND) flush_stage(st, out, n_rec, sel, lane, err);
-  __syncthreads();
-  uint32_t* dst = SEL == SEL_COUNT ? sel.bin_count : hist;
-  for (int k = threadIdx.x; k < n_hist; k += blockDim.x)
-    if (s_hist[k]) atomicAdd(&dst[k], s_hist[k]);
-}
+// The expansion into records at rec_off (SEL_ALL), or of selected bins.  A
+// warp takes PACK consecutive sequences: its lanes prepare their terms
+// (expand.cuh), then the warp walks the batch's records as one stream, lane
+// by lane, each lane moving to the next sequence when its position passes
+// the current one's end.  Every lane computes a record in every round and
+// the batch's records are contiguous in the output, so stores coalesce.
+constexpr int EXPAND_WARPS = EXPAND_THREADS / 32;
 
-// Packed expansion for d <= 2.  A warp takes PACK_SEQS consecutive
-// sequences; lane i < PACK_SEQS first prepares sequence i alone (prefix sums
-// of the polynomial fingerprint, run starts, canonical variant count), then
-// the whole warp walks the batch's records as one stream: record t of the
-// batch belongs to the sequence whose start (exclusive scan of the counts) is
-// the largest <= t, found by a 4-step search over the lanes' starts.  Every
-// lane computes a record in every round and the batch's records are
-// contiguous in the output, so the stores stay coalesced; no warp-wide work
-// is spent per sequence.  16 sequences a batch keep the per-warp tables at
-// about 4 KB, so that enough warps fit on an SM to hide the arithmetic's
-// latency.
-constexpr int PACK_WARPS = 8;
-constexpr int PACK_SEQS = 16;
-constexpr int PACK_STRIDE = XTN_MAX_LEN + 3;  // P[0 .. L + 2]
-
-struct PackedSeqs {
-  uint64_t P[PACK_SEQS][PACK_STRIDE];
-  uint8_t rs[PACK_SEQS][XTN_MAX_LEN + 1];
-  uint8_t ds[PACK_SEQS][XTN_MAX_LEN / 2 + 1];
+template <int KIND, int SEL>
+struct ExpandSmem {
+  using K = VK<KIND>;
+  uint64_t terms[EXPAND_WARPS][K::PACK][K::STRIDE];
+  uint64_t stage[SEL == SEL_APPEND ? EXPAND_WARPS : 1][SEL == SEL_APPEND ? STAGE_CAP : 1];
+  uint64_t pow[K::POS + 4];
+  VarMeta meta[EXPAND_WARPS][K::PACK];
+  uint32_t hist[MAX_PASSES * RADIX];
+  uint16_t comb[K::COMBS + 1];
 };
 
-// PK_SALT: sequences carry a repertoire salt (seq_rep given); PK_HIW: the
-// histogram's digits lie in the record's high word (hist_lo >= 32).
-constexpr int PK_SALT = 1, PK_HIW = 2;
-
-template <int SEL, int PK>
-__global__ void __launch_bounds__(PACK_WARPS * 32)
-    k_expand_packed(const Key128* __restrict__ keys, const uint8_t* __restrict__ lens,
-                    const uint32_t* __restrict__ eqprev, const uint64_t* __restrict__ rec_off,
-                    int64_t n, int d, const uint32_t* __restrict__ seq_rep, uint32_t id_bits,
-                    uint64_t* __restrict__ out, uint64_t n_rec, uint32_t* __restrict__ hist,
-                    int hist_lo, int hist_passes, int hist_hi, BinSel sel,
-                    uint32_t* __restrict__ err, uint4* __restrict__ zero, uint64_t n_zero) {
+// HIW: the histogram's digits lie in the record's high word (hist_lo >= 32).
+template <int KIND, int SEL, bool HIW>
+__global__ void __launch_bounds__(EXPAND_THREADS, 4)
+    k_expand(ExpandSource src, const uint64_t* __restrict__ rec_off, int64_t n, int d,
+             const uint32_t* __restrict__ seq_rep, uint32_t id_bits, uint64_t* __restrict__ out,
+             uint64_t n_rec, uint32_t* __restrict__ hist, int hist_lo, int hist_passes,
+             int hist_hi, BinSel sel, uint32_t* __restrict__ err, uint4* __restrict__ zero,
+             uint64_t n_zero) {
+  using K = VK<KIND>;
+  extern __shared__ __align__(16) unsigned char expand_smem[];
+  ExpandSmem<KIND, SEL>& S = *reinterpret_cast<ExpandSmem<KIND, SEL>*>(expand_smem);
   zero_fill(zero, n_zero);
-  __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
-  __shared__ VariantTables s_tab;
-  __shared__ PackedSeqs s_seq[PACK_WARPS];
-  constexpr int STAGE_WARPS = SEL == SEL_APPEND ? PACK_WARPS : 1;
-  __shared__ uint64_t s_stage[STAGE_WARPS][SEL == SEL_APPEND ? STAGE_CAP : 1];
-  WarpStage st{s_stage[SEL == SEL_APPEND ? threadIdx.x >> 5 : 0], 0u};
+  const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+  WarpStage st{S.stage[SEL == SEL_APPEND ? warp : 0], 0u};
   const int n_hist = SEL == SEL_COUNT ? (int)sel.mask + 1 : hist_passes * RADIX;
-  for (int k = threadIdx.x; k < n_hist; k += blockDim.x) s_hist[k] = 0;
-  init_variant_tables(&s_tab);
+  for (int k = threadIdx.x; k < n_hist; k += blockDim.x) S.hist[k] = 0;
+  load_powers<KIND>(S.pow);
+  load_combs<KIND>(S.comb);
   __syncthreads();
-  PackedSeqs* ps = &s_seq[threadIdx.x >> 5];
-  const uint32_t lane = lane_id();
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t idmask = (id_bits >= 64) ? ~0ull : ((1ull << id_bits) - 1ull);
   const int last_bits = hist_hi - hist_lo - 8 * (hist_passes - 1);
   const uint32_t last_mask = (1u << last_bits) - 1u;
-  static_assert(PACK_SEQS <= 32 && (PACK_SEQS & (PACK_SEQS - 1)) == 0, "power of two <= 32");
-  for (int64_t s0 = warp0 * PACK_SEQS; s0 < n; s0 += n_warps * PACK_SEQS) {
-    const int64_t my = s0 + lane;
-    // ---- this lane's sequence
-    uint32_t L = 0, R = 0, nD = 0, total = 0;
-    uint64_t salt = 0, base = 0;
-    if (lane < (uint32_t)PACK_SEQS && my < n) {
-      Key128 k = keys[my];
-      L = lens[my];
-      const uint32_t eq = eqprev[my];
-      base = rec_off[my];
+  const int q = (int)lane / K::LANES;  // this lane's sequence in the batch
+  VarMeta* meta = S.meta[warp];
+  for (int64_t s0 = warp0 * K::PACK; s0 < n; s0 += n_warps * K::PACK) {
+    const int64_t my = s0 + q;
+    const bool have = my < n;
+    const uint64_t salt = have && seq_rep ? rep_salt(seq_rep[my]) : 0ull;
+    VarMeta m;
+    uint32_t total = prepare_variants<KIND>(S.terms[warp][q], S.pow, src, my, have, d, salt, lane, m);
+    const uint64_t base = have ? rec_off[my] : 0ull;
+    if (have) {
       const uint64_t cnt = rec_off[my + 1] - base;
-      if ((PK & PK_SALT) && seq_rep) salt = rep_salt(seq_rep[my]);
-      if (L > XTN_MAX_LEN) L = XTN_MAX_LEN;  // encode rejects longer ones
-      uint64_t acc = 0, pw = 1;
-      ps->P[lane][0] = 0ull;
-      for (uint32_t p = 0; p < L; ++p) {
-        acc += (uint64_t)(uint32_t)(k.lo & 31u) * pw;
-        pw *= HASH_B;
-        k.lo = (k.lo >> 5) | (k.hi << 59);
-        k.hi >>= 5;
-        ps->P[lane][p + 1] = acc;
-      }
-      for (uint32_t p = L + 1; p <= L + 2; ++p) ps->P[lane][p] = acc;
-      const uint32_t all = L ? (0xffffffffu >> (32 - L)) : 0u;
-      uint32_t runs = ~eq & all;
-      uint32_t dbl = runs & (eq >> 1);
-      R = __popc(runs);
-      nD = __popc(dbl);
-      for (uint32_t i = 0; runs; ++i, runs &= runs - 1) ps->rs[lane][i] = (uint8_t)(__ffs(runs) - 1);
-      for (uint32_t i = 0; dbl; ++i, dbl &= dbl - 1) ps->ds[lane][i] = (uint8_t)(__ffs(dbl) - 1);
-      total = canonical_total_d2(SeqShape{L, R, nD}, d);
       if (total != cnt || (SEL == SEL_ALL && base + cnt > n_rec)) {
         atomicOr(err, DERR_RANGE);
         total = 0;
       }
     }
-    // ---- the batch's records, 32 at a time
-    uint32_t start = total;  // exclusive scan of the totals over lanes
+    // where each sequence of the batch ends in the stream
+    uint32_t end = total;
 #pragma unroll
-    for (int o = 1; o < PACK_SEQS; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(FULL_MASK, start, o);
-      if (lane >= (uint32_t)o) start += t;
+    for (int o = K::LANES; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL_MASK, end, o);
+      if (lane >= (uint32_t)o) end += t;
     }
-    const uint32_t T = __shfl_sync(FULL_MASK, start, PACK_SEQS - 1);
-    start -= total;
+    const uint32_t T = __shfl_sync(FULL_MASK, end, 31);
     const uint64_t base0 = __shfl_sync(FULL_MASK, base, 0);
-    __syncwarp();  // the tables written above are read by every lane below
+    if (lane % K::LANES == 0) {
+      m.end = (int32_t)end;
+      m.adj += (int32_t)(end - total);
+      meta[q] = m;
+    }
+    __syncwarp();  // terms and meta, written above, are read by every lane
+    int j = 0;
+    VarMeta cur = meta[0];
+    const uint64_t* tab = S.terms[warp][0];
     for (uint32_t t0 = 0; t0 < T; t0 += 32) {
       const uint32_t t = t0 + lane;
-      // largest j with start[j] <= t (starts do not decrease)
-      uint32_t j = 0;
-#pragma unroll
-      for (int step = PACK_SEQS / 2; step > 0; step >>= 1) {
-        const uint32_t sj = __shfl_sync(FULL_MASK, start, (int)(j + step));
-        if (sj <= t) j += step;
-      }
-      const uint32_t sj = __shfl_sync(FULL_MASK, start, (int)j);
-      const uint32_t Lj = __shfl_sync(FULL_MASK, L, (int)j);
-      const uint32_t Rj = __shfl_sync(FULL_MASK, R, (int)j);
-      const uint32_t Dj = __shfl_sync(FULL_MASK, nD, (int)j);
-      const uint64_t saltj = (PK & PK_SALT) ? __shfl_sync(FULL_MASK, salt, (int)j) : 0ull;
       uint64_t rec = 0;
       if (t < T) {
-        const uint32_t v = t - sj;
-        // canonical variant v of sequence j (numbering of canonical_fingerprint_d2)
-        const uint32_t u = v - 1 - Rj;
-        const uint32_t c2 = Rj * (Rj - 1) / 2;
-        const bool single = v >= 1 && v <= Rj;
-        const bool pair = v > Rj && u < c2;
-        const bool dbl = v > Rj && u >= c2;
-        const uint32_t pr = s_tab.pair[pair ? u : 0u];
-        const uint32_t a = ps->rs[j][single ? v - 1 : (pr & 255u)];
-        const uint32_t b = ps->rs[j][pr >> 8];
-        const uint32_t c = ps->ds[j][dbl ? u - c2 : 0u];
-        const uint32_t p1 = single || pair ? a : (dbl ? c : Lj);
-        const uint32_t p2 = pair ? b : (dbl ? c + 1 : (single ? Lj : Lj + 1));
-        auto P = [&](uint32_t x) { return ps->P[j][x]; };
-        const uint64_t h = P(p1) + HASH_BINV * ((P(p2) - P(p1 + 1)) +
-                                                HASH_BINV * (P(Lj) - P(p2 + 1)));
-        rec = (mix64((PK & PK_SALT) ? h ^ saltj : h) & ~idmask) | (uint64_t)(s0 + j);
+        while ((int32_t)t >= cur.end) {  // ends: t < T, the last sequence's end
+          cur = meta[++j];
+          tab += K::STRIDE;
+        }
+        const uint64_t h = variant_sum<KIND>(tab, S.comb, (uint32_t)((int32_t)t - cur.adj), cur.c,
+                                             cur.aux);
+        rec = (mix64(h) & ~idmask) | (uint64_t)(s0 + j);
       }
-      place_record<SEL, (PK & PK_HIW) != 0>(rec, t < T, base0 + t, out, n_rec, s_hist, hist_lo,
-                                            hist_passes, last_mask, sel, lane, st, err);
+      place_record<SEL, HIW>(rec, t < T, base0 + t, out, n_rec, S.hist, hist_lo, hist_passes,
+                             last_mask, sel, lane, st, err);
     }
     __syncwarp();  // the next batch overwrites the tables
   }
@@ -456,7 +302,7 @@ __global__ void __launch_bounds__(PACK_WARPS * 32)
   __syncthreads();
   uint32_t* dst = SEL == SEL_COUNT ? sel.bin_count : hist;
   for (int k = threadIdx.x; k < n_hist; k += blockDim.x)
-    if (s_hist[k]) atomicAdd(&dst[k], s_hist[k]);
+    if (S.hist[k]) atomicAdd(&dst[k], S.hist[k]);
 }
 
 // Match vectors: peq[i * PEQ_STRIDE + c - 1] = {positions p of sequence i with code c}.
@@ -519,57 +365,58 @@ void launch_encode(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Ke
   prof_end(s);
 }
 
-template <int SEL>
-static void expand_launch(const Key128* keys, const uint8_t* lens, const uint32_t* eqprev,
-                          const uint64_t* rec_off, int64_t n, int d, const uint32_t* seq_rep,
-                          uint32_t id_bits, uint64_t* out, uint64_t n_rec, uint32_t* hist,
-                          int hist_lo, int passes, int hist_hi, const BinSel& sel, int sms,
+template <int KIND, int SEL, bool HIW>
+static void expand_launch(const ExpandSource& src, const uint64_t* rec_off, int64_t n, int d,
+                          const uint32_t* seq_rep, uint32_t id_bits, uint64_t* out, uint64_t n_rec,
+                          uint32_t* hist, int hist_lo, int hist_hi, const BinSel& sel, int sms,
                           uint32_t* err, cudaStream_t s, uint4* zero, uint64_t n_zero) {
-  if (d <= 2) {
-    const int pblocks = (int)std::min<int64_t>(
-        (n + PACK_WARPS * PACK_SEQS - 1) / (PACK_WARPS * PACK_SEQS), (int64_t)sms * 8);
-    // the plain expansion picks its variant; the bin passes take the general one
-    auto f = k_expand_packed<SEL, PK_SALT>;
-    if (SEL == SEL_ALL) {
-      const bool hiw = hist_lo >= 32 && hist_hi <= 64;
-      f = seq_rep ? (hiw ? k_expand_packed<SEL, PK_SALT | PK_HIW> : k_expand_packed<SEL, PK_SALT>)
-                  : (hiw ? k_expand_packed<SEL, PK_HIW> : k_expand_packed<SEL, 0>);
-    }
-    f<<<pblocks > 0 ? pblocks : 1, PACK_WARPS * 32, 0, s>>>(keys, lens, eqprev, rec_off, n, d,
-                                                              seq_rep, id_bits, out, n_rec, hist,
-                                                              hist_lo, passes, hist_hi, sel, err,
-                                                              zero, n_zero);
-  } else {
-    int blocks = (int)std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
-    if (blocks < 1) blocks = 1;
-    k_expand<SEL><<<blocks, EXPAND_THREADS, 0, s>>>(keys, lens, eqprev, rec_off, n, d, seq_rep,
-                                                    id_bits, out, n_rec, hist, hist_lo, passes,
-                                                    hist_hi, sel, err, zero, n_zero);
-  }
+  auto f = k_expand<KIND, SEL, HIW>;
+  constexpr int smem = (int)sizeof(ExpandSmem<KIND, SEL>);
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  });
+  const int per_block = EXPAND_WARPS * VK<KIND>::PACK;
+  const int64_t blocks = std::min<int64_t>((n + per_block - 1) / per_block, (int64_t)sms * 8);
+  f<<<(uint32_t)blocks, EXPAND_THREADS, smem, s>>>(src, rec_off, n, d, seq_rep, id_bits, out,
+                                                   n_rec, hist, hist_lo, (hist_hi - hist_lo + 7) / 8,
+                                                   hist_hi, sel, err, zero, n_zero);
 }
 
-void launch_expand(const Key128* keys, const uint8_t* lens, const uint32_t* eqprev,
-                   const uint64_t* rec_off, int64_t n, int d, const uint32_t* seq_rep,
-                   uint32_t id_bits, uint64_t* out, uint64_t n_rec, uint32_t* hist, int hist_lo,
-                   int hist_hi, int sms, uint32_t* err, cudaStream_t s, const BinSel* sel,
-                   void* zero, size_t zero_bytes) {
+void launch_expand(const ExpandSource& src, const uint64_t* rec_off, int64_t n, int d,
+                   const uint32_t* seq_rep, uint32_t id_bits, uint64_t* out, uint64_t n_rec,
+                   uint32_t* hist, int hist_lo, int hist_hi, int sms, uint32_t* err,
+                   cudaStream_t s, const BinSel* sel, void* zero, size_t zero_bytes) {
   uint4* z = static_cast<uint4*>(zero);
   const uint64_t nz = z ? zero_bytes / 16 : 0;
   if (n <= 0) return;
-  const int passes = (hist_hi - hist_lo + 7) / 8;
   const BinSel none{};
-  if (!sel) {
-    prof_begin(s, "k_expand", (double)n_rec * 8.0 + (double)n * 29.0);
-    expand_launch<SEL_ALL>(keys, lens, eqprev, rec_off, n, d, seq_rep, id_bits, out, n_rec, hist,
-                           hist_lo, passes, hist_hi, none, sms, err, s, z, nz);
-  } else if (sel->append) {
-    prof_begin(s, "k_expand_bins", (double)n_rec * 8.0 + (double)n * 29.0);
-    expand_launch<SEL_APPEND>(keys, lens, eqprev, rec_off, n, d, seq_rep, id_bits, out, n_rec,
-                              hist, hist_lo, passes, hist_hi, *sel, sms, err, s, z, nz);
+  const bool paired = src.keys_b != nullptr;
+  const bool hiw = hist_lo >= 32 && hist_hi <= 64;
+  auto go = [&](auto kind) {
+    constexpr int KIND = decltype(kind)::value;
+    auto f = hiw ? expand_launch<KIND, SEL_ALL, true> : expand_launch<KIND, SEL_ALL, false>;
+    if constexpr (!VK<KIND>::PAIRED)  // the bin passes take the general digit count
+      if (sel)
+        f = sel->append ? expand_launch<KIND, SEL_APPEND, false>
+                        : expand_launch<KIND, SEL_COUNT, false>;
+    f(src, rec_off, n, d, seq_rep, id_bits, out, n_rec, hist, hist_lo, hist_hi, sel ? *sel : none,
+      sms, err, s, z, nz);
+  };
+  const char* name = paired ? "k_expand_paired"
+                     : !sel ? "k_expand" : sel->append ? "k_expand_bins" : "k_expand_count";
+  prof_begin(s, name, (sel && !sel->append ? 0.0 : (double)n_rec * 8.0) +
+                          (double)n * (paired ? 58.0 : 29.0));
+  if (paired) {
+    if (d <= 1) go(std::integral_constant<int, VK_PAIRED_D1>{});
+    else go(std::integral_constant<int, VK_PAIRED_D2>{});
+  } else if (d <= 1) {
+    go(std::integral_constant<int, VK_D1>{});
+  } else if (d == 2) {
+    go(std::integral_constant<int, VK_D2>{});
   } else {
-    prof_begin(s, "k_expand_count", (double)n * 29.0);
-    expand_launch<SEL_COUNT>(keys, lens, eqprev, rec_off, n, d, seq_rep, id_bits, out, n_rec,
-                             hist, hist_lo, passes, hist_hi, *sel, sms, err, s, z, nz);
+    go(std::integral_constant<int, VK_D3>{});
   }
   prof_end(s);
 }

@@ -39,14 +39,17 @@ struct BinSel {
 };
 constexpr int MAX_BIN_BITS = 11;
 
-// sel null: every record of sequence i goes to out[rec_off[i] ...].
+// The sequences (or paired receptors, when src.keys_b is set: d <= 2, no bin
+// selection) expanded into records.  sel null: every record of sequence i
+// goes to out[rec_off[i] ...].
 // zero: when not null, zero_bytes (a multiple of 16, 16-byte aligned) are
 // cleared there as well (the record sort's look-back status).
-void launch_expand(const Key128* keys, const uint8_t* lens, const uint32_t* eqprev,
-                   const uint64_t* rec_off, int64_t n, int d, const uint32_t* seq_rep,
-                   uint32_t id_bits, uint64_t* out, uint64_t n_rec, uint32_t* hist, int hist_lo,
-                   int hist_hi, int sms, uint32_t* err, cudaStream_t s,
-                   const BinSel* sel = nullptr, void* zero = nullptr, size_t zero_bytes = 0);
+struct ExpandSource;
+void launch_expand(const ExpandSource& src, const uint64_t* rec_off, int64_t n, int d,
+                   const uint32_t* seq_rep, uint32_t id_bits, uint64_t* out, uint64_t n_rec,
+                   uint32_t* hist, int hist_lo, int hist_hi, int sms, uint32_t* err,
+                   cudaStream_t s, const BinSel* sel = nullptr, void* zero = nullptr,
+                   size_t zero_bytes = 0);
 void launch_peq(const Key128* keys, const uint8_t* lens, int64_t n, uint32_t* peq,
                 cudaStream_t s);
 void launch_seq_rep(const int64_t* rep_off, int64_t n_rep, uint32_t* seq_rep, int64_t n,
@@ -200,19 +203,11 @@ void launch_tcrdist_filter(const xtn_triple* in, int64_t n, const Key128* keys,
                            uint64_t* status, uint32_t* err, uint64_t* total, cudaStream_t s);
 
 // k_paired.cu --------------------------------------------------------------
-// Canonical deletion variants (d <= 2) of receptors alpha + token + beta,
-// the token never deleted: counts per receptor, and the expansion into
-// records fingerprint | receptor id at rec_off (digit histograms of the sort
-// passes over bits [hist_lo, hist_hi) on the way).
+// Canonical deletion variants (d <= 2) per receptor alpha + token + beta, the
+// token never deleted.
 void launch_paired_counts(const uint8_t* lens_a, const uint32_t* eq_a, const uint8_t* lens_b,
                           const uint32_t* eq_b, int64_t n, int d, uint32_t* vcount,
                           cudaStream_t s);
-void launch_expand_paired(const Key128* keys_a, const uint8_t* lens_a, const uint32_t* eq_a,
-                          const Key128* keys_b, const uint8_t* lens_b, const uint32_t* eq_b,
-                          const uint64_t* rec_off, int64_t n, int d, uint32_t id_bits,
-                          uint64_t* out, uint64_t n_rec, uint32_t* hist, int hist_lo, int hist_hi,
-                          int sms, uint32_t* err, cudaStream_t s, void* zero = nullptr,
-                          size_t zero_bytes = 0);
 
 // k_query.cu ---------------------------------------------------------------
 // Directory of the sorted index (entry t = first record whose top dir_bits
