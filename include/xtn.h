@@ -356,8 +356,9 @@ XTN_API int xtn_tcrdist_filter_noalloc(const uint8_t* seqs, const int64_t* offse
 /*
  * Tuning knobs (process-wide, take effect for calls that start afterwards).
  *   XTN_TUNE_SORT_RECORDS : tile configuration of the radix sort of variant
- *                           records (0 .. xtn_tune_count(knob)-1): 0-19 rank
- *                           keys stably with ranks held in registers (the
+ *                           records, where they are sorted (an index, grouping
+ *                           modes 1 and 2; 0 .. xtn_tune_count(knob)-1): 0-19
+ *                           rank keys stably with ranks held in registers (the
  *                           first pass of a sort unstably); 20 and up count
  *                           and place keys with shared-memory atomics by
  *                           digit and run of already-sorted bits (default 22)
@@ -367,17 +368,15 @@ XTN_API int xtn_tcrdist_filter_noalloc(const uint8_t* seqs, const int64_t* offse
  *                           taken: 0 = the expand kernel counts the digits
  *                           of every pass, 1 = expand counts the first pass
  *                           and each sort pass counts the next
- *   XTN_TUNE_GROUPING     : how records are grouped: 0 = global radix passes
- *                           on the top bits only, then one shared-memory pass
- *                           per block of buckets that finishes the sort and
- *                           writes the group flags (default); 1 = global
- *                           passes on every bit, then a flag pass; 2 = as 0
- *                           with 512-record shared-memory segments (slower;
- *                           more buckets take the large-bucket path)
- *   XTN_TUNE_FILTER_SEGMENT : grouping mode 0 groups each block of buckets
- *                           with a singleton filter first; its blocks hold
- *                           2^value times the buckets of the shared-memory
- *                           pass (0..3)
+ *   XTN_TUNE_GROUPING     : how a search groups its records: 0 = expanded into
+ *                           fingerprint partitions, whose repeated keys a
+ *                           filter finds in shared memory (default); 1 =
+ *                           global radix passes on every bit, then a flag
+ *                           pass; 2 = global radix passes on the top bits,
+ *                           then one shared-memory pass per block of buckets
+ *                           (512-record segments)
+ *   XTN_TUNE_FILTER_SEGMENT : grouping mode 0 makes its partitions 2^(value-1)
+ *                           times as large as by default (0..3, default 1)
  * Every value gives the same result; they differ in threads per block, keys
  * per thread, ranking method and counting, hence in speed per GPU and size.
  * xtn_tune_set returns XTN_ERR_INVALID_ARG for an unknown knob or value.

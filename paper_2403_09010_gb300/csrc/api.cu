@@ -448,13 +448,14 @@ std::atomic<int> g_cfg_pairs{21};
 // counts every pass's digit, 1 = expand counts the first and each sort pass
 // counts the next one.
 std::atomic<int> g_record_hist{0};
-// How records are grouped: 0 = global radix passes on the top bucket bits,
-// then k_bucket_sort (shared-memory finish + group flags); 1 = global passes
-// on every group-key bit, then k_group_flags; 2 = as 0 with 512-record
-// shared-memory segments (more buckets take the large-bucket path).
+// How a self-search groups its records: 0 = scattered into fingerprint
+// partitions by the expansion, then k_group_filter; 1 = global radix passes
+// on every group-key bit, then k_group_flags; 2 = global passes on the top
+// bucket bits, then k_bucket with 512-record shared-memory segments.  An
+// index always takes global passes on the top bits, then k_bucket's sort.
 std::atomic<int> g_grouping{0};
 }  // namespace
-// Buckets per block of the singleton filter: 2^fx of k_bucket's blocks.
+// Records per partition: 2^fx times the smallest (choose_partitions).
 std::atomic<int> g_filter_fx{1};
 std::atomic<int>& cfg_records() { return g_cfg_records; }
 std::atomic<int>& cfg_pairs() { return g_cfg_pairs; }
@@ -545,6 +546,7 @@ struct Encoded {
   Key128* keys_b = nullptr;
   uint8_t* lens_b = nullptr;
   uint32_t* eq_b = nullptr;
+  ExpandSource source() const { return ExpandSource{keys, lens, eqprev, keys_b, lens_b, eq_b}; }
 };
 
 // allow_large: return the count even when it is 2^32 or more (the caller
@@ -640,15 +642,7 @@ struct GroupScratch {
   uint64_t* cand = nullptr;
   uint64_t cand_cap = 0;
   uint64_t* cand_count = nullptr;
-  // with cand (grouping mode 0): seg_area_bytes() for the singleton filter's
-  // segment counter (first 16 bytes) and one flag byte per block of buckets
-  uint8_t* seg_area = nullptr;
 };
-
-size_t seg_area_bytes(uint64_t rec_cap, int hs) {
-  const GroupingShape g = choose_grouping(rec_cap, hs, true);
-  return 16 + 4 * (((size_t)1 << g.G) >> g.kbits);
-}
 
 size_t bucket_start_words(uint64_t rec_cap, int hs, int mode) {
   if (mode == 1) return 1;
@@ -677,9 +671,7 @@ int expand_sort_launch(const Key128* keys, const uint8_t* lens, const uint32_t* 
   // the expansion: one chain, or paired receptors (no bin selection); it
   // also clears the record sort's status area
   const bool zeroed = true;
-  ExpandSource src{keys, lens, eqprev};
-  if (paired) src = ExpandSource{paired->keys, paired->lens, paired->eqprev,
-                                 paired->keys_b, paired->lens_b, paired->eq_b};
+  const ExpandSource src = paired ? paired->source() : ExpandSource{keys, lens, eqprev};
   auto expand = [&](int hist_lo, int hist_hi) {
     launch_expand(src, rec_off, n, d, seq_rep, id_bits, A, rec_cap, hist, hist_lo, hist_hi, sms,
                   err, s, sel, status, radix_status_bytes((int64_t)rec_cap, cfg));
@@ -716,23 +708,9 @@ int expand_sort_launch(const Key128* keys, const uint8_t* lens, const uint32_t* 
     XTN_CK(cudaMemsetAsync(gs.gstatus, 0, group_status_bytes((int64_t)rec_cap), s));
     tile_counts = group_tile_counts(gs.gstatus, (int64_t)rec_cap);
   }
-  if (hash && gs.cand && gs.seg_area && mode == 0) {
-    // the singleton filter groups and emits nearly every block of buckets;
-    // k_bucket takes only the blocks it lists
-    uint32_t* seg_count = reinterpret_cast<uint32_t*>(gs.seg_area);
-    uint32_t* seg_list = reinterpret_cast<uint32_t*>(gs.seg_area + 16);
-    XTN_CK(cudaMemsetAsync(seg_count, 0, 16, s));
-    launch_bucket_filter(X, (int64_t)rec_cap, n_rec_dev, gs.bucket_start, g,
-                         g_filter_fx.load(), lo, gs.cand, gs.cand_cap, gs.cand_count, id_bits,
-                         seg_list, seg_count, err, s);
-    launch_bucket(hash, X, Y, (int64_t)rec_cap, n_rec_dev, gs.bucket_start, g, lo, 0, gs.flags,
-                  tile_counts, gs.cand, gs.cand_cap, gs.cand_count, id_bits, err, s, seg_list,
-                  seg_count, sms);
-  } else {
-    launch_bucket(hash, X, Y, (int64_t)rec_cap, n_rec_dev, gs.bucket_start, g, lo,
-                  mode == 2 ? 512 : 0, gs.flags, tile_counts, hash ? gs.cand : nullptr,
-                  gs.cand_cap, gs.cand_count, id_bits, err, s);
-  }
+  launch_bucket(hash, X, Y, (int64_t)rec_cap, n_rec_dev, gs.bucket_start, g, lo,
+                mode == 2 ? 512 : 0, gs.flags, tile_counts, hash ? gs.cand : nullptr, gs.cand_cap,
+                gs.cand_count, id_bits, err, s);
   XTN_CK(cudaGetLastError());
   *sorted = Y;
   return XTN_OK;
@@ -760,7 +738,6 @@ int expand_and_sort(const Encoded& e, int64_t n, int d, const uint32_t* seq_rep,
     gs.cand = direct->cand;
     gs.cand_cap = direct->cand_cap;
     gs.cand_count = direct->cand_count;
-    if (mode == 0) gs.seg_area = ar.get<uint8_t>(seg_area_bytes(n_rec, out->hs));
   }
   gs.bucket_start = ar.get<uint64_t>(bucket_start_words(n_rec, out->hs, mode));
   if (want_flags) {
@@ -779,6 +756,57 @@ int expand_and_sort(const Encoded& e, int64_t n, int d, const uint32_t* seq_rep,
   out->gstatus = gs.gstatus;
   out->rec = sorted;
   out->spare = sorted == A ? B : A;
+  return XTN_OK;
+}
+
+// Partition buffers for n_rec records, the counters cleared (*n_spill is
+// the caller's to clear).  `rec` also serves as the second buffer of the
+// spill's sort.
+int take_partitions(uint64_t n_rec, Arena& ar, uint64_t* n_spill, cudaStream_t s, Partitions* p) {
+  static_cast<PartitionShape&>(*p) = choose_partitions(n_rec, g_filter_fx.load());
+  p->rec = ar.get<uint64_t>(std::max(p->words(), n_rec) + 8);
+  p->kept = ar.get<uint64_t>(p->words() + 8);
+  p->count = ar.get<uint32_t>(p->counts());
+  p->spill = ar.get<uint64_t>(n_rec + 8);
+  p->spill_cap = n_rec;
+  p->n_spill = n_spill;
+  XTN_ALLOC_OK(ar);
+  XTN_CK(cudaMemsetAsync(p->count, 0, p->counts() * 4, s));
+  return XTN_OK;
+}
+
+// Records up to this many are expanded in sequence order and then parted in a
+// pass of their own, so that the profile of a small search still times the
+// two stages apart (k_expand, k_onesweep_records); more are expanded straight
+// into their partitions.  Below it that would make little difference: 10,000
+// sequences 221 against 221 us a search at d = 1, 50,000 at d = 2 (5.2 M
+// records) 297 against 282 us; above, 200,000 sequences 229 against 162 us
+// for the two stages.
+constexpr uint64_t SPLIT_EXPANSION = 6u << 20;
+
+// The n spilled records sorted on their hs group-key bits, with group flags.
+int sort_spill(const Partitions& p, uint64_t n, uint32_t id_bits, int hs, int sms, Arena& ar,
+               uint32_t* err, cudaStream_t s, Sorted* out) {
+  const int lo = 64 - hs;
+  const int cfg = g_cfg_records.load();
+  const uint64_t g_cap = n / 2 + 1;
+  uint32_t* hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
+  uint64_t* digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
+  uint64_t* status = ar.get<uint64_t>(radix_status_bytes((int64_t)n, cfg) / 8 + 1);
+  const size_t gst = std::max(group_status_bytes((int64_t)n), scan_status_bytes((int64_t)g_cap));
+  out->flags = ar.get<uint64_t>(group_flag_words((int64_t)n));
+  out->gstatus = ar.get<uint64_t>(gst / 8 + 1);
+  XTN_ALLOC_OK(ar);
+  XTN_CK(cudaMemsetAsync(hist, 0, MAX_PASSES * RADIX * 4, s));
+  launch_histogram(p.spill, (int64_t)n, nullptr, lo, 64, hist, sms, s);
+  XTN_CK(radix_sort_passes(p.spill, p.rec, (int64_t)n, lo, 64, hist, digit_base, status, cfg, err,
+                           &out->rec, "k_onesweep_records", s, false, nullptr, nullptr,
+                           onesweep_unstable_config(cfg)));
+  out->spare = out->rec == p.spill ? p.rec : p.spill;
+  XTN_CK(cudaMemsetAsync(out->gstatus, 0, gst, s));
+  launch_group_flags(out->rec, (int64_t)n, nullptr, lo, out->flags, out->gstatus, s);
+  out->id_bits = id_bits;
+  out->hs = hs;
   return XTN_OK;
 }
 
@@ -1048,19 +1076,20 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   const int cfg = g_cfg_records.load();
   const int cfg_pairs = g_cfg_pairs.load();
   const int mode0 = g_grouping.load();
-  const uint64_t g_cap = P / 2 + 1;
-  uint64_t* A = ar.get<uint64_t>(P + 8);
-  uint64_t* B = ar.get<uint64_t>(P + 8);
+  uint64_t* digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
   uint32_t* hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
   uint32_t* phist = ar.get<uint32_t>(MAX_PASSES * RADIX);  // survivors, over all passes
-  uint64_t* digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
+  Partitions part0;
+  XTN_RC(take_partitions(P, ar, ctr + 3, s, &part0));
+  uint64_t* rec0 = ar.get<uint64_t>(P + 8);
+  uint64_t* A = part0.rec;  // the buffers of a pass grouped by sorting
+  uint64_t* B = part0.spill;
   uint64_t* status = ar.get<uint64_t>(radix_status_bytes(P, cfg) / 8 + 1);
+  const size_t gst = std::max(group_status_bytes((int64_t)P), scan_status_bytes(P / 2 + 1));
   GroupScratch gs0;
-  gs0.bucket_start = ar.get<uint64_t>(bucket_start_words(P, hs, 0));
-  gs0.seg_area = ar.get<uint8_t>(seg_area_bytes(P, hs));
+  gs0.bucket_start = ar.get<uint64_t>(bucket_start_words(P, hs, mode0 == 2 ? 2 : 1));
   gs0.flags = ar.get<uint64_t>(group_flag_words((int64_t)P));
-  gs0.gstatus = ar.get<uint64_t>(
-      std::max(group_status_bytes((int64_t)P), scan_status_bytes((int64_t)g_cap)) / 8 + 1);
+  gs0.gstatus = ar.get<uint64_t>(gst / 8 + 1);
   uint32_t* peq = ar.get<uint32_t>((size_t)n * PEQ_STRIDE);
   XTN_ALLOC_OK(ar);
   GrowBuf cand(s), surv(s);
@@ -1085,16 +1114,31 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
       sel.hi = w.second;
       sel.bin_count = nullptr;
       sel.append = reinterpret_cast<unsigned long long*>(ctr + 4);
-      GroupScratch gs = gs0;
-      if (mode != 1) {
-        gs.cand = cand.p;
-        gs.cand_cap = cand.cap;
-        gs.cand_count = ctr + 2;
-      }
       uint64_t* sorted = nullptr;
-      XTN_CK(expand_sort_launch(e.keys, e.lens, e.eqprev, e.rec_off, n, d, salt_rep, id_bits, A,
-                                B, np, lo, hist, digit_base, status, cfg, g_record_hist.load(),
-                                mode, gs, sms, err, s, nullptr, &sorted, &sel));
+      uint64_t* spare = nullptr;
+      if (mode == 0) {
+        Partitions part = part0;  // sized for the largest pass
+        const PartitionShape g = choose_partitions(np, g_filter_fx.load());
+        if (g.words() <= part0.words() && g.counts() <= part0.counts())
+          static_cast<PartitionShape&>(part) = g;
+        XTN_CK(cudaMemsetAsync(part.count, 0, part.counts() * 4, s));
+        launch_expand(e.source(), e.rec_off, n, d, salt_rep, id_bits, rec0, np, nullptr, 0, 0, sms,
+                      err, s, &sel);
+        launch_partition(rec0, (int64_t)np, ctr + 4, part, sms, err, s);
+        launch_group_filter(part, np, cand.p, cand.cap, ctr + 2, (int)id_bits, err, s);
+        XTN_CK(cudaGetLastError());
+      } else {
+        GroupScratch gs = gs0;
+        if (mode != 1) {
+          gs.cand = cand.p;
+          gs.cand_cap = cand.cap;
+          gs.cand_count = ctr + 2;
+        }
+        XTN_CK(expand_sort_launch(e.keys, e.lens, e.eqprev, e.rec_off, n, d, salt_rep, id_bits, A,
+                                  B, np, lo, hist, digit_base, status, cfg, g_record_hist.load(),
+                                  mode, gs, sms, err, s, nullptr, &sorted, &sel));
+        spare = sorted == A ? B : A;
+      }
       struct {
         uint64_t direct, large, appended, survivors;
         uint64_t groups, pairs;
@@ -1110,12 +1154,24 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
       }
       if (h.err) return map_device_err(h.err);
       if (h.appended != np) return XTN_ERR_CUDA;  // the two expansions disagree
-      uint32_t* S = reinterpret_cast<uint32_t*>(sorted == A ? B : A);
+      const uint64_t n_flagged = mode == 1 || h.large ? (mode == 0 ? h.large : np) : 0;
+      uint64_t* flags = gs0.flags;
+      uint64_t* gstatus = gs0.gstatus;
+      if (mode == 0 && n_flagged) {
+        Sorted so;
+        XTN_RC(sort_spill(part0, n_flagged, id_bits, hs, sms, ar, err, s, &so));
+        sorted = so.rec;
+        spare = so.spare;
+        flags = so.flags;
+        gstatus = so.gstatus;
+      }
+      const uint64_t g_cap = n_flagged / 2 + 1;
+      uint32_t* S = reinterpret_cast<uint32_t*>(spare);
       uint32_t* E = S + g_cap;
       uint64_t* pair_off = reinterpret_cast<uint64_t*>(E + g_cap);
-      if (mode == 1 || h.large > 0) {
-        launch_group_finish(gs.flags, (int64_t)np, nullptr, S, E, g_cap, gs.gstatus, err, ctr, s);
-        launch_scan_group_pairs(S, E, (int64_t)g_cap, ctr, pair_off, gs.gstatus, err, s);
+      if (n_flagged) {
+        launch_group_finish(flags, (int64_t)n_flagged, nullptr, S, E, g_cap, gstatus, err, ctr, s);
+        launch_scan_group_pairs(S, E, (int64_t)g_cap, ctr, pair_off, gstatus, err, s);
         k_pair_total<<<1, 1, 0, s>>>(pair_off, ctr, ctr + 1);
         XTN_CK(cudaGetLastError());
         XTN_CK(cudaMemcpyAsync(&h.groups, ctr, 16, cudaMemcpyDeviceToHost, s));
@@ -1138,8 +1194,8 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
         break;
       }
       if (h.pairs)
-        launch_emit_pairs(sorted, np, S, pair_off, (int64_t)h.groups, nullptr, h.pairs, id_bits,
-                          cand.p + h.direct, nullptr, nullptr, sms, err, s);
+        launch_emit_pairs(sorted, n_flagged, S, pair_off, (int64_t)h.groups, nullptr, h.pairs,
+                          id_bits, cand.p + h.direct, nullptr, nullptr, sms, err, s);
       if (n_pairs)
         launch_verify_candidates(cand.p, n_pairs, nullptr, id_bits, peq, e.lens, (uint64_t)n,
                                  e.keys, e.lens, (uint64_t)n, seq_rep, between ? 2 : 1, d, metric,
@@ -1242,11 +1298,10 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   }
   if (rc) return rc;
   Sorted so;
-  const uint64_t g_cap = e.n_rec / 2 + 1;
   if (mode < 0) mode = g_grouping.load();
-  // Bucket modes emit the candidates of every bucket that fits shared memory
-  // during grouping, into a buffer sized by a guess; past it, the search runs
-  // again with all-global grouping, which sizes its buffers exactly.
+  // Modes 0 and 2 write the candidates they find in shared memory at once,
+  // into a buffer sized by a guess; past it, the search runs again with
+  // all-global grouping, which sizes its buffers exactly.
   GroupScratch direct;
   if (mode != 1) {
     direct.cand_cap = std::max<uint64_t>(e.n_rec / 2, 1u << 20);
@@ -1254,17 +1309,33 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     direct.cand_count = counters + 2;
     XTN_ALLOC_OK(ar);
   }
-  rc = expand_and_sort(e, n, d, between ? nullptr : seq_rep, sms, ar, err, s, &so, true, g_cap,
-                       mode, mode != 1 ? &direct : nullptr);
-  if (rc) return rc;
-  uint32_t* S = reinterpret_cast<uint32_t*>(so.spare);  // groups live in the spare buffer
-  uint32_t* E = S + g_cap;
-  uint64_t* pair_off = reinterpret_cast<uint64_t*>(E + g_cap);  // 8-byte aligned
+  Partitions part;
+  const uint32_t* salt_rep = between ? nullptr : seq_rep;
+  so.id_bits = bits_for((uint64_t)n);
+  if (mode == 0) {
+    XTN_RC(take_partitions(e.n_rec, ar, counters + 3, s, &part));
+    if (e.n_rec <= SPLIT_EXPANSION) {
+      uint64_t* rec = ar.get<uint64_t>(e.n_rec + 8);
+      XTN_ALLOC_OK(ar);
+      launch_expand(e.source(), e.rec_off, n, d, salt_rep, so.id_bits, rec, e.n_rec, nullptr, 0, 0,
+                    sms, err, s);
+      launch_partition(rec, (int64_t)e.n_rec, nullptr, part, sms, err, s);
+    } else {
+      launch_expand_scatter(e.source(), e.rec_off, n, d, salt_rep, so.id_bits, e.n_rec, part, sms,
+                            err, s);
+    }
+    launch_group_filter(part, e.n_rec, direct.cand, direct.cand_cap, direct.cand_count,
+                        (int)so.id_bits, err, s);
+    XTN_CK(cudaGetLastError());
+  } else {
+    XTN_RC(expand_and_sort(e, n, d, salt_rep, sms, ar, err, s, &so, true, e.n_rec / 2 + 1, mode,
+                           mode != 1 ? &direct : nullptr));
+  }
   struct {
     uint64_t groups, pairs, direct, large;
     uint32_t err;
   } h{0, 0, 0, 0, 0};
-  bool flagged = mode == 1;  // groups to emit through flags and S/E
+  uint64_t n_flagged = mode == 1 ? e.n_rec : 0;  // records whose groups are emitted from flags
   if (mode != 1) {
     ReadBack rb(s);
     XTN_RC(rb.add(&h.direct, counters + 2));
@@ -1277,10 +1348,17 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
                               metric, between, b_seqs, b_offsets);
     }
     if (h.err) return map_device_err(h.err);
-    flagged = h.large > 0;
+    if (h.large) n_flagged = mode == 0 ? h.large : e.n_rec;
+    if (mode == 0 && h.large)
+      XTN_RC(sort_spill(part, h.large, so.id_bits, choose_hash_bits(e.n_rec, so.id_bits), sms, ar,
+                        err, s, &so));
   }
-  if (flagged) {
-    launch_group_finish(so.flags, (int64_t)e.n_rec, nullptr, S, E, g_cap, so.gstatus, err,
+  const uint64_t g_cap = n_flagged / 2 + 1;
+  uint32_t* S = reinterpret_cast<uint32_t*>(so.spare);  // groups live in the spare buffer
+  uint32_t* E = S + g_cap;
+  uint64_t* pair_off = reinterpret_cast<uint64_t*>(E + g_cap);  // 8-byte aligned
+  if (n_flagged) {
+    launch_group_finish(so.flags, (int64_t)n_flagged, nullptr, S, E, g_cap, so.gstatus, err,
                         counters, s);
     launch_scan_group_pairs(S, E, (int64_t)g_cap, counters, pair_off, so.gstatus, err, s);
     k_pair_total<<<1, 1, 0, s>>>(pair_off, counters, counters + 1);
@@ -1317,7 +1395,7 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   b.counters = ar.get<uint64_t>(2);
   XTN_ALLOC_OK(ar);
   if (h.pairs)
-    launch_emit_pairs(so.rec, e.n_rec, S, pair_off, (int64_t)h.groups, nullptr, h.pairs,
+    launch_emit_pairs(so.rec, n_flagged, S, pair_off, (int64_t)h.groups, nullptr, h.pairs,
                       so.id_bits, b.P1 + h.direct, nullptr, nullptr, sms, err, s);
   SecondChain sc;
   if (paired) {
@@ -1601,7 +1679,7 @@ struct xtn_plan {
   uint32_t id_bits = 0;
   int hs = 0, cfg_rec = 0, cfg_pair = 0, hist_mode = 0, group_mode = 0, sms = 0;
   uint64_t* bucket_start = nullptr;
-  uint8_t* seg_area = nullptr;  // singleton filter's segment counter and flags
+  xtn::Partitions part;  // grouping mode 0
   std::vector<void*> allocs;
   int64_t bytes = 0;
   int64_t* off = nullptr;
@@ -1677,7 +1755,9 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   p->cfg_pair = g_cfg_pairs.load();
   p->hist_mode = g_record_hist.load();
   p->group_mode = g_grouping.load();
-  const size_t st = std::max({radix_status_bytes((int64_t)rec_cap, p->cfg_rec),
+  const bool parted = p->group_mode == 0;
+  const size_t st = std::max({radix_status_bytes((int64_t)rec_cap,
+                                                 parted ? ONESWEEP_LOOP : p->cfg_rec),
                               group_status_bytes((int64_t)rec_cap),
                               scan_status_bytes((int64_t)p->g_cap), scan_status_bytes(n)});
   p->off = p->alloc<int64_t>(n + 1);
@@ -1686,14 +1766,18 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   p->eqprev = p->alloc<uint32_t>(n);
   p->vcount = p->alloc<uint32_t>(n);
   p->rec_off = p->alloc<uint64_t>(n + 1);
-  p->A = p->alloc<uint64_t>(rec_cap + 8);
+  PartitionShape shape;
+  if (parted) shape = choose_partitions(rec_cap, g_filter_fx.load());
+  p->A = p->alloc<uint64_t>((parted ? std::max(shape.words(), rec_cap) : rec_cap) + 8);
   p->B = p->alloc<uint64_t>(rec_cap + 8);
+  if (parted) p->part.kept = p->alloc<uint64_t>(shape.words() + 8);
   p->hist = p->alloc<uint32_t>(MAX_PASSES * RADIX);
   p->digit_base = p->alloc<uint64_t>(MAX_PASSES * RADIX);
   p->status = p->alloc<uint64_t>(st / 8 + 1);
   p->flags = p->alloc<uint64_t>(group_flag_words((int64_t)rec_cap));
-  p->bucket_start = p->alloc<uint64_t>(bucket_start_words(rec_cap, p->hs, p->group_mode));
-  p->seg_area = p->alloc<uint8_t>(seg_area_bytes(rec_cap, p->hs));
+  p->bucket_start =
+      p->alloc<uint64_t>(bucket_start_words(rec_cap, p->hs, parted ? 1 : p->group_mode));
+  p->part.count = p->alloc<uint32_t>(parted ? shape.counts() : 1);
   p->counters = p->alloc<uint64_t>(4);
   p->err = p->alloc<uint32_t>(4);
   p->peq = p->alloc<uint32_t>((size_t)n * PEQ_STRIDE);
@@ -1707,15 +1791,22 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   if (rep_offsets) p->seq_rep = p->alloc<uint32_t>(n);
   bool ok = p->rows && p->back.counters && p->back.status && p->back.digit_base && p->back.hist &&
             p->back.P2 && p->back.P1 && p->peq && p->err && p->counters && p->flags && p->status &&
-            p->bucket_start && p->seg_area &&
-            p->digit_base && p->hist && p->B && p->A && p->rec_off && p->vcount && p->eqprev &&
+            p->bucket_start && p->part.count &&
+            (!parted || p->part.kept) && p->digit_base && p->hist && p->B && p->A && p->rec_off && p->vcount && p->eqprev &&
             p->lens && p->keys && p->off && (!rep_offsets || p->seq_rep);
   if (!ok) {
     delete p;
     return XTN_ERR_OOM;
   }
   // which buffer ends up sorted depends on the pass count; groups live in the other
-  const bool in_b = sorted_in_b(rec_cap, p->hs, p->group_mode);
+  // (mode 0 sorts its spill, which sits in B, and sorts into A on an odd count)
+  const bool in_b = parted ? !sorted_in_b(rec_cap, p->hs, 1)
+                           : sorted_in_b(rec_cap, p->hs, p->group_mode);
+  static_cast<PartitionShape&>(p->part) = shape;
+  p->part.rec = p->A;
+  p->part.spill = p->B;
+  p->part.spill_cap = rec_cap;
+  p->part.n_spill = p->counters + 3;
   p->sorted = in_b ? p->B : p->A;
   uint64_t* spare = in_b ? p->A : p->B;
   p->S = reinterpret_cast<uint32_t*>(spare);
@@ -1753,23 +1844,39 @@ int plan_run_impl(xtn_plan* p, const uint8_t* seqs, cudaStream_t s) {
   launch_scan_counts(p->vcount, n, p->rec_off, p->status, p->err, s);
   uint64_t* sorted = nullptr;
   const uint64_t* n_rec = p->rec_off + n;  // known on the device only
-  GroupScratch gs;
-  gs.bucket_start = p->bucket_start;
-  gs.flags = p->flags;
-  gs.gstatus = p->status;
-  const bool direct = p->group_mode != 1;  // bucket modes emit most candidates while grouping
-  if (direct) {
-    gs.cand = p->back.P1;
-    gs.cand_cap = p->pair_cap;
-    gs.cand_count = p->counters + 2;
-    gs.seg_area = p->seg_area;
+  const bool direct = p->group_mode != 1;  // most candidates are written while grouping
+  const uint64_t* n_flagged = n_rec;       // records whose groups are emitted from flags
+  if (p->group_mode == 0) {
+    n_flagged = p->part.n_spill;  // usually none: what follows then finds nothing to do
+    XTN_CK(cudaMemsetAsync(p->part.count, 0, p->part.counts() * 4, s));
+    launch_expand_scatter(ExpandSource{p->keys, p->lens, p->eqprev}, p->rec_off, n, p->d,
+                          p->seq_rep, p->id_bits, p->rec_cap, p->part, p->sms, p->err, s);
+    launch_group_filter(p->part, p->rec_cap, p->back.P1, p->pair_cap, p->counters + 2,
+                        (int)p->id_bits, p->err, s);
+    launch_histogram(p->B, (int64_t)p->rec_cap, n_flagged, lo, 64, p->hist, p->sms, s);
+    launch_clear_status(p->status, (int64_t)p->rec_cap, n_flagged, p->sms, s);
+    XTN_CK(cudaGetLastError());
+    XTN_CK(radix_sort_passes(p->B, p->A, (int64_t)p->rec_cap, lo, 64, p->hist, p->digit_base,
+                             p->status, ONESWEEP_LOOP, p->err, &sorted, "k_onesweep_records", s,
+                             false, n_flagged, nullptr, ONESWEEP_LOOP, true));
+    launch_group_flags(sorted, (int64_t)p->rec_cap, n_flagged, lo, p->flags, p->status, s);
+  } else {
+    GroupScratch gs;
+    gs.bucket_start = p->bucket_start;
+    gs.flags = p->flags;
+    gs.gstatus = p->status;
+    if (direct) {
+      gs.cand = p->back.P1;
+      gs.cand_cap = p->pair_cap;
+      gs.cand_count = p->counters + 2;
+    }
+    XTN_CK(expand_sort_launch(p->keys, p->lens, p->eqprev, p->rec_off, n, p->d, p->seq_rep,
+                              p->id_bits, p->A, p->B, p->rec_cap, lo, p->hist, p->digit_base,
+                              p->status, p->cfg_rec, p->hist_mode, p->group_mode, gs, p->sms,
+                              p->err, s, n_rec, &sorted));
   }
-  XTN_CK(expand_sort_launch(p->keys, p->lens, p->eqprev, p->rec_off, n, p->d, p->seq_rep,
-                            p->id_bits, p->A, p->B, p->rec_cap, lo, p->hist, p->digit_base,
-                            p->status, p->cfg_rec, p->hist_mode, p->group_mode, gs, p->sms, p->err,
-                            s, n_rec, &sorted));
   if (sorted != p->sorted) return XTN_ERR_CUDA;
-  launch_group_finish(p->flags, (int64_t)p->rec_cap, n_rec, p->S, p->E, p->g_cap, p->status,
+  launch_group_finish(p->flags, (int64_t)p->rec_cap, n_flagged, p->S, p->E, p->g_cap, p->status,
                       p->err, p->counters, s);
   launch_scan_group_pairs(p->S, p->E, (int64_t)p->g_cap, p->counters, p->pair_off, p->status,
                           p->err, s);

@@ -13,20 +13,24 @@
 // and one or two 64-bit additions, where evaluating the polynomial took two
 // 64-bit multiplies and five loads.
 //
-// Only run starts are deleted first (a run of equal residues gives one
-// string whichever of its residues goes), so the terms are kept by run
-// index, and the canonical subsets are numbered so that one table of
-// combinations serves all of them, the sentinel being run index R:
+// The terms are kept by run of equal residues: every position of a run has
+// the same M and the same Z (Q grows by what R loses), as deleting any of
+// its residues gives one string.  A variant is therefore a choice of runs,
+// repeated at most as often as the run is long, in ascending order, the
+// sentinel (run index R, "no deletion") filling up to d:
 //   d = 2: v < C(R+1, 2)  : runs a < b <= R in colex order, Y[a] + M[b]
-//          then           : none; the first two residues of each long run
+//          then           : (R, R), and (a, a) for each run of two or more
 //   d = 3: v < C(R+1, 3)  : runs a < b < c <= R, Y[a] + M[b] + Z[c]
-//          then           : none; one run; the first two residues of a long
-//                           run; the first three of a run of three or more
-//          then           : the first two of a long run k and another run o
-//   d = 1: one run (R of them), none -- stored outright.
-// Exactly the distinct variant strings are numbered (canonical_total), so no
-// lane computes a variant that is thrown away.  Paired receptors are the
-// joined string alpha + token + beta with the runs of both chains.
+//          then           : (a, R, R) for a <= R; (a, a, a) for each run of
+//                           three or more; (k, k, o) in ascending order for
+//                           each run k of two or more and each o != k, o <= R
+//   d = 1: one run (R of them), none -- their sums stored outright.
+// The first kind comes from one table of combinations, the second from a
+// short list of the sequence's own ("extra"), both as the same packed run
+// indices.  Exactly the distinct variant strings are numbered
+// (canonical_total), so no lane computes a variant that is thrown away.
+// Paired receptors are the joined string alpha + token + beta with the runs
+// of both chains.
 #pragma once
 
 #include <type_traits>
@@ -52,17 +56,14 @@ struct VK {
   static constexpr int PACK = KIND == VK_D1 ? 32 : (KIND == VK_D2 || KIND == VK_PAIRED_D1) ? 8 : 4;
   static constexpr int LANES = 32 / PACK;
   static constexpr int PER = (POS + LANES - 1) / LANES;
-  // one sequence's terms (64-bit words)
+  // one sequence's terms (64-bit words), an odd number to spread the banks
   static constexpr int Y = 0;
-  static constexpr int M = D >= 2 ? RUNS : 0;
-  static constexpr int Z = M + (D >= 2 ? RUNS + 1 : 0);
-  static constexpr int ZERO = Z + (D == 3 ? RUNS + 1 : 0);
-  static constexpr int E = ZERO + (D >= 2 ? 1 : 0);
-  static constexpr int N_E = D == 1 ? RUNS + 1 : D == 2 ? 1 + DBL : 1 + RUNS + DBL + RUNS / 3;
-  static constexpr int DL = E + N_E;
-  static constexpr int DR = DL + (D == 3 ? DBL : 0);
-  static constexpr int DRUN = DR + (D == 3 ? DBL : 0);
-  static constexpr int STRIDE = (DRUN + (D == 3 ? DBL : 0)) | 1;  // odd: spreads the banks
+  static constexpr int M = D >= 2 ? RUNS + 1 : 0;
+  static constexpr int Z = D == 3 ? M + RUNS + 1 : M;
+  static constexpr int STRIDE = (Z + RUNS + 1) | 1;
+  // its extra run choices: d = 2 (R, R) and the long runs; d = 3 the first
+  // two lists, then the long runs' indices for the third
+  static constexpr int EXTRA = D == 1 ? 0 : D == 2 ? 1 + DBL : RUNS + 1 + RUNS / 3 + DBL;
   // table of combinations over RUNS + 1 run indices
   static constexpr int COMBS = D == 3   ? (RUNS + 1) * RUNS * (RUNS - 1) / 6
                                : D == 2 ? (RUNS + 1) * RUNS / 2
@@ -113,10 +114,13 @@ __device__ __forceinline__ void load_combs(uint16_t* s_comb) {
     for (int t = threadIdx.x; t < VK<KIND>::COMBS; t += blockDim.x) s_comb[t] = d_pairs.v[t];
 }
 
-// s_pow[k + 3] = B^k for k = -3 .. POS (B^-1 is an exact inverse).
+// s_pow[k + 3] = B^k for k = -3 .. (B^-1 is an exact inverse), as far as the
+// lanes' chunks reach.
+template <int KIND>
+constexpr int N_POWERS = VK<KIND>::PER * VK<KIND>::LANES + 4;
 template <int KIND>
 __device__ __forceinline__ void load_powers(uint64_t* s_pow) {
-  for (int k = threadIdx.x; k < VK<KIND>::POS + 4; k += blockDim.x) {
+  for (int k = threadIdx.x; k < N_POWERS<KIND>; k += blockDim.x) {
     uint64_t p = HASH_BINV3;
     for (int e = 0; e < k; ++e) p *= HASH_B;
     s_pow[k] = p;
@@ -135,7 +139,7 @@ struct ExpandSource {
 
 // Where a sequence's variants sit in the warp's stream of records: variant
 // v = t - adj for stream positions t < end; c: variants that come from the
-// combination table (d >= 2); aux: R | (words in E) << 8 (d = 3).
+// combination table (d >= 2); aux: R | (extra choices outright) << 8 (d = 3).
 struct __align__(16) VarMeta {
   int32_t end, adj;
   uint32_t c, aux;
@@ -164,17 +168,20 @@ __device__ __forceinline__ uint64_t group_incl_scan_u64(uint64_t v, uint32_t sub
   return v;
 }
 
-// Whole warp: the LANES lanes of this lane's group write the terms of
-// sequence `i` (nothing when !have) to `tab` and return its number of
-// variants with at most d deletions and the fields of its VarMeta but `end`
-// (adj relative to the sequence's first variant).  The caller orders the
-// writes (__syncwarp) before they are read.
-template <int KIND>
+// Whole warp: the LANES lanes of this lane's group compute the terms of
+// sequence `i` (nothing when !have) and return its number of variants with
+// at most d deletions and the fields of its VarMeta but `end` (adj relative
+// to the sequence's first variant).  d >= 2: the terms go to `tab` and
+// `extra`, and the caller orders those writes (__syncwarp) before they are
+// read.  d <= 1: put(a, h) takes the sum of deleting run a, put(R, h) that of
+// no deletion.  Codes past the end are zero, so the loops have no bounds.
+template <int KIND, class Put>
 __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
+                                                     uint16_t* __restrict__ extra,
                                                      const uint64_t* __restrict__ s_pow,
                                                      const ExpandSource& src, int64_t i, bool have,
                                                      int d, uint64_t salt, uint32_t lane,
-                                                     VarMeta& m) {
+                                                     VarMeta& m, Put put) {
   using K = VK<KIND>;
   const uint32_t sub = lane % K::LANES;
   const int p0 = (int)sub * K::PER;
@@ -216,17 +223,20 @@ __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
     return K::PAIRED ? (uint32_t)__popcll((uint64_t)x) : (uint32_t)__popc((uint32_t)x);
   };
   const uint32_t R = popc(runs), nD = popc(dbl), nT = popc(tri);
+  const Mask before = ((Mask)1 << p0) - 1;  // p0 < the mask's width
+  uint32_t a = popc(runs & before);
+  const uint32_t my_runs = (uint32_t)(runs >> p0);  // PER <= 25 bits of interest
+  auto code = [&](int q) -> uint32_t {              // q: a position of the chunk
+    const int b = 5 * q;
+    if (b + 5 <= 64) return (uint32_t)(k.lo >> b) & 31u;
+    if (b >= 64) return (uint32_t)(k.hi >> (b - 64)) & 31u;
+    return (uint32_t)((k.lo >> b) | (k.hi << (64 - b))) & 31u;
+  };
+  constexpr int UNROLL = K::PER > 13 ? 5 : K::PER;
   // prefix sums at the chunk's start and at the end
-  const uint32_t pe = min((uint32_t)(p0 + K::PER), L);
   uint64_t sum = 0;
-  {
-    Key128 w = k;
-    for (uint32_t p = p0; p < pe; ++p) {
-      sum += (uint64_t)((uint32_t)w.lo & 31u) * s_pow[p + 3];
-      w.lo = (w.lo >> 5) | (w.hi << 59);
-      w.hi >>= 5;
-    }
-  }
+#pragma unroll UNROLL
+  for (int q = 0; q < K::PER; ++q) sum += (uint64_t)code(q) * s_pow[p0 + q + 3];
   const uint64_t incl = group_incl_scan_u64<K::LANES>(sum, sub);
   const uint64_t PL = K::LANES > 1 ? __shfl_sync(FULL_MASK, incl, K::LANES - 1, K::LANES) : incl;
   const uint64_t QL = PL * HASH_BINV, RL = PL * HASH_BINV2;
@@ -235,59 +245,58 @@ __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
   uint64_t S = K::D == 3 ? P * HASH_BINV3 : 0ull;
   // what every Y carries
   const uint64_t C = (K::D == 1 ? QL : K::D == 2 ? RL : SL) + salt;
-  for (uint32_t p = p0; p < pe; ++p) {
-    const uint64_t s0 = (uint32_t)k.lo & 31u;
-    const uint64_t Pn = P + s0 * s_pow[p + 3];
-    const uint64_t Qn = Q + s0 * s_pow[p + 2];
-    const uint64_t Rn = K::D >= 2 ? Rr + s0 * s_pow[p + 1] : 0ull;
-    const uint64_t Sn = K::D == 3 ? S + s0 * s_pow[p] : 0ull;
-    if ((runs >> p) & 1u) {
-      const Mask below = ((Mask)1 << p) - 1;
-      const uint32_t a = popc(runs & below);
+  uint64_t w0 = s_pow[p0], w1 = s_pow[p0 + 1], w2 = s_pow[p0 + 2];  // B^(p-3), B^(p-2), B^(p-1)
+#pragma unroll UNROLL
+  for (int q = 0; q < K::PER; ++q) {
+    const uint64_t c = code(q);
+    const uint64_t w3 = s_pow[p0 + q + 3];
+    const uint64_t Pn = P + c * w3;
+    const uint64_t Qn = Q + c * w2;
+    const uint64_t Rn = K::D >= 2 ? Rr + c * w1 : 0ull;
+    const uint64_t Sn = K::D == 3 ? S + c * w0 : 0ull;
+    if ((my_runs >> q) & 1u) {
       const uint64_t y = P - Qn + C;
       if constexpr (K::D == 1) {
-        tab[K::E + a] = y;
+        put(a, y);
       } else {
-        const uint64_t m = Q - Rn;
         tab[K::Y + a] = y;
-        tab[K::M + a] = m;
-        if (K::D == 3) {
+        tab[K::M + a] = Q - Rn;
+        if constexpr (K::D == 3) {
           tab[K::Z + a] = Rr - Sn;
-          tab[K::E + 1 + a] = y - SL + QL;  // this run alone
-        }
-        if ((dbl >> p) & 1u) {
-          const uint32_t kd = popc(dbl & below);
-          // the run's next residue is the same code: terms at p + 1 (and p + 2)
-          const uint64_t m1 = Qn - (Rn + s0 * s_pow[p + 2]);
-          if constexpr (K::D == 2) {
-            tab[K::E + 1 + kd] = y + m1;
-          } else {
-            const uint64_t R2 = Rn + s0 * s_pow[p + 2], S2 = Sn + s0 * s_pow[p + 1];
-            tab[K::E + 1 + R + kd] = y + m1 + (RL - SL);
-            tab[K::DL + kd] = m + (Rn - S2);
-            tab[K::DR + kd] = y + m1;
-            tab[K::DRUN + kd] = a;
-            if ((tri >> p) & 1u)
-              tab[K::E + 1 + R + nD + popc(tri & below)] = y + m1 + (R2 - (S2 + s0 * s_pow[p + 2]));
-          }
+          extra[a] = (uint16_t)(a | R << 5 | R << 10);
         }
       }
+      ++a;
     }
     P = Pn;
     Q = Qn;
     Rr = Rn;
     S = Sn;
-    k.lo = (k.lo >> 5) | (k.hi << 59);
-    k.hi >>= 5;
+    w0 = w1;
+    w1 = w2;
+    w2 = w3;
   }
-  if (sub == 0 && have) {
+  if constexpr (K::D >= 2) {  // the few long runs that start in this chunk
+    for (Mask g = (dbl >> p0) & (((Mask)1 << K::PER) - 1); g; g &= g - 1) {
+      const int p = p0 + (K::PAIRED ? __ffsll((long long)g) : __ffs((int)g)) - 1;
+      const Mask below = ((Mask)1 << p) - 1;
+      const uint32_t run = popc(runs & below);
+      if constexpr (K::D == 2) {
+        extra[1 + popc(dbl & below)] = (uint16_t)(run * 0x101u);
+      } else {
+        extra[R + 1 + nT + popc(dbl & below)] = (uint16_t)run;
+        if ((tri >> p) & 1u) extra[R + 1 + popc(tri & below)] = (uint16_t)(run * 0x421u);
+      }
+    }
+  }
+  if (sub == 0 && have) {  // the sentinel
     if constexpr (K::D == 1) {
-      tab[K::E + R] = PL + salt;
+      put(R, PL + salt);
     } else {
-      tab[K::ZERO] = 0ull;
-      tab[K::E] = PL + salt;
-      if (K::D == 2) tab[K::M + R] = QL - RL;
+      tab[K::Y + R] = PL - QL + C;
+      tab[K::M + R] = QL - RL;
       if (K::D == 3) tab[K::Z + R] = RL - SL;
+      extra[K::D == 2 ? 0 : R] = (uint16_t)(K::D == 2 ? R * 0x101u : R * 0x421u);
     }
   }
   m.c = 0;
@@ -295,7 +304,7 @@ __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
   m.adj = 0;
   if (!have) return 0u;
   if constexpr (K::D == 1) {
-    if (d <= 0) {  // only "none", stored behind the runs
+    if (d <= 0) {  // only "none", numbered behind the runs
       m.adj = -(int32_t)R;
       return 1u;
     }
@@ -304,51 +313,43 @@ __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
     m.c = R * (R + 1) / 2;
     return m.c + 1u + nD;
   } else {
-    const uint32_t e = 1u + R + nD + nT;
+    const uint32_t e = 1u + R + nT;
     m.c = R ? (R + 1) * R * (R - 1) / 6 : 0u;
     m.aux = R | (e << 8);
-    return m.c + e + (R ? nD * (R - 1) : 0u);
+    return m.c + e + nD * R;
   }
 }
 
 // Fingerprint before mixing of variant v of the sequence with terms `tab`.
 template <int KIND>
 __device__ __forceinline__ uint64_t variant_sum(const uint64_t* __restrict__ tab,
+                                                const uint16_t* __restrict__ extra,
                                                 const uint16_t* __restrict__ s_comb, uint32_t v,
                                                 uint32_t c, uint32_t aux) {
   using K = VK<KIND>;
   if constexpr (K::D == 1) {
-    return tab[K::E + v];
+    return tab[K::Y + v];
   } else if constexpr (K::D == 2) {
-    const bool in = v < c;
-    const uint32_t pr = s_comb[in ? v : 0u];
-    const uint32_t a = in ? (pr & 255u) + K::Y : v - c + K::E;
-    const uint32_t b = in ? (pr >> 8) + K::M : (uint32_t)K::ZERO;
-    return tab[a] + tab[b];
+    const uint32_t pr = *(v < c ? s_comb + v : extra + (v - c));
+    return tab[K::Y + (pr & 255u)] + tab[K::M + (pr >> 8)];
   } else {
-    const bool in = v < c;
-    const uint32_t pr = s_comb[in ? v : 0u];
-    uint32_t a = (pr & 31u) + K::Y, b = ((pr >> 5) & 31u) + K::M, z = (pr >> 10) + K::Z;
-    if (!in) {
+    uint32_t x;
+    if (v < c) {
+      x = s_comb[v];
+    } else {
       const uint32_t R = aux & 255u, e = aux >> 8;
       uint32_t u = v - c;
-      z = K::ZERO;
       if (u < e) {
-        a = K::E + u;
-        b = K::ZERO;
+        x = extra[u];
       } else {
         u -= e;
-        const uint32_t k = u / (R - 1), o = u - k * (R - 1);
-        if (o < (uint32_t)tab[K::DRUN + k]) {
-          a = K::Y + o;
-          b = K::DL + k;
-        } else {
-          a = K::DR + k;
-          b = K::Z + o + 1;
-        }
+        const uint32_t q = u / R;
+        const uint32_t k = extra[e + q];
+        uint32_t o = u - q * R;
+        x = o < k ? (o | k << 5 | k << 10) : (k | k << 5 | (o + 1) << 10);
       }
     }
-    return tab[a] + tab[b] + tab[z];
+    return tab[K::Y + (x & 31u)] + tab[K::M + ((x >> 5) & 31u)] + tab[K::Z + (x >> 10)];
   }
 }
 

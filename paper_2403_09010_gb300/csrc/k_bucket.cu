@@ -620,8 +620,6 @@ __device__ __forceinline__ void bucket_block(
   }
 }
 
-// Every block of buckets, or with seg_list only the *seg_count blocks listed
-// there (the ones the singleton filter left), in a grid-stride loop.
 template <bool HASH>
 __global__ void __launch_bounds__(BK_THREADS, Bk<HASH>::MIN_BLOCKS)
     k_bucket(uint64_t* __restrict__ A, uint64_t* __restrict__ Y, int64_t n_cap,
@@ -630,24 +628,9 @@ __global__ void __launch_bounds__(BK_THREADS, Bk<HASH>::MIN_BLOCKS)
              int cap, uint64_t* __restrict__ flags, uint64_t* __restrict__ tile_counts,
              uint64_t* __restrict__ cand, uint64_t cand_cap,
              unsigned long long* __restrict__ cand_count, int id_bits,
-             const uint32_t* __restrict__ seg_list, const uint32_t* __restrict__ seg_count,
              uint32_t* __restrict__ err) {
-  if (!seg_list) {
-    bucket_block<HASH>(blockIdx.x, A, Y, n_cap, n_dev, bucket_start, G, kbits, lo, L, cap, flags,
-                       tile_counts, cand, cand_cap, cand_count, id_bits, err);
-    return;
-  }
-  const uint32_t count = *seg_count;
-  const uint64_t n_blocks = ((uint64_t)1 << G) >> kbits;
-  for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
-    const uint32_t blk = seg_list[i];
-    if (blk < n_blocks)
-      bucket_block<HASH>(blk, A, Y, n_cap, n_dev, bucket_start, G, kbits, lo, L, cap, flags,
-                         tile_counts, cand, cand_cap, cand_count, id_bits, err);
-    else if (threadIdx.x == 0)
-      atomicOr(err, DERR_RANGE);
-    __syncthreads();  // shared memory is reused by the next listed block
-  }
+  bucket_block<HASH>(blockIdx.x, A, Y, n_cap, n_dev, bucket_start, G, kbits, lo, L, cap, flags,
+                     tile_counts, cand, cand_cap, cand_count, id_bits, err);
 }
 
 }  // namespace
@@ -676,8 +659,7 @@ GroupingShape choose_grouping(uint64_t n_rec, int hs, bool hash) {
 void launch_bucket(bool hash, uint64_t* A, uint64_t* Y, int64_t n, const uint64_t* n_dev,
                    const uint64_t* bucket_start, const GroupingShape& g, int lo, int cap,
                    uint64_t* flags, uint64_t* tile_counts, uint64_t* cand, uint64_t cand_cap,
-                   uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s,
-                   const uint32_t* seg_list, const uint32_t* seg_count, int sms) {
+                   uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s) {
   if (n <= 0) return;
   static std::once_flag once;
   std::call_once(once, [] {
@@ -690,9 +672,7 @@ void launch_bucket(bool hash, uint64_t* A, uint64_t* Y, int64_t n, const uint64_
   });
   const int full = bucket_capacity(hash);
   if (cap <= 0 || cap > full) cap = full;
-  // a listed subset runs in a grid-stride loop over the list
-  const uint64_t blocks = seg_list ? (uint64_t)std::max(1, sms) * Bk<true>::MIN_BLOCKS
-                                   : ((uint64_t)1 << g.G) >> g.kbits;
+  const uint64_t blocks = ((uint64_t)1 << g.G) >> g.kbits;
   // algorithmic bytes: every record read once; written back unless the
   // candidates leave straight from shared memory (their words are not counted:
   // their number is unknown at launch and small next to the records)
@@ -700,15 +680,15 @@ void launch_bucket(bool hash, uint64_t* A, uint64_t* Y, int64_t n, const uint64_
                                       : (double)n * 16.0 + (flags ? (double)n / 4.0 : 0.0);
   const unsigned long long* bs = reinterpret_cast<const unsigned long long*>(bucket_start);
   if (hash) {
-    prof_begin(s, seg_list ? "k_bucket_group_listed" : "k_bucket_group", seg_list ? 0.0 : bytes);
+    prof_begin(s, "k_bucket_group", bytes);
     k_bucket<true><<<(unsigned)blocks, BK_THREADS, Bk<true>::bytes, s>>>(
         A, Y, n, n_dev, bs, g.G, g.kbits, lo, g.L, cap, flags, tile_counts, cand, cand_cap,
-        reinterpret_cast<unsigned long long*>(cand_count), id_bits, seg_list, seg_count, err);
+        reinterpret_cast<unsigned long long*>(cand_count), id_bits, err);
   } else {
     prof_begin(s, "k_bucket_sort", bytes);
     k_bucket<false><<<(unsigned)blocks, BK_THREADS, Bk<false>::bytes, s>>>(
         A, Y, n, n_dev, bs, g.G, g.kbits, lo, g.L, cap, flags, tile_counts, nullptr, 0, nullptr,
-        0, nullptr, nullptr, err);
+        0, err);
   }
   prof_end(s);
 }

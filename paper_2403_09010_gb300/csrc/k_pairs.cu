@@ -155,6 +155,7 @@ constexpr int GB_ITEMS = 16;   // positions per lane per chunk
 constexpr int GB_CHUNKS = 4;
 constexpr int GB_WARP_SPAN = 32 * GB_ITEMS * GB_CHUNKS;
 constexpr int GB_TILE = GB_THREADS * GB_ITEMS * GB_CHUNKS;  // 32768 positions
+constexpr int64_t GB_GRID = 152 * 4;  // blocks when only the device knows the count
 static_assert(GB_TILE == GROUP_FLAG_TILE, "flag tiles shared with k_bucket_sort");
 
 // K = uint32_t when the group key (key >> gshift) fits in 32 bits.
@@ -165,12 +166,13 @@ __global__ void __launch_bounds__(GB_THREADS)
                   uint64_t* __restrict__ tile_counts) {
   __shared__ uint64_t s_wtot[GB_WARPS];
   const int64_t n = n_dev ? min((int64_t)*n_dev, n_cap) : n_cap;
-  const int64_t tbase = (int64_t)blockIdx.x * GB_TILE;
-  if (tbase >= n) {
-    if (threadIdx.x == 0) tile_counts[blockIdx.x] = 0;
-    return;
-  }
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+  const int64_t tiles = (n_cap + GB_TILE - 1) / GB_TILE;
+  for (int64_t tile = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; tile < tiles;
+       tile += (int64_t)gridDim.x * blockDim.x)
+    if (tile * GB_TILE >= n) tile_counts[tile] = 0;
+  for (int64_t tile = blockIdx.x; tile * GB_TILE < n; tile += gridDim.x) {
+  const int64_t tbase = tile * GB_TILE;
   const int64_t wbase = tbase + (int64_t)warp * GB_WARP_SPAN;
   // the value before position wbase (made different from it at position 0)
   K carry = (wbase >= 1 && wbase - 1 < n) ? (K)(keys[wbase - 1] >> gshift) : (K)0;
@@ -215,7 +217,9 @@ __global__ void __launch_bounds__(GB_THREADS)
     uint64_t total = 0;
 #pragma unroll
     for (int w = 0; w < GB_WARPS; ++w) total += s_wtot[w];
-    tile_counts[blockIdx.x] = total;
+    tile_counts[tile] = total;
+  }
+  __syncthreads();  // s_wtot is reused by the next tile
   }
 }
 
@@ -226,9 +230,9 @@ __global__ void __launch_bounds__(GB_THREADS)
                   uint32_t* __restrict__ err) {
   __shared__ uint64_t s_w[GB_WARPS];
   const int64_t n = n_dev ? min((int64_t)*n_dev, n_cap) : n_cap;
-  const int64_t tbase = (int64_t)blockIdx.x * GB_TILE;
-  if (tbase >= n) return;
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+  for (int64_t tile = blockIdx.x; tile * GB_TILE < n; tile += gridDim.x) {
+  const int64_t tbase = tile * GB_TILE;
   // each warp owns GB_WARP_SPAN / 32 flag words; lane l holds words l, l+32, ...
   constexpr int WPW = GB_WARP_SPAN / 32;  // words per warp (64)
   const int64_t w0 = tbase / 32 + (int64_t)warp * WPW;
@@ -247,7 +251,7 @@ __global__ void __launch_bounds__(GB_THREADS)
   const uint64_t inc = warp_incl_scan_u64(mine);
   if (lane == 31) s_w[warp] = inc;
   __syncthreads();
-  uint64_t off = tile_prefix[blockIdx.x];
+  uint64_t off = tile_prefix[tile];
 #pragma unroll
   for (int w = 0; w < GB_WARPS; ++w)
     if (w < (int)warp) off += s_w[w];
@@ -285,6 +289,8 @@ __global__ void __launch_bounds__(GB_THREADS)
     hk += htot;
     tk += ttot;
   }
+  __syncthreads();  // s_w is reused by the next tile
+  }
 }
 
 __global__ void k_groups_total(const uint64_t* __restrict__ total, uint64_t* __restrict__ n_groups) {
@@ -315,12 +321,10 @@ void launch_group_flags(const uint64_t* keys, int64_t n, const uint64_t* n_dev, 
   const int64_t tiles = (n + GB_TILE - 1) / GB_TILE;
   uint64_t* tile_counts = group_tile_counts(status, n);
   prof_begin(s, "k_group_flags", (double)n * 8.0 + (double)(n / 32) * 8.0);
-  if (gshift >= 32)
-    k_group_flags<uint32_t><<<(unsigned)tiles, GB_THREADS, 0, s>>>(keys, n, n_dev, gshift, flags,
-                                                                   tile_counts);
-  else
-    k_group_flags<uint64_t><<<(unsigned)tiles, GB_THREADS, 0, s>>>(keys, n, n_dev, gshift, flags,
-                                                                   tile_counts);
+  // a count known only on the device is usually far below its capacity
+  const unsigned blocks = (unsigned)(n_dev ? std::min<int64_t>(tiles, GB_GRID) : tiles);
+  auto f = gshift >= 32 ? k_group_flags<uint32_t> : k_group_flags<uint64_t>;
+  f<<<blocks, GB_THREADS, 0, s>>>(keys, n, n_dev, gshift, flags, tile_counts);
   prof_end(s);
 }
 
@@ -339,8 +343,8 @@ void launch_group_finish(const uint64_t* flags, int64_t n, const uint64_t* n_dev
                   s>>>(CountsU64{tile_counts}, tiles, nullptr, tile_prefix, status, ctr, err);
   prof_end(s);
   prof_begin(s, "k_group_write", (double)(n / 32) * 8.0);
-  k_group_write<<<(unsigned)tiles, GB_THREADS, 0, s>>>(flags, n, n_dev, tile_prefix, S, E, cap,
-                                                       err);
+  k_group_write<<<(unsigned)(n_dev ? std::min<int64_t>(tiles, GB_GRID) : tiles), GB_THREADS, 0,
+                  s>>>(flags, n, n_dev, tile_prefix, S, E, cap, err);
   prof_end(s);
   // number of groups = heads in the total (high field of tile_prefix[tiles])
   k_groups_total<<<1, 1, 0, s>>>(tile_prefix + tiles, n_groups);

@@ -31,8 +31,10 @@
 namespace xtn {
 
 // Global digit histograms of every pass in one read of the keys.
-__global__ void k_histogram(const uint64_t* __restrict__ keys, int64_t n, int lo, int hi,
+__global__ void k_histogram(const uint64_t* __restrict__ keys, int64_t n_cap,
+                            const uint64_t* __restrict__ n_dev, int lo, int hi,
                             uint32_t* __restrict__ hist) {
+  const int64_t n = n_dev ? min((int64_t)*n_dev, n_cap) : n_cap;
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   const int passes = (hi - lo + 7) / 8;
   for (int k = threadIdx.x; k < passes * RADIX; k += blockDim.x) s_hist[k] = 0;
@@ -406,7 +408,11 @@ struct RunsSmem {
   static constexpr size_t bytes = keys_bytes + (size_t)CNT * 4 + RADIX * 4 + RADIX * 8;
 };
 
-template <int THREADS, int ITEMS, int MIN_BLOCKS, int LBW, int DB, int UW, bool HIW>
+// LOOP: a block takes tiles until the keys run out, so that a sort whose key
+// count is only known on the device (usually zero) needs no grid for its
+// capacity.
+template <int THREADS, int ITEMS, int MIN_BLOCKS, int LBW, int DB, int UW, bool HIW,
+          bool LOOP = false>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
     k_onesweep_runs(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                     const uint64_t* __restrict__ n_dev, int64_t n_cap, int shift, int bits, int lo,
@@ -434,6 +440,7 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
     for (int k = threadIdx.x; k < RADIX; k += THREADS) s_next[k] = 0;
   if (threadIdx.x == 0) s_shift = shift;
   const int64_t n = n_dev ? min((int64_t)*n_dev, n_cap) : n_cap;
+  do {
   const uint32_t tile = tile_id(ctr, &s_tile);
   const int64_t tile_base = (int64_t)tile * TILE;
   if (tile_base >= n) return;
@@ -675,6 +682,8 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
     status_next[(uint64_t)tile * RADIX + threadIdx.x] = 0ull;
     if (tile == 0 && threadIdx.x == 0) *ctr_next = 0u;
   }
+  if (LOOP) __syncthreads();  // shared memory is reused by the next tile
+  } while (LOOP);
 }
 
 // Tile configurations (id, threads, items per thread, min blocks per SM,
@@ -722,8 +731,11 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
   X(28, 256, 20, 4, 8, 0, 1)         \
   X(29, 384, 16, 3, 4, 0, 1)
 
+constexpr int LOOP_THREADS = 256, LOOP_ITEMS = 20, LOOP_BLOCKS = 4;  // ONESWEEP_LOOP
+
 int onesweep_tile(int cfg) {
   switch (cfg) {
+    case ONESWEEP_LOOP: return LOOP_THREADS * LOOP_ITEMS;
 #define X(id, T, I, B, M, C) \
   case id: return T * I;
     XTN_ONESWEEP_CONFIGS(X)
@@ -741,7 +753,9 @@ int onesweep_configs() { return 30; }  // the tunable ones, 0-29
 // Configurations 0-19 rank stably in every pass, so their first pass (whose
 // input order does not matter) takes the unstable configuration 100 with the
 // same tile; a k_onesweep_runs configuration serves every pass itself.
-int onesweep_unstable_config(int cfg) { return cfg >= 20 && cfg < 30 ? cfg : 100; }
+int onesweep_unstable_config(int cfg) {
+  return (cfg >= 20 && cfg < 30) || cfg == ONESWEEP_LOOP ? cfg : 100;
+}
 
 static cudaError_t onesweep_launch(int cfg, const uint64_t* in, uint64_t* out, int64_t n,
                                    const uint64_t* n_dev, int shift, int bits, const uint64_t* digit_base,
@@ -750,6 +764,21 @@ static cudaError_t onesweep_launch(int cfg, const uint64_t* in, uint64_t* out, i
                                    unsigned long long* bucket_start, int bucket_shift,
                                    uint64_t* status_next, uint32_t* ctr_next, cudaStream_t s) {
   switch (cfg) {
+    case ONESWEEP_LOOP: {
+      using SM = RunsSmem<LOOP_THREADS, LOOP_ITEMS>;
+      auto f = k_onesweep_runs<LOOP_THREADS, LOOP_ITEMS, LOOP_BLOCKS, 8, 0, 0, false, true>;
+      static std::once_flag once;
+      std::call_once(once, [&] {
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
+        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+      });
+      // every block is resident, so the look-back's predecessors run
+      const uint32_t tiles = std::min<uint32_t>(div_up_u32(n, SM::TILE), 148 * LOOP_BLOCKS);
+      f<<<tiles, LOOP_THREADS, SM::bytes, s>>>(in, out, n_dev, n, shift, bits, bucket_shift,
+                                               digit_base, status, ctr, err, next_hist, next_bits,
+                                               bucket_start, status_next, ctr_next);
+      return cudaGetLastError();
+    }
 #define X(id, T, I, B, M, C)                                                                  \
   case id: {                                                                                  \
     using SM = OnesweepSmem<T, I, M, C>;                                                      \
@@ -805,12 +834,38 @@ static size_t status_region_bytes(int64_t n, int cfg) {
 
 size_t radix_status_bytes(int64_t n, int cfg) { return 2 * status_region_bytes(n, cfg); }
 
-void launch_histogram(const uint64_t* keys, int64_t n, int lo, int hi, uint32_t* hist, int sms,
-                      cudaStream_t s) {
+// Clears the words of both status regions that a sort of *n_dev keys reads,
+// and the tile counters.
+__global__ void k_clear_status(uint64_t* __restrict__ status, uint64_t region_words,
+                               int64_t n_cap, const uint64_t* __restrict__ n_dev, int tile) {
+  const int64_t n = min((int64_t)*n_dev, n_cap);
+  const int64_t words = (n + tile - 1) / tile * RADIX;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < words;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    status[k] = 0ull;
+    status[region_words + k] = 0ull;
+  }
+  if (blockIdx.x == 0 && threadIdx.x < 2) {
+    status[region_words - 2 + threadIdx.x] = 0ull;
+    status[2 * region_words - 2 + threadIdx.x] = 0ull;
+  }
+}
+
+void launch_clear_status(uint64_t* status, int64_t n, const uint64_t* n_dev, int sms,
+                         cudaStream_t s) {
+  if (n <= 0) return;
+  prof_begin(s, "k_clear_status", 0.0);
+  k_clear_status<<<sms * 2, 256, 0, s>>>(status, status_region_bytes(n, ONESWEEP_LOOP) / 8, n,
+                                         n_dev, onesweep_tile(ONESWEEP_LOOP));
+  prof_end(s);
+}
+
+void launch_histogram(const uint64_t* keys, int64_t n, const uint64_t* n_dev, int lo, int hi,
+                      uint32_t* hist, int sms, cudaStream_t s) {
   if (n <= 0) return;
   int blocks = (int)std::min<int64_t>((n + 1023) / 1024, (int64_t)sms * 4);
   prof_begin(s, "k_histogram", (double)n * 8.0);
-  k_histogram<<<blocks, 512, 0, s>>>(keys, n, lo, hi, hist);
+  k_histogram<<<blocks, 512, 0, s>>>(keys, n, n_dev, lo, hi, hist);
   prof_end(s);
 }
 

@@ -5,7 +5,7 @@
 //   k_encode : ASCII sequence -> 128-bit key of 5-bit residue codes
 //              (Appendix "Compression of TCR sequences"), its length, the
 //              mask of positions equal to their left neighbour, and its
-//              number of canonical deletion subsets (see is_canonical).
+//              number of canonical deletion subsets (expand.cuh).
 //   k_expand : the records  fingerprint[63:b] | id[b-1:0]  of every canonical
 //              deletion variant, at rec_off (see expand.cuh).  The kernel also
 //              accumulates the digit histograms of the radix passes that will
@@ -103,11 +103,14 @@ constexpr int EXPAND_THREADS = 256;
 
 // One count per radix pass for record `rec` (8-bit digits from bit `lo`; the
 // last digit keeps only `last_mask`).
-// HIW: lo >= 32 and every counted digit lies in the high word (32-bit shifts)
-template <bool HIW = false>
+// H: HIST_NONE, HIST_HIGH (lo >= 32 and every counted digit lies in the high
+// word: 32-bit shifts) or HIST_ANY.
+enum { HIST_NONE = 0, HIST_HIGH, HIST_ANY };
+template <int H>
 __device__ __forceinline__ void count_digits(uint32_t* s_hist, uint64_t rec, int lo, int passes,
                                              uint32_t last_mask) {
-  if (HIW) {
+  if constexpr (H == HIST_NONE) return;
+  if constexpr (H == HIST_HIGH) {
     const uint32_t r = (uint32_t)(rec >> 32) >> (lo - 32);
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
@@ -167,7 +170,7 @@ __device__ __forceinline__ void flush_stage(WarpStage& st, uint64_t* __restrict_
 //   SEL_COUNT  only its fingerprint bin counted (s_hist holds the bins)
 //   SEL_APPEND staged for appending when its bin lies in [sel.lo, sel.hi);
 //              its digits counted
-template <int SEL, bool HIW = false>
+template <int SEL, int H>
 __device__ __forceinline__ void place_record(uint64_t rec, bool valid, uint64_t pos,
                                              uint64_t* __restrict__ out, uint64_t n_rec,
                                              uint32_t* s_hist, int hist_lo, int hist_passes,
@@ -176,7 +179,7 @@ __device__ __forceinline__ void place_record(uint64_t rec, bool valid, uint64_t 
   if constexpr (SEL == SEL_ALL) {
     if (valid) {
       out[pos] = rec;
-      count_digits<HIW>(s_hist, rec, hist_lo, hist_passes, last_mask);
+      count_digits<H>(s_hist, rec, hist_lo, hist_passes, last_mask);
     }
   } else {
     const uint32_t bin = (uint32_t)(rec >> sel.shift) & sel.mask;
@@ -187,7 +190,7 @@ __device__ __forceinline__ void place_record(uint64_t rec, bool valid, uint64_t 
       const uint32_t bal = __ballot_sync(FULL_MASK, keep);
       if (keep) {
         st.buf[st.n + __popc(bal & ((1u << lane) - 1u))] = rec;  // st.n + 32 <= STAGE_CAP
-        count_digits<HIW>(s_hist, rec, hist_lo, hist_passes, last_mask);
+        count_digits<H>(s_hist, rec, hist_lo, hist_passes, last_mask);
       }
       st.n += __popc(bal);
       if (st.n >= STAGE_FLUSH) flush_stage(st, out, n_rec, sel, lane, err);
@@ -212,19 +215,19 @@ __device__ __forceinline__ void zero_fill(uint4* __restrict__ p, uint64_t n) {
 // the batch's records are contiguous in the output, so stores coalesce.
 constexpr int EXPAND_WARPS = EXPAND_THREADS / 32;
 
-template <int KIND, int SEL>
+template <int KIND, int SEL, int H>
 struct ExpandSmem {
   using K = VK<KIND>;
   uint64_t terms[EXPAND_WARPS][K::PACK][K::STRIDE];
   uint64_t stage[SEL == SEL_APPEND ? EXPAND_WARPS : 1][SEL == SEL_APPEND ? STAGE_CAP : 1];
-  uint64_t pow[K::POS + 4];
+  uint64_t pow[N_POWERS<KIND>];
   VarMeta meta[EXPAND_WARPS][K::PACK];
-  uint32_t hist[MAX_PASSES * RADIX];
+  uint32_t hist[H != HIST_NONE || SEL == SEL_COUNT ? MAX_PASSES * RADIX : 1];
+  uint16_t extra[EXPAND_WARPS][K::PACK][K::EXTRA + 1];
   uint16_t comb[K::COMBS + 1];
 };
 
-// HIW: the histogram's digits lie in the record's high word (hist_lo >= 32).
-template <int KIND, int SEL, bool HIW>
+template <int KIND, int SEL, int H>
 __global__ void __launch_bounds__(EXPAND_THREADS, 4)
     k_expand(ExpandSource src, const uint64_t* __restrict__ rec_off, int64_t n, int d,
              const uint32_t* __restrict__ seq_rep, uint32_t id_bits, uint64_t* __restrict__ out,
@@ -233,18 +236,18 @@ __global__ void __launch_bounds__(EXPAND_THREADS, 4)
              uint64_t n_zero) {
   using K = VK<KIND>;
   extern __shared__ __align__(16) unsigned char expand_smem[];
-  ExpandSmem<KIND, SEL>& S = *reinterpret_cast<ExpandSmem<KIND, SEL>*>(expand_smem);
+  ExpandSmem<KIND, SEL, H>& S = *reinterpret_cast<ExpandSmem<KIND, SEL, H>*>(expand_smem);
   zero_fill(zero, n_zero);
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
   WarpStage st{S.stage[SEL == SEL_APPEND ? warp : 0], 0u};
-  const int n_hist = SEL == SEL_COUNT ? (int)sel.mask + 1 : hist_passes * RADIX;
+  const int n_hist = SEL == SEL_COUNT ? (int)sel.mask + 1 : H ? hist_passes * RADIX : 0;
   for (int k = threadIdx.x; k < n_hist; k += blockDim.x) S.hist[k] = 0;
   load_powers<KIND>(S.pow);
   load_combs<KIND>(S.comb);
   __syncthreads();
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const uint64_t idmask = (id_bits >= 64) ? ~0ull : ((1ull << id_bits) - 1ull);
+  const uint32_t idmask = (uint32_t)((1ull << id_bits) - 1ull);  // id_bits <= 32
   const int last_bits = hist_hi - hist_lo - 8 * (hist_passes - 1);
   const uint32_t last_mask = (1u << last_bits) - 1u;
   const int q = (int)lane / K::LANES;  // this lane's sequence in the batch
@@ -254,7 +257,10 @@ __global__ void __launch_bounds__(EXPAND_THREADS, 4)
     const bool have = my < n;
     const uint64_t salt = have && seq_rep ? rep_salt(seq_rep[my]) : 0ull;
     VarMeta m;
-    uint32_t total = prepare_variants<KIND>(S.terms[warp][q], S.pow, src, my, have, d, salt, lane, m);
+    uint64_t* terms = S.terms[warp][q];
+    uint32_t total =
+        prepare_variants<KIND>(terms, S.extra[warp][q], S.pow, src, my, have, d, salt, lane, m,
+                               [&](uint32_t a, uint64_t h) { terms[a] = h; });
     const uint64_t base = have ? rec_off[my] : 0ull;
     if (have) {
       const uint64_t cnt = rec_off[my + 1] - base;
@@ -278,22 +284,26 @@ __global__ void __launch_bounds__(EXPAND_THREADS, 4)
       meta[q] = m;
     }
     __syncwarp();  // terms and meta, written above, are read by every lane
-    int j = 0;
+    const VarMeta* at = meta;
     VarMeta cur = meta[0];
+    uint32_t id = (uint32_t)s0;
     const uint64_t* tab = S.terms[warp][0];
+    const uint16_t* extra = S.extra[warp][0];
     for (uint32_t t0 = 0; t0 < T; t0 += 32) {
       const uint32_t t = t0 + lane;
       uint64_t rec = 0;
       if (t < T) {
         while ((int32_t)t >= cur.end) {  // ends: t < T, the last sequence's end
-          cur = meta[++j];
+          cur = *++at;
+          ++id;
           tab += K::STRIDE;
+          extra += K::EXTRA + 1;
         }
-        const uint64_t h = variant_sum<KIND>(tab, S.comb, (uint32_t)((int32_t)t - cur.adj), cur.c,
-                                             cur.aux);
-        rec = (mix64(h) & ~idmask) | (uint64_t)(s0 + j);
+        const uint64_t h = mix64(variant_sum<KIND>(
+            tab, extra, S.comb, (uint32_t)((int32_t)t - cur.adj), cur.c, cur.aux));
+        rec = (h & 0xffffffff00000000ull) | (((uint32_t)h & ~idmask) | id);
       }
-      place_record<SEL, HIW>(rec, t < T, base0 + t, out, n_rec, S.hist, hist_lo, hist_passes,
+      place_record<SEL, H>(rec, t < T, base0 + t, out, n_rec, S.hist, hist_lo, hist_passes,
                              last_mask, sel, lane, st, err);
     }
     __syncwarp();  // the next batch overwrites the tables
@@ -365,13 +375,13 @@ void launch_encode(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Ke
   prof_end(s);
 }
 
-template <int KIND, int SEL, bool HIW>
+template <int KIND, int SEL, int H>
 static void expand_launch(const ExpandSource& src, const uint64_t* rec_off, int64_t n, int d,
                           const uint32_t* seq_rep, uint32_t id_bits, uint64_t* out, uint64_t n_rec,
                           uint32_t* hist, int hist_lo, int hist_hi, const BinSel& sel, int sms,
                           uint32_t* err, cudaStream_t s, uint4* zero, uint64_t n_zero) {
-  auto f = k_expand<KIND, SEL, HIW>;
-  constexpr int smem = (int)sizeof(ExpandSmem<KIND, SEL>);
+  auto f = k_expand<KIND, SEL, H>;
+  constexpr int smem = (int)sizeof(ExpandSmem<KIND, SEL, H>);
   static std::once_flag once;
   std::call_once(once, [&] {
     cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -393,14 +403,17 @@ void launch_expand(const ExpandSource& src, const uint64_t* rec_off, int64_t n, 
   if (n <= 0) return;
   const BinSel none{};
   const bool paired = src.keys_b != nullptr;
-  const bool hiw = hist_lo >= 32 && hist_hi <= 64;
+  const bool high = hist_lo >= 32 && hist_hi <= 64;
   auto go = [&](auto kind) {
     constexpr int KIND = decltype(kind)::value;
-    auto f = hiw ? expand_launch<KIND, SEL_ALL, true> : expand_launch<KIND, SEL_ALL, false>;
-    if constexpr (!VK<KIND>::PAIRED)  // the bin passes take the general digit count
+    auto f = !hist  ? expand_launch<KIND, SEL_ALL, HIST_NONE>
+             : high ? expand_launch<KIND, SEL_ALL, HIST_HIGH>
+                    : expand_launch<KIND, SEL_ALL, HIST_ANY>;
+    if constexpr (!VK<KIND>::PAIRED)
       if (sel)
-        f = sel->append ? expand_launch<KIND, SEL_APPEND, false>
-                        : expand_launch<KIND, SEL_COUNT, false>;
+        f = !sel->append ? expand_launch<KIND, SEL_COUNT, HIST_NONE>
+            : hist       ? expand_launch<KIND, SEL_APPEND, HIST_ANY>
+                         : expand_launch<KIND, SEL_APPEND, HIST_NONE>;
     f(src, rec_off, n, d, seq_rep, id_bits, out, n_rec, hist, hist_lo, hist_hi, sel ? *sel : none,
       sms, err, s, z, nz);
   };

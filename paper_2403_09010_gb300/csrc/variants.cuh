@@ -12,7 +12,7 @@
 //   v = 1 .. R                    : first residue of run v-1
 //   v = R+1 .. R+C(R,2)           : first residues of runs i < j (colex rank)
 //   v = R+C(R,2)+1 .. (+nD)       : first two residues of the v-th long run
-// which is exactly the set counted by canonical_count(), so no lane of the
+// which is exactly the set counted by canonical_total(), so no lane of the
 // warp computes a variant that is then thrown away.  d = 3 enumerates every
 // subset and keeps the canonical ones.
 #pragma once

@@ -357,27 +357,6 @@ __device__ __forceinline__ bool is_canonical(uint32_t mask, uint32_t eqprev) {
   return (eqprev & mask & ~(mask << 1)) == 0;
 }
 
-// Number of canonical subsets with at most d elements: a canonical subset
-// deletes a prefix of c_i positions from each run i, so the count is the sum
-// of the coefficients of x^0..x^d in prod_i (1 + x + ... + x^{len_i}).
-__host__ __device__ __forceinline__ uint32_t canonical_count(uint32_t eqprev, uint32_t L,
-                                                             uint32_t d) {
-  uint32_t poly[4] = {1u, 0u, 0u, 0u};
-  uint32_t p = 0;
-  while (p < L) {
-    uint32_t run = 1;
-    while (p + run < L && ((eqprev >> (p + run)) & 1u)) ++run;
-    uint32_t next[4] = {0u, 0u, 0u, 0u};
-    for (uint32_t k = 0; k <= d; ++k)
-      for (uint32_t c = 0; c <= k && c <= run; ++c) next[k] += poly[k - c];
-    for (uint32_t k = 0; k <= d; ++k) poly[k] = next[k];
-    p += run;
-  }
-  uint32_t total = 0;
-  for (uint32_t k = 0; k <= d; ++k) total += poly[k];
-  return total;
-}
-
 // ------------------------------------------------------------ host side ---
 // Launch bookkeeping: optional CUDA-event timing per kernel (see
 // xtn_profile_enable), tagged with algorithmic bytes.

@@ -42,6 +42,8 @@ constexpr int MAX_BIN_BITS = 11;
 // The sequences (or paired receptors, when src.keys_b is set: d <= 2, no bin
 // selection) expanded into records.  sel null: every record of sequence i
 // goes to out[rec_off[i] ...].
+// hist: when not null, the digit counts of the sort passes over bits
+// [hist_lo, hist_hi) are added there.
 // zero: when not null, zero_bytes (a multiple of 16, 16-byte aligned) are
 // cleared there as well (the record sort's look-back status).
 struct ExpandSource;
@@ -59,8 +61,15 @@ void launch_seq_rep(const int64_t* rep_off, int64_t n_rep, uint32_t* seq_rep, in
 int onesweep_tile(int cfg);
 int onesweep_configs();
 size_t radix_status_bytes(int64_t n, int cfg);
-void launch_histogram(const uint64_t* keys, int64_t n, int lo, int hi, uint32_t* hist, int sms,
-                      cudaStream_t s);
+void launch_histogram(const uint64_t* keys, int64_t n, const uint64_t* n_dev, int lo, int hi,
+                      uint32_t* hist, int sms, cudaStream_t s);
+// A configuration outside the tunable ones: one resident grid that loops over
+// the tiles of the (device-side) key count.
+constexpr int ONESWEEP_LOOP = 120;
+// Clears the status area (radix_status_bytes(n, ONESWEEP_LOOP)) as far as a
+// sort of *n_dev keys with that configuration reads it.
+void launch_clear_status(uint64_t* status, int64_t n, const uint64_t* n_dev, int sms,
+                         cudaStream_t s);
 // Sorts a[0:n) on bits [lo, hi) using b as the second buffer; `hist` holds the
 // digit histograms of every pass.  *sorted receives a or b.
 // hist_in_passes: `hist` holds only pass 0's digit counts; every pass counts
@@ -109,26 +118,52 @@ int bucket_capacity(bool hash);
 // to cand[0, cand_cap), counting them in cand_count[0] (DERR_CAPACITY past
 // the capacity); larger buckets go the flag route as before and add their
 // record count to cand_count[1].
-// seg_list / seg_count: when given, only the *seg_count blocks of buckets
-// listed (the ones k_bucket_filter left), by a grid of sms x 5 blocks.
 void launch_bucket(bool hash, uint64_t* A, uint64_t* Y, int64_t n, const uint64_t* n_dev,
                    const uint64_t* bucket_start, const GroupingShape& g, int lo, int cap,
                    uint64_t* flags, uint64_t* tile_counts, uint64_t* cand, uint64_t cand_cap,
-                   uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s,
-                   const uint32_t* seg_list = nullptr, const uint32_t* seg_count = nullptr,
-                   int sms = 0);
+                   uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s);
+// k_partition.cu, k_scatter.cu ----------------------------------------------
+// Partitions of the variant records by their top pbits fingerprint bits:
+// partition p fills rec[p * region ...] and counts its records in count[p]
+// (which may pass `region`; the records past it go to spill).  The filter
+// keeps a list per partition in `kept`, laid out alike.
+struct PartitionShape {
+  int pbits = 0;
+  uint32_t region = 0;
+  uint64_t words() const { return (uint64_t)region << pbits; }
+  uint64_t counts() const { return (uint64_t)2 << pbits; }
+};
+// fx: the size of the partitions (see XTN_TUNE_FILTER_SEGMENT).
+PartitionShape choose_partitions(uint64_t n_rec, int fx);
+struct Partitions : PartitionShape {
+  uint64_t* rec = nullptr;      // words()
+  uint64_t* kept = nullptr;     // words()
+  uint32_t* count = nullptr;    // counts() zeroed words: the partitions', then the lists'
+  uint64_t* spill = nullptr;    // spill_cap words
+  uint64_t spill_cap = 0;
+  uint64_t* n_spill = nullptr;  // zeroed by the caller
+  uint32_t* kept_count() const { return count + ((uint64_t)1 << pbits); }
+};
+// The records of every canonical variant, expanded straight into their
+// partitions; rec_off as launch_expand takes it, its last entry the record
+// count (at most n_rec, a capacity that sizes the grid).
+void launch_expand_scatter(const ExpandSource& src, const uint64_t* rec_off, int64_t n, int d,
+                           const uint32_t* seq_rep, uint32_t id_bits, uint64_t n_rec,
+                           const Partitions& p, int sms, uint32_t* err, cudaStream_t s);
+// The same for records already expanded to in[0, n) (n_dev: when not null the
+// count is read on the device and n is a capacity).
+void launch_partition(const uint64_t* in, int64_t n, const uint64_t* n_dev, const Partitions& p,
+                      int sms, uint32_t* err, cudaStream_t s);
+
 // k_filter.cu --------------------------------------------------------------
-// Candidate mode of the grouping for the buckets of shape g (G global bits):
-// each block takes 2^(kbits + fx) buckets, keeps only the records whose group
-// key occurs twice or more (two bitmaps), groups those exactly in shared
-// memory and appends their pairs to cand as k_bucket does.  A block whose
-// kept records overflow appends the k_bucket blocks it covers to seg_list
-// (counted in *seg_count, zeroed; room for every k_bucket block), for
-// launch_bucket(..., seg_list, seg_count).
-void launch_bucket_filter(const uint64_t* A, int64_t n, const uint64_t* n_dev,
-                          const uint64_t* bucket_start, const GroupingShape& g, int fx, int lo,
-                          uint64_t* cand, uint64_t cand_cap, uint64_t* cand_count, int id_bits,
-                          uint32_t* seg_list, uint32_t* seg_count, uint32_t* err, cudaStream_t s);
+// Appends the candidate words (min id << id_bits | max id) of every pair of
+// records with equal group keys to cand[0, cand_cap), counting them in
+// *cand_count (DERR_CAPACITY past the capacity).  What a block cannot group
+// on its own -- a partition or list that overflowed, a single key too
+// frequent for its table -- is appended to p.spill (counted in *p.n_spill)
+// for a global sort of those few.  n_rec: the expected records.
+void launch_group_filter(const Partitions& p, uint64_t n_rec, uint64_t* cand, uint64_t cand_cap,
+                         uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s);
 // k_pairs.cu ---------------------------------------------------------------
 size_t scan_status_bytes(int64_t n);
 size_t group_status_bytes(int64_t n);
