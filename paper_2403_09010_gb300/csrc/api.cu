@@ -546,13 +546,16 @@ struct Encoded {
   Key128* keys_b = nullptr;
   uint8_t* lens_b = nullptr;
   uint32_t* eq_b = nullptr;
+  PlaneRow* rows = nullptr;  // bit planes, for the distances (both chains)
+  PlaneRow* rows_b = nullptr;
+  PairSide side(int64_t n) const { return PairSide{rows, rows_b, (uint64_t)n}; }
   ExpandSource source() const { return ExpandSource{keys, lens, eqprev, keys_b, lens_b, eq_b}; }
 };
 
 // allow_large: return the count even when it is 2^32 or more (the caller
 // then searches in passes); otherwise that is TOO_LARGE.
 int encode_and_count(const DevSeqs& in, int d, Arena& ar, uint32_t* err, cudaStream_t s,
-                     Encoded* e, bool allow_large = false, uint32_t* peq = nullptr) {
+                     Encoded* e, bool allow_large = false, bool planes = true) {
   const int64_t n = in.n;
   e->keys = ar.get<Key128>(n);
   e->lens = ar.get<uint8_t>(n);
@@ -561,7 +564,9 @@ int encode_and_count(const DevSeqs& in, int d, Arena& ar, uint32_t* err, cudaStr
   e->rec_off = ar.get<uint64_t>(n + 1);
   uint64_t* status = ar.get<uint64_t>(scan_status_bytes(n) / 8 + 1);
   XTN_ALLOC_OK(ar);
-  launch_encode(in.seqs, in.off, n, d, e->keys, e->lens, e->eqprev, vcount, err, s);
+  if (planes) e->rows = ar.get<PlaneRow>(n);
+  XTN_ALLOC_OK(ar);
+  launch_encode(in.seqs, in.off, n, d, e->keys, e->lens, e->eqprev, vcount, e->rows, err, s);
   launch_scan_counts(vcount, n, e->rec_off, status, err, s);
   XTN_CK(cudaGetLastError());
   struct {
@@ -571,10 +576,7 @@ int encode_and_count(const DevSeqs& in, int d, Arena& ar, uint32_t* err, cudaStr
   ReadBack rb(s);
   XTN_RC(rb.add(&h.n_rec, e->rec_off + n));
   XTN_RC(rb.add(&h.err, err));
-  // the match vectors need only the encoded keys: they run during the wait
-  XTN_RC(rb.wait([&] {
-    if (peq) launch_peq(e->keys, e->lens, n, peq, s);
-  }));
+  XTN_RC(rb.wait());
   if (h.err) return map_device_err(h.err);
   e->n_rec = h.n_rec;
   if (!allow_large && h.n_rec >= (1ull << 32)) return XTN_ERR_TOO_LARGE;
@@ -584,8 +586,7 @@ int encode_and_count(const DevSeqs& in, int d, Arena& ar, uint32_t* err, cudaStr
 // Paired receptors: both chains encoded, the canonical variant counts of the
 // joined strings (the token never deleted) and their record offsets.
 int encode_and_count_paired(const DevSeqs& a, const DevSeqs& b, int d, Arena& ar, uint32_t* err,
-                            cudaStream_t s, Encoded* e, uint32_t* peq = nullptr,
-                            uint32_t* peq_b = nullptr) {
+                            cudaStream_t s, Encoded* e) {
   const int64_t n = a.n;
   e->keys = ar.get<Key128>(n);
   e->lens = ar.get<uint8_t>(n);
@@ -593,12 +594,14 @@ int encode_and_count_paired(const DevSeqs& a, const DevSeqs& b, int d, Arena& ar
   e->keys_b = ar.get<Key128>(n);
   e->lens_b = ar.get<uint8_t>(n);
   e->eq_b = ar.get<uint32_t>(n);
+  e->rows = ar.get<PlaneRow>(n);
+  e->rows_b = ar.get<PlaneRow>(n);
   uint32_t* vcount = ar.get<uint32_t>(n);
   e->rec_off = ar.get<uint64_t>(n + 1);
   uint64_t* status = ar.get<uint64_t>(scan_status_bytes(n) / 8 + 1);
   XTN_ALLOC_OK(ar);
-  launch_encode(a.seqs, a.off, n, d, e->keys, e->lens, e->eqprev, vcount, err, s);
-  launch_encode(b.seqs, b.off, n, d, e->keys_b, e->lens_b, e->eq_b, vcount, err, s);
+  launch_encode(a.seqs, a.off, n, d, e->keys, e->lens, e->eqprev, vcount, e->rows, err, s);
+  launch_encode(b.seqs, b.off, n, d, e->keys_b, e->lens_b, e->eq_b, vcount, e->rows_b, err, s);
   launch_paired_counts(e->lens, e->eqprev, e->lens_b, e->eq_b, n, d, vcount, s);
   launch_scan_counts(vcount, n, e->rec_off, status, err, s);
   XTN_CK(cudaGetLastError());
@@ -609,10 +612,7 @@ int encode_and_count_paired(const DevSeqs& a, const DevSeqs& b, int d, Arena& ar
   ReadBack rb(s);
   XTN_RC(rb.add(&h.n_rec, e->rec_off + n));
   XTN_RC(rb.add(&h.err, err));
-  XTN_RC(rb.wait([&] {
-    if (peq) launch_peq(e->keys, e->lens, n, peq, s);
-    if (peq_b) launch_peq(e->keys_b, e->lens_b, n, peq_b, s);
-  }));
+  XTN_RC(rb.wait());
   if (h.err) return map_device_err(h.err);
   e->n_rec = h.n_rec;
   if (h.n_rec >= (1ull << 32)) return XTN_ERR_TOO_LARGE;
@@ -834,36 +834,30 @@ size_t back_status_bytes(uint64_t cand_cap, int cfg) {
 // *n_rows receives the row count.
 int launch_sort_unique(uint64_t* surv, uint64_t* tmp, uint64_t cap, const uint64_t* n_dev,
                        uint32_t pair_bits, uint32_t j_bits, uint32_t* hist, uint64_t* digit_base,
-                       uint64_t* status, const uint32_t* peq_i, const uint8_t* lens_i,
-                       uint64_t n_i, const Key128* keys_j, const uint8_t* lens_j, uint64_t n_j,
-                       int metric, xtn_triple* rows, int64_t row_cap, uint32_t* err,
-                       uint64_t* n_rows, cudaStream_t s, int cfg,
-                       const SecondChain& sc = SecondChain()) {
+                       uint64_t* status, const PairSide& si, const PairSide& sj, int d, int metric,
+                       xtn_triple* rows, int64_t row_cap, uint32_t* err, uint64_t* n_rows,
+                       cudaStream_t s, int cfg) {
   uint64_t* sorted = nullptr;
   XTN_CK(radix_sort_passes(surv, tmp, (int64_t)cap, 0, (int)pair_bits, hist, digit_base, status,
                            cfg, err, &sorted, "k_onesweep_pairs", s, false, n_dev, nullptr,
                            onesweep_unstable_config(cfg)));
-  launch_unique_finalize(sorted, (int64_t)cap, n_dev, j_bits, peq_i, lens_i, n_i, keys_j, lens_j,
-                         n_j, metric, rows, row_cap, status, err, n_rows, s, sc,
-                         pair_bits + 8 <= 64 ? (int)pair_bits : 0);
+  launch_unique_finalize(sorted, (int64_t)cap, n_dev, j_bits, si, sj, d, metric, rows, row_cap,
+                         status, err, n_rows, s, pair_bits + 8 <= 64 ? (int)pair_bits : 0);
   XTN_CK(cudaGetLastError());
   return XTN_OK;
 }
 
 int launch_back(const BackStage& b, uint64_t cand_cap, const uint64_t* n_cand_dev,
-                uint32_t pair_bits, uint32_t j_bits, const uint32_t* peq_i, const uint8_t* lens_i,
-                uint64_t n_i, const Key128* keys_j, const uint8_t* lens_j, uint64_t n_j,
+                uint32_t pair_bits, uint32_t j_bits, const PairSide& si, const PairSide& sj,
                 const uint32_t* seq_rep, int self_mode, int d, xtn_triple* rows, int64_t row_cap,
-                int sms, uint32_t* err, cudaStream_t s, int cfg, int metric = 0,
-                const SecondChain& sc = SecondChain()) {
+                int sms, uint32_t* err, cudaStream_t s, int cfg, int metric = 0) {
   XTN_CK(cudaMemsetAsync(b.hist, 0, MAX_PASSES * RADIX * 4, s));
   XTN_CK(cudaMemsetAsync(b.counters, 0, 16, s));
-  launch_verify_candidates(b.P1, cand_cap, n_cand_dev, j_bits, peq_i, lens_i, n_i, keys_j, lens_j,
-                           n_j, seq_rep, self_mode, d, metric, b.P2, cand_cap, b.counters, b.hist,
-                           (int)pair_bits, sms, err, s, sc);
+  launch_verify_candidates(b.P1, cand_cap, n_cand_dev, j_bits, si, sj, seq_rep, self_mode, d,
+                           metric, b.P2, cand_cap, b.counters, b.hist, (int)pair_bits, sms, err, s);
   return launch_sort_unique(b.P2, b.P1, cand_cap, b.counters, pair_bits, j_bits, b.hist,
-                            b.digit_base, b.status, peq_i, lens_i, n_i, keys_j, lens_j, n_j, metric,
-                            rows, row_cap, err, b.counters + 1, s, cfg, sc);
+                            b.digit_base, b.status, si, sj, d, metric, rows, row_cap, err,
+                            b.counters + 1, s, cfg);
 }
 
 // Result rows go to `out` directly when it is device memory; otherwise into
@@ -1090,14 +1084,13 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   gs0.bucket_start = ar.get<uint64_t>(bucket_start_words(P, hs, mode0 == 2 ? 2 : 1));
   gs0.flags = ar.get<uint64_t>(group_flag_words((int64_t)P));
   gs0.gstatus = ar.get<uint64_t>(gst / 8 + 1);
-  uint32_t* peq = ar.get<uint32_t>((size_t)n * PEQ_STRIDE);
   XTN_ALLOC_OK(ar);
   GrowBuf cand(s), surv(s);
   if (!cand.reserve(std::max<uint64_t>(P / 2, 1u << 20), 0) ||
       !surv.reserve(std::max<uint64_t>((uint64_t)n, 1u << 20), 0))
     return XTN_ERR_OOM;
   XTN_CK(cudaMemsetAsync(phist, 0, MAX_PASSES * RADIX * 4, s));
-  launch_peq(e.keys, e.lens, n, peq, s);
+  const PairSide side = e.side(n);
   const uint32_t pair_bits = 2 * id_bits;
 
   int64_t passes_run = 0;
@@ -1197,9 +1190,9 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
         launch_emit_pairs(sorted, n_flagged, S, pair_off, (int64_t)h.groups, nullptr, h.pairs,
                           id_bits, cand.p + h.direct, nullptr, nullptr, sms, err, s);
       if (n_pairs)
-        launch_verify_candidates(cand.p, n_pairs, nullptr, id_bits, peq, e.lens, (uint64_t)n,
-                                 e.keys, e.lens, (uint64_t)n, seq_rep, between ? 2 : 1, d, metric,
-                                 surv.p, surv.cap, ctr + 5, phist, (int)pair_bits, sms, err, s);
+        launch_verify_candidates(cand.p, n_pairs, nullptr, id_bits, side, side, seq_rep,
+                                 between ? 2 : 1, d, metric, surv.p, surv.cap, ctr + 5, phist,
+                                 (int)pair_bits, sms, err, s);
       XTN_CK(cudaGetLastError());
       break;
     }
@@ -1225,8 +1218,8 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   rc = prepare_out(out, cap, f.survivors, ar, &o);
   if (rc) return rc;
   rc = launch_sort_unique(surv.p, tmp.p, f.survivors, nullptr, pair_bits, id_bits, phist,
-                          digit_base, pstatus, peq, e.lens, (uint64_t)n, e.keys, e.lens,
-                          (uint64_t)n, metric, o.dev, o.dev_cap, err, ctr + 6, s, cfg_pairs);
+                          digit_base, pstatus, side, side, d, metric, o.dev, o.dev_cap, err,
+                          ctr + 6, s, cfg_pairs);
   if (rc) return rc;
   uint64_t rows = 0;
   XTN_CK(cudaMemcpyAsync(&rows, ctr + 6, 8, cudaMemcpyDeviceToHost, s));
@@ -1283,14 +1276,10 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     if (rc) return rc;
   }
 
-  // front: encode (read back the record count; the match vectors are
-  // computed meanwhile), expand, sort, group, offsets
-  uint32_t* peq = ar.get<uint32_t>((size_t)n * PEQ_STRIDE);
-  uint32_t* peq_b = paired ? ar.get<uint32_t>((size_t)n * PEQ_STRIDE) : nullptr;
-  XTN_ALLOC_OK(ar);
+  // front: encode (read back the record count), expand, group
   Encoded e;
-  rc = paired ? encode_and_count_paired(in, in_b, d, ar, err, s, &e, peq, peq_b)
-              : encode_and_count(in, d, ar, err, s, &e, false, peq);
+  rc = paired ? encode_and_count_paired(in, in_b, d, ar, err, s, &e)
+              : encode_and_count(in, d, ar, err, s, &e);
   if (rc == XTN_ERR_TOO_LARGE && !paired) {  // 2^32 records or more: search in passes
     ar.release();
     return search_stream_impl(seqs, offsets, n, d, rep_offsets, n_rep, metric, between, 0, out,
@@ -1397,19 +1386,11 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   if (h.pairs)
     launch_emit_pairs(so.rec, n_flagged, S, pair_off, (int64_t)h.groups, nullptr, h.pairs,
                       so.id_bits, b.P1 + h.direct, nullptr, nullptr, sms, err, s);
-  SecondChain sc;
-  if (paired) {
-    sc.peq_i = peq_b;
-    sc.lens_i = e.lens_b;
-    sc.keys_j = e.keys_b;
-    sc.lens_j = e.lens_b;
-  }
   OutRows o;
   rc = prepare_out(out, cap, n_pairs, ar, &o);
   if (rc) return rc;
-  rc = launch_back(b, n_pairs, nullptr, 2 * so.id_bits, so.id_bits, peq, e.lens, n, e.keys, e.lens,
-                   n, seq_rep, between ? 2 : 1, d, o.dev, o.dev_cap, sms, err, s, cfg_pairs,
-                   metric, sc);
+  rc = launch_back(b, n_pairs, nullptr, 2 * so.id_bits, so.id_bits, e.side(n), e.side(n), seq_rep,
+                   between ? 2 : 1, d, o.dev, o.dev_cap, sms, err, s, cfg_pairs, metric);
   if (rc) return rc;
   ReadBack rb(s);
   XTN_RC(rb.add(&h.pairs, b.counters + 1));
@@ -1433,8 +1414,7 @@ struct xtn_index {
   uint32_t id_bits = 0;
   int hs = 0;
   int dir_bits = 0;
-  xtn::Key128* keys = nullptr;
-  uint8_t* lens = nullptr;
+  xtn::PlaneRow* rows = nullptr;
   uint64_t* rec = nullptr;
   uint32_t* dir = nullptr;
   int64_t bytes = 0;
@@ -1484,10 +1464,9 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     while (db < 28 && db < so.hs && ((uint64_t)1 << (db + 2)) < e.n_rec) ++db;
     idx->dir_bits = db;
   }
-  const size_t b_keys = n * sizeof(Key128), b_lens = n, b_rec = e.n_rec * 8,
+  const size_t b_rows = n * sizeof(PlaneRow), b_rec = e.n_rec * 8,
                b_dir = ((size_t(1) << idx->dir_bits) + 1) * 4;
-  bool ok = cudaMalloc(&idx->keys, b_keys) == cudaSuccess &&
-            cudaMalloc(&idx->lens, b_lens + 16) == cudaSuccess &&
+  bool ok = cudaMalloc(&idx->rows, b_rows) == cudaSuccess &&
             cudaMalloc(&idx->rec, b_rec + 8) == cudaSuccess &&
             cudaMalloc(&idx->dir, b_dir) == cudaSuccess;
   if (!ok) {
@@ -1495,9 +1474,8 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     xtn_index_free(idx);
     return XTN_ERR_OOM;
   }
-  idx->bytes = (int64_t)(b_keys + b_lens + b_rec + b_dir);
-  bool cp = cudaMemcpyAsync(idx->keys, e.keys, b_keys, cudaMemcpyDeviceToDevice, s) == cudaSuccess &&
-            cudaMemcpyAsync(idx->lens, e.lens, b_lens, cudaMemcpyDeviceToDevice, s) == cudaSuccess &&
+  idx->bytes = (int64_t)(b_rows + b_rec + b_dir);
+  bool cp = cudaMemcpyAsync(idx->rows, e.rows, b_rows, cudaMemcpyDeviceToDevice, s) == cudaSuccess &&
             cudaMemcpyAsync(idx->rec, so.rec, b_rec, cudaMemcpyDeviceToDevice, s) == cudaSuccess;
   uint64_t* groups = ar.get<uint64_t>(1);
   if (!groups) cp = false;
@@ -1588,18 +1566,16 @@ int search_query_impl(const xtn_index* idx, const uint8_t* q_seqs, const int64_t
   const int cfg_pairs = g_cfg_pairs.load();
   b.status = ar.get<uint64_t>(back_status_bytes(n_cand, cfg_pairs) / 8 + 1);
   b.counters = ar.get<uint64_t>(2);
-  uint32_t* peq = ar.get<uint32_t>((size_t)n_q * PEQ_STRIDE);
   XTN_ALLOC_OK(ar);
   launch_query_emit(idx->rec, idx->n_rec, idx->id_bits, qv_start, qv_q, cand_off, n_qv, n_cand,
                     b.P1, sms, err, s);
-  launch_peq(e.keys, e.lens, n_q, peq, s);
   XTN_CK(cudaGetLastError());
   OutRows o;
   rc = prepare_out(out, cap, n_cand, ar, &o);
   if (rc) return rc;
-  rc = launch_back(b, n_cand, nullptr, pair_bits, idx->id_bits, peq, e.lens, (uint64_t)n_q,
-                   idx->keys, idx->lens, (uint64_t)idx->n, nullptr, 0, idx->d, o.dev, o.dev_cap,
-                   sms, err, s, cfg_pairs, metric);
+  rc = launch_back(b, n_cand, nullptr, pair_bits, idx->id_bits, e.side(n_q),
+                   PairSide{idx->rows, nullptr, (uint64_t)idx->n}, nullptr, 0, idx->d, o.dev,
+                   o.dev_cap, sms, err, s, cfg_pairs, metric);
   if (rc) return rc;
   struct {
     uint64_t rows;
@@ -1634,7 +1610,7 @@ int tcrdist_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, const x
   rc = stage_seqs(seqs, offsets, n, ar, s, &in);
   if (rc) return rc;
   Encoded e;
-  rc = encode_and_count(in, 0, ar, err, s, &e);
+  rc = encode_and_count(in, 0, ar, err, s, &e, false, false);
   if (rc) return rc;
   const xtn_triple* d_in = in_rows;
   if (!is_device_ptr(in_rows)) {
@@ -1686,7 +1662,8 @@ struct xtn_plan {
   uint32_t* seq_rep = nullptr;
   xtn::Key128* keys = nullptr;
   uint8_t* lens = nullptr;
-  uint32_t *eqprev = nullptr, *vcount = nullptr, *hist = nullptr, *peq = nullptr, *err = nullptr;
+  uint32_t *eqprev = nullptr, *vcount = nullptr, *hist = nullptr, *err = nullptr;
+  xtn::PlaneRow* planes = nullptr;
   uint64_t *rec_off = nullptr, *A = nullptr, *B = nullptr, *digit_base = nullptr;
   uint64_t *status = nullptr, *flags = nullptr, *counters = nullptr;
   uint32_t *S = nullptr, *E = nullptr;
@@ -1780,7 +1757,7 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   p->part.count = p->alloc<uint32_t>(parted ? shape.counts() : 1);
   p->counters = p->alloc<uint64_t>(4);
   p->err = p->alloc<uint32_t>(4);
-  p->peq = p->alloc<uint32_t>((size_t)n * PEQ_STRIDE);
+  p->planes = p->alloc<PlaneRow>(n);
   p->back.P1 = p->alloc<uint64_t>(p->pair_cap + 8);
   p->back.P2 = p->alloc<uint64_t>(p->pair_cap + 8);
   p->back.hist = p->alloc<uint32_t>(MAX_PASSES * RADIX);
@@ -1790,7 +1767,7 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   p->rows = p->alloc<xtn_triple>(p->pair_cap);
   if (rep_offsets) p->seq_rep = p->alloc<uint32_t>(n);
   bool ok = p->rows && p->back.counters && p->back.status && p->back.digit_base && p->back.hist &&
-            p->back.P2 && p->back.P1 && p->peq && p->err && p->counters && p->flags && p->status &&
+            p->back.P2 && p->back.P1 && p->planes && p->err && p->counters && p->flags && p->status &&
             p->bucket_start && p->part.count &&
             (!parted || p->part.kept) && p->digit_base && p->hist && p->B && p->A && p->rec_off && p->vcount && p->eqprev &&
             p->lens && p->keys && p->off && (!rep_offsets || p->seq_rep);
@@ -1840,7 +1817,8 @@ int plan_run_impl(xtn_plan* p, const uint8_t* seqs, cudaStream_t s) {
   XTN_CK(init_err(p->err, s));
   XTN_CK(cudaMemsetAsync(p->counters, 0, 32, s));
   XTN_CK(cudaMemsetAsync(p->hist, 0, MAX_PASSES * RADIX * 4, s));
-  launch_encode(seqs, p->off, n, p->d, p->keys, p->lens, p->eqprev, p->vcount, p->err, s);
+  launch_encode(seqs, p->off, n, p->d, p->keys, p->lens, p->eqprev, p->vcount, p->planes,
+                p->err, s);
   launch_scan_counts(p->vcount, n, p->rec_off, p->status, p->err, s);
   uint64_t* sorted = nullptr;
   const uint64_t* n_rec = p->rec_off + n;  // known on the device only
@@ -1883,11 +1861,11 @@ int plan_run_impl(xtn_plan* p, const uint8_t* seqs, cudaStream_t s) {
   launch_emit_pairs(sorted, p->rec_cap, p->S, p->pair_off, (int64_t)p->g_cap, p->counters,
                     p->pair_cap, p->id_bits, p->back.P1, direct ? p->counters + 2 : nullptr,
                     p->counters + 1, p->sms, p->err, s);
-  launch_peq(p->keys, p->lens, n, p->peq, s);
   XTN_CK(cudaGetLastError());
-  return launch_back(p->back, p->pair_cap, p->counters + 1, 2 * p->id_bits, p->id_bits, p->peq,
-                     p->lens, (uint64_t)n, p->keys, p->lens, (uint64_t)n, p->seq_rep, 1, p->d,
-                     p->rows, (int64_t)p->pair_cap, p->sms, p->err, s, p->cfg_pair);
+  const PairSide side{p->planes, nullptr, (uint64_t)n};
+  return launch_back(p->back, p->pair_cap, p->counters + 1, 2 * p->id_bits, p->id_bits, side, side,
+                     p->seq_rep, 1, p->d, p->rows, (int64_t)p->pair_cap, p->sms, p->err, s,
+                     p->cfg_pair);
 }
 
 int plan_result_impl(xtn_plan* p, xtn_triple* out, int64_t cap, int64_t* n_out, cudaStream_t s) {
@@ -1986,8 +1964,7 @@ int xtn_index_build(const uint8_t* seqs, const int64_t* offsets, int64_t n, int 
 
 int xtn_index_free(xtn_index* idx) {
   if (!idx) return XTN_OK;
-  cudaFree(idx->keys);
-  cudaFree(idx->lens);
+  cudaFree(idx->rows);
   cudaFree(idx->rec);
   cudaFree(idx->dir);
   delete idx;
@@ -2057,7 +2034,7 @@ int xtn_search_query_scratch(const xtn_index* idx, const int64_t* q_offsets, int
   b += n * (16 + 1 + 4 + 4) + 8 * (n + 1) + scan_status_bytes((int64_t)n);  // encode
   b += n_qv * 12 + 8 * (n_qv + 1) + scan_status_bytes((int64_t)n_qv);      // lookup
   b += 16 * (n_cand + 8) + MAX_PASSES * RADIX * 12 + 16;             // candidate words
-  b += back_status_bytes(n_cand, cfg) + n * 4 * PEQ_STRIDE;          // sort, match vectors
+  b += back_status_bytes(n_cand, cfg) + 32 * n;                      // sort, bit planes
   b += 12 * n_cand;                                                  // rows for host output
   b += 24 * per_buffer;
   *bytes = (int64_t)b;

@@ -4,16 +4,14 @@
 //
 //   k_encode : ASCII sequence -> 128-bit key of 5-bit residue codes
 //              (Appendix "Compression of TCR sequences"), its length, the
-//              mask of positions equal to their left neighbour, and its
+//              mask of positions equal to their left neighbour, the bit
+//              planes of its codes (for the distance, k_verify.cu), and its
 //              number of canonical deletion subsets (expand.cuh).
 //   k_expand : the records  fingerprint[63:b] | id[b-1:0]  of every canonical
 //              deletion variant, at rec_off (see expand.cuh).  The kernel also
 //              accumulates the digit histograms of the radix passes that will
 //              sort the records (all of them, or only the first when each
 //              sort pass counts the next).
-//   k_peq    : per sequence, for each residue code c, the bit mask of the
-//              positions holding c (the match vectors of the bit-parallel
-//              edit distance used in verification).
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -37,17 +35,30 @@ __device__ __forceinline__ uint32_t letter_code(uint32_t ch) {
 }
 
 constexpr int ENCODE_WARPS = 8;
+constexpr int ENCODE_SPAN = 32 * XTN_MAX_LEN;       // letters of a warp's sequences, at most
+constexpr int ENCODE_WORDS = ENCODE_SPAN / 4 + 10;  // and the words a lane reads past its own
 
 // One warp per 32 consecutive sequences: their letters form one contiguous
-// byte span, copied to shared memory with coalesced loads; each lane then
-// encodes its own sequence.  Offsets are validated per lane first; a warp
-// with an invalid offset reads each valid lane's letters directly instead.
+// byte span, copied to shared memory four at a time; each lane then takes its
+// own sequence as unaligned words, letter by letter through a 256-byte table
+// (letters lie in different banks).  Six residues at a time are spread to
+// five fields, one per code bit (one multiply and a mask each), which become
+// the bit planes the distance needs; the equal-neighbour mask and the check
+// for bad letters come from the planes.  About 250 instructions a sequence,
+// against 500 for a loop over its letters and a match-vector kernel behind it
+// (46 + 31 us for 1M sequences; 353 + 237 us for 10M).  Offsets are validated
+// per lane first; a warp with an invalid offset reads each valid lane's
+// letters directly instead.
 __global__ void __launch_bounds__(ENCODE_WARPS * 32)
     k_encode(const uint8_t* __restrict__ seqs, const int64_t* __restrict__ off, int64_t n, int d,
              Key128* __restrict__ keys, uint8_t* __restrict__ lens,
              uint32_t* __restrict__ eqprev_out, uint32_t* __restrict__ vcount,
-             uint32_t* __restrict__ err) {
-  __shared__ uint8_t s_bytes[ENCODE_WARPS][32 * XTN_MAX_LEN];
+             PlaneRow* __restrict__ rows, uint32_t* __restrict__ err) {
+  __shared__ uint32_t s_words[ENCODE_WARPS][ENCODE_WORDS];
+  __shared__ uint8_t s_code[256];
+  static_assert(ENCODE_WARPS * 32 == 256, "one table entry per thread");
+  s_code[threadIdx.x] = (uint8_t)letter_code(threadIdx.x);
+  __syncthreads();
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
   const int64_t s0 = ((int64_t)blockIdx.x * ENCODE_WARPS + warp) * 32;
   if (s0 >= n) return;  // whole warp
@@ -65,37 +76,81 @@ __global__ void __launch_bounds__(ENCODE_WARPS * 32)
   const bool all_ok = __all_sync(FULL_MASK, ok || !in);
   const int last = (int)((n - s0 < 32) ? (n - s0 - 1) : 31);
   const int64_t A = __shfl_sync(FULL_MASK, a, 0), Bend = __shfl_sync(FULL_MASK, b, last);
-  uint8_t* buf = s_bytes[warp];
-  const bool shared_span = all_ok && Bend - A <= 32 * XTN_MAX_LEN;
-  if (shared_span) {
-    for (int64_t k = lane; k < Bend - A; k += 32) buf[k] = seqs[A + k];
+  const uint32_t L = ok ? (uint32_t)(b - a) : 0u;
+  uint32_t w[7];  // the sequence's letters, zeros behind them
+  if (all_ok && Bend - A <= ENCODE_SPAN) {
+    // byte k of the span sits at byte head + k of s_words, so that whole
+    // words of the input land on whole words here
+    const uint8_t* src = seqs + A;
+    const uint32_t head = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 3u);
+    const uint32_t bytes = head + (uint32_t)(Bend - A);
+    uint8_t* dst = reinterpret_cast<uint8_t*>(s_words[warp]);
+    const uint32_t w0 = head ? 1u : 0u, w1 = bytes / 4;  // whole words [w0, w1)
+    const uint32_t* src4 = reinterpret_cast<const uint32_t*>(src - head);
+    for (uint32_t k = w0 + lane; k < w1; k += 32) s_words[warp][k] = src4[k];
+    if (head && lane >= head && lane < 4 && lane < bytes) dst[lane] = src[lane - head];
+    const uint32_t tail = max(w0, w1) * 4 + lane;
+    if (lane < 4 && tail < bytes) dst[tail] = src[tail - head];
+    __syncwarp();
+    const uint32_t o = head + (uint32_t)(a - A);
+    const uint32_t sh = 8u * (o & 3u);
+    const uint32_t* mine = s_words[warp] + (ok ? o / 4 : 0u);
+    uint32_t lo = mine[0];
+#pragma unroll
+    for (int t = 0; t < 7; ++t) {
+      const uint32_t hi = mine[t + 1];
+      w[t] = __funnelshift_r(lo, hi, sh);
+      lo = hi;
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < 7; ++t) w[t] = 0;
+#pragma unroll
+    for (int p = 0; p < XTN_MAX_LEN; ++p)
+      if ((uint32_t)p < L) w[p / 4] |= (uint32_t)seqs[a + p] << (8 * (p % 4));
   }
-  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < 7; ++t) {  // clear what lies past the end
+    const int left = (int)L - 4 * t;
+    w[t] = left >= 4 ? w[t] : left > 0 ? w[t] & (0xffffffffu >> (32 - 8 * left)) : 0u;
+  }
   Key128 key{0ull, 0ull};
-  uint32_t L = 0, eqprev = 0;
-  if (ok) {
-    L = (uint32_t)(b - a);
-    uint32_t prev = 0;
-    for (uint32_t p = 0; p < L; ++p) {
-      const uint32_t ch = shared_span ? buf[a - A + p] : seqs[a + p];
-      const uint32_t c = letter_code(ch);
-      if (c == 0) atomicOr(err, DERR_BAD_RESIDUE);
-      if (p > 0 && c == prev) eqprev |= 1u << p;
-      prev = c;
-      const uint32_t m = 5 * p;
-      if (m < 64) {
-        key.lo |= (uint64_t)c << m;
-        if (m > 59) key.hi |= (uint64_t)c >> (64 - m);
-      } else {
-        key.hi |= (uint64_t)c << (m - 64);
+  uint32_t plane[5] = {0u, 0u, 0u, 0u, 0u};
+  const uint32_t longest = __reduce_max_sync(FULL_MASK, L);
+#pragma unroll
+  for (int g = 0; g < 5; ++g) {
+    if ((uint32_t)(6 * g) >= longest) break;  // warp-uniform
+    uint32_t acc = 0;  // five fields of six bits, the code's bits 0 .. 4
+#pragma unroll
+    for (int x = 0; x < 6; ++x) {
+      const int p = 6 * g + x;
+      acc >>= 1;
+      if (p < XTN_MAX_LEN) {
+        const uint32_t c = s_code[(w[p / 4] >> (8 * (p % 4))) & 255u];
+        acc |= (c * 0x02108420u) & 0x20820820u;  // bit b of c to bit 6 b + 5
+        if (5 * p < 64) key.lo |= (uint64_t)c << (5 * p < 64 ? 5 * p : 0);
+        if (5 * p > 59) key.hi |= 5 * p < 64 ? (uint64_t)c >> (64 - 5 * p) : (uint64_t)c << (5 * p - 64);
       }
     }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) plane[k] |= ((acc >> (6 * k)) & 63u) << (6 * g);
   }
+  const uint32_t all = L ? 0xffffffffu >> (32 - L) : 0u;
+  if ((plane[0] | plane[1] | plane[2] | plane[3] | plane[4]) != all)
+    atomicOr(err, DERR_BAD_RESIDUE);  // a letter without a code
+  uint32_t differs = 1u;  // from the left neighbour
+#pragma unroll
+  for (int k = 0; k < 5; ++k) differs |= plane[k] ^ (plane[k] << 1);
+  const uint32_t eqprev = ~differs & all;
   if (in) {
     keys[i] = key;
     lens[i] = (uint8_t)L;
     eqprev_out[i] = eqprev;
     vcount[i] = canonical_total(eqprev, L, d);
+    if (rows) {
+      rows[i].a = make_uint4(plane[0], plane[1], plane[2], plane[3]);
+      rows[i].b = make_uint4(plane[4], L, 0u, 0u);
+    }
   }
 }
 
@@ -315,34 +370,6 @@ __global__ void __launch_bounds__(EXPAND_THREADS, 4)
     if (S.hist[k]) atomicAdd(&dst[k], S.hist[k]);
 }
 
-// Match vectors: peq[i * PEQ_STRIDE + c - 1] = {positions p of sequence i with code c}.
-constexpr int PEQ_THREADS = 128;
-
-__global__ void __launch_bounds__(PEQ_THREADS)
-    k_peq(const Key128* __restrict__ keys, const uint8_t* __restrict__ lens, int64_t n,
-          uint32_t* __restrict__ peq) {
-  __shared__ uint32_t s_peq[PEQ_THREADS * PEQ_STRIDE];
-  const int64_t first = (int64_t)blockIdx.x * PEQ_THREADS;
-  for (int k = threadIdx.x; k < PEQ_THREADS * PEQ_STRIDE; k += PEQ_THREADS) s_peq[k] = 0;
-  __syncthreads();
-  const int64_t i = first + threadIdx.x;
-  if (i < n) {
-    Key128 k = keys[i];
-    const uint32_t L = lens[i];
-    uint32_t* row = s_peq + threadIdx.x * PEQ_STRIDE;
-    for (uint32_t p = 0; p < L; ++p) {
-      const uint32_t c = (uint32_t)(k.lo & 31u);
-      k.lo = (k.lo >> 5) | (k.hi << 59);
-      k.hi >>= 5;
-      if (c >= 1 && c <= 20) row[c - 1] |= 1u << p;
-    }
-  }
-  __syncthreads();
-  const int64_t rows = (n - first < PEQ_THREADS) ? (n - first) : PEQ_THREADS;
-  for (int64_t k = threadIdx.x; k < rows * PEQ_STRIDE; k += PEQ_THREADS)
-    peq[first * PEQ_STRIDE + k] = s_peq[k];
-}
-
 // seq_rep[i] = repertoire of sequence i: the last r with rep_off[r] <= i.
 __global__ void k_seq_rep(const int64_t* __restrict__ rep_off, int64_t n_rep,
                           uint32_t* __restrict__ seq_rep, int64_t n) {
@@ -365,13 +392,13 @@ void launch_seq_rep(const int64_t* rep_off, int64_t n_rep, uint32_t* seq_rep, in
 }
 
 void launch_encode(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Key128* keys,
-                   uint8_t* lens, uint32_t* eqprev, uint32_t* vcount, uint32_t* err,
-                   cudaStream_t s) {
+                   uint8_t* lens, uint32_t* eqprev, uint32_t* vcount, PlaneRow* rows,
+                   uint32_t* err, cudaStream_t s) {
   if (n <= 0) return;
-  prof_begin(s, "k_encode", (double)n * (16 + 16 + 1 + 4 + 4 + 8));
+  prof_begin(s, "k_encode", (double)n * (16 + 16 + 1 + 4 + 4 + 8 + (rows ? 32 : 0)));
   k_encode<<<div_up_u32(n, ENCODE_WARPS * 32), ENCODE_WARPS * 32, 0, s>>>(seqs, off, n, d, keys,
                                                                            lens, eqprev, vcount,
-                                                                           err);
+                                                                           rows, err);
   prof_end(s);
 }
 
@@ -431,14 +458,6 @@ void launch_expand(const ExpandSource& src, const uint64_t* rec_off, int64_t n, 
   } else {
     go(std::integral_constant<int, VK_D3>{});
   }
-  prof_end(s);
-}
-
-void launch_peq(const Key128* keys, const uint8_t* lens, int64_t n, uint32_t* peq,
-                cudaStream_t s) {
-  if (n <= 0) return;
-  prof_begin(s, "k_peq", (double)n * (17.0 + 4.0 * PEQ_STRIDE));
-  k_peq<<<div_up_u32(n, PEQ_THREADS), PEQ_THREADS, 0, s>>>(keys, lens, n, peq);
   prof_end(s);
 }
 

@@ -21,10 +21,15 @@
 //                         {i, j, dist} rows in order (single-pass compaction
 //                         with decoupled look-back).
 //
-// Edit distance: the bit-vector algorithm of Myers (1999) in the global-
-// distance form of Hyyro (2001).  Pattern i (<= 25 residues) lives in one
-// 32-bit word; its match vectors come from the per-sequence table built by
-// k_peq; the text j is streamed from its packed key, 5 bits per step.
+// Edit distance: only distances up to d <= 3 matter, so instead of a table
+// (or a bit-vector recurrence over every residue of the text) each edit count
+// e = 0 .. d gets the furthest position reached on every diagonal with e edits
+// (Ukkonen 1985; Landau & Vishkin 1989).  With the sequences as bit planes
+// (PlaneRow) the differing positions of a diagonal are one 32-bit word, and
+// sliding along equal residues is one count of trailing zeros.  About 110
+// instructions a pair at d = 2, two row loads and no per-sequence tables,
+// against 450, 16 gathered words and a table of 80 bytes per sequence for the
+// bit-vector form (146 us for the 1M workload's 4.3 M candidates).
 #include <algorithm>
 
 #include "xtn_common.cuh"
@@ -37,92 +42,105 @@ constexpr int VER_ITEMS = 8;
 constexpr int VER_TILE = VER_THREADS * VER_ITEMS;
 static_assert(VER_TILE == VERIFY_TILE, "status sizing in xtn_kernels.h assumes this tile");
 
-// Levenshtein distance between pattern (match vectors peq, length m) and the
-// text held in packed key t (length n <= XTN_MAX_LEN).  All match vectors the
-// text needs are loaded first (independent loads, one latency), then the
-// bit-vector recurrence runs from registers, unrolled over XTN_MAX_LEN steps
-// with the steps past n switched off.
-__device__ __forceinline__ uint32_t edit_distance(const uint32_t* __restrict__ peq, uint32_t m,
-                                                  Key128 t, uint32_t n) {
-  uint32_t eqv[XTN_MAX_LEN];
+struct Planes {
+  uint32_t p[5];
+  uint32_t n;  // length
+};
+
+__device__ __forceinline__ Planes load_planes(const PlaneRow* __restrict__ rows, uint64_t i) {
+  const uint4 a = __ldg(&rows[i].a), b = __ldg(&rows[i].b);
+  return Planes{{a.x, a.y, a.z, a.w, b.x}, b.y};
+}
+
+// Diagonal k = (position in y) - (position in x), -3 <= k <= 3: bit p set
+// where x[p] and y[p + k] differ, and past the diagonal's end, min(m, n - k).
+__device__ __forceinline__ uint32_t diagonal(const Planes& x, const Planes& y, int k) {
+  uint32_t diff = 0;
 #pragma unroll
-  for (int j = 0; j < XTN_MAX_LEN; ++j) {
-    const uint32_t c = (uint32_t)(t.lo & 31u);
-    t.lo = (t.lo >> 5) | (t.hi << 59);
-    t.hi >>= 5;
-    eqv[j] = ((uint32_t)j < n && c - 1u < 20u) ? __ldg(peq + (c - 1u)) : 0u;
-  }
-  if (m == 0) return n;
-  uint32_t pv = (m >= 32) ? ~0u : ((1u << m) - 1u);
-  uint32_t mv = 0;
-  uint32_t score = m;
-  const uint32_t hb = 1u << (m - 1);
+  for (int b = 0; b < 5; ++b) diff |= x.p[b] ^ ((y.p[b] << 3) >> (3 + k));
+  const int end = max(0, min((int)x.n, (int)y.n - k));  // <= 25
+  return diff | (0xffffffffu << end);
+}
+
+// The position reached from p on a diagonal without further edits.
+__device__ __forceinline__ int slide(uint32_t diff, int p) {
+  return p + __ffs((int)(diff >> p)) - 1;  // p <= end: a bit is left
+}
+
+// Levenshtein distance of x and y if it is at most D, else D + 1.
+template <int D>
+__device__ __forceinline__ uint32_t bounded_distance(const Planes& x, const Planes& y) {
+  const int m = (int)x.n, n = (int)y.n, t = n - m;
+  if (t > D || -t > D) return (uint32_t)D + 1u;
+  // f[D + k]: furthest position in x on diagonal k with the edits so far
+  constexpr int NONE = -64;
+  const uint32_t diff0 = diagonal(x, y, 0);
+  int f[2 * D + 1];
 #pragma unroll
-  for (int j = 0; j < XTN_MAX_LEN; ++j) {
-    // a lane leaves after its own text, so a warp runs the steps of its
-    // longest text, not XTN_MAX_LEN
-    if ((uint32_t)j >= n) break;
-    {
-      const uint32_t eq = eqv[j];
-      const uint32_t xv = eq | mv;
-      const uint32_t xh = (((eq & pv) + pv) ^ pv) | eq;
-      uint32_t ph = mv | ~(xh | pv);
-      uint32_t mh = pv & xh;
-      score += (ph & hb) ? 1u : 0u;
-      score -= (mh & hb) ? 1u : 0u;
-      ph = (ph << 1) | 1u;
-      mh <<= 1;
-      pv = mh | ~(xv | ph);
-      mv = ph & xv;
+  for (int k = 0; k < 2 * D + 1; ++k) f[k] = NONE;
+  f[D] = slide(diff0, 0);
+  if (t == 0 && f[D] >= m) return 0u;
+  // from diagonal k's neighbours: a substitution; a residue of x left out
+  // (from k + 1); one of y (from k - 1)
+  auto start = [&](int k) {
+    int p = f[D + k] + 1;
+    if (k < D) p = max(p, f[D + k + 1 <= 2 * D ? D + k + 1 : 0] + 1);
+    if (k > -D) p = max(p, f[D + k - 1 >= 0 ? D + k - 1 : 0]);
+    return min(p, min(m, n - k));
+  };
+  // a diagonal that no path has reached yet, or of no length, gives NONE
+  auto run = [&](int k, int p) {
+    return p >= 0 && p + k >= 0 ? slide(k == 0 ? diff0 : diagonal(x, y, k), p) : NONE;
+  };
+#pragma unroll
+  for (int e = 1; e < D; ++e) {
+    int g[2 * D + 1];
+#pragma unroll
+    for (int k = -D; k <= D; ++k) g[D + k] = k < -e || k > e ? NONE : run(k, start(k));
+    int last = NONE;
+#pragma unroll
+    for (int k = -D; k <= D; ++k) {
+      f[D + k] = g[D + k];
+      if (k == t) last = g[D + k];
     }
+    if (last >= m) return (uint32_t)e;
   }
-  return score;
-}
-
-// Hamming distance (the last step of the Hamming variant, Results) between
-// pattern (match vectors peq) and text t of the same length n: the positions
-// p whose text residue's match vector lacks bit p.
-__device__ __forceinline__ uint32_t hamming_distance(const uint32_t* __restrict__ peq, Key128 t,
-                                                     uint32_t n) {
-  uint32_t match = 0;
+  if (D > 0) {  // the last edit matters on the final diagonal only
+    int p = NONE;
 #pragma unroll
-  for (int j = 0; j < XTN_MAX_LEN; ++j) {
-    const uint32_t c = (uint32_t)(t.lo & 31u);
-    t.lo = (t.lo >> 5) | (t.hi << 59);
-    t.hi >>= 5;
-    if ((uint32_t)j < n && c - 1u < 20u) match |= __ldg(peq + (c - 1u)) & (1u << j);
+    for (int k = -D; k <= D; ++k)
+      if (k == t) p = start(k);
+    if (run(t, p) >= m) return (uint32_t)D;
   }
-  return n - (uint32_t)__popc(match);
+  return (uint32_t)D + 1u;
 }
 
-// The distance of the last step: metric 0 = Levenshtein (<= d needs
-// |m - n| <= d), 1 = Hamming (equal lengths only).  Returns d + 1 for a pair
-// that cannot be within d.
-__device__ __forceinline__ uint32_t pair_distance(int metric, int d,
-                                                  const uint32_t* __restrict__ peq, uint32_t m,
-                                                  Key128 t, uint32_t n) {
-  if (metric == 1) return m == n ? hamming_distance(peq, t, n) : (uint32_t)d + 1u;
-  if ((m > n ? m - n : n - m) > (uint32_t)d) return (uint32_t)d + 1u;
-  return edit_distance(peq, m, t, n);
+__device__ __forceinline__ uint32_t bounded_distance(const Planes& x, const Planes& y, int d) {
+  switch (d) {  // uniform
+    case 0: return bounded_distance<0>(x, y);
+    case 1: return bounded_distance<1>(x, y);
+    case 2: return bounded_distance<2>(x, y);
+    default: return bounded_distance<3>(x, y);
+  }
 }
 
-// Distance of candidate (i, j) for the last step: pair_distance of the one
-// chain, or for paired receptors (metric 2) the sum of both chains' edit
-// distances (a pair with |dLa| + |dLb| > d gets d + 1).  d >= XTN_MAX_LEN
-// asks for the exact distance.
-__device__ __forceinline__ uint32_t cand_distance(int metric, int d,
-                                                  const uint32_t* __restrict__ peq_i,
-                                                  const uint8_t* __restrict__ lens_i,
-                                                  const Key128* __restrict__ keys_j,
-                                                  const uint8_t* __restrict__ lens_j,
-                                                  const SecondChain& sc, uint64_t i, uint64_t j) {
-  if (metric != 2)
-    return pair_distance(metric, d, peq_i + i * PEQ_STRIDE, lens_i[i], keys_j[j], lens_j[j]);
-  const uint32_t ma = lens_i[i], na = lens_j[j], mb = sc.lens_i[i], nb = sc.lens_j[j];
-  const uint32_t gap = (ma > na ? ma - na : na - ma) + (mb > nb ? mb - nb : nb - mb);
-  if (gap > (uint32_t)d) return (uint32_t)d + 1u;
-  return edit_distance(peq_i + i * PEQ_STRIDE, ma, keys_j[j], na) +
-         edit_distance(sc.peq_i + i * PEQ_STRIDE, mb, sc.keys_j[j], nb);
+// Distance of candidate (i, j) for the last step, if it is at most d (else
+// anything above d): metric 0 = Levenshtein, 1 = Hamming (equal lengths
+// only), 2 = the sum of both chains' edit distances (paired receptors).
+__device__ __forceinline__ uint32_t cand_distance(int metric, int d, const PairSide& si,
+                                                  const PairSide& sj, uint64_t i, uint64_t j) {
+  const Planes x = load_planes(si.rows, i), y = load_planes(sj.rows, j);
+  if (metric == 1) {
+    if (x.n != y.n) return (uint32_t)d + 1u;
+    uint32_t diff = 0;
+#pragma unroll
+    for (int b = 0; b < 5; ++b) diff |= x.p[b] ^ y.p[b];
+    return (uint32_t)__popc(diff);
+  }
+  uint32_t dist = bounded_distance(x, y, d);
+  if (metric == 2 && dist <= (uint32_t)d)
+    dist += bounded_distance(load_planes(si.rows_b, i), load_planes(sj.rows_b, j), d);
+  return dist;
 }
 
 template <int THREADS>
@@ -151,14 +169,11 @@ constexpr uint32_t VER_STASH = 256;  // survivor words a warp collects before a 
 
 __global__ void __launch_bounds__(256)
     k_verify_candidates(const uint64_t* __restrict__ cand, uint64_t n_cap,
-                        const uint64_t* __restrict__ n_dev, uint32_t j_bits,
-                        const uint32_t* __restrict__ peq_i, const uint8_t* __restrict__ lens_i,
-                        uint64_t n_i, const Key128* __restrict__ keys_j,
-                        const uint8_t* __restrict__ lens_j, uint64_t n_j,
-                        const uint32_t* __restrict__ seq_rep, int self_mode, int d, int metric,
-                        uint64_t* __restrict__ surv, uint64_t surv_cap,
+                        const uint64_t* __restrict__ n_dev, uint32_t j_bits, PairSide si,
+                        PairSide sj, const uint32_t* __restrict__ seq_rep, int self_mode, int d,
+                        int metric, uint64_t* __restrict__ surv, uint64_t surv_cap,
                         unsigned long long* __restrict__ n_surv, uint32_t* __restrict__ hist,
-                        int hist_hi, uint32_t* __restrict__ err, SecondChain sc) {
+                        int hist_hi, uint32_t* __restrict__ err) {
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   // survivors collect per warp and go out VER_STASH - 31 or more at a time:
   // one reservation on the shared counter per flush, not per 32 candidates
@@ -192,12 +207,12 @@ __global__ void __launch_bounds__(256)
     if (t < n) {
       w = cand[t];
       const uint64_t i = w >> j_bits, j = w & jmask;
-      ok = i < n_i && j < n_j;
+      ok = i < si.n && j < sj.n;
       if (!ok) atomicOr(err, DERR_RANGE);
       if (self_mode) ok = ok && i != j;
       if (ok && seq_rep) ok = (seq_rep[i] == seq_rep[j]) == (self_mode != 2);
       if (ok) {
-        const uint32_t dist = cand_distance(metric, d, peq_i, lens_i, keys_j, lens_j, sc, i, j);
+        const uint32_t dist = cand_distance(metric, d, si, sj, i, j);
         ok = dist <= (uint32_t)d;
         // the distance rides above the pair bits, for the dedup to write it
         if (ok && hist_hi + 8 <= 64) w |= (uint64_t)dist << hist_hi;
@@ -223,32 +238,26 @@ __global__ void __launch_bounds__(256)
 }
 
 void launch_verify_candidates(const uint64_t* cand, uint64_t n, const uint64_t* n_dev,
-                              uint32_t j_bits,
-                              const uint32_t* peq_i, const uint8_t* lens_i, uint64_t n_i,
-                              const Key128* keys_j, const uint8_t* lens_j, uint64_t n_j,
+                              uint32_t j_bits, const PairSide& si, const PairSide& sj,
                               const uint32_t* seq_rep, int self_mode, int d, int metric,
                               uint64_t* surv, uint64_t surv_cap, uint64_t* n_surv, uint32_t* hist,
-                              int hist_hi, int sms, uint32_t* err, cudaStream_t s,
-                              const SecondChain& sc) {
+                              int hist_hi, int sms, uint32_t* err, cudaStream_t s) {
   if (n == 0) return;
   const int blocks = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)sms * 8);
-  prof_begin(s, "k_verify_candidates", (double)n * (8.0 + 2 * 17.0 + 4.0 * 4));
+  prof_begin(s, "k_verify_candidates", (double)n * (8.0 + 2 * 32.0));
   k_verify_candidates<<<blocks, 256, 0, s>>>(
-      cand, n, n_dev, j_bits, peq_i, lens_i, n_i, keys_j, lens_j, n_j, seq_rep, self_mode, d, metric, surv,
-      surv_cap, reinterpret_cast<unsigned long long*>(n_surv), hist, hist_hi, err, sc);
+      cand, n, n_dev, j_bits, si, sj, seq_rep, self_mode, d, metric, surv, surv_cap,
+      reinterpret_cast<unsigned long long*>(n_surv), hist, hist_hi, err);
   prof_end(s);
 }
 
 __global__ void __launch_bounds__(VER_THREADS)
     k_unique_finalize(const uint64_t* __restrict__ pairs, int64_t n_cap,
-                      const uint64_t* __restrict__ n_dev, uint32_t j_bits,
-                      const uint32_t* __restrict__ peq_i, const uint8_t* __restrict__ lens_i,
-                      uint64_t n_i, const Key128* __restrict__ keys_j,
-                      const uint8_t* __restrict__ lens_j, uint64_t n_j,
-                      int metric, xtn_triple* __restrict__ out, int64_t cap,
+                      const uint64_t* __restrict__ n_dev, uint32_t j_bits, PairSide si,
+                      PairSide sj, int d, int metric, xtn_triple* __restrict__ out, int64_t cap,
                       uint64_t* __restrict__ status, uint32_t* __restrict__ ctr,
                       uint32_t* __restrict__ err, uint64_t* __restrict__ total_out,
-                      SecondChain sc, int dist_shift) {
+                      int dist_shift) {
   __shared__ uint32_t s_tile;
   __shared__ uint32_t s_w[VER_THREADS / 32];
   __shared__ uint64_t s_prefix;
@@ -283,14 +292,13 @@ __global__ void __launch_bounds__(VER_THREADS)
       const uint64_t pw = dist_shift ? (w & ((1ull << dist_shift) - 1ull)) : w;
       const uint64_t i = pw >> j_bits, j = pw & jmask;
       ok = w != prev;
-      if (i >= n_i || j >= n_j) {
+      if (i >= si.n || j >= sj.n) {
         atomicOr(err, DERR_RANGE);
         ok = false;
       }
       if (ok)
         dist[it] = dist_shift ? (uint32_t)((w >> dist_shift) & 0xffu)
-                              : cand_distance(metric, 2 * XTN_MAX_LEN, peq_i, lens_i, keys_j,
-                                              lens_j, sc, i, j);
+                              : cand_distance(metric, d, si, sj, i, j);
       word[it] = pw;
     }
     const uint32_t bal = __ballot_sync(FULL_MASK, ok);
@@ -335,20 +343,16 @@ __global__ void __launch_bounds__(VER_THREADS)
 size_t verify_status_bytes(int64_t n) { return verify_status_bytes_for(n); }
 
 void launch_unique_finalize(const uint64_t* pairs, int64_t n, const uint64_t* n_dev,
-                            uint32_t j_bits,
-                            const uint32_t* peq_i, const uint8_t* lens_i, uint64_t n_i,
-                            const Key128* keys_j, const uint8_t* lens_j, uint64_t n_j,
+                            uint32_t j_bits, const PairSide& si, const PairSide& sj, int d,
                             int metric, xtn_triple* out, int64_t cap, uint64_t* status,
-                            uint32_t* err, uint64_t* total, cudaStream_t s,
-                            const SecondChain& sc, int dist_shift) {
+                            uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift) {
   if (n <= 0) return;
   const size_t st = verify_status_bytes(n);
   uint32_t* ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(status) + st - 16);
   cudaMemsetAsync(status, 0, st, s);
   prof_begin(s, "k_unique_finalize", (double)n * 8.0);
   k_unique_finalize<<<std::min<uint32_t>(div_up_u32(n, VER_TILE), 152 * 8), VER_THREADS, 0, s>>>(
-      pairs, n, n_dev, j_bits, peq_i, lens_i, n_i, keys_j, lens_j, n_j, metric, out, cap, status,
-      ctr, err, total, sc, dist_shift);
+      pairs, n, n_dev, j_bits, si, sj, d, metric, out, cap, status, ctr, err, total, dist_shift);
   prof_end(s);
 }
 

@@ -118,7 +118,7 @@ extern "C" int xtn_tcrdist_filter_noalloc(const uint8_t* seqs, const int64_t* of
     cudaGetLastError();
     return XTN_ERR_CUDA;
   }
-  launch_encode(seqs, offsets, n, 0, keys, lens, eq, vcount, err, s);
+  launch_encode(seqs, offsets, n, 0, keys, lens, eq, vcount, nullptr, err, s);
   launch_tcrdist_filter(in, n_in, keys, lens, n, max_score, out, status, err, total, s);
   if (cudaGetLastError() != cudaSuccess) return XTN_ERR_CUDA;
   uint64_t h_total = 0;

@@ -226,6 +226,14 @@ struct Key128 {
   uint64_t lo, hi;
 };
 
+// The same sequence as bit planes: bit p of plane k is bit k of residue p's
+// code (a.x .. a.w planes 0-3, b.x plane 4; b.y the length).  Two sequences'
+// differing positions, on any diagonal, are then a few operations on whole
+// words.  One row is one 32-byte sector.
+struct __align__(32) PlaneRow {
+  uint4 a, b;
+};
+
 // Residue code at position p (0 <= p < 25).
 __device__ __forceinline__ uint32_t code_at(const Key128& k, int p) {
   const int m = 5 * p;

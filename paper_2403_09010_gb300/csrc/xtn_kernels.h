@@ -12,10 +12,10 @@
 namespace xtn {
 
 struct Key128;
+struct PlaneRow;
 
 constexpr int RADIX = 256;       // 8-bit digits
 constexpr int MAX_PASSES = 8;    // 64-bit keys
-constexpr int PEQ_STRIDE = 20;   // match vectors per sequence (one per residue code)
 
 // api.cu: tuning knobs
 std::atomic<int>& cfg_records();
@@ -23,8 +23,8 @@ std::atomic<int>& cfg_pairs();
 
 // k_variants.cu ------------------------------------------------------------
 void launch_encode(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Key128* keys,
-                   uint8_t* lens, uint32_t* eqprev, uint32_t* vcount, uint32_t* err,
-                   cudaStream_t s);
+                   uint8_t* lens, uint32_t* eqprev, uint32_t* vcount, PlaneRow* rows,
+                   uint32_t* err, cudaStream_t s);  // rows may be null
 // Record selection by fingerprint bin, bin = (record >> shift) & mask, for
 // searches that take the records in several passes.  With `append` null the
 // expand kernel only counts records per bin into bin_count[0 .. mask] (mask
@@ -52,8 +52,6 @@ void launch_expand(const ExpandSource& src, const uint64_t* rec_off, int64_t n, 
                    uint32_t* hist, int hist_lo, int hist_hi, int sms, uint32_t* err,
                    cudaStream_t s, const BinSel* sel = nullptr, void* zero = nullptr,
                    size_t zero_bytes = 0);
-void launch_peq(const Key128* keys, const uint8_t* lens, int64_t n, uint32_t* peq,
-                cudaStream_t s);
 void launch_seq_rep(const int64_t* rep_off, int64_t n_rep, uint32_t* seq_rep, int64_t n,
                     cudaStream_t s);
 
@@ -199,18 +197,15 @@ constexpr int VERIFY_TILE = 2048;
 constexpr size_t verify_status_bytes_for(int64_t n) {
   return (size_t)((n + VERIFY_TILE - 1) / VERIFY_TILE) * 8 + 16;
 }
-// Second chains of paired receptors (metric 2, the sum of the two chains'
-// edit distances): match vectors of the i side, keys of the j side and both
-// sides' lengths.  All null for one chain.
-struct SecondChain {
-  const uint32_t* peq_i = nullptr;
-  const uint8_t* lens_i = nullptr;
-  const Key128* keys_j = nullptr;
-  const uint8_t* lens_j = nullptr;
+// The sequences one side of the pairs indexes: their bit planes, and for
+// paired receptors (metric 2) those of their second chains.
+struct PairSide {
+  const PlaneRow* rows = nullptr;
+  const PlaneRow* rows_b = nullptr;
+  uint64_t n = 0;
 };
 // metric: 0 = Levenshtein, 1 = Hamming (pairs of equal length only), 2 =
-// paired chains (Levenshtein of the first chains plus that of the second,
-// which `sc` describes).  Verify writes a survivor's distance into bits
+// paired chains (Levenshtein of the first chains plus that of the second).  Verify writes a survivor's distance into bits
 // [hist_hi, hist_hi + 8) of its word when they exist (hist_hi + 8 <= 64);
 // the dedup then reads it there (dist_shift = hist_hi) instead of computing
 // it again (dist_shift = 0).
@@ -219,20 +214,14 @@ struct SecondChain {
 // between different repertoires.
 size_t verify_status_bytes(int64_t n);
 void launch_verify_candidates(const uint64_t* cand, uint64_t n, const uint64_t* n_dev,
-                              uint32_t j_bits,
-                              const uint32_t* peq_i, const uint8_t* lens_i, uint64_t n_i,
-                              const Key128* keys_j, const uint8_t* lens_j, uint64_t n_j,
+                              uint32_t j_bits, const PairSide& si, const PairSide& sj,
                               const uint32_t* seq_rep, int self_mode, int d, int metric,
                               uint64_t* surv, uint64_t surv_cap, uint64_t* n_surv, uint32_t* hist,
-                              int hist_hi, int sms, uint32_t* err, cudaStream_t s,
-                              const SecondChain& sc = SecondChain());
+                              int hist_hi, int sms, uint32_t* err, cudaStream_t s);
 void launch_unique_finalize(const uint64_t* pairs, int64_t n, const uint64_t* n_dev,
-                            uint32_t j_bits,
-                            const uint32_t* peq_i, const uint8_t* lens_i, uint64_t n_i,
-                            const Key128* keys_j, const uint8_t* lens_j, uint64_t n_j,
+                            uint32_t j_bits, const PairSide& si, const PairSide& sj, int d,
                             int metric, xtn_triple* out, int64_t cap, uint64_t* status,
-                            uint32_t* err, uint64_t* total, cudaStream_t s,
-                            const SecondChain& sc = SecondChain(), int dist_shift = 0);
+                            uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift);
 void launch_tcrdist_filter(const xtn_triple* in, int64_t n, const Key128* keys,
                            const uint8_t* lens, int64_t n_seq, int max_score, xtn_triple* out,
                            uint64_t* status, uint32_t* err, uint64_t* total, cudaStream_t s);
