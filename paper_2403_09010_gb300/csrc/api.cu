@@ -342,13 +342,15 @@ class ReadBack {
   explicit ReadBack(cudaStream_t s) : s_(s) {}
   template <class T>
   int add(T* host, const T* dev) {
-    static_assert(sizeof(T) <= 8, "one word per value");
-    if (n_ == kSlots) return XTN_ERR_CUDA;
+    constexpr int words = (int)((sizeof(T) + 7) / 8);
+    if (n_ == kValues || words_ + words > kWords) return XTN_ERR_CUDA;
     Slot& m = slot();
     if (!m.buf) return XTN_ERR_CUDA;
-    XTN_CK(cudaMemcpyAsync(m.buf + n_, dev, sizeof(T), cudaMemcpyDeviceToHost, s_));
+    XTN_CK(cudaMemcpyAsync(m.buf + words_, dev, sizeof(T), cudaMemcpyDeviceToHost, s_));
     dst_[n_] = host;
+    at_[n_] = words_;
     size_[n_] = sizeof(T);
+    words_ += words;
     ++n_;
     return XTN_OK;
   }
@@ -363,8 +365,8 @@ class ReadBack {
       HostSpan span("host_stream_wait");
       XTN_CK(cudaEventSynchronize(m.ev));
     }
-    for (int k = 0; k < n_; ++k) std::memcpy(dst_[k], m.buf + k, size_[k]);
-    n_ = 0;
+    for (int k = 0; k < n_; ++k) std::memcpy(dst_[k], m.buf + at_[k], size_[k]);
+    n_ = words_ = 0;
     return XTN_OK;
   }
   int wait() {
@@ -372,7 +374,7 @@ class ReadBack {
   }
 
  private:
-  static constexpr int kSlots = 8;
+  static constexpr int kValues = 4, kWords = 16;
   struct Slot {
     uint64_t* buf = nullptr;
     cudaEvent_t ev = nullptr;
@@ -384,7 +386,7 @@ class ReadBack {
     Slot& m = per_device[dev];
     if (!m.buf) {
       void* p = nullptr;
-      if (cudaHostAlloc(&p, kSlots * sizeof(uint64_t), cudaHostAllocPortable) != cudaSuccess)
+      if (cudaHostAlloc(&p, kWords * sizeof(uint64_t), cudaHostAllocPortable) != cudaSuccess)
         return m;
       if (cudaEventCreateWithFlags(&m.ev, cudaEventDisableTiming) != cudaSuccess) {
         cudaFreeHost(p);
@@ -395,9 +397,10 @@ class ReadBack {
     return m;
   }
   cudaStream_t s_;
-  int n_ = 0;
-  void* dst_[kSlots] = {};
-  size_t size_[kSlots] = {};
+  int n_ = 0, words_ = 0;
+  void* dst_[kValues] = {};
+  int at_[kValues] = {};
+  size_t size_[kValues] = {};
 };
 
 // Poll limit of bounded device waits for calls that start from now on (0 =
@@ -406,16 +409,37 @@ std::atomic<uint32_t> g_wait_limit{0};
 
 __global__ void k_set_word(uint32_t* p, uint32_t v) { *p = v; }
 
-// Zero a call's error words (4 x u32) and, when a wait limit is set, put it
-// in the second word, where the look-back waits read it.
-int init_err(uint32_t* err, cudaStream_t s) {
-  XTN_CK(cudaMemsetAsync(err, 0, 16, s));
+// Zero a call's error words (4 x u32; `clear` bytes from there) and, when a
+// wait limit is set, put it in the second word, where the look-back waits
+// read it.
+int init_err(uint32_t* err, cudaStream_t s, size_t clear = 16) {
+  XTN_CK(cudaMemsetAsync(err, 0, clear, s));
   const uint32_t lim = g_wait_limit.load();
   if (lim) {
     k_set_word<<<1, 1, 0, s>>>(err + 1, lim);
     XTN_CK(cudaGetLastError());
   }
   return XTN_OK;
+}
+
+// What a call counts on the device, in one piece with its error words and the
+// status words of its first look-back: one clear at the start, and one copy
+// wherever the host reads any of it (a small call is mostly such pieces).
+struct Control {
+  uint32_t err[4];
+  uint64_t counters[4];  // groups, flagged pairs, direct candidates, flagged records
+  uint64_t n_rec;
+  uint64_t back[2];  // survivors, rows
+};
+
+// *status: status_bytes for the caller, cleared with the rest.
+int take_control(Arena& ar, size_t status_bytes, cudaStream_t s, Control** c, uint64_t** status) {
+  static_assert(sizeof(Control) <= 128, "the status begins at byte 128");
+  uint64_t* p = ar.get<uint64_t>((128 + status_bytes + 7) / 8);
+  XTN_ALLOC_OK(ar);
+  *c = reinterpret_cast<Control*>(p);
+  *status = p + 16;
+  return init_err((*c)->err, s, 128 + status_bytes);
 }
 
 // Read n elements of device memory into host memory and wait for the stream.
@@ -552,32 +576,33 @@ struct Encoded {
   ExpandSource source() const { return ExpandSource{keys, lens, eqprev, keys_b, lens_b, eq_b}; }
 };
 
-// allow_large: return the count even when it is 2^32 or more (the caller
-// then searches in passes); otherwise that is TOO_LARGE.
-int encode_and_count(const DevSeqs& in, int d, Arena& ar, uint32_t* err, cudaStream_t s,
-                     Encoded* e, bool allow_large = false, bool planes = true) {
+// Queues the encoding; the record offsets' total goes to ctl->n_rec.  status:
+// encode_status_bytes(n), cleared.
+int launch_front(const DevSeqs& in, int d, Arena& ar, Control* ctl, uint64_t* status,
+                 cudaStream_t s, Encoded* e) {
   const int64_t n = in.n;
   e->keys = ar.get<Key128>(n);
   e->lens = ar.get<uint8_t>(n);
   e->eqprev = ar.get<uint32_t>(n);
-  uint32_t* vcount = ar.get<uint32_t>(n);
   e->rec_off = ar.get<uint64_t>(n + 1);
-  uint64_t* status = ar.get<uint64_t>(scan_status_bytes(n) / 8 + 1);
+  e->rows = ar.get<PlaneRow>(n);
   XTN_ALLOC_OK(ar);
-  if (planes) e->rows = ar.get<PlaneRow>(n);
-  XTN_ALLOC_OK(ar);
-  launch_encode(in.seqs, in.off, n, d, e->keys, e->lens, e->eqprev, vcount, e->rows, err, s);
-  launch_scan_counts(vcount, n, e->rec_off, status, err, s);
+  launch_encode_scan(in.seqs, in.off, n, d, e->keys, e->lens, e->eqprev, e->rec_off, &ctl->n_rec,
+                     status, e->rows, ctl->err, s);
   XTN_CK(cudaGetLastError());
-  struct {
-    uint64_t n_rec;
-    uint32_t err;
-  } h{0, 0};
+  return XTN_OK;
+}
+
+// allow_large: return the count even when it is 2^32 or more (the caller
+// then searches in passes); otherwise that is TOO_LARGE.
+int encode_and_count(const DevSeqs& in, int d, Arena& ar, Control* ctl, uint64_t* status,
+                     cudaStream_t s, Encoded* e, bool allow_large = false) {
+  XTN_RC(launch_front(in, d, ar, ctl, status, s, e));
+  Control h{};
   ReadBack rb(s);
-  XTN_RC(rb.add(&h.n_rec, e->rec_off + n));
-  XTN_RC(rb.add(&h.err, err));
+  XTN_RC(rb.add(&h, ctl));
   XTN_RC(rb.wait());
-  if (h.err) return map_device_err(h.err);
+  if (h.err[0]) return map_device_err(h.err[0]);
   e->n_rec = h.n_rec;
   if (!allow_large && h.n_rec >= (1ull << 32)) return XTN_ERR_TOO_LARGE;
   return XTN_OK;
@@ -784,6 +809,14 @@ int take_partitions(uint64_t n_rec, Arena& ar, uint64_t* n_spill, cudaStream_t s
 // for the two stages.
 constexpr uint64_t SPLIT_EXPANSION = 6u << 20;
 
+// A self-search whose sequences, were they all of the greatest length, would
+// make at most this many records runs up to its candidates on buffers of that
+// size, without the wait for the record count in between (10 us or so, of a
+// call of 140).  Past the limit the larger buffers' clears and the partitions
+// chosen for too many records would take it back.
+constexpr uint64_t UNREAD_RECORDS = 4u << 20;
+static_assert(UNREAD_RECORDS <= SPLIT_EXPANSION, "the split expansion takes a device count");
+
 // The n spilled records sorted on their hs group-key bits, with group flags.
 int sort_spill(const Partitions& p, uint64_t n, uint32_t id_bits, int hs, int sms, Arena& ar,
                uint32_t* err, cudaStream_t s, Sorted* out) {
@@ -821,6 +854,10 @@ struct BackStage {
   uint64_t* digit_base = nullptr;  // MAX_PASSES * RADIX
   uint64_t* status = nullptr;      // back_status_bytes(cand_cap)
   uint64_t* counters = nullptr;    // 2
+  // one clear for all: hist, status (the sort's) and unique_status lie in
+  // one piece of zero_bytes, and the counters are zero already
+  uint64_t* unique_status = nullptr;
+  size_t zero_bytes = 0;
 };
 
 size_t back_status_bytes(uint64_t cand_cap, int cfg) {
@@ -836,13 +873,15 @@ int launch_sort_unique(uint64_t* surv, uint64_t* tmp, uint64_t cap, const uint64
                        uint32_t pair_bits, uint32_t j_bits, uint32_t* hist, uint64_t* digit_base,
                        uint64_t* status, const PairSide& si, const PairSide& sj, int d, int metric,
                        xtn_triple* rows, int64_t row_cap, uint32_t* err, uint64_t* n_rows,
-                       cudaStream_t s, int cfg) {
+                       cudaStream_t s, int cfg, uint64_t* unique_status = nullptr) {
   uint64_t* sorted = nullptr;
+  const bool zeroed = unique_status != nullptr;  // both status areas are clear
   XTN_CK(radix_sort_passes(surv, tmp, (int64_t)cap, 0, (int)pair_bits, hist, digit_base, status,
                            cfg, err, &sorted, "k_onesweep_pairs", s, false, n_dev, nullptr,
-                           onesweep_unstable_config(cfg)));
+                           onesweep_unstable_config(cfg), zeroed));
   launch_unique_finalize(sorted, (int64_t)cap, n_dev, j_bits, si, sj, d, metric, rows, row_cap,
-                         status, err, n_rows, s, pair_bits + 8 <= 64 ? (int)pair_bits : 0);
+                         zeroed ? unique_status : status, err, n_rows, s,
+                         pair_bits + 8 <= 64 ? (int)pair_bits : 0, zeroed);
   XTN_CK(cudaGetLastError());
   return XTN_OK;
 }
@@ -851,13 +890,48 @@ int launch_back(const BackStage& b, uint64_t cand_cap, const uint64_t* n_cand_de
                 uint32_t pair_bits, uint32_t j_bits, const PairSide& si, const PairSide& sj,
                 const uint32_t* seq_rep, int self_mode, int d, xtn_triple* rows, int64_t row_cap,
                 int sms, uint32_t* err, cudaStream_t s, int cfg, int metric = 0) {
-  XTN_CK(cudaMemsetAsync(b.hist, 0, MAX_PASSES * RADIX * 4, s));
-  XTN_CK(cudaMemsetAsync(b.counters, 0, 16, s));
+  if (b.zero_bytes) {
+    XTN_CK(cudaMemsetAsync(b.hist, 0, b.zero_bytes, s));
+  } else {
+    XTN_CK(cudaMemsetAsync(b.hist, 0, MAX_PASSES * RADIX * 4, s));
+    XTN_CK(cudaMemsetAsync(b.counters, 0, 16, s));
+  }
   launch_verify_candidates(b.P1, cand_cap, n_cand_dev, j_bits, si, sj, seq_rep, self_mode, d,
                            metric, b.P2, cand_cap, b.counters, b.hist, (int)pair_bits, sms, err, s);
   return launch_sort_unique(b.P2, b.P1, cand_cap, b.counters, pair_bits, j_bits, b.hist,
                             b.digit_base, b.status, si, sj, d, metric, rows, row_cap, err,
-                            b.counters + 1, s, cfg);
+                            b.counters + 1, s, cfg, b.zero_bytes ? b.unique_status : nullptr);
+}
+
+// The last step of a call whose n_pairs candidate words stand in P1: in one
+// block's launch when they are few, through launch_back otherwise.  The row
+// count goes to ctl->back[1].
+int finish_pairs(uint64_t* P1, uint64_t n_pairs, uint32_t pair_bits, uint32_t j_bits,
+                 const PairSide& si, const PairSide& sj, const uint32_t* seq_rep, int self_mode,
+                 int d, int metric, xtn_triple* rows, int64_t row_cap, int sms, Control* ctl,
+                 Arena& ar, cudaStream_t s) {
+  if (n_pairs <= SMALL_PAIRS && pair_bits + 2 <= 64) {
+    launch_small_rows(P1, n_pairs, j_bits, si, sj, seq_rep, self_mode, d, metric, rows, row_cap,
+                      ctl->back + 1, ctl->err, s);
+    XTN_CK(cudaGetLastError());
+    return XTN_OK;
+  }
+  const int cfg = g_cfg_pairs.load();
+  const size_t hist_b = MAX_PASSES * RADIX * 4;
+  const size_t sort_b = (radix_status_bytes((int64_t)n_pairs, cfg) + 15) & ~size_t(15);
+  BackStage b;
+  b.P1 = P1;
+  b.P2 = ar.get<uint64_t>(n_pairs + 8);
+  b.digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
+  b.zero_bytes = hist_b + sort_b + verify_status_bytes((int64_t)n_pairs);
+  char* z = ar.get<char>(b.zero_bytes);
+  XTN_ALLOC_OK(ar);
+  b.hist = reinterpret_cast<uint32_t*>(z);
+  b.status = reinterpret_cast<uint64_t*>(z + hist_b);
+  b.unique_status = reinterpret_cast<uint64_t*>(z + hist_b + sort_b);
+  b.counters = ctl->back;
+  return launch_back(b, n_pairs, nullptr, pair_bits, j_bits, si, sj, seq_rep, self_mode, d, rows,
+                     row_cap, sms, ctl->err, s, cfg, metric);
 }
 
 // Result rows go to `out` directly when it is device memory; otherwise into
@@ -1005,13 +1079,15 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   if (rc) return rc;
   Arena ar(s);
   constexpr uint32_t NB = 1u << MAX_BIN_BITS;
-  uint32_t* err = ar.get<uint32_t>(4);
+  Control* ctl = nullptr;
+  uint64_t* front_status = nullptr;
+  XTN_RC(take_control(ar, encode_status_bytes(n), s, &ctl, &front_status));
+  uint32_t* err = ctl->err;
   // [0] groups [1] pairs [2] direct candidates [3] large-bucket records
   // [4] records appended [5] survivors [6] rows
   uint64_t* ctr = ar.get<uint64_t>(8);
   uint32_t* bins = ar.get<uint32_t>(NB);
   XTN_ALLOC_OK(ar);
-  XTN_CK(init_err(err, s));
   XTN_CK(cudaMemsetAsync(ctr, 0, 64, s));
   XTN_CK(cudaMemsetAsync(bins, 0, NB * 4, s));
   DevSeqs in;
@@ -1025,7 +1101,7 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
     if (rc) return rc;
   }
   Encoded e;
-  rc = encode_and_count(in, d, ar, err, s, &e, true);
+  rc = encode_and_count(in, d, ar, ctl, front_status, s, &e, true);
   if (rc) return rc;
   const uint32_t id_bits = bits_for((uint64_t)n);
   const uint32_t* salt_rep = between ? nullptr : seq_rep;
@@ -1256,11 +1332,11 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   int rc = current_device_info(&sms);
   if (rc) return rc;
   Arena ar(s);
-  uint32_t* err = ar.get<uint32_t>(4);
-  uint64_t* counters = ar.get<uint64_t>(4);
-  XTN_ALLOC_OK(ar);
-  XTN_CK(init_err(err, s));
-  XTN_CK(cudaMemsetAsync(counters, 0, 32, s));
+  Control* ctl = nullptr;
+  uint64_t* front_status = nullptr;
+  XTN_RC(take_control(ar, encode_status_bytes(n), s, &ctl, &front_status));
+  uint32_t* err = ctl->err;
+  uint64_t* counters = ctl->counters;
   DevSeqs in, in_b;
   rc = stage_seqs(seqs, offsets, n, ar, s, &in);
   if (rc) return rc;
@@ -1276,10 +1352,19 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     if (rc) return rc;
   }
 
-  // front: encode (read back the record count), expand, group
+  // front: encode (read back the record count unless its bound is small),
+  // expand, group
+  if (mode < 0) mode = g_grouping.load();
   Encoded e;
-  rc = paired ? encode_and_count_paired(in, in_b, d, ar, err, s, &e)
-              : encode_and_count(in, d, ar, err, s, &e);
+  const uint64_t n_max = (uint64_t)n * variant_count(XTN_MAX_LEN, (uint32_t)d);
+  const bool unread = mode == 0 && !paired && n_max <= UNREAD_RECORDS;
+  if (unread) {
+    rc = launch_front(in, d, ar, ctl, front_status, s, &e);
+    e.n_rec = n_max;
+  } else {
+    rc = paired ? encode_and_count_paired(in, in_b, d, ar, err, s, &e)
+                : encode_and_count(in, d, ar, ctl, front_status, s, &e);
+  }
   if (rc == XTN_ERR_TOO_LARGE && !paired) {  // 2^32 records or more: search in passes
     ar.release();
     return search_stream_impl(seqs, offsets, n, d, rep_offsets, n_rep, metric, between, 0, out,
@@ -1287,7 +1372,6 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   }
   if (rc) return rc;
   Sorted so;
-  if (mode < 0) mode = g_grouping.load();
   // Modes 0 and 2 write the candidates they find in shared memory at once,
   // into a buffer sized by a guess; past it, the search runs again with
   // all-global grouping, which sizes its buffers exactly.
@@ -1308,7 +1392,7 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
       XTN_ALLOC_OK(ar);
       launch_expand(e.source(), e.rec_off, n, d, salt_rep, so.id_bits, rec, e.n_rec, nullptr, 0, 0,
                     sms, err, s);
-      launch_partition(rec, (int64_t)e.n_rec, nullptr, part, sms, err, s);
+      launch_partition(rec, (int64_t)e.n_rec, unread ? &ctl->n_rec : nullptr, part, sms, err, s);
     } else {
       launch_expand_scatter(e.source(), e.rec_off, n, d, salt_rep, so.id_bits, e.n_rec, part, sms,
                             err, s);
@@ -1322,21 +1406,21 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   }
   struct {
     uint64_t groups, pairs, direct, large;
-    uint32_t err;
-  } h{0, 0, 0, 0, 0};
+  } h{0, 0, 0, 0};
+  Control c{};
   uint64_t n_flagged = mode == 1 ? e.n_rec : 0;  // records whose groups are emitted from flags
   if (mode != 1) {
     ReadBack rb(s);
-    XTN_RC(rb.add(&h.direct, counters + 2));
-    XTN_RC(rb.add(&h.large, counters + 3));
-    XTN_RC(rb.add(&h.err, err));
+    XTN_RC(rb.add(&c, ctl));
     XTN_RC(rb.wait());
-    if (h.err == DERR_CAPACITY) {  // candidate overflow alone: regroup sized exactly
+    h.direct = c.counters[2];
+    h.large = c.counters[3];
+    if (c.err[0] == DERR_CAPACITY) {  // candidate overflow alone: regroup sized exactly
       ar.release();
       return search_self_impl(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out, s, 1,
                               metric, between, b_seqs, b_offsets);
     }
-    if (h.err) return map_device_err(h.err);
+    if (c.err[0]) return map_device_err(c.err[0]);
     if (h.large) n_flagged = mode == 0 ? h.large : e.n_rec;
     if (mode == 0 && h.large)
       XTN_RC(sort_spill(part, h.large, so.id_bits, choose_hash_bits(e.n_rec, so.id_bits), sms, ar,
@@ -1353,11 +1437,11 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     k_pair_total<<<1, 1, 0, s>>>(pair_off, counters, counters + 1);
     XTN_CK(cudaGetLastError());
     ReadBack rb(s);
-    XTN_RC(rb.add(&h.groups, counters));
-    XTN_RC(rb.add(&h.pairs, counters + 1));
-    XTN_RC(rb.add(&h.err, err));
+    XTN_RC(rb.add(&c, ctl));
     XTN_RC(rb.wait());
-    if (h.err) return map_device_err(h.err);
+    if (c.err[0]) return map_device_err(c.err[0]);
+    h.groups = c.counters[0];
+    h.pairs = c.counters[1];
   }
   const uint64_t n_pairs = h.direct + h.pairs;
   if (n_pairs == 0) return XTN_OK;
@@ -1374,30 +1458,21 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   }
 
   // back: the remaining candidates, verify, sort survivors, dedup
-  BackStage b;
-  b.P1 = mode != 1 ? direct.cand : ar.get<uint64_t>(n_pairs + 8);
-  b.P2 = ar.get<uint64_t>(n_pairs + 8);
-  b.hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
-  b.digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
-  const int cfg_pairs = g_cfg_pairs.load();
-  b.status = ar.get<uint64_t>(back_status_bytes(n_pairs, cfg_pairs) / 8 + 1);
-  b.counters = ar.get<uint64_t>(2);
+  uint64_t* P1 = mode != 1 ? direct.cand : ar.get<uint64_t>(n_pairs + 8);
   XTN_ALLOC_OK(ar);
   if (h.pairs)
     launch_emit_pairs(so.rec, n_flagged, S, pair_off, (int64_t)h.groups, nullptr, h.pairs,
-                      so.id_bits, b.P1 + h.direct, nullptr, nullptr, sms, err, s);
+                      so.id_bits, P1 + h.direct, nullptr, nullptr, sms, err, s);
   OutRows o;
   rc = prepare_out(out, cap, n_pairs, ar, &o);
   if (rc) return rc;
-  rc = launch_back(b, n_pairs, nullptr, 2 * so.id_bits, so.id_bits, e.side(n), e.side(n), seq_rep,
-                   between ? 2 : 1, d, o.dev, o.dev_cap, sms, err, s, cfg_pairs, metric);
-  if (rc) return rc;
+  XTN_RC(finish_pairs(P1, n_pairs, 2 * so.id_bits, so.id_bits, e.side(n), e.side(n), seq_rep,
+                      between ? 2 : 1, d, metric, o.dev, o.dev_cap, sms, ctl, ar, s));
   ReadBack rb(s);
-  XTN_RC(rb.add(&h.pairs, b.counters + 1));
-  XTN_RC(rb.add(&h.err, err));
+  XTN_RC(rb.add(&c, ctl));
   XTN_RC(rb.wait());
-  if (h.err) return map_device_err(h.err);
-  return finish_out(o, out, cap, h.pairs, s, n_out);
+  if (c.err[0]) return map_device_err(c.err[0]);
+  return finish_out(o, out, cap, c.back[1], s, n_out);
 }
 
 }  // namespace
@@ -1436,14 +1511,15 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   int rc = current_device_info(&sms);
   if (rc) return rc;
   Arena ar(s);
-  uint32_t* err = ar.get<uint32_t>(4);
-  XTN_ALLOC_OK(ar);
-  XTN_CK(init_err(err, s));
+  Control* ctl = nullptr;
+  uint64_t* front_status = nullptr;
+  XTN_RC(take_control(ar, encode_status_bytes(n), s, &ctl, &front_status));
+  uint32_t* err = ctl->err;
   DevSeqs in;
   rc = stage_seqs(seqs, offsets, n, ar, s, &in);
   if (rc) return rc;
   Encoded e;
-  rc = encode_and_count(in, d, ar, err, s, &e);
+  rc = encode_and_count(in, d, ar, ctl, front_status, s, &e);
   if (rc) return rc;
   Sorted so;
   rc = expand_and_sort(e, n, d, nullptr, sms, ar, err, s, &so);
@@ -1518,14 +1594,15 @@ int search_query_impl(const xtn_index* idx, const uint8_t* q_seqs, const int64_t
   int rc = current_device_info(&sms);
   if (rc) return rc;
   Arena ar(s);
-  uint32_t* err = ar.get<uint32_t>(4);
-  XTN_ALLOC_OK(ar);
-  XTN_CK(init_err(err, s));
+  Control* ctl = nullptr;
+  uint64_t* front_status = nullptr;
+  XTN_RC(take_control(ar, encode_status_bytes(n_q), s, &ctl, &front_status));
+  uint32_t* err = ctl->err;
   DevSeqs in;
   rc = stage_seqs(q_seqs, q_offsets, n_q, ar, s, &in);
   if (rc) return rc;
   Encoded e;
-  rc = encode_and_count(in, idx->d, ar, err, s, &e);
+  rc = encode_and_count(in, idx->d, ar, ctl, front_status, s, &e);
   if (rc) return rc;
   const uint64_t n_qv = e.n_rec;
   uint32_t* qv_start = ar.get<uint32_t>(n_qv);
@@ -1558,38 +1635,23 @@ int search_query_impl(const xtn_index* idx, const uint8_t* q_seqs, const int64_t
   const uint32_t q_bits = bits_for((uint64_t)n_q);
   const uint32_t pair_bits = q_bits + idx->id_bits;
   if (pair_bits > 64) return XTN_ERR_TOO_LARGE;
-  BackStage b;
-  b.P1 = ar.get<uint64_t>(n_cand + 8);
-  b.P2 = ar.get<uint64_t>(n_cand + 8);
-  b.hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
-  b.digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
-  const int cfg_pairs = g_cfg_pairs.load();
-  b.status = ar.get<uint64_t>(back_status_bytes(n_cand, cfg_pairs) / 8 + 1);
-  b.counters = ar.get<uint64_t>(2);
+  uint64_t* P1 = ar.get<uint64_t>(n_cand + 8);
   XTN_ALLOC_OK(ar);
   launch_query_emit(idx->rec, idx->n_rec, idx->id_bits, qv_start, qv_q, cand_off, n_qv, n_cand,
-                    b.P1, sms, err, s);
+                    P1, sms, err, s);
   XTN_CK(cudaGetLastError());
   OutRows o;
   rc = prepare_out(out, cap, n_cand, ar, &o);
   if (rc) return rc;
-  rc = launch_back(b, n_cand, nullptr, pair_bits, idx->id_bits, e.side(n_q),
-                   PairSide{idx->rows, nullptr, (uint64_t)idx->n}, nullptr, 0, idx->d, o.dev,
-                   o.dev_cap, sms, err, s, cfg_pairs, metric);
-  if (rc) return rc;
-  struct {
-    uint64_t rows;
-    uint32_t err;
-  } h{0, 0};
-  {
-    ReadBack rb(s);
-    XTN_RC(rb.add(&h.rows, b.counters + 1));
-    XTN_RC(rb.add(&h.err, err));
-    XTN_RC(rb.wait());
-  }
-  if (h.err) return map_device_err(h.err);
-  const uint64_t n_rows = h.rows;
-  return finish_out(o, out, cap, n_rows, s, n_out);
+  XTN_RC(finish_pairs(P1, n_cand, pair_bits, idx->id_bits, e.side(n_q),
+                      PairSide{idx->rows, nullptr, (uint64_t)idx->n}, nullptr, 0, idx->d, metric,
+                      o.dev, o.dev_cap, sms, ctl, ar, s));
+  Control h{};
+  ReadBack rb(s);
+  XTN_RC(rb.add(&h, ctl));
+  XTN_RC(rb.wait());
+  if (h.err[0]) return map_device_err(h.err[0]);
+  return finish_out(o, out, cap, h.back[1], s, n_out);
 }
 
 int tcrdist_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, const xtn_triple* in_rows,
@@ -1603,15 +1665,18 @@ int tcrdist_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, const x
   int rc = current_device_info(&sms);
   if (rc) return rc;
   Arena ar(s);
-  uint32_t* err = ar.get<uint32_t>(4);
-  XTN_ALLOC_OK(ar);
-  XTN_CK(init_err(err, s));
+  Control* ctl = nullptr;
+  uint64_t* unused = nullptr;
+  XTN_RC(take_control(ar, 0, s, &ctl, &unused));
   DevSeqs in;
   rc = stage_seqs(seqs, offsets, n, ar, s, &in);
   if (rc) return rc;
   Encoded e;
-  rc = encode_and_count(in, 0, ar, err, s, &e, false, false);
-  if (rc) return rc;
+  e.keys = ar.get<Key128>(n);
+  e.lens = ar.get<uint8_t>(n);
+  e.eqprev = ar.get<uint32_t>(n);
+  XTN_ALLOC_OK(ar);
+  launch_encode(in.seqs, in.off, n, 0, e.keys, e.lens, e.eqprev, nullptr, nullptr, ctl->err, s);
   const xtn_triple* d_in = in_rows;
   if (!is_device_ptr(in_rows)) {
     xtn_triple* t = ar.get<xtn_triple>(n_in);
@@ -1622,17 +1687,16 @@ int tcrdist_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, const x
   const bool host_out = !is_device_ptr(out);
   xtn_triple* d_out = host_out ? ar.get<xtn_triple>(n_in) : out;
   uint64_t* status = ar.get<uint64_t>(verify_status_bytes(n_in) / 8 + 1);
-  uint64_t* d_total = ar.get<uint64_t>(1);
   XTN_ALLOC_OK(ar);
-  launch_tcrdist_filter(d_in, n_in, e.keys, e.lens, n, max_score, d_out, status, err, d_total, s);
+  launch_tcrdist_filter(d_in, n_in, e.keys, e.lens, n, max_score, d_out, status, ctl->err,
+                        ctl->back, s);
   XTN_CK(cudaGetLastError());
-  uint64_t total = 0;
-  rc = read_back(&total, d_total, 1, s);
-  if (rc) return rc;
-  uint32_t herr = 0;
-  rc = read_back(&herr, err, 1, s);
-  if (rc) return rc;
-  if (herr) return map_device_err(herr);
+  Control h{};
+  ReadBack rb(s);
+  XTN_RC(rb.add(&h, ctl));
+  XTN_RC(rb.wait());
+  if (h.err[0]) return map_device_err(h.err[0]);
+  const uint64_t total = h.back[0];
   if (host_out && total > 0) {
     XTN_CK(cudaMemcpyAsync(out, d_out, total * sizeof(xtn_triple), cudaMemcpyDeviceToHost, s));
     XTN_CK(host_sync(s));
@@ -1662,7 +1726,7 @@ struct xtn_plan {
   uint32_t* seq_rep = nullptr;
   xtn::Key128* keys = nullptr;
   uint8_t* lens = nullptr;
-  uint32_t *eqprev = nullptr, *vcount = nullptr, *hist = nullptr, *err = nullptr;
+  uint32_t *eqprev = nullptr, *hist = nullptr, *err = nullptr;
   xtn::PlaneRow* planes = nullptr;
   uint64_t *rec_off = nullptr, *A = nullptr, *B = nullptr, *digit_base = nullptr;
   uint64_t *status = nullptr, *flags = nullptr, *counters = nullptr;
@@ -1736,12 +1800,11 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   const size_t st = std::max({radix_status_bytes((int64_t)rec_cap,
                                                  parted ? ONESWEEP_LOOP : p->cfg_rec),
                               group_status_bytes((int64_t)rec_cap),
-                              scan_status_bytes((int64_t)p->g_cap), scan_status_bytes(n)});
+                              scan_status_bytes((int64_t)p->g_cap), encode_status_bytes(n)});
   p->off = p->alloc<int64_t>(n + 1);
   p->keys = p->alloc<Key128>(n);
   p->lens = p->alloc<uint8_t>(n);
   p->eqprev = p->alloc<uint32_t>(n);
-  p->vcount = p->alloc<uint32_t>(n);
   p->rec_off = p->alloc<uint64_t>(n + 1);
   PartitionShape shape;
   if (parted) shape = choose_partitions(rec_cap, g_filter_fx.load());
@@ -1767,10 +1830,10 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   p->rows = p->alloc<xtn_triple>(p->pair_cap);
   if (rep_offsets) p->seq_rep = p->alloc<uint32_t>(n);
   bool ok = p->rows && p->back.counters && p->back.status && p->back.digit_base && p->back.hist &&
-            p->back.P2 && p->back.P1 && p->planes && p->err && p->counters && p->flags && p->status &&
-            p->bucket_start && p->part.count &&
-            (!parted || p->part.kept) && p->digit_base && p->hist && p->B && p->A && p->rec_off && p->vcount && p->eqprev &&
-            p->lens && p->keys && p->off && (!rep_offsets || p->seq_rep);
+            p->back.P2 && p->back.P1 && p->planes && p->err && p->counters && p->flags &&
+            p->status && p->bucket_start && p->part.count && (!parted || p->part.kept) &&
+            p->digit_base && p->hist && p->B && p->A && p->rec_off && p->eqprev && p->lens &&
+            p->keys && p->off && (!rep_offsets || p->seq_rep);
   if (!ok) {
     delete p;
     return XTN_ERR_OOM;
@@ -1817,9 +1880,9 @@ int plan_run_impl(xtn_plan* p, const uint8_t* seqs, cudaStream_t s) {
   XTN_CK(init_err(p->err, s));
   XTN_CK(cudaMemsetAsync(p->counters, 0, 32, s));
   XTN_CK(cudaMemsetAsync(p->hist, 0, MAX_PASSES * RADIX * 4, s));
-  launch_encode(seqs, p->off, n, p->d, p->keys, p->lens, p->eqprev, p->vcount, p->planes,
-                p->err, s);
-  launch_scan_counts(p->vcount, n, p->rec_off, p->status, p->err, s);
+  XTN_CK(cudaMemsetAsync(p->status, 0, encode_status_bytes(n), s));
+  launch_encode_scan(seqs, p->off, n, p->d, p->keys, p->lens, p->eqprev, p->rec_off,
+                     p->rec_off + n, p->status, p->planes, p->err, s);
   uint64_t* sorted = nullptr;
   const uint64_t* n_rec = p->rec_off + n;  // known on the device only
   const bool direct = p->group_mode != 1;  // most candidates are written while grouping

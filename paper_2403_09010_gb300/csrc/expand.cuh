@@ -145,12 +145,6 @@ struct __align__(16) VarMeta {
   uint32_t c, aux;
 };
 
-__device__ __forceinline__ Key128 shr128(const Key128& k, uint32_t s) {
-  if (s >= 128) return Key128{0ull, 0ull};
-  if (s >= 64) return Key128{k.hi >> (s - 64), 0ull};
-  if (s == 0) return k;
-  return Key128{(k.lo >> s) | (k.hi << (64 - s)), k.hi >> s};
-}
 __device__ __forceinline__ Key128 shl128(const Key128& k, uint32_t s) {
   if (s >= 128) return Key128{0ull, 0ull};
   if (s >= 64) return Key128{0ull, k.lo << (s - 64)};

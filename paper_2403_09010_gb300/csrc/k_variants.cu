@@ -49,108 +49,167 @@ constexpr int ENCODE_WORDS = ENCODE_SPAN / 4 + 10;  // and the words a lane read
 // (46 + 31 us for 1M sequences; 353 + 237 us for 10M).  Offsets are validated
 // per lane first; a warp with an invalid offset reads each valid lane's
 // letters directly instead.
-__global__ void __launch_bounds__(ENCODE_WARPS * 32)
+//
+// SCAN: the variant counts are not written but summed up to record offsets
+// (single pass with decoupled look-back over the blocks), the total also to
+// *total_out.  ROUNDS times 256 sequences a block, so that long inputs have
+// fewer blocks to look back over: 1M sequences 53, 42, 39 and 44 us with 1, 2,
+// 4 and 8 rounds, 10M 423, 283, 229 and 234 us (a scan kernel behind this one:
+// 49 and 316 us for the two).
+template <bool SCAN, int ROUNDS>
+__global__ void __launch_bounds__(ENCODE_WARPS * 32, 8)
     k_encode(const uint8_t* __restrict__ seqs, const int64_t* __restrict__ off, int64_t n, int d,
              Key128* __restrict__ keys, uint8_t* __restrict__ lens,
              uint32_t* __restrict__ eqprev_out, uint32_t* __restrict__ vcount,
+             uint64_t* __restrict__ rec_off, uint64_t* __restrict__ status,
+             uint32_t* __restrict__ ctr, uint64_t* __restrict__ total_out,
              PlaneRow* __restrict__ rows, uint32_t* __restrict__ err) {
   __shared__ uint32_t s_words[ENCODE_WARPS][ENCODE_WORDS];
   __shared__ uint8_t s_code[256];
+  __shared__ uint32_t s_sum[ENCODE_WARPS * ROUNDS];  // of each 32 sequences, then of all before
+  __shared__ uint32_t s_before[SCAN ? ENCODE_WARPS * 32 * ROUNDS : 1];  // within its 32
+  __shared__ uint64_t s_prefix;
+  __shared__ uint32_t s_tile;
   static_assert(ENCODE_WARPS * 32 == 256, "one table entry per thread");
+  static_assert(ENCODE_WARPS * ROUNDS <= 32, "one warp scans the sums");
   s_code[threadIdx.x] = (uint8_t)letter_code(threadIdx.x);
-  __syncthreads();
   const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-  const int64_t s0 = ((int64_t)blockIdx.x * ENCODE_WARPS + warp) * 32;
-  if (s0 >= n) return;  // whole warp
-  const int64_t i = s0 + lane;
-  const bool in = i < n;
+  uint32_t tile = blockIdx.x;
+  if (SCAN) tile = tile_id(ctr, &s_tile);  // in start order, for the look-back
+  __syncthreads();
   const int64_t total = off[n];
-  const int64_t a = in ? off[i] : 0, b = in ? off[i + 1] : 0;
-  bool ok = in && a >= 0 && b >= a && b <= total;
-  if (in && !ok) atomicOr(err, DERR_RANGE);
-  if (i == 0 && a != 0) atomicOr(err, DERR_RANGE);  // offsets start at 0
-  if (ok && b - a > XTN_MAX_LEN) {
-    atomicOr(err, DERR_TOO_LONG);
-    ok = false;
-  }
-  const bool all_ok = __all_sync(FULL_MASK, ok || !in);
-  const int last = (int)((n - s0 < 32) ? (n - s0 - 1) : 31);
-  const int64_t A = __shfl_sync(FULL_MASK, a, 0), Bend = __shfl_sync(FULL_MASK, b, last);
-  const uint32_t L = ok ? (uint32_t)(b - a) : 0u;
-  uint32_t w[7];  // the sequence's letters, zeros behind them
-  if (all_ok && Bend - A <= ENCODE_SPAN) {
-    // byte k of the span sits at byte head + k of s_words, so that whole
-    // words of the input land on whole words here
-    const uint8_t* src = seqs + A;
-    const uint32_t head = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 3u);
-    const uint32_t bytes = head + (uint32_t)(Bend - A);
-    uint8_t* dst = reinterpret_cast<uint8_t*>(s_words[warp]);
-    const uint32_t w0 = head ? 1u : 0u, w1 = bytes / 4;  // whole words [w0, w1)
-    const uint32_t* src4 = reinterpret_cast<const uint32_t*>(src - head);
-    for (uint32_t k = w0 + lane; k < w1; k += 32) s_words[warp][k] = src4[k];
-    if (head && lane >= head && lane < 4 && lane < bytes) dst[lane] = src[lane - head];
-    const uint32_t tail = max(w0, w1) * 4 + lane;
-    if (lane < 4 && tail < bytes) dst[tail] = src[tail - head];
-    __syncwarp();
-    const uint32_t o = head + (uint32_t)(a - A);
-    const uint32_t sh = 8u * (o & 3u);
-    const uint32_t* mine = s_words[warp] + (ok ? o / 4 : 0u);
-    uint32_t lo = mine[0];
-#pragma unroll
-    for (int t = 0; t < 7; ++t) {
-      const uint32_t hi = mine[t + 1];
-      w[t] = __funnelshift_r(lo, hi, sh);
-      lo = hi;
+#pragma unroll 1  // 32 registers, eight blocks an SM
+  for (int round = 0; round < ROUNDS; ++round) {
+    const int64_t s0 = (((int64_t)tile * ROUNDS + round) * ENCODE_WARPS + warp) * 32;
+    const int64_t i = s0 + lane;
+    const bool in = i < n;
+    const int64_t a = in ? off[i] : 0, b = in ? off[i + 1] : 0;
+    bool ok = in && a >= 0 && b >= a && b <= total;
+    if (in && !ok) atomicOr(err, DERR_RANGE);
+    if (i == 0 && a != 0) atomicOr(err, DERR_RANGE);  // offsets start at 0
+    if (ok && b - a > XTN_MAX_LEN) {
+      atomicOr(err, DERR_TOO_LONG);
+      ok = false;
     }
-  } else {
+    const bool all_ok = __all_sync(FULL_MASK, ok || !in);
+    const int last = (int)max((int64_t)0, min((int64_t)31, n - s0 - 1));
+    const int64_t A = __shfl_sync(FULL_MASK, a, 0), Bend = __shfl_sync(FULL_MASK, b, last);
+    const uint32_t L = ok ? (uint32_t)(b - a) : 0u;
+    uint32_t w[7];  // the sequence's letters, zeros behind them
+    if (all_ok && Bend - A <= ENCODE_SPAN) {
+      // byte k of the span sits at byte head + k of s_words, so that whole
+      // words of the input land on whole words here
+      __syncwarp();  // the round before is done with the words
+      const uint8_t* src = seqs + A;
+      const uint32_t head = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 3u);
+      const uint32_t bytes = head + (uint32_t)(Bend - A);
+      uint8_t* dst = reinterpret_cast<uint8_t*>(s_words[warp]);
+      const uint32_t w0 = head ? 1u : 0u, w1 = bytes / 4;  // whole words [w0, w1)
+      const uint32_t* src4 = reinterpret_cast<const uint32_t*>(src - head);
+      for (uint32_t k = w0 + lane; k < w1; k += 32) s_words[warp][k] = src4[k];
+      if (head && lane >= head && lane < 4 && lane < bytes) dst[lane] = src[lane - head];
+      const uint32_t tail = max(w0, w1) * 4 + lane;
+      if (lane < 4 && tail < bytes) dst[tail] = src[tail - head];
+      __syncwarp();
+      const uint32_t o = head + (uint32_t)(a - A);
+      const uint32_t sh = 8u * (o & 3u);
+      const uint32_t* mine = s_words[warp] + (ok ? o / 4 : 0u);
+      uint32_t lo = mine[0];
 #pragma unroll
-    for (int t = 0; t < 7; ++t) w[t] = 0;
+      for (int t = 0; t < 7; ++t) {
+        const uint32_t hi = mine[t + 1];
+        w[t] = __funnelshift_r(lo, hi, sh);
+        lo = hi;
+      }
+    } else {
 #pragma unroll
-    for (int p = 0; p < XTN_MAX_LEN; ++p)
-      if ((uint32_t)p < L) w[p / 4] |= (uint32_t)seqs[a + p] << (8 * (p % 4));
+      for (int t = 0; t < 7; ++t) w[t] = 0;
+#pragma unroll
+      for (int p = 0; p < XTN_MAX_LEN; ++p)
+        if ((uint32_t)p < L) w[p / 4] |= (uint32_t)seqs[a + p] << (8 * (p % 4));
+    }
+#pragma unroll
+    for (int t = 0; t < 7; ++t) {  // clear what lies past the end
+      const int left = (int)L - 4 * t;
+      w[t] = left >= 4 ? w[t] : left > 0 ? w[t] & (0xffffffffu >> (32 - 8 * left)) : 0u;
+    }
+    Key128 key{0ull, 0ull};
+    uint32_t plane[5] = {0u, 0u, 0u, 0u, 0u};
+    const uint32_t longest = __reduce_max_sync(FULL_MASK, L);
+#pragma unroll
+    for (int g = 0; g < 5; ++g) {
+      if ((uint32_t)(6 * g) >= longest) break;  // warp-uniform
+      uint32_t acc = 0;  // five fields of six bits, the code's bits 0 .. 4
+#pragma unroll
+      for (int x = 0; x < 6; ++x) {
+        const int p = 6 * g + x;
+        acc >>= 1;
+        if (p < XTN_MAX_LEN) {
+          const uint32_t c = s_code[(w[p / 4] >> (8 * (p % 4))) & 255u];
+          acc |= (c * 0x02108420u) & 0x20820820u;  // bit b of c to bit 6 b + 5
+          if (5 * p < 64) key.lo |= (uint64_t)c << (5 * p < 64 ? 5 * p : 0);
+          if (5 * p > 59)
+            key.hi |= 5 * p < 64 ? (uint64_t)c >> (64 - 5 * p) : (uint64_t)c << (5 * p - 64);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 5; ++k) plane[k] |= ((acc >> (6 * k)) & 63u) << (6 * g);
+    }
+    const uint32_t all = L ? 0xffffffffu >> (32 - L) : 0u;
+    if ((plane[0] | plane[1] | plane[2] | plane[3] | plane[4]) != all)
+      atomicOr(err, DERR_BAD_RESIDUE);  // a letter without a code
+    uint32_t differs = 1u;  // from the left neighbour
+#pragma unroll
+    for (int k = 0; k < 5; ++k) differs |= plane[k] ^ (plane[k] << 1);
+    const uint32_t eqprev = ~differs & all;
+    const uint32_t count = in ? canonical_total(eqprev, L, d) : 0u;
+    if (in) {
+      keys[i] = key;
+      lens[i] = (uint8_t)L;
+      eqprev_out[i] = eqprev;
+      if (!SCAN && vcount) vcount[i] = count;
+      if (rows)
+        store_row(rows + i, PlaneRow{make_uint4(plane[0], plane[1], plane[2], plane[3]),
+                                     make_uint4(plane[4], L, 0u, 0u)});
+    }
+    if (SCAN) {
+      uint32_t inc = count;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL_MASK, inc, o);
+        if (lane >= (uint32_t)o) inc += t;
+      }
+      s_before[round * ENCODE_WARPS * 32 + threadIdx.x] = inc - count;
+      if (lane == 31) s_sum[round * ENCODE_WARPS + warp] = inc;
+    }
   }
+  if (!SCAN) return;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t v = lane < ENCODE_WARPS * ROUNDS ? s_sum[lane] : 0u;
+    uint32_t inc = v;
 #pragma unroll
-  for (int t = 0; t < 7; ++t) {  // clear what lies past the end
-    const int left = (int)L - 4 * t;
-    w[t] = left >= 4 ? w[t] : left > 0 ? w[t] & (0xffffffffu >> (32 - 8 * left)) : 0u;
-  }
-  Key128 key{0ull, 0ull};
-  uint32_t plane[5] = {0u, 0u, 0u, 0u, 0u};
-  const uint32_t longest = __reduce_max_sync(FULL_MASK, L);
-#pragma unroll
-  for (int g = 0; g < 5; ++g) {
-    if ((uint32_t)(6 * g) >= longest) break;  // warp-uniform
-    uint32_t acc = 0;  // five fields of six bits, the code's bits 0 .. 4
-#pragma unroll
-    for (int x = 0; x < 6; ++x) {
-      const int p = 6 * g + x;
-      acc >>= 1;
-      if (p < XTN_MAX_LEN) {
-        const uint32_t c = s_code[(w[p / 4] >> (8 * (p % 4))) & 255u];
-        acc |= (c * 0x02108420u) & 0x20820820u;  // bit b of c to bit 6 b + 5
-        if (5 * p < 64) key.lo |= (uint64_t)c << (5 * p < 64 ? 5 * p : 0);
-        if (5 * p > 59) key.hi |= 5 * p < 64 ? (uint64_t)c >> (64 - 5 * p) : (uint64_t)c << (5 * p - 64);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL_MASK, inc, o);
+      if (lane >= (uint32_t)o) inc += t;
+    }
+    if (lane < ENCODE_WARPS * ROUNDS) s_sum[lane] = inc - v;
+    const uint32_t all = __shfl_sync(FULL_MASK, inc, 31);
+    const uint64_t pre = warp_lookback(status, tile, all, err);
+    if (lane == 0) {
+      s_prefix = pre;
+      if (((int64_t)tile + 1) * ROUNDS * ENCODE_WARPS * 32 >= n) {
+        rec_off[n] = pre + all;
+        *total_out = pre + all;
       }
     }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) plane[k] |= ((acc >> (6 * k)) & 63u) << (6 * g);
   }
-  const uint32_t all = L ? 0xffffffffu >> (32 - L) : 0u;
-  if ((plane[0] | plane[1] | plane[2] | plane[3] | plane[4]) != all)
-    atomicOr(err, DERR_BAD_RESIDUE);  // a letter without a code
-  uint32_t differs = 1u;  // from the left neighbour
+  __syncthreads();
 #pragma unroll
-  for (int k = 0; k < 5; ++k) differs |= plane[k] ^ (plane[k] << 1);
-  const uint32_t eqprev = ~differs & all;
-  if (in) {
-    keys[i] = key;
-    lens[i] = (uint8_t)L;
-    eqprev_out[i] = eqprev;
-    vcount[i] = canonical_total(eqprev, L, d);
-    if (rows) {
-      rows[i].a = make_uint4(plane[0], plane[1], plane[2], plane[3]);
-      rows[i].b = make_uint4(plane[4], L, 0u, 0u);
-    }
+  for (int round = 0; round < ROUNDS; ++round) {
+    const int64_t i = (((int64_t)tile * ROUNDS + round) * ENCODE_WARPS + warp) * 32 + lane;
+    if (i < n) rec_off[i] = s_prefix + s_sum[round * ENCODE_WARPS + warp] +
+                             s_before[round * ENCODE_WARPS * 32 + threadIdx.x];
   }
 }
 
@@ -396,9 +455,31 @@ void launch_encode(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Ke
                    uint32_t* err, cudaStream_t s) {
   if (n <= 0) return;
   prof_begin(s, "k_encode", (double)n * (16 + 16 + 1 + 4 + 4 + 8 + (rows ? 32 : 0)));
-  k_encode<<<div_up_u32(n, ENCODE_WARPS * 32), ENCODE_WARPS * 32, 0, s>>>(seqs, off, n, d, keys,
-                                                                           lens, eqprev, vcount,
-                                                                           rows, err);
+  k_encode<false, 1><<<div_up_u32(n, ENCODE_WARPS * 32), ENCODE_WARPS * 32, 0, s>>>(
+      seqs, off, n, d, keys, lens, eqprev, vcount, nullptr, nullptr, nullptr, nullptr, rows, err);
+  prof_end(s);
+}
+
+// Above this many sequences (two blocks an SM with four rounds each) a block
+// takes four rounds of them; below, more blocks are worth more.
+constexpr int64_t ENCODE_LONG = 1 << 18;
+
+size_t encode_status_bytes(int64_t n) {
+  const int64_t per = ENCODE_WARPS * 32 * (n > ENCODE_LONG ? 4 : 1);
+  return (size_t)((n + per - 1) / per) * 8 + 16;
+}
+
+void launch_encode_scan(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Key128* keys,
+                        uint8_t* lens, uint32_t* eqprev, uint64_t* rec_off, uint64_t* total,
+                        uint64_t* status, PlaneRow* rows, uint32_t* err, cudaStream_t s) {
+  if (n <= 0) return;
+  const size_t st = encode_status_bytes(n);
+  uint32_t* ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(status) + st - 16);
+  prof_begin(s, "k_encode", (double)n * (16 + 16 + 1 + 4 + 8 + 8 + (rows ? 32 : 0)));
+  auto f = n > ENCODE_LONG ? k_encode<true, 4> : k_encode<true, 1>;
+  f<<<(uint32_t)((st - 16) / 8), ENCODE_WARPS * 32, 0, s>>>(seqs, off, n, d, keys, lens, eqprev,
+                                                            nullptr, rec_off, status, ctr, total,
+                                                            rows, err);
   prof_end(s);
 }
 

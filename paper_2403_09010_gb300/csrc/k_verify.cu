@@ -48,8 +48,8 @@ struct Planes {
 };
 
 __device__ __forceinline__ Planes load_planes(const PlaneRow* __restrict__ rows, uint64_t i) {
-  const uint4 a = __ldg(&rows[i].a), b = __ldg(&rows[i].b);
-  return Planes{{a.x, a.y, a.z, a.w, b.x}, b.y};
+  const PlaneRow r = load_row(rows + i);
+  return Planes{{r.a.x, r.a.y, r.a.z, r.a.w, r.b.x}, r.b.y};
 }
 
 // Diagonal k = (position in y) - (position in x), -3 <= k <= 3: bit p set
@@ -165,6 +165,22 @@ __device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t* s_
   return total;
 }
 
+// Whether candidate word w is a row, and its distance.
+__device__ __forceinline__ bool verified(uint64_t w, uint32_t j_bits, const PairSide& si,
+                                         const PairSide& sj, const uint32_t* __restrict__ seq_rep,
+                                         int self_mode, int d, int metric,
+                                         uint32_t* __restrict__ err, uint32_t& dist) {
+  const uint64_t i = w >> j_bits, j = w & ((1ull << j_bits) - 1ull);
+  if (i >= si.n || j >= sj.n) {
+    atomicOr(err, DERR_RANGE);
+    return false;
+  }
+  if (self_mode && i == j) return false;
+  if (seq_rep && (seq_rep[i] == seq_rep[j]) != (self_mode != 2)) return false;
+  dist = cand_distance(metric, d, si, sj, i, j);
+  return dist <= (uint32_t)d;
+}
+
 constexpr uint32_t VER_STASH = 256;  // survivor words a warp collects before a flush
 
 __global__ void __launch_bounds__(256)
@@ -197,7 +213,6 @@ __global__ void __launch_bounds__(256)
     held = 0;
   };
   const uint32_t lt_mask = (1u << lane) - 1u;
-  const uint64_t jmask = (1ull << j_bits) - 1ull;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); t0 < n;
        t0 += stride) {
@@ -206,17 +221,10 @@ __global__ void __launch_bounds__(256)
     uint64_t w = 0;
     if (t < n) {
       w = cand[t];
-      const uint64_t i = w >> j_bits, j = w & jmask;
-      ok = i < si.n && j < sj.n;
-      if (!ok) atomicOr(err, DERR_RANGE);
-      if (self_mode) ok = ok && i != j;
-      if (ok && seq_rep) ok = (seq_rep[i] == seq_rep[j]) == (self_mode != 2);
-      if (ok) {
-        const uint32_t dist = cand_distance(metric, d, si, sj, i, j);
-        ok = dist <= (uint32_t)d;
-        // the distance rides above the pair bits, for the dedup to write it
-        if (ok && hist_hi + 8 <= 64) w |= (uint64_t)dist << hist_hi;
-      }
+      uint32_t dist = 0;
+      ok = verified(w, j_bits, si, sj, seq_rep, self_mode, d, metric, err, dist);
+      // the distance rides above the pair bits, for the dedup to write it
+      if (ok && hist_hi + 8 <= 64) w |= (uint64_t)dist << hist_hi;
     }
     const uint32_t bal = __ballot_sync(FULL_MASK, ok);
     if (ok) {
@@ -345,14 +353,163 @@ size_t verify_status_bytes(int64_t n) { return verify_status_bytes_for(n); }
 void launch_unique_finalize(const uint64_t* pairs, int64_t n, const uint64_t* n_dev,
                             uint32_t j_bits, const PairSide& si, const PairSide& sj, int d,
                             int metric, xtn_triple* out, int64_t cap, uint64_t* status,
-                            uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift) {
+                            uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift,
+                            bool status_zeroed) {
   if (n <= 0) return;
   const size_t st = verify_status_bytes(n);
   uint32_t* ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(status) + st - 16);
-  cudaMemsetAsync(status, 0, st, s);
+  if (!status_zeroed) cudaMemsetAsync(status, 0, st, s);
   prof_begin(s, "k_unique_finalize", (double)n * 8.0);
   k_unique_finalize<<<std::min<uint32_t>(div_up_u32(n, VER_TILE), 152 * 8), VER_THREADS, 0, s>>>(
       pairs, n, n_dev, j_bits, si, sj, d, metric, out, cap, status, ctr, err, total, dist_shift);
+  prof_end(s);
+}
+
+// ----------------------------------------------------------- small results ---
+// Drop duplicates (a hash table in shared memory), verify, sort and write rows
+// in one block of one launch: for a few thousand candidates the general path
+// (ten launches and clears) is all latency.  Duplicates go first because most
+// candidates are some: a pair has one candidate per variant it shares.  The
+// sort is bitonic with a thread's words in registers: exchanges across less
+// than a warp are shuffles, and only those across warps go through shared
+// memory, with a barrier each (15 of 55 steps for 1,024 words, 25 of 78 for
+// 4,096).  10,000 sequences, d = 1: 18 us instead of about 70 for verify,
+// sort passes and dedup; with every candidate verified and sorted it took 61.
+// The limit is the table: 4,096 words in half of 64 KB.
+constexpr int SR_THREADS = 1024;
+
+// Sorts the block's SR_THREADS * K words, thread t holding words t + k *
+// SR_THREADS; s_w: two buffers of SR_THREADS words for the exchanges.
+template <int K>
+__device__ __forceinline__ void block_sort(uint64_t (&r)[K], uint64_t* s_w) {
+  const uint32_t t = threadIdx.x;
+  uint32_t flip = 0;
+  for (uint32_t size = 2; size <= (uint32_t)(SR_THREADS * K); size <<= 1) {
+    for (uint32_t step = size >> 1; step > 0; step >>= 1) {
+      if (step >= SR_THREADS) {  // between the thread's own words
+        const int ks = (int)(step / SR_THREADS);
+#pragma unroll
+        for (int x = 0; x < K; ++x) {
+#pragma unroll
+          for (int y = x + 1; y < K; ++y) {
+            if (y != (x ^ ks)) continue;
+            const bool up = ((x * SR_THREADS + t) & size) == 0;
+            const uint64_t lo = min(r[x], r[y]), hi = max(r[x], r[y]);
+            r[x] = up ? lo : hi;
+            r[y] = up ? hi : lo;
+          }
+        }
+        continue;
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        uint64_t o;
+        if (step < 32) {
+          o = __shfl_xor_sync(FULL_MASK, r[k], step);
+        } else {
+          // two buffers in turn: a barrier between a word's write and its
+          // read also lies between that read and the buffer's next write
+          uint64_t* buf = s_w + (flip & 1u) * SR_THREADS;
+          ++flip;
+          buf[t] = r[k];
+          __syncthreads();
+          o = buf[t ^ step];
+        }
+        const bool up = ((k * SR_THREADS + t) & size) == 0, low = (t & step) == 0;
+        r[k] = up == low ? min(r[k], o) : max(r[k], o);
+      }
+    }
+  }
+}
+
+// Words s_w[0, m) in order, as rows.
+template <int K>
+__device__ __forceinline__ void sorted_rows(const uint64_t* s_w, uint64_t* s_buf, uint32_t m,
+                                            uint32_t j_bits, xtn_triple* __restrict__ rows,
+                                            int64_t row_cap) {
+  uint64_t r[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t x = threadIdx.x + k * SR_THREADS;
+    r[k] = x < m ? s_w[x] : ~0ull;
+  }
+  block_sort<K>(r, s_buf);
+  const uint64_t jmask = (1ull << j_bits) - 1ull;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const uint32_t x = threadIdx.x + k * SR_THREADS;
+    if (x < m && (int64_t)x < row_cap) {
+      xtn_triple t;
+      t.i = (uint32_t)(r[k] >> 2 >> j_bits);
+      t.j = (uint32_t)(r[k] >> 2 & jmask);
+      t.dist = (uint32_t)(r[k] & 3u);
+      rows[x] = t;
+    }
+  }
+}
+
+// Shared memory, in words: the hash table (later the sort's exchange
+// buffers), the rows' words.
+constexpr uint32_t SR_SLOTS = 2 * (uint32_t)SMALL_PAIRS;  // at most half full
+constexpr size_t SR_SMEM = (SR_SLOTS + SMALL_PAIRS) * 8;
+
+__global__ void __launch_bounds__(SR_THREADS)
+    k_small_rows(const uint64_t* __restrict__ cand, uint32_t n, uint32_t j_bits, PairSide si,
+                 PairSide sj, const uint32_t* __restrict__ seq_rep, int self_mode, int d,
+                 int metric, xtn_triple* __restrict__ rows, int64_t row_cap,
+                 uint64_t* __restrict__ n_rows, uint32_t* __restrict__ err) {
+  static_assert(SMALL_PAIRS == 4 * SR_THREADS, "up to four words a thread");
+  extern __shared__ uint64_t s_slot[];
+  uint64_t* s_w = s_slot + SR_SLOTS;  // pair << 2 | distance (at most 3)
+  __shared__ uint32_t s_n;
+  if (threadIdx.x == 0) s_n = 0;
+  for (uint32_t k = threadIdx.x; k < SR_SLOTS; k += SR_THREADS) s_slot[k] = ~0ull;
+  __syncthreads();
+  for (uint32_t t0 = threadIdx.x & ~31u; t0 < n; t0 += SR_THREADS) {
+    const uint32_t t = t0 + lane_id();
+    uint64_t w = 0;
+    uint32_t dist = 0;
+    bool ok = false;
+    if (t < n) {
+      w = cand[t];  // not ~0: two bits are free above the pair
+      uint32_t h = (uint32_t)((w * HASH_B) >> 32) % SR_SLOTS;
+      for (;;) {  // ends: the table has free slots
+        const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(s_slot + h), ~0ull,
+                                       (unsigned long long)w);
+        if (old == w) break;
+        if (old == ~0ull) {
+          ok = true;
+          break;
+        }
+        h = (h + 1) % SR_SLOTS;
+      }
+      ok = ok && verified(w, j_bits, si, sj, seq_rep, self_mode, d, metric, err, dist);
+    }
+    const uint32_t bal = __ballot_sync(FULL_MASK, ok);
+    uint32_t at = 0;
+    if (lane_id() == 0 && bal) at = atomicAdd(&s_n, (uint32_t)__popc(bal));
+    at = __shfl_sync(FULL_MASK, at, 0) + __popc(bal & ((1u << lane_id()) - 1u));
+    if (ok) s_w[at] = w << 2 | dist;  // at < n <= SMALL_PAIRS
+  }
+  __syncthreads();
+  const uint32_t m = s_n;
+  if (threadIdx.x == 0) *n_rows = m;
+  if (m <= SR_THREADS)
+    sorted_rows<1>(s_w, s_slot, m, j_bits, rows, row_cap);
+  else if (m <= 2 * SR_THREADS)
+    sorted_rows<2>(s_w, s_slot, m, j_bits, rows, row_cap);
+  else
+    sorted_rows<4>(s_w, s_slot, m, j_bits, rows, row_cap);
+}
+
+void launch_small_rows(const uint64_t* cand, uint64_t n, uint32_t j_bits, const PairSide& si,
+                       const PairSide& sj, const uint32_t* seq_rep, int self_mode, int d,
+                       int metric, xtn_triple* rows, int64_t row_cap, uint64_t* n_rows,
+                       uint32_t* err, cudaStream_t s) {
+  cudaFuncSetAttribute(k_small_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SR_SMEM);
+  prof_begin(s, "k_small_rows", (double)n * (8.0 + 2 * 32.0));
+  k_small_rows<<<1, SR_THREADS, SR_SMEM, s>>>(cand, (uint32_t)n, j_bits, si, sj, seq_rep, self_mode, d,
+                                        metric, rows, row_cap, n_rows, err);
   prof_end(s);
 }
 
@@ -384,43 +541,65 @@ __constant__ int8_t c_blosum62[20][20] = {
 
 // TCRdist-style CDR3 score: gaps after the first floor(m/2) residues of the
 // shorter sequence, mismatch cost min(4, 4 - BLOSUM62), gap cost 4, weight 3.
-__device__ __forceinline__ int tcrdist_score(const Key128& a, int la, const Key128& b, int lb) {
+// cost: the mismatch costs by residue codes, 32 bytes a row.
+__device__ __forceinline__ int tcrdist_score(const uint8_t* cost, const Key128& a, int la,
+                                             const Key128& b, int lb) {
   const bool a_short = la <= lb;
-  const Key128& sk = a_short ? a : b;
-  const Key128& lk = a_short ? b : a;
+  const Key128 s = a_short ? a : b;
+  const Key128 l = a_short ? b : a;
   const int m = a_short ? la : lb;
   const int g = (a_short ? lb : la) - m;
+  int sum = 4 * g;
+  // the halves before and behind the gaps, residue by residue off the keys
+  auto half = [&](Key128 x, Key128 y, int count) {
+    for (int k = 0; k < count; ++k) {
+      sum += cost[((uint32_t)x.lo & 31u) << 5 | ((uint32_t)y.lo & 31u)];
+      x.lo = (x.lo >> 5) | (x.hi << 59);
+      x.hi >>= 5;
+      y.lo = (y.lo >> 5) | (y.hi << 59);
+      y.hi >>= 5;
+    }
+  };
   const int p = m / 2;
-  int sum = 0;
-  for (int k = 0; k < m; ++k) {
-    const uint32_t x = code_at(sk, k);
-    const uint32_t y = code_at(lk, k < p ? k : k + g);
-    if (x != y) sum += min(4, 4 - (int)c_blosum62[x - 1][y - 1]);
-  }
-  return 3 * (sum + 4 * g);
+  half(s, l, p);
+  half(shr128(s, 5 * p), shr128(l, 5 * (p + g)), m - p);
+  return 3 * sum;
 }
 
+// ITEMS rows a thread, in the order of the input.
+template <int ITEMS>
 __global__ void __launch_bounds__(VER_THREADS)
     k_tcrdist_filter(const xtn_triple* __restrict__ in, int64_t n, const Key128* __restrict__ keys,
                      const uint8_t* __restrict__ lens, int64_t n_seq, int max_score,
                      xtn_triple* __restrict__ out, uint64_t* __restrict__ status,
                      uint32_t* __restrict__ ctr, uint32_t* __restrict__ err,
                      uint64_t* __restrict__ total_out) {
+  constexpr int TILE = VER_THREADS * ITEMS;
+  __shared__ uint8_t s_cost[32 * 32];
   __shared__ uint32_t s_tile;
   __shared__ uint32_t s_w[VER_THREADS / 32];
   __shared__ uint64_t s_prefix;
-  const uint32_t tile = tile_id(ctr, &s_tile);
-  const int64_t tbase = (int64_t)tile * VER_TILE;
-  const int64_t base = tbase + (int64_t)threadIdx.x * VER_ITEMS;
+  // codes 0 (a letter outside the alphabet: the call reports it) and past 20
+  // cost like a gap
+  for (int k = threadIdx.x; k < 32 * 32; k += VER_THREADS) {
+    const int x = k >> 5, y = k & 31;
+    s_cost[k] = x == y ? 0
+                : x >= 1 && x <= 20 && y >= 1 && y <= 20
+                    ? (uint8_t)min(4, 4 - (int)c_blosum62[x - 1][y - 1])
+                    : 4;
+  }
+  const uint32_t tile = tile_id(ctr, &s_tile);  // a barrier: the costs are complete
+  const int64_t tbase = (int64_t)tile * TILE;
+  const int64_t base = tbase + (int64_t)threadIdx.x * ITEMS;
   uint32_t keep = 0, cnt = 0;
 #pragma unroll
-  for (int it = 0; it < VER_ITEMS; ++it) {
+  for (int it = 0; it < ITEMS; ++it) {
     const int64_t p = base + it;
     if (p < n) {
       const xtn_triple t = in[p];
       bool ok = false;
       if (t.i < n_seq && t.j < n_seq) {
-        ok = tcrdist_score(keys[t.i], lens[t.i], keys[t.j], lens[t.j]) <= max_score;
+        ok = tcrdist_score(s_cost, keys[t.i], lens[t.i], keys[t.j], lens[t.j]) <= max_score;
       } else {
         atomicOr(err, DERR_RANGE);
       }
@@ -434,13 +613,13 @@ __global__ void __launch_bounds__(VER_THREADS)
     const uint64_t pre = warp_lookback(status, tile, total, err);
     if (threadIdx.x == 0) {
       s_prefix = pre;
-      if (tbase + VER_TILE >= n) *total_out = pre + total;
+      if (tbase + TILE >= n) *total_out = pre + total;
     }
   }
   __syncthreads();
   int64_t o = (int64_t)(s_prefix + excl);
 #pragma unroll
-  for (int it = 0; it < VER_ITEMS; ++it)
+  for (int it = 0; it < ITEMS; ++it)
     if (keep >> it & 1u) {
       if (o < n) out[o] = in[base + it];
       ++o;
@@ -453,10 +632,20 @@ void launch_tcrdist_filter(const xtn_triple* in, int64_t n, const Key128* keys,
   if (n <= 0) return;
   const size_t st = verify_status_bytes(n);
   uint32_t* ctr = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(status) + st - 16);
+  // one row a thread while the blocks fit the chip at once: 11,700 rows on 6
+  // blocks took 37 us, most of it the serial walk of eight rows; past it
+  // eight rows amortise the look-back
+  const bool few = n <= FEW_ROWS;
+  static_assert(VER_TILE == VERIFY_TILE && VER_THREADS == VERIFY_TILE / 8,
+                "the status is sized for both");
   cudaMemsetAsync(status, 0, st, s);
   prof_begin(s, "k_tcrdist_filter", (double)n * (12.0 * 2 + 2 * 17.0));
-  k_tcrdist_filter<<<div_up_u32(n, VER_TILE), VER_THREADS, 0, s>>>(
-      in, n, keys, lens, n_seq, max_score, out, status, ctr, err, total);
+  if (few)
+    k_tcrdist_filter<1><<<div_up_u32(n, VER_THREADS), VER_THREADS, 0, s>>>(
+        in, n, keys, lens, n_seq, max_score, out, status, ctr, err, total);
+  else
+    k_tcrdist_filter<VER_ITEMS><<<div_up_u32(n, VER_TILE), VER_THREADS, 0, s>>>(
+        in, n, keys, lens, n_seq, max_score, out, status, ctr, err, total);
   prof_end(s);
 }
 

@@ -226,6 +226,13 @@ struct Key128 {
   uint64_t lo, hi;
 };
 
+__device__ __forceinline__ Key128 shr128(const Key128& k, uint32_t s) {
+  if (s >= 128) return Key128{0ull, 0ull};
+  if (s >= 64) return Key128{k.hi >> (s - 64), 0ull};
+  if (s == 0) return k;
+  return Key128{(k.lo >> s) | (k.hi << (64 - s)), k.hi >> s};
+}
+
 // The same sequence as bit planes: bit p of plane k is bit k of residue p's
 // code (a.x .. a.w planes 0-3, b.x plane 4; b.y the length).  Two sequences'
 // differing positions, on any diagonal, are then a few operations on whole
@@ -233,6 +240,23 @@ struct Key128 {
 struct __align__(32) PlaneRow {
   uint4 a, b;
 };
+
+// A row as one 32-byte access: a gather of rows, or a warp's stores of 32 of
+// them, are then half as many requests to the memory system as 16-byte
+// accesses make.
+__device__ __forceinline__ PlaneRow load_row(const PlaneRow* p) {
+  PlaneRow r;
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r.a.x), "=r"(r.a.y), "=r"(r.a.z), "=r"(r.a.w), "=r"(r.b.x), "=r"(r.b.y),
+                 "=r"(r.b.z), "=r"(r.b.w)
+               : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void store_row(PlaneRow* p, const PlaneRow& r) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r.a.x),
+               "r"(r.a.y), "r"(r.a.z), "r"(r.a.w), "r"(r.b.x), "r"(r.b.y), "r"(r.b.z), "r"(r.b.w)
+               : "memory");
+}
 
 // Residue code at position p (0 <= p < 25).
 __device__ __forceinline__ uint32_t code_at(const Key128& k, int p) {

@@ -24,7 +24,13 @@ std::atomic<int>& cfg_pairs();
 // k_variants.cu ------------------------------------------------------------
 void launch_encode(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Key128* keys,
                    uint8_t* lens, uint32_t* eqprev, uint32_t* vcount, PlaneRow* rows,
-                   uint32_t* err, cudaStream_t s);  // rows may be null
+                   uint32_t* err, cudaStream_t s);  // vcount and rows may be null
+// The same with the counts summed up: rec_off[0, n], the total also to
+// *total.  status: encode_status_bytes(n), zeroed.
+size_t encode_status_bytes(int64_t n);
+void launch_encode_scan(const uint8_t* seqs, const int64_t* off, int64_t n, int d, Key128* keys,
+                        uint8_t* lens, uint32_t* eqprev, uint64_t* rec_off, uint64_t* total,
+                        uint64_t* status, PlaneRow* rows, uint32_t* err, cudaStream_t s);
 // Record selection by fingerprint bin, bin = (record >> shift) & mask, for
 // searches that take the records in several passes.  With `append` null the
 // expand kernel only counts records per bin into bin_count[0 .. mask] (mask
@@ -191,11 +197,16 @@ void launch_emit_pairs(const uint64_t* keys, uint64_t n_keys, const uint32_t* S,
                        cudaStream_t s);
 
 // k_verify.cu --------------------------------------------------------------
-// Rows per tile of the verify, dedup and TCRdist kernels, and the look-back
-// status those kernels need for n rows (one word per tile plus a tile counter).
+// Rows per tile of the dedup and TCRdist kernels, and the look-back status
+// those kernels need for n rows (one word per tile plus a tile counter).  Up
+// to FEW_ROWS the TCRdist kernel takes tiles of an eighth.
 constexpr int VERIFY_TILE = 2048;
+constexpr int64_t FEW_ROWS = 1 << 18;
 constexpr size_t verify_status_bytes_for(int64_t n) {
-  return (size_t)((n + VERIFY_TILE - 1) / VERIFY_TILE) * 8 + 16;
+  const int64_t few = n < FEW_ROWS ? n : FEW_ROWS;
+  constexpr int64_t eighth = VERIFY_TILE / 8;
+  const int64_t a = (n + VERIFY_TILE - 1) / VERIFY_TILE, b = (few + eighth - 1) / eighth;
+  return (size_t)(a > b ? a : b) * 8 + 16;
 }
 // The sequences one side of the pairs indexes: their bit planes, and for
 // paired receptors (metric 2) those of their second chains.
@@ -205,8 +216,8 @@ struct PairSide {
   uint64_t n = 0;
 };
 // metric: 0 = Levenshtein, 1 = Hamming (pairs of equal length only), 2 =
-// paired chains (Levenshtein of the first chains plus that of the second).  Verify writes a survivor's distance into bits
-// [hist_hi, hist_hi + 8) of its word when they exist (hist_hi + 8 <= 64);
+// paired chains (Levenshtein of the first chains plus that of the second).
+// Verify writes a survivor's distance into bits [hist_hi, hist_hi + 8) of its word when they exist (hist_hi + 8 <= 64);
 // the dedup then reads it there (dist_shift = hist_hi) instead of computing
 // it again (dist_shift = 0).
 // self_mode: 0 = query vs reference, 1 = self-search (pairs within a
@@ -221,7 +232,15 @@ void launch_verify_candidates(const uint64_t* cand, uint64_t n, const uint64_t* 
 void launch_unique_finalize(const uint64_t* pairs, int64_t n, const uint64_t* n_dev,
                             uint32_t j_bits, const PairSide& si, const PairSide& sj, int d,
                             int metric, xtn_triple* out, int64_t cap, uint64_t* status,
-                            uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift);
+                            uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift,
+                            bool status_zeroed = false);
+// The whole last step for at most SMALL_PAIRS candidates in one block: their
+// distances, the sort, the duplicates out, the rows (*n_rows of them).
+constexpr uint64_t SMALL_PAIRS = 4096;
+void launch_small_rows(const uint64_t* cand, uint64_t n, uint32_t j_bits, const PairSide& si,
+                       const PairSide& sj, const uint32_t* seq_rep, int self_mode, int d,
+                       int metric, xtn_triple* rows, int64_t row_cap, uint64_t* n_rows,
+                       uint32_t* err, cudaStream_t s);
 void launch_tcrdist_filter(const xtn_triple* in, int64_t n, const Key128* keys,
                            const uint8_t* lens, int64_t n_seq, int max_score, xtn_triple* out,
                            uint64_t* status, uint32_t* err, uint64_t* total, cudaStream_t s);
