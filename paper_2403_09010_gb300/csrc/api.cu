@@ -1494,8 +1494,9 @@ struct xtn_index {
   uint32_t* dir = nullptr;
   int64_t bytes = 0;
   uint64_t n_groups = 0;  // distinct variant fingerprints in the index
-  // candidates and query variants of the searches so far (scratch estimates)
-  mutable std::atomic<uint64_t> seen_cand{0}, seen_qv{0};
+  // candidates, query variants and queries of the searches so far (scratch
+  // estimates)
+  mutable std::atomic<uint64_t> seen_cand{0}, seen_qv{0}, seen_q{0};
 };
 
 namespace xtn {
@@ -1579,6 +1580,15 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   return XTN_OK;
 }
 
+// Candidate words a query search makes room for before it knows their number:
+// twice what this index has given per query so far, else 32 a query.
+uint64_t query_cand_guess(const xtn_index* idx, int64_t n_q) {
+  const uint64_t q = idx->seen_q.load(), c = idx->seen_cand.load();
+  const double rate = q ? 2.0 * (double)c / (double)q : 32.0;
+  return std::max<uint64_t>(1u << 17, (uint64_t)(rate * (double)n_q));
+}
+constexpr uint64_t QUERY_LIST = 1u << 13;  // chunks of large groups, likewise
+
 // metric: 0 = Levenshtein, 1 = Hamming (the index's candidates serve both:
 // Hamming neighbours within d share the string left after deleting the
 // differing positions).
@@ -1596,49 +1606,52 @@ int search_query_impl(const xtn_index* idx, const uint8_t* q_seqs, const int64_t
   Arena ar(s);
   Control* ctl = nullptr;
   uint64_t* front_status = nullptr;
-  XTN_RC(take_control(ar, encode_status_bytes(n_q), s, &ctl, &front_status));
+  XTN_RC(take_control(ar, 0, s, &ctl, &front_status));
   uint32_t* err = ctl->err;
   DevSeqs in;
   rc = stage_seqs(q_seqs, q_offsets, n_q, ar, s, &in);
   if (rc) return rc;
   Encoded e;
-  rc = encode_and_count(in, idx->d, ar, ctl, front_status, s, &e);
-  if (rc) return rc;
-  const uint64_t n_qv = e.n_rec;
-  uint32_t* qv_start = ar.get<uint32_t>(n_qv);
-  uint32_t* qv_cnt = ar.get<uint32_t>(n_qv);
-  uint32_t* qv_q = ar.get<uint32_t>(n_qv);
-  uint64_t* cand_off = ar.get<uint64_t>(n_qv + 1);
-  uint64_t* status = ar.get<uint64_t>(scan_status_bytes(n_qv) / 8 + 1);
+  e.keys = ar.get<Key128>(n_q);
+  e.lens = ar.get<uint8_t>(n_q);
+  e.eqprev = ar.get<uint32_t>(n_q);
+  e.rows = ar.get<PlaneRow>(n_q);
+  // buffers by a guess; past it the lookup runs again with what it counted
+  uint64_t cand_cap = query_cand_guess(idx, n_q), list_cap = QUERY_LIST;
+  uint64_t* P1 = ar.get<uint64_t>(cand_cap + 8);
+  QueryChunk* list = ar.get<QueryChunk>(list_cap);
   XTN_ALLOC_OK(ar);
-  launch_query_lookup(e.keys, e.lens, e.eqprev, e.rec_off, n_q, n_qv, idx->d, idx->rec,
-                      idx->n_rec, idx->dir, idx->dir_bits, 64 - idx->hs, qv_start, qv_cnt, qv_q,
-                      sms, err, s);
-  launch_scan_counts(qv_cnt, (int64_t)n_qv, cand_off, status, err, s);
-  XTN_CK(cudaGetLastError());
-  struct {
-    uint64_t cand;
-    uint32_t err;
-  } hc{0, 0};
-  {
+  launch_encode(in.seqs, in.off, n_q, idx->d, e.keys, e.lens, e.eqprev, nullptr, e.rows, err, s);
+  Control h{};
+  uint64_t n_cand = 0, n_list = 0;
+  for (;;) {  // at most twice
+    launch_query_candidates(e.source(), n_q, idx->d, idx->rec, idx->n_rec, idx->dir,
+                            idx->dir_bits, 64 - idx->hs, idx->id_bits, P1, cand_cap,
+                            ctl->counters, list, list_cap, ctl->counters + 1, &ctl->n_rec, sms,
+                            err, s);
+    XTN_CK(cudaGetLastError());
     ReadBack rb(s);
-    XTN_RC(rb.add(&hc.cand, cand_off + n_qv));
-    XTN_RC(rb.add(&hc.err, err));
+    XTN_RC(rb.add(&h, ctl));
     XTN_RC(rb.wait());
+    if (h.err[0]) return map_device_err(h.err[0]);
+    n_cand = h.counters[0];
+    n_list = h.counters[1];
+    if (h.n_rec >= (1ull << 32) || n_cand >= (1ull << 32)) return XTN_ERR_TOO_LARGE;
+    if (n_cand <= cand_cap && n_list <= list_cap) break;
+    if (n_cand > cand_cap) P1 = ar.get<uint64_t>((cand_cap = n_cand) + 8);
+    if (n_list > list_cap) list = ar.get<QueryChunk>(list_cap = n_list);
+    XTN_ALLOC_OK(ar);
+    XTN_CK(cudaMemsetAsync(ctl->counters, 0, 16, s));
+    XTN_CK(cudaMemsetAsync(&ctl->n_rec, 0, 8, s));
   }
-  if (hc.err) return map_device_err(hc.err);
-  const uint64_t n_cand = hc.cand;
   idx->seen_cand += n_cand;
-  idx->seen_qv += n_qv;
+  idx->seen_qv += h.n_rec;
+  idx->seen_q += (uint64_t)n_q;
   if (n_cand == 0) return XTN_OK;
-  if (n_cand >= (1ull << 32)) return XTN_ERR_TOO_LARGE;
   const uint32_t q_bits = bits_for((uint64_t)n_q);
   const uint32_t pair_bits = q_bits + idx->id_bits;
   if (pair_bits > 64) return XTN_ERR_TOO_LARGE;
-  uint64_t* P1 = ar.get<uint64_t>(n_cand + 8);
-  XTN_ALLOC_OK(ar);
-  launch_query_emit(idx->rec, idx->n_rec, idx->id_bits, qv_start, qv_q, cand_off, n_qv, n_cand,
-                    P1, sms, err, s);
+  launch_query_spread(idx->rec, idx->n_rec, idx->id_bits, list, n_list, P1, cand_cap, sms, err, s);
   XTN_CK(cudaGetLastError());
   OutRows o;
   rc = prepare_out(out, cap, n_cand, ar, &o);
@@ -1646,7 +1659,6 @@ int search_query_impl(const xtn_index* idx, const uint8_t* q_seqs, const int64_t
   XTN_RC(finish_pairs(P1, n_cand, pair_bits, idx->id_bits, e.side(n_q),
                       PairSide{idx->rows, nullptr, (uint64_t)idx->n}, nullptr, 0, idx->d, metric,
                       o.dev, o.dev_cap, sms, ctl, ar, s));
-  Control h{};
   ReadBack rb(s);
   XTN_RC(rb.add(&h, ctl));
   XTN_RC(rb.wait());
@@ -2094,8 +2106,8 @@ int xtn_search_query_scratch(const xtn_index* idx, const int64_t* q_offsets, int
   const uint64_t per_buffer = 64 + 256;  // arena spare bytes and alignment
   uint64_t b = 0;
   b += 16 + letters + 8 * (n + 1);                                   // errors, staging
-  b += n * (16 + 1 + 4 + 4) + 8 * (n + 1) + scan_status_bytes((int64_t)n);  // encode
-  b += n_qv * 12 + 8 * (n_qv + 1) + scan_status_bytes((int64_t)n_qv);      // lookup
+  b += n * (16 + 1 + 4);                                             // encode
+  b += QUERY_LIST * sizeof(QueryChunk) + 8 * query_cand_guess(idx, n_q);  // lookup
   b += 16 * (n_cand + 8) + MAX_PASSES * RADIX * 12 + 16;             // candidate words
   b += back_status_bytes(n_cand, cfg) + 32 * n;                      // sort, bit planes
   b += 12 * n_cand;                                                  // rows for host output

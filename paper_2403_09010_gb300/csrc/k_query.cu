@@ -7,16 +7,22 @@
 //                    range of ~n_rec / 2^dir_bits records (a few, with the
 //                    directory sized at about one entry per 4 records)
 //                    instead of all.
-//   k_query_lookup : one warp per query, one lane per deletion variant (same
-//                    order as the self-search expansion): binary search of the
-//                    variant's fingerprint group inside its directory range;
-//                    writes the group's start and size.
-//   k_query_emit   : candidate t finds its query variant by binary search over
-//                    the candidate offsets, reads the reference id at the
-//                    matching index position and writes (q << ref_bits) | r.
+//   k_query_candidates : the queries' variants (expand.cuh), a lane each: the
+//                    variant's directory range is read and compared, and the
+//                    references of equal fingerprint go out at once as
+//                    candidate words (q << ref_bits) | r, collected per warp.
+//                    Bound by the memory system's rate of random requests
+//                    (about 30 G lines/s for reads of this kind, whatever
+//                    their locality): a lookup is one line of the directory
+//                    and 1.3 of the records, so 1.1 M of them (10,000 queries,
+//                    d = 2, a 10M index) take 85 us alone, 120 here.  Lookup,
+//                    count scan and emission as kernels of their own took
+//                    128 + 19 + 16 us, through 20 bytes written and read a
+//                    variant; 40 queries 17 + 8 + 11 us instead of 10.
+//   k_query_spread : groups too large for one lane, a warp per 1,024 records.
 #include <algorithm>
 
-#include "variants.cuh"
+#include "expand.cuh"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -54,145 +60,253 @@ void launch_build_dir(const uint64_t* rec, uint64_t n_rec, int dir_bits, int gsh
   prof_end(s);
 }
 
-// Group [lo, hi) of fingerprint fp in the sorted index (empty if absent).
-__device__ __forceinline__ void index_range(const uint64_t* __restrict__ rec, uint64_t n_rec,
-                                            const uint32_t* __restrict__ dir, int dir_bits,
-                                            int gshift, uint64_t fp, uint32_t* err, uint64_t& a,
-                                            uint64_t& c) {
-  const uint64_t g = fp >> gshift;
-  const uint64_t top = fp >> (64 - dir_bits);
-  uint64_t lo = dir[top], hi = dir[top + 1];
+constexpr int QC_THREADS = 256;
+constexpr int QC_WARPS = QC_THREADS / 32;
+constexpr int QC_BLOCKS = 4;           // of an SM
+constexpr uint32_t QC_FLUSH = 96;      // words a warp collects before a flush
+constexpr uint32_t QC_DIRECT = 256;    // records of a group a warp emits by itself
+constexpr uint32_t QC_CHUNK = 1024;    // and of larger ones, per entry of the list
+constexpr uint64_t QC_SCAN = 32;       // longer directory ranges are searched
+
+template <int KIND>
+struct QuerySmem {
+  using K = VK<KIND>;
+  uint64_t terms[QC_WARPS][K::PACK][K::STRIDE];
+  uint64_t stash[QC_WARPS][QC_FLUSH + 32];
+  uint64_t pow[N_POWERS<KIND>];
+  VarMeta meta[QC_WARPS][K::PACK];
+  uint16_t extra[QC_WARPS][K::PACK][K::EXTRA + 1];
+  uint16_t comb[K::COMBS + 1];
+};
+
+// Group of key g in the index: first record *at, number of records.
+__device__ __forceinline__ uint32_t index_group(const uint64_t* __restrict__ rec, uint64_t n_rec,
+                                                const uint32_t* __restrict__ dir, uint64_t top,
+                                                int gshift, uint64_t g, uint32_t* err,
+                                                uint32_t& at) {
+  uint64_t lo = __ldg(dir + top), hi = __ldg(dir + top + 1);
   if (hi > n_rec || lo > hi) {
     atomicOr(err, DERR_RANGE);
-    lo = hi = 0;
+    return 0u;
   }
-  a = lo;
-  uint64_t b = hi;  // lower bound of g
-  while (a < b) {
-    const uint64_t mid = (a + b) >> 1;
-    if ((rec[mid] >> gshift) < g) a = mid + 1; else b = mid;
+  if (hi - lo > QC_SCAN) {
+    uint64_t e = hi;  // lower bound
+    while (lo < e) {
+      const uint64_t mid = (lo + e) >> 1;
+      if ((__ldg(rec + mid) >> gshift) < g) lo = mid + 1; else e = mid;
+    }
+    uint64_t c = lo;  // upper bound
+    e = hi;
+    while (c < e) {
+      const uint64_t mid = (c + e) >> 1;
+      if ((__ldg(rec + mid) >> gshift) <= g) c = mid + 1; else e = mid;
+    }
+    at = (uint32_t)lo;
+    return (uint32_t)(c - lo);
   }
-  c = a;
-  uint64_t e = hi;  // upper bound of g
-  while (c < e) {
-    const uint64_t mid = (c + e) >> 1;
-    if ((rec[mid] >> gshift) <= g) c = mid + 1; else e = mid;
+  uint32_t below = 0, equal = 0;
+  for (uint64_t p = lo; p < hi; p += 4) {  // four at a time: one round trip, not four
+    uint64_t r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[k] = p + k < hi ? __ldg(rec + p + k) >> gshift : ~0ull;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      below += r[k] < g;
+      equal += r[k] == g && p + k < hi;
+    }
+    if (r[3] > g) break;
   }
+  at = (uint32_t)lo + below;
+  return equal;
 }
 
-__global__ void __launch_bounds__(256)
-    k_query_lookup(const Key128* __restrict__ qkeys, const uint8_t* __restrict__ qlens,
-                   const uint32_t* __restrict__ qeqprev, const uint64_t* __restrict__ q_rec_off,
-                   int64_t n_q, uint64_t n_qv, int d, const uint64_t* __restrict__ rec,
-                   uint64_t n_rec, const uint32_t* __restrict__ dir, int dir_bits, int gshift,
-                   uint32_t* __restrict__ qv_start, uint32_t* __restrict__ qv_cnt,
-                   uint32_t* __restrict__ qv_q, uint32_t* __restrict__ err) {
-  __shared__ VariantTables s_tab;
-  __shared__ WarpVariants s_warp[8];
-  init_variant_tables(&s_tab);
+// A warp takes `pack` consecutive queries (or a share of them, `parts` warps
+// the same ones): few queries would otherwise leave most of the chip idle
+// and give a lane many lookups in turn.
+template <int KIND>
+__global__ void __launch_bounds__(QC_THREADS, QC_BLOCKS)
+    k_query_candidates(ExpandSource src, int64_t n_q, int d, const uint64_t* __restrict__ rec,
+                       uint64_t n_rec, const uint32_t* __restrict__ dir, int dir_bits, int gshift,
+                       uint32_t ref_bits, int pack, int parts, uint64_t* __restrict__ cand,
+                       uint64_t cand_cap, unsigned long long* __restrict__ n_cand,
+                       QueryChunk* __restrict__ list, uint64_t list_cap,
+                       unsigned long long* __restrict__ n_list,
+                       unsigned long long* __restrict__ n_variants, uint32_t* __restrict__ err) {
+  using K = VK<KIND>;
+  extern __shared__ __align__(16) unsigned char query_smem[];
+  QuerySmem<KIND>& S = *reinterpret_cast<QuerySmem<KIND>*>(query_smem);
+  load_powers<KIND>(S.pow);
+  load_combs<KIND>(S.comb);
   __syncthreads();
-  WarpVariants* w = &s_warp[threadIdx.x >> 5];
-  const uint32_t lane = lane_id();
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t q = warp0; q < n_q; q += n_warps) {
-    const uint32_t L = qlens[q];
-    const uint32_t eq = qeqprev[q];
-    const uint64_t base = q_rec_off[q];
-    uint32_t cnt = (uint32_t)(q_rec_off[q + 1] - base);
-    if (base + cnt > n_qv) {
-      if (lane == 0) atomicOr(err, DERR_RANGE);
-      cnt = 0;
+  const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+  const uint64_t idmask = (1ull << ref_bits) - 1ull;
+  uint64_t* stash = S.stash[warp];
+  uint32_t held = 0;  // words in the stash, the same in every lane
+  auto flush = [&] {
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(n_cand, (unsigned long long)held);
+    base = __shfl_sync(FULL_MASK, base, 0);
+    __syncwarp();  // every lane's words are visible
+    for (uint32_t k = lane; k < held; k += 32)
+      if (base + k < cand_cap) cand[base + k] = stash[k];  // past it: counted, the caller reruns
+    __syncwarp();
+    held = 0;
+  };
+  const int q = (int)lane / K::LANES;
+  VarMeta* meta = S.meta[warp];
+  uint64_t variants = 0;
+  const int64_t units = (n_q + pack - 1) / pack * parts;
+  const int64_t n_warps = (int64_t)gridDim.x * QC_WARPS;
+  for (int64_t u = (int64_t)blockIdx.x * QC_WARPS + warp; u < units; u += n_warps) {
+    const int64_t s0 = u / parts * pack;
+    const uint32_t part = (uint32_t)(u % parts);
+    const int64_t my = s0 + q;
+    const bool have = q < pack && my < n_q;
+    VarMeta m;
+    uint64_t* terms = S.terms[warp][q];
+    const uint32_t total =
+        prepare_variants<KIND>(terms, S.extra[warp][q], S.pow, src, my, have, d, 0ull, lane, m,
+                               [&](uint32_t a, uint64_t h) { terms[a] = h; });
+    uint32_t end = total;
+#pragma unroll
+    for (int o = K::LANES; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(FULL_MASK, end, o);
+      if (lane >= (uint32_t)o) end += t;
     }
-    const SeqShape sh = warp_prepare(w, &s_tab, qkeys[q], L, eq, lane);
-    if (d <= 2) {
-      uint32_t total = canonical_total_d2(sh, d);
-      if (total != cnt) {
-        if (lane == 0) atomicOr(err, DERR_RANGE);
-        total = 0;
-      }
-      for (uint32_t v = lane; v < total; v += 32) {
-        uint64_t a, c;
-        index_range(rec, n_rec, dir, dir_bits, gshift,
-                    canonical_fingerprint_d2(w, &s_tab, sh, v, 0ull), err, a, c);
-        qv_start[base + v] = (uint32_t)a;
-        qv_cnt[base + v] = (uint32_t)(c - a);
-        qv_q[base + v] = (uint32_t)q;
-      }
-    } else {
-      const uint32_t total = cnt ? variant_count(L, (uint32_t)d) : 0u;
-      uint32_t written = 0;
-      for (uint32_t v0 = 0; v0 < total; v0 += 32) {
-        const uint32_t v = v0 + lane;
-        bool keep = false;
-        Subset ss{0u, 0u, 0u, 0u};
-        if (v < total) {
-          ss = unrank_subset(L, v);
-          keep = is_canonical(subset_mask(ss), eq);
+    const uint32_t T = __shfl_sync(FULL_MASK, end, 31);
+    if (part == 0) variants += T;
+    if (lane % K::LANES == 0) {
+      m.end = (int32_t)end;
+      m.adj += (int32_t)(end - total);
+      meta[q] = m;
+    }
+    __syncwarp();  // terms and meta, written above, are read by every lane
+    const VarMeta* at = meta;
+    VarMeta cur = meta[0];
+    uint32_t id = (uint32_t)s0;
+    const uint64_t* tab = S.terms[warp][0];
+    const uint16_t* extra = S.extra[warp][0];
+    for (uint32_t t0 = part * 32; t0 < T; t0 += 32u * (uint32_t)parts) {
+      const uint32_t t = t0 + lane;
+      uint32_t first = 0, count = 0;
+      if (t < T) {
+        while ((int32_t)t >= cur.end) {  // ends: t < T, the last query's end
+          cur = *++at;
+          ++id;
+          tab += K::STRIDE;
+          extra += K::EXTRA + 1;
         }
-        const uint32_t bal = __ballot_sync(FULL_MASK, keep);
-        const uint32_t slot = written + __popc(bal & lt_mask);
-        written += __popc(bal);
-        if (keep && slot < cnt) {
-          uint64_t a, c;
-          index_range(rec, n_rec, dir, dir_bits, gshift, subset_fingerprint(w, L, ss, 0ull), err,
-                      a, c);
-          qv_start[base + slot] = (uint32_t)a;
-          qv_cnt[base + slot] = (uint32_t)(c - a);
-          qv_q[base + slot] = (uint32_t)q;
+        const uint64_t h = mix64(variant_sum<KIND>(
+            tab, extra, S.comb, (uint32_t)((int32_t)t - cur.adj), cur.c, cur.aux));
+        count = index_group(rec, n_rec, dir, h >> (64 - dir_bits), gshift, h >> gshift, err,
+                            first);
+        if (count > QC_DIRECT) {
+          const uint32_t chunks = (count + QC_CHUNK - 1) / QC_CHUNK;
+          const uint64_t base = atomicAdd(n_cand, (unsigned long long)count);
+          const uint64_t slot = atomicAdd(n_list, (unsigned long long)chunks);
+          for (uint32_t k = 0; k < chunks; ++k) {
+            const uint32_t o = k * QC_CHUNK;
+            if (slot + k < list_cap)
+              list[slot + k] = QueryChunk{base + o, first + o, min(QC_CHUNK, count - o), id, 0u};
+          }
+          count = 0;
         }
+      }
+      // the round's records, 32 at a time whosever they are: a lane finds the
+      // lane that a record belongs to among the counts' prefix sums
+      uint32_t ends = count;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(FULL_MASK, ends, o);
+        if (lane >= (uint32_t)o) ends += x;
+      }
+      const uint32_t words = __shfl_sync(FULL_MASK, ends, 31);
+      const uint32_t from = first - (ends - count);  // word k of its own is record from + k
+      for (uint32_t k0 = 0; k0 < words; k0 += 32) {
+        const uint32_t k = k0 + lane;
+        int owner = 0;  // lanes whose words all come before k
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(FULL_MASK, ends, owner + o - 1) <= k) owner += o;
+        owner = min(owner, 31);
+        const uint32_t p = __shfl_sync(FULL_MASK, from, owner) + k;
+        const uint32_t whose = __shfl_sync(FULL_MASK, id, owner);
+        if (k < words)
+          stash[held + lane] = ((uint64_t)whose << ref_bits) | (__ldg(rec + p) & idmask);
+        held += min(32u, words - k0);
+        if (held >= QC_FLUSH) flush();  // at most QC_FLUSH + 31 words
       }
     }
+    __syncwarp();  // the next queries reuse terms and meta
   }
+  if (held) flush();
+  if (lane == 0 && variants) atomicAdd(n_variants, (unsigned long long)variants);
 }
 
-void launch_query_lookup(const Key128* qkeys, const uint8_t* qlens, const uint32_t* qeqprev,
-                         const uint64_t* q_rec_off, int64_t n_q, uint64_t n_qv, int d,
-                         const uint64_t* rec, uint64_t n_rec, const uint32_t* dir,
-                         int dir_bits, int gshift, uint32_t* qv_start, uint32_t* qv_cnt,
-                         uint32_t* qv_q, int sms, uint32_t* err, cudaStream_t s) {
+template <int KIND>
+static void query_launch(const ExpandSource& src, int64_t n_q, int d, const uint64_t* rec,
+                         uint64_t n_rec, const uint32_t* dir, int dir_bits, int gshift,
+                         uint32_t ref_bits, uint64_t* cand, uint64_t cand_cap, uint64_t* n_cand,
+                         QueryChunk* list, uint64_t list_cap, uint64_t* n_list,
+                         uint64_t* n_variants, int sms, uint32_t* err, cudaStream_t s) {
+  using ull = unsigned long long;
+  auto f = k_query_candidates<KIND>;
+  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)sizeof(QuerySmem<KIND>));
+  // `pack` as large as leaves a resident warp four units of work: one query a
+  // unit for 10,000 (132 us with two), 30,000 of a 36M-record index 125 us
+  // against 147 with six
+  const int64_t warps = (int64_t)sms * QC_BLOCKS * QC_WARPS;  // resident at once
+  const int pack =
+      (int)std::min<int64_t>(VK<KIND>::PACK, std::max<int64_t>(1, n_q / (4 * warps)));
+  const int64_t groups = (n_q + pack - 1) / pack;
+  const int parts = (int)std::min<int64_t>(8, std::max<int64_t>(1, warps / groups));
+  const uint32_t blocks =
+      (uint32_t)std::min<int64_t>((groups * parts + QC_WARPS - 1) / QC_WARPS, sms * QC_BLOCKS);
+  f<<<blocks, QC_THREADS, sizeof(QuerySmem<KIND>), s>>>(
+      src, n_q, d, rec, n_rec, dir, dir_bits, gshift, ref_bits, pack, parts, cand, cand_cap,
+      reinterpret_cast<ull*>(n_cand), list, list_cap, reinterpret_cast<ull*>(n_list),
+      reinterpret_cast<ull*>(n_variants), err);
+}
+
+void launch_query_candidates(const ExpandSource& src, int64_t n_q, int d, const uint64_t* rec,
+                             uint64_t n_rec, const uint32_t* dir, int dir_bits, int gshift,
+                             uint32_t ref_bits, uint64_t* cand, uint64_t cand_cap,
+                             uint64_t* n_cand, QueryChunk* list, uint64_t list_cap,
+                             uint64_t* n_list, uint64_t* n_variants, int sms, uint32_t* err,
+                             cudaStream_t s) {
   if (n_q <= 0) return;
-  const int blocks = (int)std::min<int64_t>((n_q + 7) / 8, (int64_t)sms * 8);
-  prof_begin(s, "k_query_lookup", (double)n_q * 30.0);
-  k_query_lookup<<<blocks, 256, 0, s>>>(qkeys, qlens, qeqprev, q_rec_off, n_q, n_qv, d, rec, n_rec,
-                                        dir, dir_bits, gshift, qv_start, qv_cnt, qv_q, err);
+  prof_begin(s, "k_query_candidates", (double)n_q * 32.0);
+  auto f = d <= 1 ? query_launch<VK_D1> : d == 2 ? query_launch<VK_D2> : query_launch<VK_D3>;
+  f(src, n_q, d, rec, n_rec, dir, dir_bits, gshift, ref_bits, cand, cand_cap, n_cand, list,
+    list_cap, n_list, n_variants, sms, err, s);
   prof_end(s);
 }
 
 __global__ void __launch_bounds__(256)
-    k_query_emit(const uint64_t* __restrict__ rec, uint64_t n_rec, uint32_t ref_bits,
-                 const uint32_t* __restrict__ qv_start, const uint32_t* __restrict__ qv_q,
-                 const uint64_t* __restrict__ cand_off, uint64_t n_qv, uint64_t n_cand,
-                 uint64_t* __restrict__ out, uint32_t* __restrict__ err) {
+    k_query_spread(const uint64_t* __restrict__ rec, uint64_t n_rec, uint32_t ref_bits,
+                   const QueryChunk* __restrict__ list, uint64_t n_list,
+                   uint64_t* __restrict__ cand, uint64_t cand_cap, uint32_t* __restrict__ err) {
   const uint64_t idmask = (1ull << ref_bits) - 1ull;
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_cand;
-       t += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t lo = 0, hi = n_qv;  // largest v with cand_off[v] <= t
-    while (hi - lo > 1) {
-      const uint64_t mid = (lo + hi) >> 1;
-      if (cand_off[mid] <= t) lo = mid; else hi = mid;
+  const uint64_t stride = (uint64_t)gridDim.x * 8;
+  for (uint64_t e = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5); e < n_list; e += stride) {
+    const QueryChunk c = list[e];
+    if ((uint64_t)c.first + c.count > n_rec || c.base + c.count > cand_cap) {
+      if (lane_id() == 0) atomicOr(err, DERR_RANGE);
+      continue;
     }
-    const uint64_t pos = (uint64_t)qv_start[lo] + (t - cand_off[lo]);
-    uint64_t w = 0;
-    if (pos < n_rec) {
-      w = ((uint64_t)qv_q[lo] << ref_bits) | (rec[pos] & idmask);
-    } else {
-      atomicOr(err, DERR_RANGE);
-    }
-    out[t] = w;
+    for (uint32_t k = lane_id(); k < c.count; k += 32)
+      cand[c.base + k] = ((uint64_t)c.q << ref_bits) | (rec[c.first + k] & idmask);
   }
 }
 
-void launch_query_emit(const uint64_t* rec, uint64_t n_rec, uint32_t ref_bits,
-                       const uint32_t* qv_start, const uint32_t* qv_q, const uint64_t* cand_off,
-                       uint64_t n_qv, uint64_t n_cand, uint64_t* out, int sms, uint32_t* err,
-                       cudaStream_t s) {
-  if (n_cand == 0) return;
-  const int blocks = (int)std::min<uint64_t>((n_cand + 255) / 256, (uint64_t)sms * 8);
-  prof_begin(s, "k_query_emit", (double)n_cand * 24.0);
-  k_query_emit<<<blocks, 256, 0, s>>>(rec, n_rec, ref_bits, qv_start, qv_q, cand_off, n_qv, n_cand,
-                                      out, err);
+void launch_query_spread(const uint64_t* rec, uint64_t n_rec, uint32_t ref_bits,
+                         const QueryChunk* list, uint64_t n_list, uint64_t* cand,
+                         uint64_t cand_cap, int sms, uint32_t* err, cudaStream_t s) {
+  if (n_list == 0) return;
+  const int blocks = (int)std::min<uint64_t>((n_list + 7) / 8, (uint64_t)sms * 8);
+  prof_begin(s, "k_query_spread", (double)n_list * QC_CHUNK * 16.0);
+  k_query_spread<<<blocks, 256, 0, s>>>(rec, n_rec, ref_bits, list, n_list, cand, cand_cap, err);
   prof_end(s);
 }
 

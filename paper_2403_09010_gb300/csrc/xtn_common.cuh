@@ -258,19 +258,6 @@ __device__ __forceinline__ void store_row(PlaneRow* p, const PlaneRow& r) {
                : "memory");
 }
 
-// Residue code at position p (0 <= p < 25).
-__device__ __forceinline__ uint32_t code_at(const Key128& k, int p) {
-  const int m = 5 * p;
-  uint64_t v;
-  if (m < 64) {
-    v = k.lo >> m;
-    if (m > 59) v |= k.hi << (64 - m);
-  } else {
-    v = k.hi >> (m - 64);
-  }
-  return (uint32_t)(v & 31u);
-}
-
 // ------------------------------------------------------- fingerprints ---
 // A residue string s_0..s_{L-1} (codes 1..20) is fingerprinted through the
 // polynomial H(s) = sum_k s_k B^k mod 2^64 (B odd, so B is invertible mod

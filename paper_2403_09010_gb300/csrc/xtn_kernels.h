@@ -258,14 +258,25 @@ void launch_paired_counts(const uint8_t* lens_a, const uint32_t* eq_a, const uin
 // (bits from gshift up).
 void launch_build_dir(const uint64_t* rec, uint64_t n_rec, int dir_bits, int gshift,
                       uint32_t* dir, uint64_t* n_groups, cudaStream_t s);
-void launch_query_lookup(const Key128* qkeys, const uint8_t* qlens, const uint32_t* qeqprev,
-                         const uint64_t* q_rec_off, int64_t n_q, uint64_t n_qv, int d,
-                         const uint64_t* rec, uint64_t n_rec, const uint32_t* dir,
-                         int dir_bits, int gshift, uint32_t* qv_start, uint32_t* qv_cnt,
-                         uint32_t* qv_q, int sms, uint32_t* err, cudaStream_t s);
-void launch_query_emit(const uint64_t* rec, uint64_t n_rec, uint32_t ref_bits,
-                       const uint32_t* qv_start, const uint32_t* qv_q, const uint64_t* cand_off,
-                       uint64_t n_qv, uint64_t n_cand, uint64_t* out, int sms, uint32_t* err,
-                       cudaStream_t s);
+// Records [first, first + count) of the index, candidates of query q, to
+// cand[base ...]: a part of a group too large for one lane.
+struct QueryChunk {
+  uint64_t base;
+  uint32_t first, count, q, unused;
+};
+// Candidate words of the queries: cand[0, *n_cand) but for the large groups,
+// whose places are reserved and which `list` names (launch_query_spread
+// writes them).  *n_cand above cand_cap or *n_list above list_cap: nothing is
+// written past either, and the counts say what a rerun needs.  *n_variants
+// receives the queries' variants.  The three counts begin at zero.
+void launch_query_candidates(const ExpandSource& src, int64_t n_q, int d, const uint64_t* rec,
+                             uint64_t n_rec, const uint32_t* dir, int dir_bits, int gshift,
+                             uint32_t ref_bits, uint64_t* cand, uint64_t cand_cap,
+                             uint64_t* n_cand, QueryChunk* list, uint64_t list_cap,
+                             uint64_t* n_list, uint64_t* n_variants, int sms, uint32_t* err,
+                             cudaStream_t s);
+void launch_query_spread(const uint64_t* rec, uint64_t n_rec, uint32_t ref_bits,
+                         const QueryChunk* list, uint64_t n_list, uint64_t* cand,
+                         uint64_t cand_cap, int sms, uint32_t* err, cudaStream_t s);
 
 }  // namespace xtn

@@ -80,3 +80,23 @@ def test_tcrdist_rows(xtn, n_rows):
         want = oracle.tcrdist_filter(seqs, off, rows, top)
         got = xtn.tcrdist_filter(seqs, off, rows, top)
         assert np.array_equal(_rows(got), want)
+
+
+@pytest.mark.parametrize("d", [0, 1, 2, 3])
+def test_lookup(xtn, d):
+    """Groups a lane emits alone, groups spread over warps, one query (split
+    between warps) to several a warp, more candidates than the first guess."""
+    rng = np.random.default_rng(d)
+    refs = (["CASSLGTDTQYF"] * 3000 + ["CASSPGQGAYEQYF"] * 256 + ["CATSDLNEQYF"] * 257
+            + ["CA", "", "A" * 25])
+    refs += ["".join(rng.choice(list("ACDEFGHIKLMNPQRSTVWY"), rng.integers(0, 26)))
+             for _ in range(2000)]
+    seqs, off = gen.from_strings([refs[i] for i in rng.permutation(len(refs))])
+    idx = xtn.index_build(*_cuda(seqs, off), d)
+    for qs in (["CASSLGTDTQYF"], ["A" * 25, "CASSPGQGAYEQYF", "CATSDLNEQYF", ""],
+               (refs[2990:3540] + refs[-900:]) * (1 if d == 3 else 7),
+               ["CASSLGTDTQYF"] * 300):
+        q, qo = gen.from_strings(qs)
+        want = oracle.bruteforce_query(seqs, off, q, qo, d, threads=0)
+        for _ in range(2):  # the second guess knows the first call's counts
+            assert np.array_equal(_rows(xtn.search_query(idx, *_cuda(q, qo), cap=len(want))), want)
