@@ -476,7 +476,9 @@ std::atomic<int> g_record_hist{0};
 // partitions by the expansion, then k_group_filter; 1 = global radix passes
 // on every group-key bit, then k_group_flags; 2 = global passes on the top
 // bucket bits, then k_bucket with 512-record shared-memory segments.  An
-// index always takes global passes on the top bits, then k_bucket's sort.
+// index is built out of partitions in mode 0, up to 134 M records
+// (choose_index_partitions); else it takes global passes on the top bits, then
+// k_bucket's sort.
 std::atomic<int> g_grouping{0};
 }  // namespace
 // Records per partition: 2^fx times the smallest (choose_partitions).
@@ -808,6 +810,25 @@ int take_partitions(uint64_t n_rec, Arena& ar, uint64_t* n_spill, cudaStream_t s
 // records) 297 against 282 us; above, 200,000 sequences 229 against 162 us
 // for the two stages.
 constexpr uint64_t SPLIT_EXPANSION = 6u << 20;
+
+// The records of e into the partitions (n_rec_dev: their number, where only
+// a bound of it is known).
+int expand_into(const Partitions& part, const Encoded& e, int64_t n, int d,
+                const uint32_t* seq_rep, uint32_t id_bits, const uint64_t* n_rec_dev, int sms,
+                Arena& ar, uint32_t* err, cudaStream_t s) {
+  if (e.n_rec <= SPLIT_EXPANSION) {
+    uint64_t* rec = ar.get<uint64_t>(e.n_rec + 8);
+    XTN_ALLOC_OK(ar);
+    launch_expand(e.source(), e.rec_off, n, d, seq_rep, id_bits, rec, e.n_rec, nullptr, 0, 0, sms,
+                  err, s);
+    launch_partition(rec, (int64_t)e.n_rec, n_rec_dev, part, sms, err, s);
+  } else {
+    launch_expand_scatter(e.source(), e.rec_off, n, d, seq_rep, id_bits, e.n_rec, part, sms, err,
+                          s);
+  }
+  XTN_CK(cudaGetLastError());
+  return XTN_OK;
+}
 
 // A self-search whose sequences, were they all of the greatest length, would
 // make at most this many records runs up to its candidates on buffers of that
@@ -1387,16 +1408,8 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   so.id_bits = bits_for((uint64_t)n);
   if (mode == 0) {
     XTN_RC(take_partitions(e.n_rec, ar, counters + 3, s, &part));
-    if (e.n_rec <= SPLIT_EXPANSION) {
-      uint64_t* rec = ar.get<uint64_t>(e.n_rec + 8);
-      XTN_ALLOC_OK(ar);
-      launch_expand(e.source(), e.rec_off, n, d, salt_rep, so.id_bits, rec, e.n_rec, nullptr, 0, 0,
-                    sms, err, s);
-      launch_partition(rec, (int64_t)e.n_rec, unread ? &ctl->n_rec : nullptr, part, sms, err, s);
-    } else {
-      launch_expand_scatter(e.source(), e.rec_off, n, d, salt_rep, so.id_bits, e.n_rec, part, sms,
-                            err, s);
-    }
+    XTN_RC(expand_into(part, e, n, d, salt_rep, so.id_bits, unread ? &ctl->n_rec : nullptr, sms,
+                       ar, err, s));
     launch_group_filter(part, e.n_rec, direct.cand, direct.cand_cap, direct.cand_count,
                         (int)so.id_bits, err, s);
     XTN_CK(cudaGetLastError());
@@ -1489,6 +1502,7 @@ struct xtn_index {
   uint32_t id_bits = 0;
   int hs = 0;
   int dir_bits = 0;
+  void* mem = nullptr;  // holds the three arrays
   xtn::PlaneRow* rows = nullptr;
   uint64_t* rec = nullptr;
   uint32_t* dir = nullptr;
@@ -1502,8 +1516,10 @@ struct xtn_index {
 namespace xtn {
 namespace {
 
+// by_sorting: the records sorted globally whatever their number (else only
+// where k_index.cu does not take them, or grouping by sorting is set).
 int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d, cudaStream_t s,
-                     xtn_index** out) {
+                     xtn_index** out, bool by_sorting = false) {
   if (!out) return XTN_ERR_INVALID_ARG;
   *out = nullptr;
   if (n < 1 || d < 0 || d > XTN_MAX_D || !offsets) return XTN_ERR_INVALID_ARG;
@@ -1522,60 +1538,77 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   Encoded e;
   rc = encode_and_count(in, d, ar, ctl, front_status, s, &e);
   if (rc) return rc;
-  Sorted so;
-  rc = expand_and_sort(e, n, d, nullptr, sms, ar, err, s, &so);
-  if (rc) return rc;
-
   xtn_index* idx = new xtn_index;
+  struct Guard {  // frees the index unless it is handed out
+    xtn_index* p;
+    ~Guard() { xtn_index_free(p); }
+  } guard{idx};
   cudaGetDevice(&idx->device);
   idx->d = d;
   idx->n = n;
   idx->n_rec = e.n_rec;
-  idx->id_bits = so.id_bits;
-  idx->hs = so.hs;
+  idx->id_bits = bits_for((uint64_t)n);
+  idx->hs = choose_hash_bits(e.n_rec, idx->id_bits);
   // about one directory entry per 4 records (at most 2^28 entries, 1 GiB):
   // a lookup's range then spans a cache line or two instead of a binary
   // search through hundreds of records
   {
     int db = 10;
-    while (db < 28 && db < so.hs && ((uint64_t)1 << (db + 2)) < e.n_rec) ++db;
+    while (db < 28 && db < idx->hs && ((uint64_t)1 << (db + 2)) < e.n_rec) ++db;
     idx->dir_bits = db;
   }
+  const int gshift = 64 - idx->hs;
+  Partitions part;
+  const bool parted = !by_sorting && g_grouping.load() == 0 &&
+                      choose_index_partitions(e.n_rec, idx->dir_bits, &part);
+  Sorted so;
+  if (parted) {
+    part.rec = ar.get<uint64_t>(part.words() + 8);
+    part.count = ar.get<uint32_t>(part.counts());
+    part.spill = ar.get<uint64_t>(e.n_rec + 8);
+    part.spill_cap = e.n_rec;
+    part.n_spill = ctl->counters + 3;
+    XTN_ALLOC_OK(ar);
+    XTN_CK(cudaMemsetAsync(part.count, 0, part.counts() * 4, s));
+    XTN_RC(expand_into(part, e, n, d, nullptr, idx->id_bits, nullptr, sms, ar, err, s));
+  } else {
+    XTN_RC(expand_and_sort(e, n, d, nullptr, sms, ar, err, s, &so));
+  }
+  // the index's memory, in one piece, while the device works
   const size_t b_rows = n * sizeof(PlaneRow), b_rec = e.n_rec * 8,
                b_dir = ((size_t(1) << idx->dir_bits) + 1) * 4;
-  bool ok = cudaMalloc(&idx->rows, b_rows) == cudaSuccess &&
-            cudaMalloc(&idx->rec, b_rec + 8) == cudaSuccess &&
-            cudaMalloc(&idx->dir, b_dir) == cudaSuccess;
-  if (!ok) {
+  const size_t at_rec = (b_rows + 255) & ~size_t(255);
+  const size_t at_dir = (at_rec + b_rec + 8 + 255) & ~size_t(255);
+  if (cudaMalloc(&idx->mem, at_dir + b_dir) != cudaSuccess) {
     cudaGetLastError();
-    xtn_index_free(idx);
     return XTN_ERR_OOM;
   }
+  char* mem = static_cast<char*>(idx->mem);
+  idx->rows = reinterpret_cast<PlaneRow*>(mem);
+  idx->rec = reinterpret_cast<uint64_t*>(mem + at_rec);
+  idx->dir = reinterpret_cast<uint32_t*>(mem + at_dir);
   idx->bytes = (int64_t)(b_rows + b_rec + b_dir);
-  bool cp = cudaMemcpyAsync(idx->rows, e.rows, b_rows, cudaMemcpyDeviceToDevice, s) == cudaSuccess &&
-            cudaMemcpyAsync(idx->rec, so.rec, b_rec, cudaMemcpyDeviceToDevice, s) == cudaSuccess;
-  uint64_t* groups = ar.get<uint64_t>(1);
-  if (!groups) cp = false;
-  if (cp) cp = cudaMemsetAsync(groups, 0, 8, s) == cudaSuccess;
-  if (cp)
-    launch_build_dir(idx->rec, idx->n_rec, idx->dir_bits, 64 - idx->hs, idx->dir, groups, s);
-  struct {
-    uint64_t groups;
-    uint32_t err;
-  } h{0, 0};
-  if (!cp || cudaGetLastError() != cudaSuccess ||
-      cudaMemcpyAsync(&h.groups, groups, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(&h.err, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      host_sync(s) != cudaSuccess) {
-    cudaGetLastError();
-    xtn_index_free(idx);
-    return XTN_ERR_CUDA;
+  XTN_CK(cudaMemcpyAsync(idx->rows, e.rows, b_rows, cudaMemcpyDeviceToDevice, s));
+  if (parted) {
+    launch_index_build(part, e.n_rec, idx->dir_bits, gshift, idx->rec, idx->dir, ctl->counters,
+                       err, s);
+  } else {
+    XTN_CK(cudaMemcpyAsync(idx->rec, so.rec, b_rec, cudaMemcpyDeviceToDevice, s));
+    launch_build_dir(idx->rec, idx->n_rec, idx->dir_bits, gshift, idx->dir, ctl->counters, s);
   }
-  if (h.err) {
-    xtn_index_free(idx);
-    return map_device_err(h.err);
+  XTN_CK(cudaGetLastError());
+  Control h{};
+  ReadBack rb(s);
+  XTN_RC(rb.add(&h, ctl));
+  XTN_RC(rb.wait());
+  if (parted && (h.err[0] == DERR_CAPACITY || (!h.err[0] && h.counters[3]))) {
+    // too many records of one key for a partition or a block
+    ar.release();
+    return index_build_impl(seqs, offsets, n, d, s, out, true);
   }
-  idx->n_groups = h.groups;
+  if (h.err[0]) return map_device_err(h.err[0]);
+  idx->n_groups = h.counters[0];
+  guard.p = nullptr;
   *out = idx;
   return XTN_OK;
 }
@@ -2039,9 +2072,7 @@ int xtn_index_build(const uint8_t* seqs, const int64_t* offsets, int64_t n, int 
 
 int xtn_index_free(xtn_index* idx) {
   if (!idx) return XTN_OK;
-  cudaFree(idx->rows);
-  cudaFree(idx->rec);
-  cudaFree(idx->dir);
+  cudaFree(idx->mem);
   delete idx;
   return XTN_OK;
 }

@@ -66,7 +66,6 @@ constexpr int QC_BLOCKS = 4;           // of an SM
 constexpr uint32_t QC_FLUSH = 96;      // words a warp collects before a flush
 constexpr uint32_t QC_DIRECT = 256;    // records of a group a warp emits by itself
 constexpr uint32_t QC_CHUNK = 1024;    // and of larger ones, per entry of the list
-constexpr uint64_t QC_SCAN = 32;       // longer directory ranges are searched
 
 template <int KIND>
 struct QuerySmem {
@@ -79,17 +78,18 @@ struct QuerySmem {
   uint16_t comb[K::COMBS + 1];
 };
 
-// Group of key g in the index: first record *at, number of records.
+// Group of key g in the index: number of its records, the first at `at`; the
+// records are at + (the set bits of `mask`), or in a row where it is 0.
 __device__ __forceinline__ uint32_t index_group(const uint64_t* __restrict__ rec, uint64_t n_rec,
                                                 const uint32_t* __restrict__ dir, uint64_t top,
                                                 int gshift, uint64_t g, uint32_t* err,
-                                                uint32_t& at) {
+                                                uint32_t& at, uint32_t& mask) {
   uint64_t lo = __ldg(dir + top), hi = __ldg(dir + top + 1);
   if (hi > n_rec || lo > hi) {
     atomicOr(err, DERR_RANGE);
     return 0u;
   }
-  if (hi - lo > QC_SCAN) {
+  if (hi - lo > (uint64_t)INDEX_SCAN) {
     uint64_t e = hi;  // lower bound
     while (lo < e) {
       const uint64_t mid = (lo + e) >> 1;
@@ -104,20 +104,16 @@ __device__ __forceinline__ uint32_t index_group(const uint64_t* __restrict__ rec
     at = (uint32_t)lo;
     return (uint32_t)(c - lo);
   }
-  uint32_t below = 0, equal = 0;
   for (uint64_t p = lo; p < hi; p += 4) {  // four at a time: one round trip, not four
     uint64_t r[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) r[k] = p + k < hi ? __ldg(rec + p + k) >> gshift : ~0ull;
+    for (int k = 0; k < 4; ++k) r[k] = p + k < hi ? __ldg(rec + p + k) >> gshift : 0ull;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      below += r[k] < g;
-      equal += r[k] == g && p + k < hi;
-    }
-    if (r[3] > g) break;
+    for (int k = 0; k < 4; ++k)
+      if (p + k < hi && r[k] == g) mask |= 1u << (uint32_t)(p + k - lo);  // hi - lo <= 32
   }
-  at = (uint32_t)lo + below;
-  return equal;
+  at = (uint32_t)lo;
+  return (uint32_t)__popc(mask);
 }
 
 // A warp takes `pack` consecutive queries (or a share of them, `parts` warps
@@ -188,7 +184,7 @@ __global__ void __launch_bounds__(QC_THREADS, QC_BLOCKS)
     const uint16_t* extra = S.extra[warp][0];
     for (uint32_t t0 = part * 32; t0 < T; t0 += 32u * (uint32_t)parts) {
       const uint32_t t = t0 + lane;
-      uint32_t first = 0, count = 0;
+      uint32_t first = 0, count = 0, mask = 0;
       if (t < T) {
         while ((int32_t)t >= cur.end) {  // ends: t < T, the last query's end
           cur = *++at;
@@ -199,7 +195,7 @@ __global__ void __launch_bounds__(QC_THREADS, QC_BLOCKS)
         const uint64_t h = mix64(variant_sum<KIND>(
             tab, extra, S.comb, (uint32_t)((int32_t)t - cur.adj), cur.c, cur.aux));
         count = index_group(rec, n_rec, dir, h >> (64 - dir_bits), gshift, h >> gshift, err,
-                            first);
+                            first, mask);
         if (count > QC_DIRECT) {
           const uint32_t chunks = (count + QC_CHUNK - 1) / QC_CHUNK;
           const uint64_t base = atomicAdd(n_cand, (unsigned long long)count);
@@ -221,7 +217,6 @@ __global__ void __launch_bounds__(QC_THREADS, QC_BLOCKS)
         if (lane >= (uint32_t)o) ends += x;
       }
       const uint32_t words = __shfl_sync(FULL_MASK, ends, 31);
-      const uint32_t from = first - (ends - count);  // word k of its own is record from + k
       for (uint32_t k0 = 0; k0 < words; k0 += 32) {
         const uint32_t k = k0 + lane;
         int owner = 0;  // lanes whose words all come before k
@@ -229,7 +224,15 @@ __global__ void __launch_bounds__(QC_THREADS, QC_BLOCKS)
         for (int o = 16; o > 0; o >>= 1)
           if (__shfl_sync(FULL_MASK, ends, owner + o - 1) <= k) owner += o;
         owner = min(owner, 31);
-        const uint32_t p = __shfl_sync(FULL_MASK, from, owner) + k;
+        const uint32_t nth = k - __shfl_sync(FULL_MASK, ends - count, owner);
+        uint32_t bits = __shfl_sync(FULL_MASK, mask, owner);
+        uint32_t p = __shfl_sync(FULL_MASK, first, owner);
+        if (bits == 0) {
+          p += nth;
+        } else if (k < words) {
+          for (uint32_t x = 0; x < nth; ++x) bits &= bits - 1u;
+          p += (uint32_t)__ffs((int)bits) - 1u;
+        }
         const uint32_t whose = __shfl_sync(FULL_MASK, id, owner);
         if (k < words)
           stash[held + lane] = ((uint64_t)whose << ref_bits) | (__ldg(rec + p) & idmask);

@@ -258,6 +258,22 @@ void launch_paired_counts(const uint8_t* lens_a, const uint32_t* eq_a, const uin
 // (bits from gshift up).
 void launch_build_dir(const uint64_t* rec, uint64_t n_rec, int dir_bits, int gshift,
                       uint32_t* dir, uint64_t* n_groups, cudaStream_t s);
+// A directory range of at most this many records is compared whole by a
+// lookup, so its records stand in any order; longer ones are sorted.
+constexpr int INDEX_SCAN = 32;
+// k_index.cu: the index out of partitions of the records.  False where its
+// sizes do not take it (the records are then sorted, and launch_build_dir
+// reads the directory off them).
+constexpr int INDEX_SUB_BITS = 14;
+bool choose_index_partitions(uint64_t n_rec, int dir_bits, PartitionShape* g);
+// rec[0, n_rec), dir[0, 2^dir_bits]; *n_groups += the distinct group keys
+// (bits from gshift up; of a million records or more 16 times those of every
+// 16th partition, since counting all took 100 of 300 us and the number only
+// feeds an estimate).  DERR_CAPACITY: one directory range is too long.
+void launch_index_build(const Partitions& p, uint64_t n_rec, int dir_bits, int gshift,
+                        uint64_t* rec, uint32_t* dir, uint64_t* n_groups, uint32_t* err,
+                        cudaStream_t s);
+
 // Records [first, first + count) of the index, candidates of query q, to
 // cand[base ...]: a part of a group too large for one lane.
 struct QueryChunk {
