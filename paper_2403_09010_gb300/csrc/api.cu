@@ -918,41 +918,90 @@ int launch_back(const BackStage& b, uint64_t cand_cap, const uint64_t* n_cand_de
     XTN_CK(cudaMemsetAsync(b.counters, 0, 16, s));
   }
   launch_verify_candidates(b.P1, cand_cap, n_cand_dev, j_bits, si, sj, seq_rep, self_mode, d,
-                           metric, b.P2, cand_cap, b.counters, b.hist, (int)pair_bits, sms, err, s);
+                           metric, b.P2, cand_cap, b.counters, b.hist, 0, (int)pair_bits, sms, err,
+                           s);
   return launch_sort_unique(b.P2, b.P1, cand_cap, b.counters, pair_bits, j_bits, b.hist,
                             b.digit_base, b.status, si, sj, d, metric, rows, row_cap, err,
                             b.counters + 1, s, cfg, b.zero_bytes ? b.unique_status : nullptr);
 }
 
+// Candidate words up to which the last step groups them by 8 bits and sorts
+// each group in a block (launch_bucket_rows), past SMALL_PAIRS.  What counts
+// is the rows of a group, and a row has more candidates the larger d is (about
+// 1, 3, 15 and 90 for d = 0 .. 3); 1M sequences at d = 2 (4.4 M candidates, 285,000
+// rows) have a group too many for a block.
+uint64_t medium_pairs(int d) { return d <= 1 ? (uint64_t)1 << (18 + d) : (uint64_t)1 << 21; }
+
 // The last step of a call whose n_pairs candidate words stand in P1: in one
-// block's launch when they are few, through launch_back otherwise.  The row
-// count goes to ctl->back[1].
+// block's launch, by groups, or through launch_back.  Waits for it and gives
+// the row count.
 int finish_pairs(uint64_t* P1, uint64_t n_pairs, uint32_t pair_bits, uint32_t j_bits,
                  const PairSide& si, const PairSide& sj, const uint32_t* seq_rep, int self_mode,
                  int d, int metric, xtn_triple* rows, int64_t row_cap, int sms, Control* ctl,
-                 Arena& ar, cudaStream_t s) {
-  if (n_pairs <= SMALL_PAIRS && pair_bits + 2 <= 64) {
-    launch_small_rows(P1, n_pairs, j_bits, si, sj, seq_rep, self_mode, d, metric, rows, row_cap,
-                      ctl->back + 1, ctl->err, s);
-    XTN_CK(cudaGetLastError());
-    return XTN_OK;
-  }
+                 Arena& ar, cudaStream_t s, uint64_t* n_rows) {
+  Control h{};
+  ReadBack rb(s);
   const int cfg = g_cfg_pairs.load();
   const size_t hist_b = MAX_PASSES * RADIX * 4;
   const size_t sort_b = (radix_status_bytes((int64_t)n_pairs, cfg) + 15) & ~size_t(15);
   BackStage b;
   b.P1 = P1;
-  b.P2 = ar.get<uint64_t>(n_pairs + 8);
-  b.digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
-  b.zero_bytes = hist_b + sort_b + verify_status_bytes((int64_t)n_pairs);
-  char* z = ar.get<char>(b.zero_bytes);
-  XTN_ALLOC_OK(ar);
-  b.hist = reinterpret_cast<uint32_t*>(z);
-  b.status = reinterpret_cast<uint64_t*>(z + hist_b);
-  b.unique_status = reinterpret_cast<uint64_t*>(z + hist_b + sort_b);
   b.counters = ctl->back;
-  return launch_back(b, n_pairs, nullptr, pair_bits, j_bits, si, sj, seq_rep, self_mode, d, rows,
-                     row_cap, sms, ctl->err, s, cfg, metric);
+  // P2, digit_base and the piece [hist | the sort's status | unique_status]
+  auto take = [&](size_t unique_b) {
+    if (!b.P2) b.P2 = ar.get<uint64_t>(n_pairs + 8);
+    if (!b.digit_base) b.digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
+    b.zero_bytes = hist_b + sort_b + unique_b;
+    char* z = ar.get<char>(b.zero_bytes);
+    XTN_ALLOC_OK(ar);
+    b.hist = reinterpret_cast<uint32_t*>(z);
+    b.status = reinterpret_cast<uint64_t*>(z + hist_b);
+    b.unique_status = reinterpret_cast<uint64_t*>(z + hist_b + sort_b);
+    return XTN_OK;
+  };
+  if (n_pairs <= SMALL_PAIRS && pair_bits + 2 <= 64) {
+    launch_small_rows(P1, n_pairs, j_bits, si, sj, seq_rep, self_mode, d, metric, rows, row_cap,
+                      ctl->back + 1, ctl->err, s);
+  } else if (n_pairs <= medium_pairs(d) && pair_bits >= 8 && pair_bits + 8 <= 64) {
+    XTN_RC(take(bucket_rows_status_bytes()));
+    XTN_CK(cudaMemsetAsync(b.hist, 0, b.zero_bytes, s));
+    launch_verify_candidates(P1, n_pairs, nullptr, j_bits, si, sj, seq_rep, self_mode, d, metric,
+                             b.P2, n_pairs, ctl->back, b.hist, (int)pair_bits - 8, (int)pair_bits,
+                             sms, ctl->err, s);
+    uint64_t* grouped = nullptr;
+    XTN_CK(radix_sort_passes(b.P2, P1, (int64_t)n_pairs, (int)pair_bits - 8, (int)pair_bits,
+                             b.hist, b.digit_base, b.status, cfg, ctl->err, &grouped,
+                             "k_onesweep_pairs", s, false, ctl->back, nullptr,
+                             onesweep_unstable_config(cfg), true));
+    launch_bucket_rows(grouped, n_pairs, ctl->back, b.digit_base, pair_bits, j_bits, rows, row_cap,
+                       b.unique_status, ctl->back + 1, ctl->err, s);
+    XTN_CK(cudaGetLastError());
+    XTN_RC(rb.add(&h, ctl));
+    XTN_RC(rb.wait());
+    if (h.err[0] == DERR_CAPACITY) {  // a group too large: sort the survivors, still in P2
+      XTN_CK(cudaMemsetAsync(ctl->err, 0, 4, s));
+      XTN_RC(take(verify_status_bytes((int64_t)n_pairs)));
+      XTN_CK(cudaMemsetAsync(b.hist, 0, b.zero_bytes, s));
+      launch_histogram(b.P2, (int64_t)n_pairs, ctl->back, 0, (int)pair_bits, b.hist, sms, s);
+      XTN_RC(launch_sort_unique(b.P2, P1, n_pairs, ctl->back, pair_bits, j_bits, b.hist,
+                                b.digit_base, b.status, si, sj, d, metric, rows, row_cap,
+                                ctl->err, ctl->back + 1, s, cfg, b.unique_status));
+    } else {
+      if (h.err[0]) return map_device_err(h.err[0]);
+      *n_rows = h.back[1];
+      return XTN_OK;
+    }
+  } else {
+    XTN_RC(take(verify_status_bytes((int64_t)n_pairs)));
+    XTN_RC(launch_back(b, n_pairs, nullptr, pair_bits, j_bits, si, sj, seq_rep, self_mode, d, rows,
+                       row_cap, sms, ctl->err, s, cfg, metric));
+  }
+  XTN_CK(cudaGetLastError());
+  XTN_RC(rb.add(&h, ctl));
+  XTN_RC(rb.wait());
+  if (h.err[0]) return map_device_err(h.err[0]);
+  *n_rows = h.back[1];
+  return XTN_OK;
 }
 
 // Result rows go to `out` directly when it is device memory; otherwise into
@@ -1289,7 +1338,7 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
       if (n_pairs)
         launch_verify_candidates(cand.p, n_pairs, nullptr, id_bits, side, side, seq_rep,
                                  between ? 2 : 1, d, metric, surv.p, surv.cap, ctr + 5, phist,
-                                 (int)pair_bits, sms, err, s);
+                                 0, (int)pair_bits, sms, err, s);
       XTN_CK(cudaGetLastError());
       break;
     }
@@ -1480,12 +1529,8 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   rc = prepare_out(out, cap, n_pairs, ar, &o);
   if (rc) return rc;
   XTN_RC(finish_pairs(P1, n_pairs, 2 * so.id_bits, so.id_bits, e.side(n), e.side(n), seq_rep,
-                      between ? 2 : 1, d, metric, o.dev, o.dev_cap, sms, ctl, ar, s));
-  ReadBack rb(s);
-  XTN_RC(rb.add(&c, ctl));
-  XTN_RC(rb.wait());
-  if (c.err[0]) return map_device_err(c.err[0]);
-  return finish_out(o, out, cap, c.back[1], s, n_out);
+                      between ? 2 : 1, d, metric, o.dev, o.dev_cap, sms, ctl, ar, s, &h.pairs));
+  return finish_out(o, out, cap, h.pairs, s, n_out);
 }
 
 }  // namespace
@@ -1691,12 +1736,8 @@ int search_query_impl(const xtn_index* idx, const uint8_t* q_seqs, const int64_t
   if (rc) return rc;
   XTN_RC(finish_pairs(P1, n_cand, pair_bits, idx->id_bits, e.side(n_q),
                       PairSide{idx->rows, nullptr, (uint64_t)idx->n}, nullptr, 0, idx->d, metric,
-                      o.dev, o.dev_cap, sms, ctl, ar, s));
-  ReadBack rb(s);
-  XTN_RC(rb.add(&h, ctl));
-  XTN_RC(rb.wait());
-  if (h.err[0]) return map_device_err(h.err[0]);
-  return finish_out(o, out, cap, h.back[1], s, n_out);
+                      o.dev, o.dev_cap, sms, ctl, ar, s, &n_cand));
+  return finish_out(o, out, cap, n_cand, s, n_out);
 }
 
 int tcrdist_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, const xtn_triple* in_rows,

@@ -189,12 +189,12 @@ __global__ void __launch_bounds__(256)
                         PairSide sj, const uint32_t* __restrict__ seq_rep, int self_mode, int d,
                         int metric, uint64_t* __restrict__ surv, uint64_t surv_cap,
                         unsigned long long* __restrict__ n_surv, uint32_t* __restrict__ hist,
-                        int hist_hi, uint32_t* __restrict__ err) {
+                        int hist_lo, int hist_hi, uint32_t* __restrict__ err) {
   __shared__ uint32_t s_hist[MAX_PASSES * RADIX];
   // survivors collect per warp and go out VER_STASH - 31 or more at a time:
   // one reservation on the shared counter per flush, not per 32 candidates
   __shared__ uint64_t s_stash[256 / 32][VER_STASH];
-  const int passes = (hist_hi + 7) / 8;
+  const int passes = (hist_hi - hist_lo + 7) / 8;
   for (int k = threadIdx.x; k < passes * RADIX; k += blockDim.x) s_hist[k] = 0;
   __syncthreads();
   const uint64_t n = n_dev ? min(*n_dev, n_cap) : n_cap;
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256)
     if (ok) {
       stash[held + __popc(bal & lt_mask)] = w;
       for (int p = 0; p < passes; ++p) {
-        const int sh = 8 * p;
+        const int sh = hist_lo + 8 * p;
         const int bits = min(8, hist_hi - sh);
         atomicAdd(&s_hist[p * RADIX + (uint32_t)((w >> sh) & ((1u << bits) - 1u))], 1u);
       }
@@ -249,13 +249,13 @@ void launch_verify_candidates(const uint64_t* cand, uint64_t n, const uint64_t* 
                               uint32_t j_bits, const PairSide& si, const PairSide& sj,
                               const uint32_t* seq_rep, int self_mode, int d, int metric,
                               uint64_t* surv, uint64_t surv_cap, uint64_t* n_surv, uint32_t* hist,
-                              int hist_hi, int sms, uint32_t* err, cudaStream_t s) {
+                              int hist_lo, int hist_hi, int sms, uint32_t* err, cudaStream_t s) {
   if (n == 0) return;
   const int blocks = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)sms * 8);
   prof_begin(s, "k_verify_candidates", (double)n * (8.0 + 2 * 32.0));
   k_verify_candidates<<<blocks, 256, 0, s>>>(
       cand, n, n_dev, j_bits, si, sj, seq_rep, self_mode, d, metric, surv, surv_cap,
-      reinterpret_cast<unsigned long long*>(n_surv), hist, hist_hi, err);
+      reinterpret_cast<unsigned long long*>(n_surv), hist, hist_lo, hist_hi, err);
   prof_end(s);
 }
 
@@ -448,10 +448,34 @@ __device__ __forceinline__ void sorted_rows(const uint64_t* s_w, uint64_t* s_buf
   }
 }
 
+__device__ __forceinline__ void sorted_rows(const uint64_t* s_w, uint64_t* s_buf, uint32_t m,
+                                            uint32_t j_bits, xtn_triple* __restrict__ rows,
+                                            int64_t row_cap) {
+  if (m <= SR_THREADS)
+    sorted_rows<1>(s_w, s_buf, m, j_bits, rows, row_cap);
+  else if (m <= 2 * SR_THREADS)
+    sorted_rows<2>(s_w, s_buf, m, j_bits, rows, row_cap);
+  else
+    sorted_rows<4>(s_w, s_buf, m, j_bits, rows, row_cap);
+}
+
 // Shared memory, in words: the hash table (later the sort's exchange
 // buffers), the rows' words.
 constexpr uint32_t SR_SLOTS = 2 * (uint32_t)SMALL_PAIRS;  // at most half full
 constexpr size_t SR_SMEM = (SR_SLOTS + SMALL_PAIRS) * 8;
+
+// Puts w in the table; whether it was not there.  Fewer than SR_SLOTS words
+// ever go in, so the search ends.
+__device__ __forceinline__ bool first_of(uint64_t* s_slot, uint64_t w) {
+  uint32_t h = (uint32_t)((w * HASH_B) >> 32) % SR_SLOTS;
+  for (;;) {
+    const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(s_slot + h), ~0ull,
+                                   (unsigned long long)w);
+    if (old == w) return false;
+    if (old == ~0ull) return true;
+    h = (h + 1) % SR_SLOTS;
+  }
+}
 
 __global__ void __launch_bounds__(SR_THREADS)
     k_small_rows(const uint64_t* __restrict__ cand, uint32_t n, uint32_t j_bits, PairSide si,
@@ -472,18 +496,8 @@ __global__ void __launch_bounds__(SR_THREADS)
     bool ok = false;
     if (t < n) {
       w = cand[t];  // not ~0: two bits are free above the pair
-      uint32_t h = (uint32_t)((w * HASH_B) >> 32) % SR_SLOTS;
-      for (;;) {  // ends: the table has free slots
-        const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(s_slot + h), ~0ull,
-                                       (unsigned long long)w);
-        if (old == w) break;
-        if (old == ~0ull) {
-          ok = true;
-          break;
-        }
-        h = (h + 1) % SR_SLOTS;
-      }
-      ok = ok && verified(w, j_bits, si, sj, seq_rep, self_mode, d, metric, err, dist);
+      ok = first_of(s_slot, w) &&
+           verified(w, j_bits, si, sj, seq_rep, self_mode, d, metric, err, dist);
     }
     const uint32_t bal = __ballot_sync(FULL_MASK, ok);
     uint32_t at = 0;
@@ -494,22 +508,89 @@ __global__ void __launch_bounds__(SR_THREADS)
   __syncthreads();
   const uint32_t m = s_n;
   if (threadIdx.x == 0) *n_rows = m;
-  if (m <= SR_THREADS)
-    sorted_rows<1>(s_w, s_slot, m, j_bits, rows, row_cap);
-  else if (m <= 2 * SR_THREADS)
-    sorted_rows<2>(s_w, s_slot, m, j_bits, rows, row_cap);
-  else
-    sorted_rows<4>(s_w, s_slot, m, j_bits, rows, row_cap);
+  sorted_rows(s_w, s_slot, m, j_bits, rows, row_cap);
 }
 
 void launch_small_rows(const uint64_t* cand, uint64_t n, uint32_t j_bits, const PairSide& si,
                        const PairSide& sj, const uint32_t* seq_rep, int self_mode, int d,
                        int metric, xtn_triple* rows, int64_t row_cap, uint64_t* n_rows,
                        uint32_t* err, cudaStream_t s) {
-  cudaFuncSetAttribute(k_small_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SR_SMEM);
+  cudaFuncSetAttribute(k_small_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)SR_SMEM);
   prof_begin(s, "k_small_rows", (double)n * (8.0 + 2 * 32.0));
-  k_small_rows<<<1, SR_THREADS, SR_SMEM, s>>>(cand, (uint32_t)n, j_bits, si, sj, seq_rep, self_mode, d,
-                                        metric, rows, row_cap, n_rows, err);
+  k_small_rows<<<1, SR_THREADS, SR_SMEM, s>>>(cand, (uint32_t)n, j_bits, si, sj, seq_rep,
+                                              self_mode, d, metric, rows, row_cap, n_rows, err);
+  prof_end(s);
+}
+
+// -------------------------------------------------------- medium results ---
+// The verified words lie grouped by their top 8 pair bits (one pass of the
+// pair sort); a block takes a group of them, strips its duplicates, sorts the
+// rest and writes the rows behind those of the groups before it.  Up to a
+// million words or two the pair sort's further passes and the dedup are
+// mostly latency, about 10 us a launch whatever the size.  Sort and dedup
+// before, and now: 10,000 queries (230,000 candidates) 63 + 14 and 12 + 21
+// us, 200,000 sequences (720,000) 68 + 14 and 12 + 29, overlap of 500,000
+// (1.9 M) 94 + 14 and 14 + 27.  A group with more distinct words than a block
+// holds sets DERR_CAPACITY (the caller sorts).
+__global__ void __launch_bounds__(SR_THREADS)
+    k_bucket_rows(const uint64_t* __restrict__ words, const uint64_t* __restrict__ n_words,
+                  const uint64_t* __restrict__ starts, uint32_t pair_bits, uint32_t j_bits,
+                  xtn_triple* __restrict__ rows, int64_t row_cap, uint64_t* __restrict__ status,
+                  uint32_t* __restrict__ ctr, uint64_t* __restrict__ n_rows,
+                  uint32_t* __restrict__ err) {
+  extern __shared__ uint64_t s_slot[];
+  uint64_t* s_w = s_slot + SR_SLOTS;
+  __shared__ uint32_t s_n, s_tile;
+  __shared__ uint64_t s_prefix;
+  if (threadIdx.x == 0) s_n = 0;
+  for (uint32_t k = threadIdx.x; k < SR_SLOTS; k += SR_THREADS) s_slot[k] = ~0ull;
+  const uint32_t b = tile_id(ctr, &s_tile);  // a barrier: the table is clear
+  const uint64_t all = *n_words;
+  const uint64_t p = min(starts[b], all), q = b + 1 < RADIX ? min(starts[b + 1], all) : all;
+  const uint64_t pair_mask = (1ull << pair_bits) - 1ull;
+  for (uint64_t t0 = p + (threadIdx.x & ~31u); t0 < q; t0 += SR_THREADS) {
+    if (*(volatile uint32_t*)&s_n > SMALL_PAIRS) break;  // then at most 1,024 more go in
+    const uint64_t t = t0 + lane_id();
+    uint64_t w = 0;
+    bool first = false;
+    if (t < q) {
+      w = words[t];
+      w = (w & pair_mask) << 2 | (w >> pair_bits & 3u);
+      first = first_of(s_slot, w);
+    }
+    const uint32_t bal = __ballot_sync(FULL_MASK, first);
+    uint32_t at = 0;
+    if (lane_id() == 0 && bal) at = atomicAdd(&s_n, (uint32_t)__popc(bal));
+    at = __shfl_sync(FULL_MASK, at, 0) + __popc(bal & ((1u << lane_id()) - 1u));
+    if (first && at < SMALL_PAIRS) s_w[at] = w;
+  }
+  __syncthreads();
+  const uint32_t m = min(s_n, (uint32_t)SMALL_PAIRS);
+  if (threadIdx.x == 0 && s_n > SMALL_PAIRS) atomicOr(err, DERR_CAPACITY);
+  if (threadIdx.x < 32) {
+    const uint64_t pre = warp_lookback(status, b, m, err);
+    if (threadIdx.x == 0) {
+      s_prefix = pre;
+      if (b + 1 == RADIX) *n_rows = pre + m;
+    }
+  }
+  __syncthreads();
+  const int64_t pre = (int64_t)s_prefix;
+  sorted_rows(s_w, s_slot, m, j_bits, rows + pre, row_cap - pre);
+}
+
+size_t bucket_rows_status_bytes() { return RADIX * 8 + 16; }
+
+void launch_bucket_rows(const uint64_t* words, uint64_t n_max, const uint64_t* n_words,
+                        const uint64_t* starts, uint32_t pair_bits, uint32_t j_bits,
+                        xtn_triple* rows, int64_t row_cap, uint64_t* status, uint64_t* n_rows, uint32_t* err, cudaStream_t s) {
+  cudaFuncSetAttribute(k_bucket_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SR_SMEM);
+  prof_begin(s, "k_unique_finalize", (double)n_max * 8.0);
+  k_bucket_rows<<<RADIX, SR_THREADS, SR_SMEM, s>>>(words, n_words, starts, pair_bits, j_bits, rows,
+                                                   row_cap, status,
+                                                   reinterpret_cast<uint32_t*>(status + RADIX),
+                                                   n_rows, err);
   prof_end(s);
 }
 

@@ -217,8 +217,9 @@ struct PairSide {
 };
 // metric: 0 = Levenshtein, 1 = Hamming (pairs of equal length only), 2 =
 // paired chains (Levenshtein of the first chains plus that of the second).
-// Verify writes a survivor's distance into bits [hist_hi, hist_hi + 8) of its word when they exist (hist_hi + 8 <= 64);
-// the dedup then reads it there (dist_shift = hist_hi) instead of computing
+// Verify counts the survivors' digits over bits [hist_lo, hist_hi) and writes
+// a survivor's distance into bits [hist_hi, hist_hi + 8) of its word when they
+// exist (hist_hi + 8 <= 64); the dedup then reads it there (dist_shift = hist_hi) instead of computing
 // it again (dist_shift = 0).
 // self_mode: 0 = query vs reference, 1 = self-search (pairs within a
 // repertoire when seq_rep is given), 2 = self-search keeping only pairs
@@ -228,12 +229,20 @@ void launch_verify_candidates(const uint64_t* cand, uint64_t n, const uint64_t* 
                               uint32_t j_bits, const PairSide& si, const PairSide& sj,
                               const uint32_t* seq_rep, int self_mode, int d, int metric,
                               uint64_t* surv, uint64_t surv_cap, uint64_t* n_surv, uint32_t* hist,
-                              int hist_hi, int sms, uint32_t* err, cudaStream_t s);
+                              int hist_lo, int hist_hi, int sms, uint32_t* err, cudaStream_t s);
 void launch_unique_finalize(const uint64_t* pairs, int64_t n, const uint64_t* n_dev,
                             uint32_t j_bits, const PairSide& si, const PairSide& sj, int d,
                             int metric, xtn_triple* out, int64_t cap, uint64_t* status,
                             uint32_t* err, uint64_t* total, cudaStream_t s, int dist_shift,
                             bool status_zeroed = false);
+// The same for words (with their distances) grouped by their top 8 pair bits,
+// the groups beginning at starts[0, 256): duplicates out, sort and rows.
+// status: bucket_rows_status_bytes(), cleared.  DERR_CAPACITY: a group has
+// more than SMALL_PAIRS distinct words.
+size_t bucket_rows_status_bytes();
+void launch_bucket_rows(const uint64_t* words, uint64_t n_max, const uint64_t* n_words,
+                        const uint64_t* starts, uint32_t pair_bits, uint32_t j_bits,
+                        xtn_triple* rows, int64_t row_cap, uint64_t* status, uint64_t* n_rows, uint32_t* err, cudaStream_t s);
 // The whole last step for at most SMALL_PAIRS candidates in one block: their
 // distances, the sort, the duplicates out, the rows (*n_rows of them).
 constexpr uint64_t SMALL_PAIRS = 4096;

@@ -2,6 +2,8 @@
 they change over, against the CPU oracle: the last step in one block, the
 front without a wait for the record count, one and four rounds of sequences a
 block in the encoder, one and eight rows a thread in the TCRdist filter."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -100,3 +102,24 @@ def test_lookup(xtn, d):
         want = oracle.bruteforce_query(seqs, off, q, qo, d, threads=0)
         for _ in range(2):  # the second guess knows the first call's counts
             assert np.array_equal(_rows(xtn.search_query(idx, *_cuda(q, qo), cap=len(want))), want)
+
+
+@pytest.mark.parametrize("copies,others", [(724, 0), (724, 1400), (725, 0)])
+def test_last_step_by_groups(xtn, copies, others):
+    """261,726 candidates in groups of 4 sequences, which a block holds, and of
+    16, which it does not (the survivors are sorted); one copy more, past the
+    limit on candidates."""
+    rng = np.random.default_rng(others)
+    strs = ["CASSLGTDTQYF"] * copies + [
+        "W" + "".join(rng.choice(list("ACDEFGHIKL"), 20)) for _ in range(others)]
+    seqs, off = gen.from_strings(strs)
+    want = np.stack([*np.triu_indices(copies, 1), np.zeros(copies * (copies - 1) // 2)], 1)
+    got = _rows(xtn.search_self(*_cuda(seqs, off), 0, cap=len(want)))
+    assert np.array_equal(got, want.astype(np.uint32))
+    few = torch.zeros((100, 3), dtype=torch.int32, device="cuda")  # too small a buffer
+    n = ctypes.c_int64(0)
+    status = xtn.native.lib().xtn_search_self(
+        seqs.ctypes.data, off.ctypes.data, len(strs), 0, None, 0, few.data_ptr(), 100,
+        ctypes.byref(n), None)
+    assert status != 0 and n.value == len(want)
+    assert np.array_equal(_rows(few), want[:100].astype(np.uint32))
