@@ -38,9 +38,9 @@ METRIC = "1M-seq d≤2 all-neighbour search time (s), verified pairs/s; query p5
 UNIT = "verified pairs/s"
 L2_FLUSH_BYTES = 256 << 20
 CPU_SAMPLE_N = 100_000
-ROOFLINE_KERNEL = "k_onesweep_records"
-ROOFLINE_SOURCE = os.path.join(ROOT, "paper_2403_09010_gb300", "csrc", "k_radix.cu")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_onesweep_records_traffic.txt")
+ROOFLINE_KERNEL = "k_expand"
+ROOFLINE_SOURCE = os.path.join(ROOT, "paper_2403_09010_gb300", "csrc", "k_scatter.cu")
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_expand_scatter_traffic.txt")
 
 
 def _dist():
@@ -79,7 +79,7 @@ def _peaks():
 
 
 def _traffic_per_record():
-    """DRAM bytes per sorted record from the committed ncu summary, or None
+    """DRAM bytes per expanded record from the committed ncu summary, or None
     when the kernel source changed since the counters were taken."""
     try:
         text = open(TRAFFIC_FILE).read()
@@ -659,7 +659,8 @@ def main():
         name, (nl, ms, nbytes) = top
         achieved = nbytes / (ms / 1000.0) / 1e9
         tpr = _traffic_per_record() if name == ROOFLINE_KERNEL else None
-        n_rec_per_launch = nbytes / nl / 16.0 if name == ROOFLINE_KERNEL else None
+        # k_expand accounts 8 bytes a record and 29 a sequence
+        n_rec_per_launch = (nbytes / nl - 29.0 * n) / 8.0 if name == ROOFLINE_KERNEL else None
         roofline = {"kernel": name, "bound": "hbm", "achieved": achieved, "peak": peak,
                     "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / peak,
                     "traffic": (tpr * n_rec_per_launch) if tpr and n_rec_per_launch else None,

@@ -13,7 +13,7 @@
 //                         residues) and pairs from different repertoires
 //                         (from the same one when searching between them),
 //                         reject |len_i - len_j| > d, compute the edit
-//                         distance bit-parallel, keep it if <= d.  Survivors
+//                         distance up to d, keep it if <= d.  Survivors
 //                         are appended with one atomic per warp; their radix
 //                         histograms are accumulated on the way.
 //   k_unique_finalize   : over the sorted survivors, drop a word equal to its
