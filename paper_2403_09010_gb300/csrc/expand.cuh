@@ -127,6 +127,13 @@ __device__ __forceinline__ void load_powers(uint64_t* s_pow) {
   }
 }
 
+// B^k, a constant where k is one.
+__host__ __device__ constexpr uint64_t power_of_b(int k) {
+  uint64_t p = 1;
+  for (int e = 0; e < k; ++e) p *= HASH_B;
+  return p;
+}
+
 // The sequences a kernel expands: one chain, or two with `b` fields set.
 struct ExpandSource {
   const Key128* keys = nullptr;
@@ -226,6 +233,32 @@ __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
     if (b >= 64) return (uint32_t)(k.hi >> (b - 64)) & 31u;
     return (uint32_t)((k.lo >> b) | (k.hi << (64 - b))) & 31u;
   };
+  if constexpr (KIND == VK_D1) {
+    // a lane has its sequence to itself: from one deleted position to the next
+    // the sum changes by (c[p] - c[p+1]) B^p, and with the loops unrolled the
+    // powers and the codes' shifts are constants: k_expand of 10M sequences
+    // 1,000 us, 1,250 with prefix sums by a loop over the longest length
+    const uint32_t longest = __reduce_max_sync(FULL_MASK, L);
+    uint64_t y = 0;  // the sum without position 0
+#pragma unroll
+    for (int q = 1; q < XTN_MAX_LEN; ++q) {
+      if ((uint32_t)q >= longest) break;  // uniform
+      y += (uint64_t)code(q) * power_of_b(q - 1);
+    }
+    const uint64_t none = y * HASH_B + code(0) + salt;
+    y += salt;
+#pragma unroll
+    for (int q = 0; q < XTN_MAX_LEN; ++q) {
+      if ((uint32_t)q >= longest) break;
+      if (my_runs >> q & 1u) put(a++, y);
+      y += (uint64_t)((int64_t)code(q) - (int64_t)code(q + 1)) * power_of_b(q);
+    }
+    m.c = m.aux = 0;
+    m.adj = d <= 0 ? -(int32_t)R : 0;  // only "none", numbered behind the runs
+    if (!have) return 0u;
+    put(R, none);
+    return d <= 0 ? 1u : R + 1u;
+  }
   constexpr int UNROLL = K::PER > 13 ? 5 : K::PER;
   // prefix sums at the chunk's start and at the end
   uint64_t sum = 0;
@@ -235,38 +268,36 @@ __device__ __forceinline__ uint32_t prepare_variants(uint64_t* __restrict__ tab,
   const uint64_t PL = K::LANES > 1 ? __shfl_sync(FULL_MASK, incl, K::LANES - 1, K::LANES) : incl;
   const uint64_t QL = PL * HASH_BINV, RL = PL * HASH_BINV2;
   const uint64_t SL = K::D == 3 ? PL * HASH_BINV3 : 0ull;
-  uint64_t P = incl - sum, Q = P * HASH_BINV, Rr = K::D >= 2 ? P * HASH_BINV2 : 0ull;
-  uint64_t S = K::D == 3 ? P * HASH_BINV3 : 0ull;
   // what every Y carries
   const uint64_t C = (K::D == 1 ? QL : K::D == 2 ? RL : SL) + salt;
-  uint64_t w0 = s_pow[p0], w1 = s_pow[p0 + 1], w2 = s_pow[p0 + 2];  // B^(p-3), B^(p-2), B^(p-1)
+  uint64_t w1 = s_pow[p0 + 1], w2 = s_pow[p0 + 2];  // B^(p-2), B^(p-1)
+  // the terms at p: Y - C = P[p] - Q[p+1], M = B^-1 (Y - C), Z = B^-1 M; one
+  // position on, Y changes by (c[p] - c[p+1]) B^p, M by B^-1 of that, Z by B^-2
+  // (1M sequences, d = 2: k_expand 633 us, 650 with P, Q, R carried along)
+  const uint64_t P = incl - sum;
+  const uint64_t y0 = P - P * HASH_BINV - (uint64_t)code(0) * w2;
+  uint64_t y = y0 + C, mm = K::D >= 2 ? y0 * HASH_BINV : 0ull;
+  uint64_t z = K::D == 3 ? mm * HASH_BINV : 0ull;
 #pragma unroll UNROLL
   for (int q = 0; q < K::PER; ++q) {
-    const uint64_t c = code(q);
     const uint64_t w3 = s_pow[p0 + q + 3];
-    const uint64_t Pn = P + c * w3;
-    const uint64_t Qn = Q + c * w2;
-    const uint64_t Rn = K::D >= 2 ? Rr + c * w1 : 0ull;
-    const uint64_t Sn = K::D == 3 ? S + c * w0 : 0ull;
     if ((my_runs >> q) & 1u) {
-      const uint64_t y = P - Qn + C;
       if constexpr (K::D == 1) {
         put(a, y);
       } else {
         tab[K::Y + a] = y;
-        tab[K::M + a] = Q - Rn;
+        tab[K::M + a] = mm;
         if constexpr (K::D == 3) {
-          tab[K::Z + a] = Rr - Sn;
+          tab[K::Z + a] = z;
           extra[a] = (uint16_t)(a | R << 5 | R << 10);
         }
       }
       ++a;
     }
-    P = Pn;
-    Q = Qn;
-    Rr = Rn;
-    S = Sn;
-    w0 = w1;
+    const uint64_t step = (uint64_t)((int64_t)code(q) - (int64_t)code(q + 1));
+    y += step * w3;
+    if (K::D >= 2) mm += step * w2;
+    if (K::D == 3) z += step * w1;
     w1 = w2;
     w2 = w3;
   }
