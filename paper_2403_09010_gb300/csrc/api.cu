@@ -1659,11 +1659,13 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
 }
 
 // Candidate words a query search makes room for before it knows their number:
-// twice what this index has given per query so far, else 32 a query.
+// twice what this index has given per query so far (no more than 256 a query
+// and 4 M, whatever earlier queries found), else 32 a query.
 uint64_t query_cand_guess(const xtn_index* idx, int64_t n_q) {
   const uint64_t q = idx->seen_q.load(), c = idx->seen_cand.load();
   const double rate = q ? 2.0 * (double)c / (double)q : 32.0;
-  return std::max<uint64_t>(1u << 17, (uint64_t)(rate * (double)n_q));
+  const uint64_t most = ((uint64_t)1 << 22) + 256 * (uint64_t)n_q;
+  return std::max<uint64_t>(1u << 17, (uint64_t)std::min(rate * (double)n_q, (double)most));
 }
 constexpr uint64_t QUERY_LIST = 1u << 13;  // chunks of large groups, likewise
 

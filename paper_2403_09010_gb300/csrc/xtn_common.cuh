@@ -180,43 +180,6 @@ __device__ __forceinline__ uint32_t tile_id(uint32_t* ctr, uint32_t* s_slot) {
   return *s_slot;
 }
 
-// ------------------------------------------------- bulk copies, mbarriers ---
-// One-dimensional bulk asynchronous copies (global -> this block's shared
-// memory) whose completion is counted on an mbarrier in shared memory.
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) from
-// global memory into this block's shared memory, counted on `bar`.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
-                                          uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
 // ------------------------------------------------------ packed sequences ---
 // A sequence of length L <= 25 is a 128-bit integer (lo, hi): residue p sits
 // at bits [5p, 5p+5) with codes 1..20 (alphabetical one-letter order), zero
@@ -266,8 +229,7 @@ __device__ __forceinline__ void store_row(PlaneRow* p, const PlaneRow& r) {
 // With prefix sums P[x] = sum_{k<x} s_k B^k, deleting positions
 // p1 < p2 < p3 gives
 //   H = P[p1] + (P[p2] - P[p1+1]) B^-1 + (P[p3] - P[p2+1]) B^-2 + (P[L] - P[p3+1]) B^-3,
-// (fewer deletions: the missing positions are L, L+1, L+2 and P[x] = P[L]
-// for x >= L), so a variant costs four table reads and three multiplies.
+// a sum of one term per deleted position (expand.cuh).
 // Equal strings give equal fingerprints whatever they were derived from, so
 // grouping by fingerprint finds every shared variant; unequal strings that
 // collide only add candidate pairs, which the exact distance check removes.
@@ -317,64 +279,9 @@ __host__ __device__ __forceinline__ uint32_t variant_count(uint32_t L, uint32_t 
   return c;
 }
 
-// Deletion subsets of the positions {0..L-1} with at most d elements, ranked
-// v = 0 (empty set), then every single position, every pair, every triple;
-// each size in colexicographic order ({p<q} has rank C(q,2)+p among pairs,
-// {p<q<r} has rank C(r,3)+C(q,2)+p among triples).  sum_{k<=d} C(L,k)
-// subsets in all (variant_count).
-struct Subset {
-  uint32_t k, p, q, r;  // size and positions (p < q < r, unused ones 0)
-};
-
-__device__ __forceinline__ Subset unrank_subset(uint32_t L, uint32_t v) {
-  Subset s{0u, 0u, 0u, 0u};
-  if (v == 0) return s;
-  if (v <= L) {
-    s.k = 1;
-    s.p = v - 1;
-    return s;
-  }
-  uint32_t t = v - 1 - L;
-  const uint32_t c2 = L * (L - 1) / 2;
-  if (t < c2) {
-    uint32_t q = (uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);
-    while (q * (q - 1) / 2 > t) --q;
-    while ((q + 1) * q / 2 <= t) ++q;
-    s.k = 2;
-    s.q = q;
-    s.p = t - q * (q - 1) / 2;
-    return s;
-  }
-  t -= c2;
-  uint32_t r = 2;
-  while (binom_small(r + 1, 3) <= t) ++r;
-  t -= binom_small(r, 3);
-  uint32_t q = 1;
-  while (binom_small(q + 1, 2) <= t) ++q;
-  t -= binom_small(q, 2);
-  s.k = 3;
-  s.r = r;
-  s.q = q;
-  s.p = t;
-  return s;
-}
-
-__device__ __forceinline__ uint32_t subset_mask(const Subset& s) {
-  uint32_t m = 0;
-  if (s.k >= 1) m |= 1u << s.p;
-  if (s.k >= 2) m |= 1u << s.q;
-  if (s.k >= 3) m |= 1u << s.r;
-  return m;
-}
-
 // Within a run of equal residues, deleting any c of its positions leaves the
-// same string, so only the leftmost-c choice is kept: a subset is canonical
-// when every deleted position p whose left neighbour holds the same residue
-// (bit p of `eqprev`) has that neighbour deleted too.  Every deletion variant
-// string still arises from exactly one canonical subset per run pattern.
-__device__ __forceinline__ bool is_canonical(uint32_t mask, uint32_t eqprev) {
-  return (eqprev & mask & ~(mask << 1)) == 0;
-}
+// same string, so only one choice of each run and count is kept: every
+// deletion variant string arises exactly once (expand.cuh).
 
 // ------------------------------------------------------------ host side ---
 // Launch bookkeeping: optional CUDA-event timing per kernel (see
