@@ -244,11 +244,11 @@ XTN_API int xtn_search_query(const xtn_index* idx, const uint8_t* q_seqs, const 
  * batches: *bytes receives the device bytes xtn_search_query (or its Hamming
  * variant) takes for n_q queries with these offsets (a host pointer, n_q+1
  * entries; the letters are not needed), counting host input and output
- * buffers.  The part set by the queries' lengths is an upper bound (every
- * deletion subset of at most d positions); the candidate part is estimated
- * from the candidates per query variant this index has produced in the
- * searches so far (before any: its mean number of records per variant
- * fingerprint), with a margin of 1.5x.  The call only reads host memory.
+ * buffers.  The candidate part is estimated from the candidates per query
+ * variant this index has produced in the searches so far (before any: its
+ * mean number of records per variant fingerprint) and an upper bound of the
+ * queries' variants (every deletion subset of at most d positions), with a
+ * margin of 1.5x.  The call only reads host memory.
  * Errors: INVALID_ARG, SEQ_TOO_LONG.
  */
 XTN_API int xtn_search_query_scratch(const xtn_index* idx, const int64_t* q_offsets, int64_t n_q,

@@ -802,26 +802,27 @@ int take_partitions(uint64_t n_rec, Arena& ar, uint64_t* n_spill, cudaStream_t s
   return XTN_OK;
 }
 
-// Records up to this many are expanded in sequence order and then parted in a
-// pass of their own, so that the profile of a small search still times the
-// two stages apart (k_expand, k_onesweep_records); more are expanded straight
-// into their partitions.  Below it that would make little difference: 10,000
-// sequences 221 against 221 us a search at d = 1, 50,000 at d = 2 (5.2 M
-// records) 297 against 282 us; above, 200,000 sequences 229 against 162 us
-// for the two stages.
+// Up to this many records, where their number is known, are expanded in
+// sequence order and then parted in a pass of their own, so that the profile
+// of a small search still times the two stages apart (k_expand,
+// k_onesweep_records).  More, and those of which only a bound is known, are
+// expanded straight into their partitions: 10,000 sequences at d = 1 128
+// against 137 us a search, 30,000 160 against 167, 50,000 at d = 2 (5.2 M
+// records, kept apart) 232 against 248, and for 200,000 162 against 229 us for
+// the two stages.
 constexpr uint64_t SPLIT_EXPANSION = 6u << 20;
 
-// The records of e into the partitions (n_rec_dev: their number, where only
-// a bound of it is known).
+// The records of e into the partitions (is_bound: e.n_rec is only a bound of
+// their number).
 int expand_into(const Partitions& part, const Encoded& e, int64_t n, int d,
-                const uint32_t* seq_rep, uint32_t id_bits, const uint64_t* n_rec_dev, int sms,
-                Arena& ar, uint32_t* err, cudaStream_t s) {
-  if (e.n_rec <= SPLIT_EXPANSION) {
+                const uint32_t* seq_rep, uint32_t id_bits, bool is_bound, int sms, Arena& ar,
+                uint32_t* err, cudaStream_t s) {
+  if (e.n_rec <= SPLIT_EXPANSION && !is_bound) {
     uint64_t* rec = ar.get<uint64_t>(e.n_rec + 8);
     XTN_ALLOC_OK(ar);
     launch_expand(e.source(), e.rec_off, n, d, seq_rep, id_bits, rec, e.n_rec, nullptr, 0, 0, sms,
                   err, s);
-    launch_partition(rec, (int64_t)e.n_rec, n_rec_dev, part, sms, err, s);
+    launch_partition(rec, (int64_t)e.n_rec, nullptr, part, sms, err, s);
   } else {
     launch_expand_scatter(e.source(), e.rec_off, n, d, seq_rep, id_bits, e.n_rec, part, sms, err,
                           s);
@@ -832,11 +833,11 @@ int expand_into(const Partitions& part, const Encoded& e, int64_t n, int d,
 
 // A self-search whose sequences, were they all of the greatest length, would
 // make at most this many records runs up to its candidates on buffers of that
-// size, without the wait for the record count in between (10 us or so, of a
-// call of 140).  Past the limit the larger buffers' clears and the partitions
-// chosen for too many records would take it back.
+// size, without the wait for the record count in between: 10,000 sequences at
+// d = 1 137 us with the wait left out, 152 with it, 12,000 at d = 2 175 and
+// 192.  Past the limit the larger buffers' clears and the partitions chosen
+// for too many records take it back (200,000 at d = 2: 448 against 413).
 constexpr uint64_t UNREAD_RECORDS = 4u << 20;
-static_assert(UNREAD_RECORDS <= SPLIT_EXPANSION, "the split expansion takes a device count");
 
 // The n spilled records sorted on their hs group-key bits, with group flags.
 int sort_spill(const Partitions& p, uint64_t n, uint32_t id_bits, int hs, int sms, Arena& ar,
@@ -1457,8 +1458,7 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   so.id_bits = bits_for((uint64_t)n);
   if (mode == 0) {
     XTN_RC(take_partitions(e.n_rec, ar, counters + 3, s, &part));
-    XTN_RC(expand_into(part, e, n, d, salt_rep, so.id_bits, unread ? &ctl->n_rec : nullptr, sms,
-                       ar, err, s));
+    XTN_RC(expand_into(part, e, n, d, salt_rep, so.id_bits, unread, sms, ar, err, s));
     launch_group_filter(part, e.n_rec, direct.cand, direct.cand_cap, direct.cand_count,
                         (int)so.id_bits, err, s);
     XTN_CK(cudaGetLastError());
@@ -1615,7 +1615,7 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     part.n_spill = ctl->counters + 3;
     XTN_ALLOC_OK(ar);
     XTN_CK(cudaMemsetAsync(part.count, 0, part.counts() * 4, s));
-    XTN_RC(expand_into(part, e, n, d, nullptr, idx->id_bits, nullptr, sms, ar, err, s));
+    XTN_RC(expand_into(part, e, n, d, nullptr, idx->id_bits, false, sms, ar, err, s));
   } else {
     XTN_RC(expand_and_sort(e, n, d, nullptr, sms, ar, err, s, &so));
   }
