@@ -550,7 +550,11 @@ __global__ void __launch_bounds__(SR_THREADS)
   const uint64_t p = min(starts[b], all), q = b + 1 < RADIX ? min(starts[b + 1], all) : all;
   const uint64_t pair_mask = (1ull << pair_bits) - 1ull;
   for (uint64_t t0 = p + (threadIdx.x & ~31u); t0 < q; t0 += SR_THREADS) {
-    if (*(volatile uint32_t*)&s_n > SMALL_PAIRS) break;  // then at most 1,024 more go in
+    // one lane reads the counter that other warps add to: a warp whose lanes
+    // read different values would part here, before the ballot of all 32
+    uint32_t listed = 0;
+    if (lane_id() == 0) listed = *(volatile uint32_t*)&s_n;
+    if (__shfl_sync(FULL_MASK, listed, 0) > SMALL_PAIRS) break;  // at most 1,024 more go in
     const uint64_t t = t0 + lane_id();
     uint64_t w = 0;
     bool first = false;
