@@ -42,10 +42,11 @@ struct FilterSmem {
   unsigned long long base;
 };
 
-template <int THREADS, int SEEN, int AGAIN, int MIN_BLOCKS>
+// LOW: the bits reach below the high word (shift < 32).
+template <int THREADS, int SEEN, int AGAIN, int MIN_BLOCKS, bool LOW>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
     k_bucket_filter(const uint64_t* __restrict__ rec, const uint32_t* __restrict__ count,
-                    uint32_t region, int pbits, uint64_t* __restrict__ kept,
+                    uint32_t region, int shift, uint64_t* __restrict__ kept,
                     uint32_t* __restrict__ kept_count, uint64_t* __restrict__ spill, uint64_t spill_cap,
                     unsigned long long* __restrict__ n_spill, uint32_t* __restrict__ err) {
   using SM = FilterSmem<SEEN, AGAIN>;
@@ -69,9 +70,8 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
     reinterpret_cast<uint4*>(S.seen)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (threadIdx.x == 0) S.n_kept = 0;
   __syncthreads();
-  // Bit h of `seen`: the SEEN record bits below the partition's.  They lie in
-  // the high word but for pbits + SEEN > 32, where the lowest are left out.
-  const int hshift = max(32 - pbits - SEEN, 0);
+  // Bit h of `seen`: the SEEN record bits below the partition's, from `shift`
+  // up (id bits are left out: then fewer, above them)
   constexpr uint32_t HMASK = (1u << SEEN) - 1u;
   constexpr int DROP = SEEN - AGAIN;  // `again` tells the bits above the lowest DROP apart
   // The records two by two (regions start on 16-byte boundaries), in chunks
@@ -93,7 +93,11 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS)
     }
   };
   auto rec_of = [&](int u) { return u & 1 ? v[u / 2].y : v[u / 2].x; };
-  auto bits_of = [&](int u) { return (uint32_t)(rec_of(u) >> 32) >> hshift; };
+  auto bits_of = [&](int u) {
+    const uint64_t r = rec_of(u);
+    return LOW ? __funnelshift_r((uint32_t)r, (uint32_t)(r >> 32), shift)
+               : (uint32_t)(r >> 32) >> (shift - 32);
+  };
   // the records of this thread's chunk at i0 that exist, a bit each
   auto there = [&](uint32_t i0) {
     uint32_t mask = (1u << (2 * U)) - 1u;
@@ -308,30 +312,40 @@ __global__ void __launch_bounds__(GK_THREADS, 2)
   if (held) flush();
 }
 
-template <int THREADS, int SEEN, int AGAIN, int MIN_BLOCKS>
-void filter_launch(const Partitions& p, uint32_t* err, cudaStream_t s) {
+template <int THREADS, int SEEN, int AGAIN, int MIN_BLOCKS, bool LOW>
+void filter_launch(const Partitions& p, int shift, uint32_t* err, cudaStream_t s) {
   using SM = FilterSmem<SEEN, AGAIN>;
-  auto f = k_bucket_filter<THREADS, SEEN, AGAIN, MIN_BLOCKS>;
+  auto f = k_bucket_filter<THREADS, SEEN, AGAIN, MIN_BLOCKS, LOW>;
   static std::once_flag once;
   std::call_once(once, [&] {
     cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM));
     cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   });
   f<<<1u << p.pbits, THREADS, sizeof(SM), s>>>(
-      p.rec, p.count, p.region, p.pbits, p.kept, p.kept_count(), p.spill, p.spill_cap,
+      p.rec, p.count, p.region, shift, p.kept, p.kept_count(), p.spill, p.spill_cap,
       reinterpret_cast<unsigned long long*>(p.n_spill), err);
+}
+
+template <int THREADS, int SEEN, int AGAIN, int MIN_BLOCKS>
+void filter_launch(const Partitions& p, int id_bits, uint32_t* err, cudaStream_t s) {
+  const int shift = std::max(64 - p.pbits - SEEN, id_bits);
+  if (shift < 32) filter_launch<THREADS, SEEN, AGAIN, MIN_BLOCKS, true>(p, shift, err, s);
+  else filter_launch<THREADS, SEEN, AGAIN, MIN_BLOCKS, false>(p, shift, err, s);
 }
 
 }  // namespace
 
-void launch_group_filter(const Partitions& p, uint64_t n_rec, uint64_t* cand, uint64_t cand_cap,
-                         uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s) {
+void launch_group_filter(const Partitions& q, uint64_t n_rec, uint64_t* cand, uint64_t cand_cap,
+                         uint64_t* cand_count, int id_bits, int sms, uint32_t* err,
+                         cudaStream_t s) {
+  if (q.sub) launch_split(q, n_rec, sms, err, s);
+  const Partitions p = q.sub ? q.fine() : q;
   // the bitmaps hold about 20 bits per record of the expected partition
   const uint64_t mean = n_rec >> p.pbits;
   prof_begin(s, "k_bucket_filter", (double)n_rec * 8.0);
-  if (mean <= 6500) filter_launch<256, 17, 15, 4>(p, err, s);
-  else if (mean <= 26500) filter_launch<512, 19, 17, 2>(p, err, s);
-  else filter_launch<1024, 20, 18, 1>(p, err, s);
+  if (mean <= 6500) filter_launch<256, 17, 15, 4>(p, id_bits, err, s);
+  else if (mean <= 26500) filter_launch<512, 19, 17, 2>(p, id_bits, err, s);
+  else filter_launch<1024, 20, 18, 1>(p, id_bits, err, s);
   prof_end(s);
   static std::once_flag once;
   std::call_once(once, [] {

@@ -35,6 +35,8 @@ namespace xtn {
 namespace {
 
 constexpr int PT_THREADS = 512;
+constexpr int SPLIT_COARSE_BITS = 9;  // partitions of the first of two levels
+constexpr int SPLIT_MAX_BITS = 8;     // and of each of those
 
 // A tile's records, then the bins' counters and output offsets.
 template <int ITEMS>
@@ -161,6 +163,148 @@ void partition_launch(const uint64_t* in, int64_t n, const uint64_t* n_dev, cons
       reinterpret_cast<unsigned long long*>(p.n_spill), err);
 }
 
+// The second level: every coarse partition once more by the `sub` bits below
+// its own, in tiles of one partition each, with k_partition's steps.  With 2^5
+// to 2^8 bins a tile's runs are 44 to 350 records long, against five at the
+// end of one level: 3.97 G records (36M sequences, d = 2) 18.4 ms, 3.4 TB/s.
+template <int ITEMS, int MIN_BLOCKS>
+__global__ void __launch_bounds__(PT_THREADS, MIN_BLOCKS)
+    k_split(const uint64_t* __restrict__ in, const uint32_t* __restrict__ count, uint32_t region,
+            int pbits, int sub, uint64_t* __restrict__ out, uint32_t fine_region,
+            uint32_t* __restrict__ fine_count, uint64_t* __restrict__ spill, uint64_t spill_cap,
+            unsigned long long* __restrict__ n_spill, uint32_t* __restrict__ err) {
+  constexpr uint32_t TILE = PT_THREADS * ITEMS;
+  constexpr int BATCH = ITEMS / 2;
+  extern __shared__ __align__(16) unsigned char pt_smem[];
+  uint64_t* s_stage = reinterpret_cast<uint64_t*>(pt_smem);
+  __shared__ __align__(16) uint32_t s_cnt[1 << SPLIT_MAX_BITS];
+  __shared__ uint32_t s_pos[1 << SPLIT_MAX_BITS];
+  __shared__ uint32_t s_wsum[8];
+  __shared__ uint32_t s_held, s_over;
+  __shared__ unsigned long long s_base;
+  static_assert((1 << SPLIT_MAX_BITS) == 256, "one bin a thread in scan_bins");
+  const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+  const uint32_t F = 1u << sub;
+  const uint32_t per = (region + TILE - 1) / TILE;  // tiles of a partition
+  const uint32_t n_tiles = per << pbits;
+  const bool wide = ((uint64_t)fine_region << (pbits + sub)) >> 32 != 0;  // past 32-bit indices
+  if (threadIdx.x < 256) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_over = 0;  // a region has run over
+  uint64_t rec[ITEMS];
+  const uint32_t first = warp * 32 * ITEMS + lane;  // of this thread in a tile
+  // tile -> its partition, its records and whether the partition ran over
+  auto locate = [&](uint32_t tile, uint32_t& part, uint32_t& at, bool& ran_over) -> uint32_t {
+    part = tile / per;
+    at = (tile - part * per) * TILE;
+    ran_over = false;
+    if (tile >= n_tiles) return 0u;
+    const uint32_t m = count[part];
+    ran_over = m > region;
+    const uint32_t have = min(m, region);
+    return have > at ? min(have - at, TILE) : 0u;
+  };
+  auto load = [&](uint32_t part, uint32_t at, uint32_t held) {
+    const uint64_t* src = in + (uint64_t)part * region + at + first;
+    if (held == TILE) {
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) rec[i] = __ldcs(src + i * 32);
+    } else {
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) rec[i] = first + i * 32 < held ? __ldcs(src + i * 32) : 0ull;
+    }
+  };
+  auto bin_of = [&](uint64_t r) { return (uint32_t)(r >> 32) << pbits >> (32 - sub); };
+  uint32_t part, next_part, next_at;
+  bool ran_over, next_over;
+  uint32_t held = locate(blockIdx.x, part, next_at, ran_over);
+  load(part, next_at, held);
+  __syncthreads();
+  for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const uint32_t f0 = part << sub;  // its first fine partition
+    const bool full = held == TILE;
+    const uint32_t next = locate(tile + gridDim.x, next_part, next_at, next_over);
+    if (ran_over) {  // uniform: the region's records to the global grouping
+      if (threadIdx.x == 0 && held) s_base = atomicAdd(n_spill, (unsigned long long)held);
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        const uint32_t k = first + i * 32;
+        if (k < held) {
+          if (s_base + k < spill_cap) spill[s_base + k] = rec[i];
+          else atomicOr(err, DERR_RANGE);
+        }
+      }
+      load(next_part, next_at, next);
+    } else if (held) {
+      // 1. count
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i)
+        if (full || first + i * 32 < held) atomicAdd(&s_cnt[bin_of(rec[i])], 1u);
+      __syncthreads();
+      // 2. exclusive scan of the bins, then room in every fine partition
+      scan_bins(s_cnt, 1, s_wsum, &s_held);
+      if (threadIdx.x < F) {
+        const uint32_t b = threadIdx.x, at = s_cnt[b];
+        const uint32_t c = (b + 1 < F ? s_cnt[b + 1] : held) - at;
+        const uint32_t room = c ? atomicAdd(&fine_count[f0 + b], c) : 0u;
+        s_pos[b] = (f0 + b) * fine_region + room - at;  // modulo 2^32
+        if (room + c > fine_region) s_over = 1;
+      }
+      __syncthreads();
+      // 3. place in partition order
+#pragma unroll
+      for (int i0 = 0; i0 < ITEMS; i0 += BATCH) {
+        uint32_t at[BATCH];
+#pragma unroll
+        for (int x = 0; x < BATCH; ++x) {
+          const int i = i0 + x;
+          at[x] = TILE;
+          if (full || first + i * 32 < held) at[x] = atomicAdd(&s_cnt[bin_of(rec[i])], 1u);
+        }
+#pragma unroll
+        for (int x = 0; x < BATCH; ++x)
+          if (at[x] < TILE) s_stage[at[x]] = rec[i0 + x];
+      }
+      __syncthreads();
+      // 4. write the runs out, the next tile's loads under way
+      const bool over = s_over || wide;
+      load(next_part, next_at, next);
+      if (threadIdx.x < 256) s_cnt[threadIdx.x] = 0;
+      if (!over) {
+#pragma unroll 4
+        for (uint32_t j = threadIdx.x; j < held; j += PT_THREADS) {
+          const uint64_t v = s_stage[j];
+          out[s_pos[bin_of(v)] + j] = v;
+        }
+      } else {
+        for (uint32_t j = threadIdx.x; j < held; j += PT_THREADS) {
+          const uint64_t v = s_stage[j];
+          const uint32_t b = bin_of(v), f = f0 + b;
+          const uint32_t at = s_pos[b] + j - f * fine_region;
+          if (at < fine_region) {
+            out[(uint64_t)f * fine_region + at] = v;
+          } else {  // past the region's end
+            const uint64_t o = atomicAdd(n_spill, 1ull);
+            if (o < spill_cap) spill[o] = v;
+            else atomicOr(err, DERR_RANGE);
+          }
+        }
+      }
+    } else {
+      load(next_part, next_at, next);
+    }
+    __syncthreads();  // the stage and the bins are reused
+    part = next_part;
+    ran_over = next_over;
+    held = next;
+  }
+}
+
+// Records of a region for `mean` expected ones.
+uint32_t region_of(double mean) {
+  return ((uint32_t)(mean + 8.0 * std::sqrt(mean)) + 128u + 15u) & ~15u;
+}
+
 }  // namespace
 
 // 2^11 partitions where that leaves 20,000 to 80,000 records in one on
@@ -170,6 +314,12 @@ void partition_launch(const uint64_t* in, int64_t n, const uint64_t* n_dev, cons
 // + 0.47 against 1.53 + 0.49 ms), and smaller ones let the last blocks of
 // small inputs end together.  No more than 2^13 partitions, what a tile's
 // counters leave room for, and no fewer than 2^8, so that every SM has some.
+// More records than 2^13 such partitions take go through two levels, 2^9 and up
+// to 2^8 each: fuller bitmaps keep more and more lone records, and a list is
+// read once for every 5,600 of them.  Whole searches at d = 2, one level against
+// two: 0.55 G records 8.8 and 9.2 ms, 0.77 G 13.2 and 12.4, 0.99 G 17.7 and
+// 16.2 (17.1 with 2^11 in the first level); 2.0 G 33 with two and 96 with one
+// whose bitmap had a bit less to go by, 4.0 G 68 and 734.
 PartitionShape choose_partitions(uint64_t n_rec, int fx) {
   PartitionShape g;
   const uint64_t most = (uint64_t)40000 << fx, least = (uint64_t)10000 << fx;
@@ -177,9 +327,34 @@ PartitionShape choose_partitions(uint64_t n_rec, int fx) {
   while (b > 8 && (n_rec >> b) < least) --b;
   while (b < PART_MAX_BITS && (n_rec >> b) > most) ++b;
   g.pbits = b;
-  const double mean = (double)n_rec / (double)(1u << b);
-  g.region = ((uint32_t)(mean + 8.0 * std::sqrt(mean)) + 128u + 15u) & ~15u;
+  if ((n_rec >> b) > most) {
+    // split again before the filter
+    int t = b;
+    while (t < SPLIT_COARSE_BITS + SPLIT_MAX_BITS && (n_rec >> t) > most) ++t;
+    b = SPLIT_COARSE_BITS;
+    g.sub = t - b;
+    g.fine_region = region_of(std::ldexp((double)n_rec, -t));
+  }
+  g.pbits = b;
+  g.region = region_of(std::ldexp((double)n_rec, -b));
   return g;
+}
+
+void launch_split(const Partitions& p, uint64_t n_rec, int sms, uint32_t* err, cudaStream_t s) {
+  constexpr int ITEMS = 22, MIN_BLOCKS = 2;
+  constexpr int smem = PT_THREADS * ITEMS * 8;
+  auto f = k_split<ITEMS, MIN_BLOCKS>;
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  });
+  const Partitions q = p.fine();
+  prof_begin(s, "k_split", (double)n_rec * 16.0);
+  f<<<(uint32_t)sms * MIN_BLOCKS, PT_THREADS, smem, s>>>(
+      p.rec, p.count, p.region, p.pbits, p.sub, q.rec, q.region, q.count, p.spill, p.spill_cap,
+      reinterpret_cast<unsigned long long*>(p.n_spill), err);
+  prof_end(s);
 }
 
 void launch_partition(const uint64_t* in, int64_t n, const uint64_t* n_dev, const Partitions& p,

@@ -131,22 +131,45 @@ void launch_bucket(bool hash, uint64_t* A, uint64_t* Y, int64_t n, const uint64_
 // partition p fills rec[p * region ...] and counts its records in count[p]
 // (which may pass `region`; the records past it go to spill).  The filter
 // keeps a list per partition in `kept`, laid out alike.
+// sub: when not 0, each partition is split once more, by the sub bits below,
+// before the filter (launch_group_filter): into `kept`, fine_region words
+// each, and the filter's lists then lie in `rec`.
 struct PartitionShape {
   int pbits = 0;
   uint32_t region = 0;
-  uint64_t words() const { return (uint64_t)region << pbits; }
-  uint64_t counts() const { return (uint64_t)2 << pbits; }
+  int sub = 0;
+  uint32_t fine_region = 0;
+  uint64_t words() const {
+    const uint64_t a = (uint64_t)region << pbits, b = (uint64_t)fine_region << (pbits + sub);
+    return a > b ? a : b;
+  }
+  uint64_t counts() const {
+    return ((uint64_t)2 << (pbits + sub)) + (sub ? (uint64_t)1 << pbits : 0);
+  }
 };
 // fx: the size of the partitions (see XTN_TUNE_FILTER_SEGMENT).
 PartitionShape choose_partitions(uint64_t n_rec, int fx);
 struct Partitions : PartitionShape {
   uint64_t* rec = nullptr;      // words()
   uint64_t* kept = nullptr;     // words()
-  uint32_t* count = nullptr;    // counts() zeroed words: the partitions', then the lists'
+  uint32_t* count = nullptr;    // counts() zeroed words: (the coarse partitions',) the
+                                // partitions', then the lists'
   uint64_t* spill = nullptr;    // spill_cap words
   uint64_t spill_cap = 0;
   uint64_t* n_spill = nullptr;  // zeroed by the caller
   uint32_t* kept_count() const { return count + ((uint64_t)1 << pbits); }
+  // the partitions after the split (sub != 0)
+  Partitions fine() const {
+    Partitions f = *this;
+    f.pbits = pbits + sub;
+    f.region = fine_region;
+    f.sub = 0;
+    f.fine_region = 0;
+    f.rec = kept;
+    f.kept = rec;
+    f.count = count + ((uint64_t)1 << pbits);
+    return f;
+  }
 };
 // The records of every canonical variant, expanded straight into their
 // partitions; rec_off as launch_expand takes it, its last entry the record
@@ -158,6 +181,9 @@ void launch_expand_scatter(const ExpandSource& src, const uint64_t* rec_off, int
 // count is read on the device and n is a capacity).
 void launch_partition(const uint64_t* in, int64_t n, const uint64_t* n_dev, const Partitions& p,
                       int sms, uint32_t* err, cudaStream_t s);
+// The split of coarse partitions (p.sub != 0) into p.fine(); a partition that
+// ran over goes to the spill whole.
+void launch_split(const Partitions& p, uint64_t n_rec, int sms, uint32_t* err, cudaStream_t s);
 
 // k_filter.cu --------------------------------------------------------------
 // Appends the candidate words (min id << id_bits | max id) of every pair of
@@ -167,7 +193,8 @@ void launch_partition(const uint64_t* in, int64_t n, const uint64_t* n_dev, cons
 // frequent for its table -- is appended to p.spill (counted in *p.n_spill)
 // for a global sort of those few.  n_rec: the expected records.
 void launch_group_filter(const Partitions& p, uint64_t n_rec, uint64_t* cand, uint64_t cand_cap,
-                         uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s);
+                         uint64_t* cand_count, int id_bits, int sms, uint32_t* err,
+                         cudaStream_t s);
 // k_pairs.cu ---------------------------------------------------------------
 size_t scan_status_bytes(int64_t n);
 size_t group_status_bytes(int64_t n);
