@@ -1265,7 +1265,8 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
         launch_expand(e.source(), e.rec_off, n, d, salt_rep, id_bits, rec0, np, nullptr, 0, 0, sms,
                       err, s, &sel);
         launch_partition(rec0, (int64_t)np, ctr + 4, part, sms, err, s);
-        launch_group_filter(part, np, cand.p, cand.cap, ctr + 2, (int)id_bits, sms, err, s);
+        launch_group_filter(part, np, cand.p, cand.cap, ctr + 2, false, (int)id_bits, sms, err,
+                            s);
         XTN_CK(cudaGetLastError());
       } else {
         GroupScratch gs = gs0;
@@ -1460,7 +1461,7 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     XTN_RC(take_partitions(e.n_rec, ar, counters + 3, s, &part));
     XTN_RC(expand_into(part, e, n, d, salt_rep, so.id_bits, unread, sms, ar, err, s));
     launch_group_filter(part, e.n_rec, direct.cand, direct.cand_cap, direct.cand_count,
-                        (int)so.id_bits, sms, err, s);
+                        false, (int)so.id_bits, sms, err, s);
     XTN_CK(cudaGetLastError());
   } else {
     XTN_RC(expand_and_sort(e, n, d, salt_rep, sms, ar, err, s, &so, true, e.n_rec / 2 + 1, mode,
@@ -1981,7 +1982,7 @@ int plan_run_impl(xtn_plan* p, const uint8_t* seqs, cudaStream_t s) {
     launch_expand_scatter(ExpandSource{p->keys, p->lens, p->eqprev}, p->rec_off, n, p->d,
                           p->seq_rep, p->id_bits, p->rec_cap, p->part, p->sms, p->err, s);
     launch_group_filter(p->part, p->rec_cap, p->back.P1, p->pair_cap, p->counters + 2,
-                        (int)p->id_bits, p->sms, p->err, s);
+                        true, (int)p->id_bits, p->sms, p->err, s);
     launch_histogram(p->B, (int64_t)p->rec_cap, n_flagged, lo, 64, p->hist, p->sms, s);
     launch_clear_status(p->status, (int64_t)p->rec_cap, n_flagged, p->sms, s);
     XTN_CK(cudaGetLastError());

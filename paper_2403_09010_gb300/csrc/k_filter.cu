@@ -178,20 +178,27 @@ struct GroupSmem {
   uint64_t stash[GK_WARPS][GK_STASH];
   uint16_t next[GK_LIST];
   uint32_t n_list;
+  bool full;  // the candidates are past their buffer
 };
 
 // skip: key bits that all records of a list share (the partition's).
+// count_all: the candidates are counted to the end, past cand_cap too; else
+// blocks that begin after that leave, as the caller starts over (100,000
+// sequences ten times each, d = 2: 472 M candidates of which 52 M fit, 1.4 ms
+// instead of 14.6).
 __global__ void __launch_bounds__(GK_THREADS, 2)
     k_group_kept(const uint64_t* __restrict__ kept, const uint32_t* __restrict__ kept_count,
                  uint32_t region, int skip, uint64_t* __restrict__ spill, uint64_t spill_cap,
                  unsigned long long* __restrict__ n_spill, uint64_t* __restrict__ cand,
-                 uint64_t cand_cap, unsigned long long* __restrict__ cand_count, int id_bits,
-                 uint32_t* __restrict__ err) {
+                 uint64_t cand_cap, unsigned long long* __restrict__ cand_count, bool count_all,
+                 int id_bits, uint32_t* __restrict__ err) {
   constexpr int THREADS = GK_THREADS;
   extern __shared__ __align__(16) unsigned char gk_smem[];
   GroupSmem& S = *reinterpret_cast<GroupSmem*>(gk_smem);
   const uint32_t lane = lane_id();
   const uint64_t idmask = (1ull << id_bits) - 1ull;
+  if (threadIdx.x == 0)  // read once for the block: other blocks add to it
+    S.full = !count_all && *(volatile unsigned long long*)cand_count > cand_cap;
   const uint32_t m = kept_count[blockIdx.x];
   if (m < 2) return;
   const uint64_t* __restrict__ in = kept + (uint64_t)blockIdx.x * region;
@@ -221,6 +228,7 @@ __global__ void __launch_bounds__(GK_THREADS, 2)
       reinterpret_cast<uint4*>(S.head)[k] = make_uint4(GK_NIL, GK_NIL, GK_NIL, GK_NIL);
     if (threadIdx.x == 0) S.n_list = 0;
     __syncthreads();
+    if (S.full) return;
     // 1. list the part's records, each put at the head of its slot's chain
     for (uint32_t k0 = 0; k0 < m; k0 += GK_LOADS * THREADS) {
       uint64_t r[GK_LOADS];
@@ -336,8 +344,8 @@ void filter_launch(const Partitions& p, int id_bits, uint32_t* err, cudaStream_t
 }  // namespace
 
 void launch_group_filter(const Partitions& q, uint64_t n_rec, uint64_t* cand, uint64_t cand_cap,
-                         uint64_t* cand_count, int id_bits, int sms, uint32_t* err,
-                         cudaStream_t s) {
+                         uint64_t* cand_count, bool count_all, int id_bits, int sms,
+                         uint32_t* err, cudaStream_t s) {
   if (q.sub) launch_split(q, n_rec, sms, err, s);
   const Partitions p = q.sub ? q.fine() : q;
   // the bitmaps hold about 20 bits per record of the expected partition
@@ -357,7 +365,7 @@ void launch_group_filter(const Partitions& q, uint64_t n_rec, uint64_t* cand, ui
   k_group_kept<<<1u << p.pbits, GK_THREADS, sizeof(GroupSmem), s>>>(
       p.kept, p.kept_count(), p.region, p.pbits, p.spill, p.spill_cap,
       reinterpret_cast<unsigned long long*>(p.n_spill), cand, cand_cap,
-      reinterpret_cast<unsigned long long*>(cand_count), id_bits, err);
+      reinterpret_cast<unsigned long long*>(cand_count), count_all, id_bits, err);
   prof_end(s);
 }
 

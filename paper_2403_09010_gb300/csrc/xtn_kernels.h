@@ -188,13 +188,14 @@ void launch_split(const Partitions& p, uint64_t n_rec, int sms, uint32_t* err, c
 // k_filter.cu --------------------------------------------------------------
 // Appends the candidate words (min id << id_bits | max id) of every pair of
 // records with equal group keys to cand[0, cand_cap), counting them in
-// *cand_count (DERR_CAPACITY past the capacity).  What a block cannot group
+// *cand_count (DERR_CAPACITY past the capacity, and without count_all perhaps
+// not all of them counted then).  What a block cannot group
 // on its own -- a partition or list that overflowed, a single key too
 // frequent for its table -- is appended to p.spill (counted in *p.n_spill)
 // for a global sort of those few.  n_rec: the expected records.
 void launch_group_filter(const Partitions& p, uint64_t n_rec, uint64_t* cand, uint64_t cand_cap,
-                         uint64_t* cand_count, int id_bits, int sms, uint32_t* err,
-                         cudaStream_t s);
+                         uint64_t* cand_count, bool count_all, int id_bits, int sms,
+                         uint32_t* err, cudaStream_t s);
 // k_pairs.cu ---------------------------------------------------------------
 size_t scan_status_bytes(int64_t n);
 size_t group_status_bytes(int64_t n);
