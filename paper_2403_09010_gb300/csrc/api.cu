@@ -788,11 +788,11 @@ int expand_and_sort(const Encoded& e, int64_t n, int d, const uint32_t* seq_rep,
 
 // Partition buffers for n_rec records, the counters cleared (*n_spill is
 // the caller's to clear).  `rec` also serves as the second buffer of the
-// spill's sort.
+// spill's sort, and `kept` may hold the records before they are parted.
 int take_partitions(uint64_t n_rec, Arena& ar, uint64_t* n_spill, cudaStream_t s, Partitions* p) {
   static_cast<PartitionShape&>(*p) = choose_partitions(n_rec, g_filter_fx.load());
   p->rec = ar.get<uint64_t>(std::max(p->words(), n_rec) + 8);
-  p->kept = ar.get<uint64_t>(p->words() + 8);
+  p->kept = ar.get<uint64_t>(std::max(p->words(), n_rec) + 8);
   p->count = ar.get<uint32_t>(p->counts());
   p->spill = ar.get<uint64_t>(n_rec + 8);
   p->spill_cap = n_rec;
@@ -839,26 +839,44 @@ int expand_into(const Partitions& part, const Encoded& e, int64_t n, int d,
 // for too many records take it back (200,000 at d = 2: 448 against 413).
 constexpr uint64_t UNREAD_RECORDS = 4u << 20;
 
-// The n spilled records sorted on their hs group-key bits, with group flags.
-int sort_spill(const Partitions& p, uint64_t n, uint32_t id_bits, int hs, int sms, Arena& ar,
-               uint32_t* err, cudaStream_t s, Sorted* out) {
-  const int lo = 64 - hs;
-  const int cfg = g_cfg_records.load();
-  const uint64_t g_cap = n / 2 + 1;
-  uint32_t* hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
-  uint64_t* digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
-  uint64_t* status = ar.get<uint64_t>(radix_status_bytes((int64_t)n, cfg) / 8 + 1);
-  const size_t gst = std::max(group_status_bytes((int64_t)n), scan_status_bytes((int64_t)g_cap));
-  out->flags = ar.get<uint64_t>(group_flag_words((int64_t)n));
-  out->gstatus = ar.get<uint64_t>(gst / 8 + 1);
+// Scratch of a sort of up to n records and of their group flags.
+struct SortScratch {
+  uint32_t* hist = nullptr;        // MAX_PASSES * RADIX
+  uint64_t* digit_base = nullptr;  // MAX_PASSES * RADIX
+  uint64_t* status = nullptr;      // radix_status_bytes(n, cfg)
+  uint64_t* flags = nullptr;       // group_flag_words(n)
+  uint64_t* gstatus = nullptr;     // sort_gstatus_bytes(n)
+};
+
+// Of the group-bound and the group-pair scans.
+size_t sort_gstatus_bytes(uint64_t n) {
+  return std::max(group_status_bytes((int64_t)n), scan_status_bytes((int64_t)(n / 2 + 1)));
+}
+
+int take_sort_scratch(uint64_t n, int cfg, Arena& ar, SortScratch* w) {
+  w->hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
+  w->digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
+  w->status = ar.get<uint64_t>(radix_status_bytes((int64_t)n, cfg) / 8 + 1);
+  w->flags = ar.get<uint64_t>(group_flag_words((int64_t)n));
+  w->gstatus = ar.get<uint64_t>(sort_gstatus_bytes(n) / 8 + 1);
   XTN_ALLOC_OK(ar);
-  XTN_CK(cudaMemsetAsync(hist, 0, MAX_PASSES * RADIX * 4, s));
-  launch_histogram(p.spill, (int64_t)n, nullptr, lo, 64, hist, sms, s);
-  XTN_CK(radix_sort_passes(p.spill, p.rec, (int64_t)n, lo, 64, hist, digit_base, status, cfg, err,
-                           &out->rec, "k_onesweep_records", s, false, nullptr, nullptr,
+  return XTN_OK;
+}
+
+// The n spilled records sorted on their hs group-key bits by configuration
+// cfg, with group flags.
+int sort_spill(const Partitions& p, uint64_t n, uint32_t id_bits, int hs, int cfg,
+               const SortScratch& w, int sms, uint32_t* err, cudaStream_t s, Sorted* out) {
+  const int lo = 64 - hs;
+  out->flags = w.flags;
+  out->gstatus = w.gstatus;
+  XTN_CK(cudaMemsetAsync(w.hist, 0, MAX_PASSES * RADIX * 4, s));
+  launch_histogram(p.spill, (int64_t)n, nullptr, lo, 64, w.hist, sms, s);
+  XTN_CK(radix_sort_passes(p.spill, p.rec, (int64_t)n, lo, 64, w.hist, w.digit_base, w.status, cfg,
+                           err, &out->rec, "k_onesweep_records", s, false, nullptr, nullptr,
                            onesweep_unstable_config(cfg)));
   out->spare = out->rec == p.spill ? p.rec : p.spill;
-  XTN_CK(cudaMemsetAsync(out->gstatus, 0, gst, s));
+  XTN_CK(cudaMemsetAsync(out->gstatus, 0, sort_gstatus_bytes(n), s));
   launch_group_flags(out->rec, (int64_t)n, nullptr, lo, out->flags, out->gstatus, s);
   out->id_bits = id_bits;
   out->hs = hs;
@@ -1105,8 +1123,9 @@ struct GrowBuf {
 };
 
 // Records one pass may hold when the caller sets no budget: what a pass needs
-// (two record buffers, candidate words, flags: about 32 bytes per record) in
-// half the free device memory, below 2^32.
+// (three record buffers of 8 to 8.3 bytes a record, candidate words 4, status
+// and flags 0.9: 29 bytes, about 32 for passes of a million) in half the free
+// device memory, below 2^32.
 uint64_t default_pass_records() {
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
@@ -1217,20 +1236,21 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   const int cfg = g_cfg_records.load();
   const int cfg_pairs = g_cfg_pairs.load();
   const int mode0 = g_grouping.load();
-  uint64_t* digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
-  uint32_t* hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
   uint32_t* phist = ar.get<uint32_t>(MAX_PASSES * RADIX);  // survivors, over all passes
   Partitions part0;
   XTN_RC(take_partitions(P, ar, ctr + 3, s, &part0));
-  uint64_t* rec0 = ar.get<uint64_t>(P + 8);
+  uint64_t* rec0 = part0.kept;  // in sequence order: read before the lists are made
   uint64_t* A = part0.rec;  // the buffers of a pass grouped by sorting
   uint64_t* B = part0.spill;
-  uint64_t* status = ar.get<uint64_t>(radix_status_bytes(P, cfg) / 8 + 1);
-  const size_t gst = std::max(group_status_bytes((int64_t)P), scan_status_bytes(P / 2 + 1));
+  SortScratch sort0;
+  XTN_RC(take_sort_scratch(P, cfg, ar, &sort0));
+  uint64_t* digit_base = sort0.digit_base;
+  uint32_t* hist = sort0.hist;
+  uint64_t* status = sort0.status;
   GroupScratch gs0;
   gs0.bucket_start = ar.get<uint64_t>(bucket_start_words(P, hs, mode0 == 2 ? 2 : 1));
-  gs0.flags = ar.get<uint64_t>(group_flag_words((int64_t)P));
-  gs0.gstatus = ar.get<uint64_t>(gst / 8 + 1);
+  gs0.flags = sort0.flags;
+  gs0.gstatus = sort0.gstatus;
   XTN_ALLOC_OK(ar);
   GrowBuf cand(s), surv(s);
   if (!cand.reserve(std::max<uint64_t>(P / 2, 1u << 20), 0) ||
@@ -1300,7 +1320,7 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
       uint64_t* gstatus = gs0.gstatus;
       if (mode == 0 && n_flagged) {
         Sorted so;
-        XTN_RC(sort_spill(part0, n_flagged, id_bits, hs, sms, ar, err, s, &so));
+        XTN_RC(sort_spill(part0, n_flagged, id_bits, hs, cfg, sort0, sms, err, s, &so));
         sorted = so.rec;
         spare = so.spare;
         flags = so.flags;
@@ -1485,9 +1505,13 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     }
     if (c.err[0]) return map_device_err(c.err[0]);
     if (h.large) n_flagged = mode == 0 ? h.large : e.n_rec;
-    if (mode == 0 && h.large)
-      XTN_RC(sort_spill(part, h.large, so.id_bits, choose_hash_bits(e.n_rec, so.id_bits), sms, ar,
-                        err, s, &so));
+    if (mode == 0 && h.large) {
+      const int cfg = g_cfg_records.load();
+      SortScratch w;
+      XTN_RC(take_sort_scratch(h.large, cfg, ar, &w));
+      XTN_RC(sort_spill(part, h.large, so.id_bits, choose_hash_bits(e.n_rec, so.id_bits), cfg, w,
+                        sms, err, s, &so));
+    }
   }
   const uint64_t g_cap = n_flagged / 2 + 1;
   uint32_t* S = reinterpret_cast<uint32_t*>(so.spare);  // groups live in the spare buffer

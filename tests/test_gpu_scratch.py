@@ -1,0 +1,90 @@
+"""Device memory a call takes for its scratch: a search in passes within what
+its budget of records stands for, however many passes and spilled partitions."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import cdr3_synth as gen
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def xtn():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import paper_2403_09010_gb300 as pkg
+    pkg.build()
+    torch.zeros(1, device="cuda")
+    return pkg
+
+
+def _cuda(*arrays):
+    return [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in arrays]
+
+
+class PoolPeak:
+    """The most bytes of the device's default memory pool in use at a time
+    (scratch comes from there) while the block runs, from an empty cache."""
+    USED_HIGH = 8  # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+
+    def __init__(self, xtn):
+        self.xtn = xtn
+        self.cuda = ctypes.CDLL("libcuda.so.1")
+        self.pool = ctypes.c_void_p()
+        assert self.cuda.cuDeviceGetDefaultMemPool(
+            ctypes.byref(self.pool), torch.cuda.current_device()) == 0
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        self.xtn.scratch_trim()
+        zero = ctypes.c_uint64(0)
+        assert self.cuda.cuMemPoolSetAttribute(self.pool, self.USED_HIGH, ctypes.byref(zero)) == 0
+        return self
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        high = ctypes.c_uint64(0)
+        assert self.cuda.cuMemPoolGetAttribute(self.pool, self.USED_HIGH, ctypes.byref(high)) == 0
+        self.bytes = high.value
+        return False
+
+
+def test_passes_take_32_bytes_a_record(xtn):
+    """The documented size of a pass, besides the sequences (80 bytes: keys,
+    lengths, masks, planes, offsets) and the verified pairs (growing to 1.5
+    times their number, and once more where they are sorted)."""
+    n, per_pass = 500_000, 20_000_000
+    ds, do = _cuda(*gen.generate(n, 5, 0.15, 0.01))
+    want = xtn.search_self(ds, do, 2)
+    with PoolPeak(xtn) as peak:
+        rows, passes = xtn.search_self_streaming(ds, do, 2, max_pass_records=per_pass)
+    assert passes >= 3 and torch.equal(rows, want)
+    assert peak.bytes <= 32 * per_pass + 80 * n + 8 * (1 << 20) + 3 * 8 * len(want) + (8 << 20)
+
+
+def test_passes_that_all_spill_take_their_scratch_once(xtn):
+    """190 passes of 5,000 records in keys of 300 copies each: every pass has
+    partitions that run over (256 regions of about 180 records)."""
+    rng = np.random.default_rng(3)
+    one = gen.to_strings(*gen.generate(200, 1, 0.0, 0.0))
+    strs = [one[k] for k in rng.permutation(np.repeat(np.arange(200), 300))]
+    ds, do = _cuda(*gen.from_strings(strs))
+    cap = 200 * 300 * 299 // 2 + 2000 * 300 * 300
+    want = xtn.search_self(ds, do, 1, cap=cap)
+    peaks = []
+    for per_pass in (5_000, 20_000):
+        with PoolPeak(xtn) as peak:
+            xtn.profile_report()
+            xtn.profile_enable(True)
+            rows, passes = xtn.search_self_streaming(ds, do, 1, max_pass_records=per_pass, cap=cap)
+            xtn.profile_enable(False)
+            spans = xtn.profile_report()
+        assert torch.equal(rows, want)
+        peaks.append((peak.bytes, passes, spans["host_scratch_alloc"][0]))
+    assert peaks[0][1] > 100 and peaks[0][1] > 3 * peaks[1][1]
+    # a pass's buffers, and the few times that the pair words' buffers grow
+    assert peaks[0][2] < 80 and peaks[0][0] <= peaks[1][0] + (8 << 20)
