@@ -219,7 +219,7 @@ class Arena {
     for (void* p : ptrs_) cudaFreeAsync(p, s_);
     ptrs_.clear();
     if (ws_) {
-      ws_->want = std::max(ws_->want, total_);
+      if (!failed_) ws_->want = std::max(ws_->want, total_);
       cudaEventRecord(ws_->done, s_);
       std::lock_guard<std::mutex> g(g_ws_mu);
       g_ws[dev_].idle.push_back(ws_);
@@ -486,6 +486,18 @@ std::atomic<int> g_filter_fx{1};
 std::atomic<int>& cfg_records() { return g_cfg_records; }
 std::atomic<int>& cfg_pairs() { return g_cfg_pairs; }
 namespace {
+
+// run(mode) in the tuned grouping mode.  Where the device has no room for
+// partitions (28 bytes a record with their candidates), the records are
+// sorted instead (16, the candidates counted first).
+template <class F>
+int partitioned_or_sorted(F&& run) {
+  const int mode = g_grouping.load();
+  const int rc = run(mode);
+  if (rc != XTN_ERR_OOM || mode != 0) return rc;
+  trim_scratch();
+  return run(1);
+}
 
 // Sequences resident on the device for one call.
 struct DevSeqs {
@@ -1149,12 +1161,12 @@ uint64_t default_pass_records() {
 // min(i, j) instead, so that it can remove repeats before verifying; here
 // verification comes first, and only its survivors are kept.)  A pass whose
 // candidates exceed 2^32 words or device memory is split in two at its
-// middle bin.  Arguments as search_self_impl; max_pass <= 0 takes
+// middle bin.  Arguments as search_self_once; max_pass <= 0 takes
 // default_pass_records(); *n_passes receives the passes run.
-int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
+int search_stream_once(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
                        const int64_t* rep_offsets, int64_t n_rep, int metric, bool between,
                        int64_t max_pass, xtn_triple* out, int64_t cap, int64_t* n_out,
-                       int64_t* n_passes, cudaStream_t s) {
+                       int64_t* n_passes, cudaStream_t s, int mode0) {
   if (!n_out) return XTN_ERR_INVALID_ARG;
   *n_out = 0;
   if (n_passes) *n_passes = 0;
@@ -1235,10 +1247,14 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   const int lo = 64 - hs;
   const int cfg = g_cfg_records.load();
   const int cfg_pairs = g_cfg_pairs.load();
-  const int mode0 = g_grouping.load();
   uint32_t* phist = ar.get<uint32_t>(MAX_PASSES * RADIX);  // survivors, over all passes
   Partitions part0;
-  XTN_RC(take_partitions(P, ar, ctr + 3, s, &part0));
+  if (mode0 == 0) {
+    XTN_RC(take_partitions(P, ar, ctr + 3, s, &part0));
+  } else {
+    part0.rec = ar.get<uint64_t>(P + 8);
+    part0.spill = ar.get<uint64_t>(P + 8);
+  }
   uint64_t* rec0 = part0.kept;  // in sequence order: read before the lists are made
   uint64_t* A = part0.rec;  // the buffers of a pass grouped by sorting
   uint64_t* B = part0.spill;
@@ -1397,7 +1413,18 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
   return finish_out(o, out, cap, rows, s, n_out);
 }
 
-// mode: grouping mode (see g_grouping), -1 = the tuned one.  metric: 0 =
+int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
+                       const int64_t* rep_offsets, int64_t n_rep, int metric, bool between,
+                       int64_t max_pass, xtn_triple* out, int64_t cap, int64_t* n_out,
+                       int64_t* n_passes, cudaStream_t s) {
+  auto run = [&](int mode) {
+    return search_stream_once(seqs, offsets, n, d, rep_offsets, n_rep, metric, between, max_pass,
+                              out, cap, n_out, n_passes, s, mode);
+  };
+  return partitioned_or_sorted(run);
+}
+
+// mode: grouping mode (see g_grouping).  metric: 0 =
 // Levenshtein, 1 = Hamming (the Hamming variant: the same candidates, the
 // last step filters by Hamming distance).  between: report the pairs between
 // different repertoires instead of those within one; the variants then carry
@@ -1405,11 +1432,10 @@ int search_stream_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
 // b_seqs / b_offsets (paired receptors, the paired-chain search): the second
 // chains; seqs / offsets then hold the first chains, d <= 2, one repertoire,
 // and the last step takes metric 2 (the sum of the two chains' distances).
-int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
+int search_self_once(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
                      const int64_t* rep_offsets, int64_t n_rep, xtn_triple* out, int64_t cap,
-                     int64_t* n_out, cudaStream_t s, int mode = -1, int metric = 0,
-                     bool between = false, const uint8_t* b_seqs = nullptr,
-                     const int64_t* b_offsets = nullptr) {
+                     int64_t* n_out, cudaStream_t s, int mode, int metric, bool between,
+                     const uint8_t* b_seqs, const int64_t* b_offsets) {
   if (!n_out) return XTN_ERR_INVALID_ARG;
   *n_out = 0;
   if (n < 0 || d < 0 || d > XTN_MAX_D || cap < 0 || !offsets) return XTN_ERR_INVALID_ARG;
@@ -1446,7 +1472,6 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
 
   // front: encode (read back the record count unless its bound is small),
   // expand, group
-  if (mode < 0) mode = g_grouping.load();
   Encoded e;
   const uint64_t n_max = (uint64_t)n * variant_count(XTN_MAX_LEN, (uint32_t)d);
   const bool unread = mode == 0 && !paired && n_max <= UNREAD_RECORDS;
@@ -1500,7 +1525,7 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
     h.large = c.counters[3];
     if (c.err[0] == DERR_CAPACITY) {  // candidate overflow alone: regroup sized exactly
       ar.release();
-      return search_self_impl(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out, s, 1,
+      return search_self_once(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out, s, 1,
                               metric, between, b_seqs, b_offsets);
     }
     if (c.err[0]) return map_device_err(c.err[0]);
@@ -1540,7 +1565,7 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   }
   if (mode != 1 && n_pairs > direct.cand_cap) {
     ar.release();
-    return search_self_impl(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out, s, 1,
+    return search_self_once(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out, s, 1,
                             metric, between, b_seqs, b_offsets);
   }
 
@@ -1556,6 +1581,17 @@ int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   XTN_RC(finish_pairs(P1, n_pairs, 2 * so.id_bits, so.id_bits, e.side(n), e.side(n), seq_rep,
                       between ? 2 : 1, d, metric, o.dev, o.dev_cap, sms, ctl, ar, s, &h.pairs));
   return finish_out(o, out, cap, h.pairs, s, n_out);
+}
+
+int search_self_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
+                     const int64_t* rep_offsets, int64_t n_rep, xtn_triple* out, int64_t cap,
+                     int64_t* n_out, cudaStream_t s, int metric = 0, bool between = false,
+                     const uint8_t* b_seqs = nullptr, const int64_t* b_offsets = nullptr) {
+  auto run = [&](int mode) {
+    return search_self_once(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out, s, mode,
+                            metric, between, b_seqs, b_offsets);
+  };
+  return partitioned_or_sorted(run);
 }
 
 }  // namespace
@@ -1869,8 +1905,8 @@ struct xtn_plan {
 namespace xtn {
 namespace {
 
-int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* rep_offsets,
-                     int64_t n_rep, int64_t pair_capacity, xtn_plan** out) {
+int plan_create_once(const int64_t* offsets, int64_t n, int d, const int64_t* rep_offsets,
+                     int64_t n_rep, int64_t pair_capacity, xtn_plan** out, int mode) {
   if (!out) return XTN_ERR_INVALID_ARG;
   *out = nullptr;
   if (n < 1 || d < 0 || d > XTN_MAX_D || !offsets) return XTN_ERR_INVALID_ARG;
@@ -1908,7 +1944,7 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   p->cfg_rec = g_cfg_records.load();
   p->cfg_pair = g_cfg_pairs.load();
   p->hist_mode = g_record_hist.load();
-  p->group_mode = g_grouping.load();
+  p->group_mode = mode;
   const bool parted = p->group_mode == 0;
   const size_t st = std::max({radix_status_bytes((int64_t)rec_cap,
                                                  parted ? ONESWEEP_LOOP : p->cfg_rec),
@@ -1982,6 +2018,14 @@ int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* re
   }
   *out = p;
   return XTN_OK;
+}
+
+int plan_create_impl(const int64_t* offsets, int64_t n, int d, const int64_t* rep_offsets,
+                     int64_t n_rep, int64_t pair_capacity, xtn_plan** out) {
+  auto run = [&](int mode) {
+    return plan_create_once(offsets, n, d, rep_offsets, n_rep, pair_capacity, out, mode);
+  };
+  return partitioned_or_sorted(run);
 }
 
 int plan_run_impl(xtn_plan* p, const uint8_t* seqs, cudaStream_t s) {
@@ -2109,7 +2153,7 @@ int xtn_search_self_hamming(const uint8_t* seqs, const int64_t* offsets, int64_t
                             int64_t cap, int64_t* n_out, xtn_stream_t stream) {
   xtn::HostSpan span("host_call_search_self");
   return xtn::search_self_impl(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out,
-                               reinterpret_cast<cudaStream_t>(stream), -1, 1);
+                               reinterpret_cast<cudaStream_t>(stream), 1);
 }
 
 int xtn_search_between(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
@@ -2120,7 +2164,7 @@ int xtn_search_between(const uint8_t* seqs, const int64_t* offsets, int64_t n, i
     return XTN_ERR_INVALID_ARG;
   xtn::HostSpan span("host_call_search_between");
   return xtn::search_self_impl(seqs, offsets, n, d, rep_offsets, n_rep, out, cap, n_out,
-                               reinterpret_cast<cudaStream_t>(stream), -1, metric, true);
+                               reinterpret_cast<cudaStream_t>(stream), metric, true);
 }
 
 int xtn_search_self_streaming(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d,
@@ -2164,7 +2208,7 @@ int xtn_search_paired(const uint8_t* a_seqs, const int64_t* a_offsets, const uin
     return XTN_ERR_INVALID_ARG;
   }
   return xtn::search_self_impl(a_seqs, a_offsets, n, d, nullptr, 0, out, cap, n_out,
-                               reinterpret_cast<cudaStream_t>(stream), -1, 2, false, b_seqs,
+                               reinterpret_cast<cudaStream_t>(stream), 2, false, b_seqs,
                                b_offsets);
 }
 

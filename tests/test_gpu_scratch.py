@@ -88,3 +88,54 @@ def test_passes_that_all_spill_take_their_scratch_once(xtn):
     assert peaks[0][1] > 100 and peaks[0][1] > 3 * peaks[1][1]
     # a pass's buffers, and the few times that the pair words' buffers grow
     assert peaks[0][2] < 80 and peaks[0][0] <= peaks[1][0] + (8 << 20)
+
+
+class LittleMemory:
+    """All of the device's memory but `free` bytes taken, the scratch cache empty."""
+
+    def __init__(self, xtn, free):
+        self.xtn, self.free = xtn, free
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        self.xtn.scratch_trim()
+        have = torch.cuda.mem_get_info()[0]
+        self.hog = torch.empty(have - self.free, dtype=torch.uint8, device="cuda")
+
+    def __exit__(self, *exc):
+        del self.hog
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        self.xtn.scratch_trim()
+        return False
+
+
+# 104.8 M records (115.5 M in a plan's bound).  With partitions a search takes
+# 29 bytes a record and 93 a sequence (3.1 GB), a plan 25 and 28 a pair of its
+# capacity (3.2 GB); sorted, 17 and 17 (1.9 and 2.3 GB).
+@pytest.mark.parametrize("what,free", [("search", 2_500 << 20), ("passes", 2_600 << 20),
+                                       ("plan", 2_750 << 20), ("search", 8_000 << 20)])
+def test_sorted_where_partitions_do_not_fit(xtn, what, free):
+    n, cap = 1_000_000, 400_000
+    seqs, off = gen.workload(gen.SELF_1M)
+    ds, do = _cuda(seqs, off)
+    want = xtn.search_self(ds, do, 2, cap=cap)
+    with LittleMemory(xtn, free):
+        for _ in range(2):
+            xtn.profile_report()
+            xtn.profile_enable(True)
+            if what == "plan":
+                plan = xtn.Plan(off, 2, pair_capacity=6_000_000)
+                plan.run(ds)
+                got = plan.result(cap=cap, like=ds)
+                plan.free()
+            elif what == "passes":
+                got, _ = xtn.search_self_streaming(ds, do, 2, max_pass_records=120_000_000,
+                                                   cap=cap)
+            else:
+                got = xtn.search_self(ds, do, 2, cap=cap)
+            xtn.profile_enable(False)
+            kernels = xtn.profile_report()
+            assert torch.equal(got, want)
+            assert ("k_bucket_filter" in kernels) == (free > 4_000 << 20)
