@@ -757,17 +757,19 @@ int expand_sort_launch(const Key128* keys, const uint8_t* lens, const uint32_t* 
 
 // want_flags: also make the group flags (out->flags, out->gstatus, the latter
 // sized for the group-bound and group-pair scans of up to g_cap groups).
+// A, B: two buffers of n_rec + 8 words, taken here when null.
 int expand_and_sort(const Encoded& e, int64_t n, int d, const uint32_t* seq_rep, int sms,
                     Arena& ar, uint32_t* err, cudaStream_t s, Sorted* out,
                     bool want_flags = false, uint64_t g_cap = 0, int mode = -1,
-                    const GroupScratch* direct = nullptr) {
+                    const GroupScratch* direct = nullptr, uint64_t* A = nullptr,
+                    uint64_t* B = nullptr) {
   const uint64_t n_rec = e.n_rec;
   out->id_bits = bits_for((uint64_t)n);
   out->hs = choose_hash_bits(n_rec, out->id_bits);
   const int lo = 64 - out->hs;
   const int cfg = g_cfg_records.load();
-  uint64_t* A = ar.get<uint64_t>(n_rec + 8);
-  uint64_t* B = ar.get<uint64_t>(n_rec + 8);
+  if (!A) A = ar.get<uint64_t>(n_rec + 8);
+  if (!B) B = ar.get<uint64_t>(n_rec + 8);
   uint32_t* hist = ar.get<uint32_t>(MAX_PASSES * RADIX);
   uint64_t* digit_base = ar.get<uint64_t>(MAX_PASSES * RADIX);
   uint64_t* status = ar.get<uint64_t>(radix_status_bytes(n_rec, cfg) / 8 + 1);
@@ -1622,10 +1624,10 @@ struct xtn_index {
 namespace xtn {
 namespace {
 
-// by_sorting: the records sorted globally whatever their number (else only
-// where k_index.cu does not take them, or grouping by sorting is set).
-int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d, cudaStream_t s,
-                     xtn_index** out, bool by_sorting = false) {
+// mode: 0 = out of partitions where k_index.cu takes them, else the records
+// sorted globally.
+int index_build_once(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d, cudaStream_t s,
+                     xtn_index** out, int mode) {
   if (!out) return XTN_ERR_INVALID_ARG;
   *out = nullptr;
   if (n < 1 || d < 0 || d > XTN_MAX_D || !offsets) return XTN_ERR_INVALID_ARG;
@@ -1665,11 +1667,10 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   }
   const int gshift = 64 - idx->hs;
   Partitions part;
-  const bool parted = !by_sorting && g_grouping.load() == 0 &&
-                      choose_index_partitions(e.n_rec, idx->dir_bits, &part);
+  const bool parted = mode == 0 && choose_index_partitions(e.n_rec, idx->dir_bits, &part);
   Sorted so;
   if (parted) {
-    part.rec = ar.get<uint64_t>(part.words() + 8);
+    part.rec = ar.get<uint64_t>(std::max(part.words(), e.n_rec) + 8);
     part.count = ar.get<uint32_t>(part.counts());
     part.spill = ar.get<uint64_t>(e.n_rec + 8);
     part.spill_cap = e.n_rec;
@@ -1695,28 +1696,44 @@ int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int
   idx->dir = reinterpret_cast<uint32_t*>(mem + at_dir);
   idx->bytes = (int64_t)(b_rows + b_rec + b_dir);
   XTN_CK(cudaMemcpyAsync(idx->rows, e.rows, b_rows, cudaMemcpyDeviceToDevice, s));
-  if (parted) {
-    launch_index_build(part, e.n_rec, idx->dir_bits, gshift, idx->rec, idx->dir, ctl->counters,
-                       err, s);
-  } else {
+  auto from_sorted = [&]() -> int {
     XTN_CK(cudaMemcpyAsync(idx->rec, so.rec, b_rec, cudaMemcpyDeviceToDevice, s));
     launch_build_dir(idx->rec, idx->n_rec, idx->dir_bits, gshift, idx->dir, ctl->counters, s);
-  }
+    return XTN_OK;
+  };
+  if (parted)
+    launch_index_build(part, e.n_rec, idx->dir_bits, gshift, idx->rec, idx->dir, ctl->counters,
+                       err, s);
+  else
+    XTN_RC(from_sorted());
   XTN_CK(cudaGetLastError());
   Control h{};
   ReadBack rb(s);
   XTN_RC(rb.add(&h, ctl));
   XTN_RC(rb.wait());
   if (parted && (h.err[0] == DERR_CAPACITY || (!h.err[0] && h.counters[3]))) {
-    // too many records of one key for a partition or a block
-    ar.release();
-    return index_build_impl(seqs, offsets, n, d, s, out, true);
+    // too many records of one key for a partition or a block: sorted instead,
+    // in the partitions' buffers, into the memory that is there
+    XTN_CK(cudaMemsetAsync(ctl->err, 0, 4, s));
+    XTN_CK(cudaMemsetAsync(ctl->counters, 0, sizeof ctl->counters, s));
+    XTN_RC(expand_and_sort(e, n, d, nullptr, sms, ar, err, s, &so, false, 0, -1, nullptr,
+                           part.rec, part.spill));
+    XTN_RC(from_sorted());
+    XTN_CK(cudaGetLastError());
+    XTN_RC(rb.add(&h, ctl));
+    XTN_RC(rb.wait());
   }
   if (h.err[0]) return map_device_err(h.err[0]);
   idx->n_groups = h.counters[0];
   guard.p = nullptr;
   *out = idx;
   return XTN_OK;
+}
+
+int index_build_impl(const uint8_t* seqs, const int64_t* offsets, int64_t n, int d, cudaStream_t s,
+                     xtn_index** out) {
+  return partitioned_or_sorted(
+      [&](int mode) { return index_build_once(seqs, offsets, n, d, s, out, mode); });
 }
 
 // Candidate words a query search makes room for before it knows their number:
