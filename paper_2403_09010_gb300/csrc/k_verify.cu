@@ -651,7 +651,8 @@ __device__ __forceinline__ int tcrdist_score(const uint8_t* cost, const Key128& 
   return 3 * sum;
 }
 
-// ITEMS rows a thread, in the order of the input.
+// ITEMS rows a thread, in the order of the input.  `out` is left alone when
+// the encoder has found a bad letter, length or offset.
 template <int ITEMS>
 __global__ void __launch_bounds__(VER_THREADS)
     k_tcrdist_filter(const xtn_triple* __restrict__ in, int64_t n, const Key128* __restrict__ keys,
@@ -673,6 +674,8 @@ __global__ void __launch_bounds__(VER_THREADS)
                     ? (uint8_t)min(4, 4 - (int)c_blosum62[x - 1][y - 1])
                     : 4;
   }
+  // (a row out of range, which other blocks may report by now, spoils `out` anyway)
+  const bool failed = *(volatile uint32_t*)err != 0;
   const uint32_t tile = tile_id(ctr, &s_tile);  // a barrier: the costs are complete
   const int64_t tbase = (int64_t)tile * TILE;
   const int64_t base = tbase + (int64_t)threadIdx.x * ITEMS;
@@ -706,7 +709,7 @@ __global__ void __launch_bounds__(VER_THREADS)
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it)
     if (keep >> it & 1u) {
-      if (o < n) out[o] = in[base + it];
+      if (o < n && !failed) out[o] = in[base + it];
       ++o;
     }
 }
