@@ -26,8 +26,8 @@
 // alternating between the input buffer (scratch within the bucket's own
 // range) and the output.
 #include <algorithm>
-#include <mutex>
 
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -661,14 +661,11 @@ void launch_bucket(bool hash, uint64_t* A, uint64_t* Y, int64_t n, const uint64_
                    uint64_t* flags, uint64_t* tile_counts, uint64_t* cand, uint64_t cand_cap,
                    uint64_t* cand_count, int id_bits, uint32_t* err, cudaStream_t s) {
   if (n <= 0) return;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_bucket<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)Bk<true>::bytes);
-    cudaFuncSetAttribute(k_bucket<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    cudaFuncSetAttribute(k_bucket<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)Bk<false>::bytes);
-    cudaFuncSetAttribute(k_bucket<false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  static PerDevice shared;
+  shared([] {
+    const cudaError_t e = allow_shared((const void*)k_bucket<true>, (int)Bk<true>::bytes);
+    return e != cudaSuccess ? e
+                            : allow_shared((const void*)k_bucket<false>, (int)Bk<false>::bytes);
   });
   const int full = bucket_capacity(hash);
   if (cap <= 0 || cap > full) cap = full;

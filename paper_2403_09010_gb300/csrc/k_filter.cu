@@ -25,8 +25,8 @@
 // key compared is every fingerprint bit the record holds above its id, so
 // unequal variants hardly ever make a candidate.
 #include <algorithm>
-#include <mutex>
 
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -324,11 +324,8 @@ template <int THREADS, int SEEN, int AGAIN, int MIN_BLOCKS, bool LOW>
 void filter_launch(const Partitions& p, int shift, uint32_t* err, cudaStream_t s) {
   using SM = FilterSmem<SEEN, AGAIN>;
   auto f = k_bucket_filter<THREADS, SEEN, AGAIN, MIN_BLOCKS, LOW>;
-  static std::once_flag once;
-  std::call_once(once, [&] {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM));
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  });
+  static PerDevice shared;
+  shared([&] { return allow_shared((const void*)f, (int)sizeof(SM)); });
   f<<<1u << p.pbits, THREADS, sizeof(SM), s>>>(
       p.rec, p.count, p.region, shift, p.kept, p.kept_count(), p.spill, p.spill_cap,
       reinterpret_cast<unsigned long long*>(p.n_spill), err);
@@ -355,12 +352,8 @@ void launch_group_filter(const Partitions& q, uint64_t n_rec, uint64_t* cand, ui
   else if (mean <= 26500) filter_launch<512, 19, 17, 2>(p, id_bits, err, s);
   else filter_launch<1024, 20, 18, 1>(p, id_bits, err, s);
   prof_end(s);
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_group_kept, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(GroupSmem));
-    cudaFuncSetAttribute(k_group_kept, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  });
+  static PerDevice shared;
+  shared([] { return allow_shared((const void*)k_group_kept, (int)sizeof(GroupSmem)); });
   prof_begin(s, "k_group_kept", 0.0);
   k_group_kept<<<1u << p.pbits, GK_THREADS, sizeof(GroupSmem), s>>>(
       p.kept, p.kept_count(), p.region, p.pbits, p.spill, p.spill_cap,

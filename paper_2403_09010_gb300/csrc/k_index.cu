@@ -22,6 +22,7 @@
 #include <cmath>
 
 #include "partition.cuh"
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -214,8 +215,8 @@ bool choose_index_partitions(uint64_t n_rec, int dir_bits, PartitionShape* g) {
 void launch_index_build(const Partitions& p, uint64_t n_rec, int dir_bits, int gshift,
                         uint64_t* rec, uint32_t* dir, uint64_t* n_groups, uint32_t* err,
                         cudaStream_t s) {
-  cudaFuncSetAttribute(k_index_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sizeof(IndexSmem));
+  static PerDevice shared;
+  shared([] { return allow_shared((const void*)k_index_build, (int)sizeof(IndexSmem), false); });
   prof_begin(s, "k_index_build", (double)n_rec * 24.0 + 4.0 * (double)(1ull << dir_bits));
   k_index_build<<<1u << p.pbits, IX_THREADS, sizeof(IndexSmem), s>>>(
       p.rec, p.count, p.region, p.pbits, dir_bits, gshift, rec, n_rec, dir,

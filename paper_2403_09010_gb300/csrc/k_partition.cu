@@ -24,9 +24,9 @@
 // the write-out, into the registers that the placing has freed.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
 #include "partition.cuh"
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -150,11 +150,9 @@ template <int ITEMS, int MIN_BLOCKS>
 void partition_launch(const uint64_t* in, int64_t n, const uint64_t* n_dev, const Partitions& p,
                       int max_bits, int sms, uint32_t* err, cudaStream_t s) {
   auto f = k_partition<ITEMS, MIN_BLOCKS>;
-  static std::once_flag once;
-  std::call_once(once, [&] {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)partition_smem_bytes<ITEMS>(max_bits));
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  static PerDevice shared;
+  shared([&] {
+    return allow_shared((const void*)f, (int)partition_smem_bytes<ITEMS>(max_bits));
   });
   const int64_t tiles = (n + PT_THREADS * ITEMS - 1) / (PT_THREADS * ITEMS);
   f<<<(uint32_t)std::min<int64_t>(tiles, (int64_t)sms * MIN_BLOCKS), PT_THREADS,
@@ -344,11 +342,8 @@ void launch_split(const Partitions& p, uint64_t n_rec, int sms, uint32_t* err, c
   constexpr int ITEMS = 22, MIN_BLOCKS = 2;
   constexpr int smem = PT_THREADS * ITEMS * 8;
   auto f = k_split<ITEMS, MIN_BLOCKS>;
-  static std::once_flag once;
-  std::call_once(once, [&] {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  });
+  static PerDevice shared;
+  shared([&] { return allow_shared((const void*)f, smem); });
   const Partitions q = p.fine();
   prof_begin(s, "k_split", (double)n_rec * 16.0);
   f<<<(uint32_t)sms * MIN_BLOCKS, PT_THREADS, smem, s>>>(

@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "expand.cuh"
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -254,8 +255,8 @@ static void query_launch(const ExpandSource& src, int64_t n_q, int d, const uint
                          uint64_t* n_variants, int sms, uint32_t* err, cudaStream_t s) {
   using ull = unsigned long long;
   auto f = k_query_candidates<KIND>;
-  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)sizeof(QuerySmem<KIND>));
+  static PerDevice shared;
+  shared([&] { return allow_shared((const void*)f, (int)sizeof(QuerySmem<KIND>), false); });
   // `pack` as large as leaves a resident warp four units of work: one query a
   // unit for 10,000 (132 us with two), 30,000 of a 36M-record index 125 us
   // against 147 with six

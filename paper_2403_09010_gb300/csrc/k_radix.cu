@@ -23,8 +23,8 @@
 // k_onesweep_runs (further down) keeps the same steps but counts and places
 // keys with shared-memory atomics instead of keeping ranks in registers.
 #include <algorithm>
-#include <mutex>
 
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -767,11 +767,8 @@ static cudaError_t onesweep_launch(int cfg, const uint64_t* in, uint64_t* out, i
     case ONESWEEP_LOOP: {
       using SM = RunsSmem<LOOP_THREADS, LOOP_ITEMS>;
       auto f = k_onesweep_runs<LOOP_THREADS, LOOP_ITEMS, LOOP_BLOCKS, 8, 0, 0, false, true>;
-      static std::once_flag once;
-      std::call_once(once, [&] {
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
-        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      });
+      static PerDevice shared;
+      shared([&] { return allow_shared((const void*)f, (int)SM::bytes); });
       // every block is resident, so the look-back's predecessors run
       const uint32_t tiles = std::min<uint32_t>(div_up_u32(n, SM::TILE), 148 * LOOP_BLOCKS);
       f<<<tiles, LOOP_THREADS, SM::bytes, s>>>(in, out, n_dev, n, shift, bits, bucket_shift,
@@ -782,12 +779,9 @@ static cudaError_t onesweep_launch(int cfg, const uint64_t* in, uint64_t* out, i
 #define X(id, T, I, B, M, C)                                                                  \
   case id: {                                                                                  \
     using SM = OnesweepSmem<T, I, M, C>;                                                      \
-    static std::once_flag once;                                                               \
-    std::call_once(once, [] {                                                                 \
-      cudaFuncSetAttribute(k_onesweep<T, I, B, M, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           (int)SM::bytes);                                                   \
-      cudaFuncSetAttribute(k_onesweep<T, I, B, M, C>,                                            \
-                           cudaFuncAttributePreferredSharedMemoryCarveout, 100);              \
+    static PerDevice shared;                                                                  \
+    shared([] {                                                                               \
+      return allow_shared((const void*)k_onesweep<T, I, B, M, C>, (int)SM::bytes);            \
     });                                                                                       \
     /* one tile per block; with the count on the device, n is its capacity */                \
     const uint32_t tiles = div_up_u32(n, SM::TILE);                                           \
@@ -803,13 +797,13 @@ static cudaError_t onesweep_launch(int cfg, const uint64_t* in, uint64_t* out, i
 #define X(id, T, I, B, W, D, U)                                                               \
   case id: {                                                                                  \
     using SM = RunsSmem<T, I>;                                                                \
-    static std::once_flag once;                                                               \
-    std::call_once(once, [] {                                                                 \
+    static PerDevice shared;                                                                  \
+    shared([] {                                                                               \
+      cudaError_t e = cudaSuccess;                                                            \
       for (auto f : {k_onesweep_runs<T, I, B, W, D, U, false>,                                \
-                     k_onesweep_runs<T, I, B, W, D, U, true>}) {                              \
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes); \
-        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);         \
-      }                                                                                       \
+                     k_onesweep_runs<T, I, B, W, D, U, true>})                                \
+        if (e == cudaSuccess) e = allow_shared((const void*)f, (int)SM::bytes);               \
+      return e;                                                                               \
     });                                                                                       \
     const uint32_t tiles = div_up_u32(n, SM::TILE);                                           \
     auto f = bucket_shift >= 32 ? k_onesweep_runs<T, I, B, W, D, U, true>                     \

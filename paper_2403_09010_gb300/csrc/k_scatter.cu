@@ -10,11 +10,11 @@
 // an expansion in sequence order and a pass over its records this saves
 // writing and reading them once (16 of 24 bytes per record).
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "expand.cuh"
 #include "partition.cuh"
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -288,11 +288,9 @@ void scatter_launch(const ExpandSource& src, const uint64_t* rec_off, int64_t n,
                     uint64_t spill_cap, uint64_t* n_spill, int sms, uint32_t* err,
                     cudaStream_t s) {
   auto f = k_expand_scatter<KIND>;
-  static std::once_flag once;
-  std::call_once(once, [&] {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)scatter_smem_bytes<KIND>(PART_MAX_BITS));
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  static PerDevice shared;
+  shared([&] {
+    return allow_shared((const void*)f, (int)scatter_smem_bytes<KIND>(PART_MAX_BITS));
   });
   // small inputs: fewer records a warp, so that every SM has some
   using C = SC<KIND>;

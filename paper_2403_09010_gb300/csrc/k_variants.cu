@@ -13,10 +13,10 @@
 //              sort the records (all of them, or only the first when each
 //              sort pass counts the next).
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "expand.cuh"
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -490,11 +490,8 @@ static void expand_launch(const ExpandSource& src, const uint64_t* rec_off, int6
                           uint32_t* err, cudaStream_t s, uint4* zero, uint64_t n_zero) {
   auto f = k_expand<KIND, SEL, H>;
   constexpr int smem = (int)sizeof(ExpandSmem<KIND, SEL, H>);
-  static std::once_flag once;
-  std::call_once(once, [&] {
-    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  });
+  static PerDevice shared;
+  shared([&] { return allow_shared((const void*)f, smem); });
   const int per_block = EXPAND_WARPS * VK<KIND>::PACK;
   const int64_t blocks = std::min<int64_t>((n + per_block - 1) / per_block, (int64_t)sms * 8);
   f<<<(uint32_t)blocks, EXPAND_THREADS, smem, s>>>(src, rec_off, n, d, seq_rep, id_bits, out,

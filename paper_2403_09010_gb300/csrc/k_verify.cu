@@ -32,6 +32,7 @@
 // bit-vector form (146 us for the 1M workload's 4.3 M candidates).
 #include <algorithm>
 
+#include "per_device.h"
 #include "xtn_common.cuh"
 #include "xtn_kernels.h"
 
@@ -515,8 +516,8 @@ void launch_small_rows(const uint64_t* cand, uint64_t n, uint32_t j_bits, const 
                        const PairSide& sj, const uint32_t* seq_rep, int self_mode, int d,
                        int metric, xtn_triple* rows, int64_t row_cap, uint64_t* n_rows,
                        uint32_t* err, cudaStream_t s) {
-  cudaFuncSetAttribute(k_small_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)SR_SMEM);
+  static PerDevice shared;
+  shared([] { return allow_shared((const void*)k_small_rows, (int)SR_SMEM, false); });
   prof_begin(s, "k_small_rows", (double)n * (8.0 + 2 * 32.0));
   k_small_rows<<<1, SR_THREADS, SR_SMEM, s>>>(cand, (uint32_t)n, j_bits, si, sj, seq_rep,
                                               self_mode, d, metric, rows, row_cap, n_rows, err);
@@ -589,7 +590,8 @@ size_t bucket_rows_status_bytes() { return RADIX * 8 + 16; }
 void launch_bucket_rows(const uint64_t* words, uint64_t n_max, const uint64_t* n_words,
                         const uint64_t* starts, uint32_t pair_bits, uint32_t j_bits,
                         xtn_triple* rows, int64_t row_cap, uint64_t* status, uint64_t* n_rows, uint32_t* err, cudaStream_t s) {
-  cudaFuncSetAttribute(k_bucket_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SR_SMEM);
+  static PerDevice shared;
+  shared([] { return allow_shared((const void*)k_bucket_rows, (int)SR_SMEM, false); });
   prof_begin(s, "k_unique_finalize", (double)n_max * 8.0);
   k_bucket_rows<<<RADIX, SR_THREADS, SR_SMEM, s>>>(words, n_words, starts, pair_bits, j_bits, rows,
                                                    row_cap, status,
