@@ -115,11 +115,12 @@ __device__ __forceinline__ void load_combs(uint16_t* s_comb) {
 }
 
 // s_pow[k + 3] = B^k for k = -3 .. (B^-1 is an exact inverse), as far as the
-// lanes' chunks reach.
+// lanes' chunks reach; none for VK_D1, whose powers are constants.
 template <int KIND>
-constexpr int N_POWERS = VK<KIND>::PER * VK<KIND>::LANES + 4;
+constexpr int N_POWERS = KIND == VK_D1 ? 1 : VK<KIND>::PER * VK<KIND>::LANES + 4;
 template <int KIND>
 __device__ __forceinline__ void load_powers(uint64_t* s_pow) {
+  if constexpr (KIND == VK_D1) return;
   for (int k = threadIdx.x; k < N_POWERS<KIND>; k += blockDim.x) {
     uint64_t p = HASH_BINV3;
     for (int e = 0; e < k; ++e) p *= HASH_B;

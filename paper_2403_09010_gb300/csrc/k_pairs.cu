@@ -350,14 +350,6 @@ void launch_group_finish(const uint64_t* flags, int64_t n, const uint64_t* n_dev
   k_groups_total<<<1, 1, 0, s>>>(tile_prefix + tiles, n_groups);
 }
 
-void launch_group_bounds(const uint64_t* keys, int64_t n, const uint64_t* n_dev, int gshift,
-                         uint32_t* S, uint32_t* E, uint64_t cap, uint64_t* flags,
-                         uint64_t* status, uint32_t* err, uint64_t* n_groups, cudaStream_t s) {
-  launch_group_flags(keys, n, n_dev, gshift, flags, status, s);
-  launch_group_finish(flags, n, n_dev, S, E, cap, status, err, n_groups, s);
-}
-
-
 // ------------------------------------------------------------ pair emit ---
 constexpr int EMIT_THREADS = 256;
 constexpr int EMIT_ITEMS = 8;

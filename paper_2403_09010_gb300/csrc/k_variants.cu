@@ -24,8 +24,9 @@ namespace xtn {
 
 // 'A'..'Z' -> residue code (alphabetical order of the 20 one-letter codes),
 // 0 for letters outside the alphabet (B J O U X Z) and for anything else.
-// Computed, not looked up: lanes of a warp read different letters, which a
-// constant-memory table would serve one at a time.
+// Computed once a block for the encoder's table in shared memory (lanes of a
+// warp read different letters, which a constant-memory table would serve one
+// at a time).
 constexpr uint32_t NOT_RESIDUE = (1u << 1) | (1u << 9) | (1u << 14) | (1u << 20) | (1u << 23) |
                                  (1u << 25);  // B J O U X Z
 __device__ __forceinline__ uint32_t letter_code(uint32_t ch) {

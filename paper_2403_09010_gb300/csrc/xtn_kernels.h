@@ -207,9 +207,6 @@ void launch_scan_group_pairs(const uint32_t* S, const uint32_t* E, int64_t n_gro
 size_t group_flag_words(int64_t n);
 // Group bounds = flags (k_group_flags, or k_bucket_sort) + finish (tile
 // prefix, k_group_write, group count).  `status` holds group_status_bytes(n).
-void launch_group_bounds(const uint64_t* keys, int64_t n, const uint64_t* n_dev, int gshift,
-                         uint32_t* S, uint32_t* E, uint64_t cap, uint64_t* flags,
-                         uint64_t* status, uint32_t* err, uint64_t* n_groups, cudaStream_t s);
 uint64_t* group_tile_counts(uint64_t* status, int64_t n);
 void launch_group_flags(const uint64_t* keys, int64_t n, const uint64_t* n_dev, int gshift,
                         uint64_t* flags, uint64_t* status, cudaStream_t s);
