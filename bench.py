@@ -39,7 +39,9 @@ UNIT = "verified pairs/s"
 L2_FLUSH_BYTES = 256 << 20
 CPU_SAMPLE_N = 100_000
 ROOFLINE_KERNEL = "k_expand"
-ROOFLINE_SOURCE = os.path.join(ROOT, "paper_2403_09010_gb300", "csrc", "k_scatter.cu")
+# k_expand_scatter and what it is made of (its body is in the headers)
+ROOFLINE_SOURCES = [os.path.join(ROOT, "paper_2403_09010_gb300", "csrc", f)
+                    for f in ("k_scatter.cu", "expand.cuh", "partition.cuh", "xtn_common.cuh")]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_expand_scatter_traffic.txt")
 
 
@@ -78,6 +80,15 @@ def _peaks():
         return 6800.0, "fallback"
 
 
+def _source_hash():
+    """First 16 hex digits of the SHA-256 of ROOFLINE_SOURCES, one after another."""
+    h = hashlib.sha256()
+    for path in ROOFLINE_SOURCES:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def _traffic_per_record():
     """DRAM bytes per expanded record from the committed ncu summary, or None
     when the kernel source changed since the counters were taken."""
@@ -86,8 +97,7 @@ def _traffic_per_record():
     except OSError:
         return None
     kv = dict(l.split("=", 1) for l in text.splitlines() if "=" in l and not l.startswith("#"))
-    src_hash = hashlib.sha256(open(ROOFLINE_SOURCE, "rb").read()).hexdigest()[:16]
-    if kv.get("source_sha256_16", "").strip() != src_hash:
+    if kv.get("source_sha256_16", "").strip() != _source_hash():
         return None
     try:
         return float(kv["dram_bytes_per_record"])
