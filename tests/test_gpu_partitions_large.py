@@ -106,3 +106,49 @@ def test_partitions_of_either_level_run_over(xtn):
         ds, do, 1, max_pass_records=800_000_000, cap=cap))
     assert passes == 1 and kernels["k_split"][0] == 1
     assert torch.equal(rows, got)
+
+
+def _subsets_d3(m):
+    """Distinct strings after at most three deletions, per row of m (their
+    number goes by the runs of equal residues: R, two or longer, three or
+    longer)."""
+    eq = m[:, 1:] == m[:, :-1]
+    start = torch.ones_like(m, dtype=torch.bool)
+    start[:, 1:] = ~eq
+    long2 = start[:, :-1] & eq
+    long3 = long2[:, :-1] & eq[:, 1:]
+    R, D, T = (x.sum(1).long() for x in (start, long2, long3))
+    return (1 + R + R * (R - 1) // 2 + D + R * (R - 1) * (R - 2) // 6 + D * (R - 1) + T)
+
+
+def test_word_indices_past_32_bits(xtn):
+    """4,285 to 4,294 M records at once: in one pass (the regions together are
+    past 2^32 words there, too, and the records come through k_partition) and in
+    one search, against passes of a quarter."""
+    n, L = 2_100_000, 25
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    letters = torch.from_numpy(gen.AA_BYTES.copy()).cuda()
+    m = letters[torch.randint(0, 20, (n, L), generator=g, device="cuda")]
+    src = torch.randint(0, n // 2, (n // 40,), generator=g, device="cuda")
+    at = n // 2 + torch.randperm(n // 2, generator=g, device="cuda")[:n // 40]
+    m[at] = m[src]  # copies, then one to three residues of most of them changed
+    for _ in range(3):
+        m[at, torch.randint(0, L, (n // 40,), generator=g, device="cuda")] = \
+            letters[torch.randint(0, 20, (n // 40,), generator=g, device="cuda")]
+    limit = (1 << 32) - (1 << 20)
+    upto = torch.cumsum(_subsets_d3(m), 0)
+    n = int((upto < limit - 1_000_000).sum())
+    total = int(upto[n - 1])
+    assert 4_285_000_000 < total < limit
+    ds = m[:n].reshape(-1).contiguous()
+    do = torch.arange(n + 1, device="cuda", dtype=torch.int64) * L
+    want, passes = xtn.search_self_streaming(ds, do, 3, max_pass_records=1 << 30)
+    assert passes > 3 and len(want) > n // 100
+    (rows, passes), kernels = _kernels(xtn, lambda: xtn.search_self_streaming(
+        ds, do, 3, max_pass_records=limit))
+    assert passes == 1 and kernels["k_split"][0] == 1
+    assert torch.equal(rows, want)
+    got, kernels = _kernels(xtn, lambda: xtn.search_self(ds, do, 3))
+    assert kernels["k_split"][0] == 1 and "k_expand_bins" not in kernels
+    assert torch.equal(got, want)
