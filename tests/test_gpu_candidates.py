@@ -55,3 +55,34 @@ def test_candidates_past_the_buffer():
     assert torch.equal(plan.result(cap=cap, like=ds), got)
     assert plan.stats()["candidates"] == needed
     plan.free()
+
+
+def test_candidates_past_the_buffer_of_a_small_search():
+    """All partitions of a small search are worked on at once, so blocks have to
+    leave in the middle of their list: 1.1 M records, 8 M candidates, room for 1 M."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import oracle
+    import paper_2403_09010_gb300 as xtn
+    xtn.build()
+    rng = np.random.default_rng(3)
+    n = 160_000
+    m = rng.choice(gen.AA_BYTES, (n, 6))
+    m[:, 0], m[:, -1] = ord("C"), ord("F")
+    off = np.arange(n + 1, dtype=np.int64) * 6
+    seqs = m.reshape(-1).copy()
+    ds, do = torch.from_numpy(seqs).cuda(), torch.from_numpy(off).cuda()
+    cap = 8_000_000
+    got = xtn.search_self(ds, do, 1, cap=cap)
+    xtn.profile_report()
+    xtn.profile_enable(True)
+    again = xtn.search_self(ds, do, 1, cap=cap)
+    xtn.profile_enable(False)
+    kernels = xtn.profile_report()
+    assert torch.equal(again, got)
+    assert kernels["k_emit_pairs"][0] == 1  # the search started over
+    assert kernels["k_group_kept"][1] < 0.3 * kernels["k_emit_pairs"][1]
+    few = 20_000
+    want = oracle.symdel_self_sharded(seqs[:6 * few], off[:few + 1], 1)
+    part = got[got[:, 1] < few].cpu().numpy().astype(np.uint32)
+    assert np.array_equal(part, want)
