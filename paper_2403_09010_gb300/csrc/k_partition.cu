@@ -163,8 +163,9 @@ void partition_launch(const uint64_t* in, int64_t n, const uint64_t* n_dev, cons
 
 // The second level: every coarse partition once more by the `sub` bits below
 // its own, in tiles of one partition each, with k_partition's steps.  With 2^5
-// to 2^8 bins a tile's runs are 44 to 350 records long, against five at the
-// end of one level: 3.97 G records (36M sequences, d = 2) 18.4 ms, 3.4 TB/s.
+// to 2^8 bins a tile's runs are 36 to 290 records long, against five at the
+// end of one level: 3.97 G records (36M sequences, d = 2) 15.4 ms, 4.1 TB/s
+// (with 22 records a thread, which spill registers, 18.3; 16 15.6).
 template <int ITEMS, int MIN_BLOCKS>
 __global__ void __launch_bounds__(PT_THREADS, MIN_BLOCKS)
     k_split(const uint64_t* __restrict__ in, const uint32_t* __restrict__ count, uint32_t region,
@@ -315,9 +316,9 @@ uint32_t region_of(double mean) {
 // More records than 2^13 such partitions take go through two levels, 2^9 and up
 // to 2^8 each: fuller bitmaps keep more and more lone records, and a list is
 // read once for every 5,600 of them.  Whole searches at d = 2, one level against
-// two: 0.55 G records 8.8 and 9.2 ms, 0.77 G 13.2 and 12.4, 0.99 G 17.7 and
-// 16.2 (17.1 with 2^11 in the first level); 2.0 G 33 with two and 96 with one
-// whose bitmap had a bit less to go by, 4.0 G 68 and 734.
+// two: 0.55 G records 8.8 and 9.2 ms, 0.77 G 13.2 and 11.9, 0.99 G 17.7 and
+// 15.7 (0.9 more with 2^11 in the first level); 2.0 G 32 with two and 96 with
+// one whose bitmap had a bit less to go by, 4.0 G 66 and 734.
 PartitionShape choose_partitions(uint64_t n_rec, int fx) {
   PartitionShape g;
   const uint64_t most = (uint64_t)40000 << fx, least = (uint64_t)10000 << fx;
@@ -339,7 +340,7 @@ PartitionShape choose_partitions(uint64_t n_rec, int fx) {
 }
 
 void launch_split(const Partitions& p, uint64_t n_rec, int sms, uint32_t* err, cudaStream_t s) {
-  constexpr int ITEMS = 22, MIN_BLOCKS = 2;
+  constexpr int ITEMS = 18, MIN_BLOCKS = 2;
   constexpr int smem = PT_THREADS * ITEMS * 8;
   auto f = k_split<ITEMS, MIN_BLOCKS>;
   static PerDevice shared;

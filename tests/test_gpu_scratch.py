@@ -113,9 +113,11 @@ class LittleMemory:
 
 # 104.8 M records (115.5 M in a plan's bound).  With partitions a search takes
 # 29 bytes a record and 93 a sequence (3.1 GB), a plan 25 and 28 a pair of its
-# capacity (3.2 GB); sorted, 17 and 17 (1.9 and 2.3 GB).
+# capacity (3.2 GB), a build 20 and 10 for the index (3.2 GB); sorted, 17, 17
+# and 27 (1.9, 2.3 and 2.9 GB).
 @pytest.mark.parametrize("what,free", [("search", 2_500 << 20), ("passes", 2_600 << 20),
-                                       ("plan", 2_750 << 20), ("search", 8_000 << 20)])
+                                       ("plan", 2_750 << 20), ("index", 2_870 << 20),
+                                       ("search", 8_000 << 20), ("index", 8_000 << 20)])
 def test_sorted_where_partitions_do_not_fit(xtn, what, free):
     n, cap = 1_000_000, 400_000
     seqs, off = gen.workload(gen.SELF_1M)
@@ -133,9 +135,17 @@ def test_sorted_where_partitions_do_not_fit(xtn, what, free):
             elif what == "passes":
                 got, _ = xtn.search_self_streaming(ds, do, 2, max_pass_records=120_000_000,
                                                    cap=cap)
+            elif what == "index":
+                idx = xtn.index_build(ds, do, 2)
+                got = want
+                info = idx.info()
+                idx.free()
+                assert info["n_records"] > 104_000_000
             else:
                 got = xtn.search_self(ds, do, 2, cap=cap)
             xtn.profile_enable(False)
             kernels = xtn.profile_report()
             assert torch.equal(got, want)
-            assert ("k_bucket_filter" in kernels) == (free > 4_000 << 20)
+            parted = "k_index_build" if what == "index" else "k_bucket_filter"
+            assert (parted in kernels) == (free > 4_000 << 20)
+            assert what != "index" or ("k_bucket_sort" in kernels) == (free < 4_000 << 20)
