@@ -41,7 +41,6 @@ struct IndexSmem {
   uint32_t bin[IX_BINS];  // 16-byte aligned
   uint32_t wsum[IX_THREADS / 32];
   uint32_t total, base, b1, o1, heads, n_list;
-  bool give_up;
   uint16_t list[IX_LIST];
 };
 
@@ -82,8 +81,8 @@ __global__ void __launch_bounds__(IX_THREADS, 1)
     k_index_build(const uint64_t* __restrict__ parts, const uint32_t* __restrict__ count,
                   uint32_t region, int pbits, int dir_bits, int gshift,
                   uint64_t* __restrict__ rec, uint64_t n_rec, uint32_t* __restrict__ dir,
-                  uint32_t sample, const uint64_t* __restrict__ n_spill,
-                  unsigned long long* __restrict__ n_groups, uint32_t* __restrict__ err) {
+                  uint32_t sample, unsigned long long* __restrict__ n_groups,
+                  uint32_t* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char index_smem[];
   IndexSmem& S = *reinterpret_cast<IndexSmem*>(index_smem);
   const uint32_t p = blockIdx.x, lane = lane_id(), warp = threadIdx.x >> 5;
@@ -93,18 +92,19 @@ __global__ void __launch_bounds__(IX_THREADS, 1)
   const uint32_t nb = 1u << sub, bmask = nb - 1u;
   const int bshift = 64 - dir_bits;
   const bool counts = p % sample == 0;  // its distinct keys, for all `sample` of them
-  // this partition's place: the records of those before it
+  // this partition's place: the records of those before it; and whether any
+  // ran over, as the caller then sorts globally
   uint32_t before = 0;
-  for (uint32_t q = threadIdx.x; q < p; q += IX_THREADS) before += min(count[q], region);
-  before = __reduce_add_sync(FULL_MASK, before);
-  if (threadIdx.x == 0) {
-    S.base = S.heads = 0;
-    // the caller will sort globally (read once for the block: others set it)
-    S.give_up = *n_spill != 0 || (*(volatile uint32_t*)err & DERR_CAPACITY) != 0;
+  bool ran_over = false;
+  for (uint32_t q = threadIdx.x; q < gridDim.x; q += IX_THREADS) {
+    const uint32_t c = count[q];
+    if (q < p) before += min(c, region);
+    ran_over |= c > region;
   }
+  before = __reduce_add_sync(FULL_MASK, before);
+  if (threadIdx.x == 0) S.base = S.heads = 0;
   for (uint32_t b = threadIdx.x; b < max(nb, 256u); b += IX_THREADS) S.bin[b] = 0;
-  __syncthreads();
-  if (S.give_up) return;
+  if (__syncthreads_or(ran_over)) return;
   if (lane == 0 && before) atomicAdd(&S.base, before);
   auto each = [&](auto f) {  // the partition's records, four loads in flight
     for (uint32_t k0 = threadIdx.x; k0 < m; k0 += 4 * IX_THREADS) {
@@ -200,9 +200,9 @@ __global__ void __launch_bounds__(IX_THREADS, 1)
 // stage) and as many directory entries as the counters hold; past those the
 // index is sorted globally.  Regions half as large again as the mean: copies
 // of one sequence all fall into one partition.  Where one overflows all the
-// same, or an entry is beyond a block's stage, the blocks leave and the caller
-// sorts: 300,000 sequences and 15,000 copies of one, d = 2, 1.97 ms, as long as
-// sorting at once; 1M and 60,000, d = 1, 1.46 (1.52).
+// same, the blocks leave and the caller sorts: 300,000 sequences and 15,000
+// copies of one, d = 2, 1.97 ms, as long as sorting at once; 1M and 60,000,
+// d = 1, 1.46 (1.52).
 bool choose_index_partitions(uint64_t n_rec, int dir_bits, PartitionShape* g) {
   int b = 8;
   while (b < 11 && (n_rec >> b) > 17000) ++b;
@@ -220,8 +220,7 @@ void launch_index_build(const Partitions& p, uint64_t n_rec, int dir_bits, int g
   prof_begin(s, "k_index_build", (double)n_rec * 24.0 + 4.0 * (double)(1ull << dir_bits));
   k_index_build<<<1u << p.pbits, IX_THREADS, sizeof(IndexSmem), s>>>(
       p.rec, p.count, p.region, p.pbits, dir_bits, gshift, rec, n_rec, dir,
-      n_rec < 1u << 20 ? 1u : 16u, p.n_spill, reinterpret_cast<unsigned long long*>(n_groups),
-      err);
+      n_rec < 1u << 20 ? 1u : 16u, reinterpret_cast<unsigned long long*>(n_groups), err);
   prof_end(s);
 }
 
