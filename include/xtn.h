@@ -113,11 +113,14 @@ XTN_API int xtn_version(void);
  *   n_out            : host; receives the exact number of result rows.
  * Scratch comes from the scratch cache (see xtn_scratch_trim) and is given
  * back before the call returns; the call synchronises the stream three times
- * (record count, candidate count, row count).  With the default grouping the
- * candidate buffer is sized at half the record count before grouping; an
- * input that needs more (thousands of copies of one sequence) is searched
- * again with all-global grouping, which sizes it exactly, so the result is
- * the same, only slower.
+ * (record count, candidate count, row count; a small search does not wait for
+ * the record count).  With the default grouping it takes about 29 bytes a
+ * variant record and 93 a sequence, and the candidate buffer is sized at half
+ * the record count before grouping; an input that needs more (thousands of
+ * copies of one sequence) is searched again with all-global grouping, which
+ * sizes it exactly, so the result is the same, only slower.  A device that has
+ * no room for that is searched with all-global grouping as well, which takes
+ * about 17 bytes a record and 16 a candidate pair.
  * Errors: INVALID_ARG, BAD_RESIDUE, SEQ_TOO_LONG, OOM, BUFFER_TOO_SMALL,
  * CUDA, DEVICE_TIMEOUT, TOO_LARGE.  An input with 2^32 variant records or more,
  * or 2^32 candidate pairs or more, is searched in passes as
@@ -193,10 +196,12 @@ XTN_API int xtn_search_paired(const uint8_t* a_seqs, const int64_t* a_offsets,
  * The rows are those of xtn_search_self (metric 0), xtn_search_self_hamming
  * (metric 1) or xtn_search_between (between != 0).
  *   max_pass_records : records per pass; <= 0 takes what fits in half the
- *                      free device memory (about 32 bytes per record).
+ *                      free device memory (at 32 bytes per record; large
+ *                      passes take 29).
  *   n_passes         : host, may be NULL; receives the passes run.
  * Other arguments as xtn_search_self.  Device memory: the sequences and
- * their match vectors, buffers for the largest pass, and the verified pairs.
+ * their bit planes, buffers for the largest pass (the same for every pass), and
+ * the verified pairs.
  * Errors: as xtn_search_self; INVALID_ARG for an unknown metric, or for
  * between != 0 without rep_offsets.
  */
@@ -212,7 +217,9 @@ XTN_API int xtn_search_self_streaming(const uint8_t* seqs, const int64_t* offset
  * 1-4; the paper's multi-value hash map of the SymDel step list, realised as a
  * sorted array as Sec. 2.2 describes).  The index owns its device memory
  * until xtn_index_free(); it is tied to the current device and may be used
- * from any stream of it.  *out receives the handle.
+ * from any stream of it.  *out receives the handle.  The build takes about 20
+ * bytes of scratch a record, 17 where it sorts them (past 134 M records, where
+ * one sequence makes up a few percent of the set, or for lack of room).
  * Errors: INVALID_ARG, BAD_RESIDUE, SEQ_TOO_LONG, OOM, CUDA, DEVICE_TIMEOUT,
  * TOO_LARGE.
  */
@@ -273,7 +280,8 @@ XTN_API int xtn_search_query_hamming(const xtn_index* idx, const uint8_t* q_seqs
  * sequence after its first floor(m/2) residues; each aligned position costs
  * 0 if the residues agree, else min(4, 4 - BLOSUM62[a][b]); each gap costs
  * 4; the sum is multiplied by 3.  Rows with score <= max_score are written
- * to `out` in input order (out must hold n_in rows).
+ * to `out` in input order (out must hold n_in rows); `out` is left alone when
+ * the sequences are refused.
  *   seqs, offsets, n : the sequences the row indices refer to.
  *   in, n_in         : input rows (i, j < n).
  * Errors: INVALID_ARG, BAD_RESIDUE, SEQ_TOO_LONG, OOM, CUDA.
@@ -293,8 +301,10 @@ XTN_API int xtn_tcrdist_filter(const uint8_t* seqs, const int64_t* offsets, int6
  * xtn_plan_create: plan for inputs with exactly these offsets (host or
  *   device, n+1 entries) and repertoire offsets (NULL for one repertoire).
  *   Record buffers are sized for every deletion subset of every sequence, an
- *   upper bound whatever the letters.  pair_capacity bounds the candidate
- *   pairs of one run (<= 0: one eighth of the record bound, at least 65,536).
+ *   upper bound whatever the letters (about 25 bytes each, 17 where a device
+ *   without room for more gets a plan that sorts all records).  pair_capacity
+ *   bounds the candidate pairs of one run (<= 0: one eighth of the record bound,
+ *   at least 65,536).
  * xtn_plan_run: search the n sequences at `seqs` (a device pointer; letters
  *   laid out as the plan's offsets say) on `stream`; returns once the work is
  *   queued.  Runs on one plan must not overlap.
@@ -315,8 +325,9 @@ XTN_API int xtn_plan_result(xtn_plan* plan, xtn_triple* out, int64_t cap, int64_
 XTN_API int xtn_plan_info(const xtn_plan* plan, int64_t* record_capacity, int64_t* pair_capacity,
                   int64_t* device_bytes);
 /* Counts of the last run (waits for `stream`): variant records, groups of
- * two or more records, candidate pairs, verified pair words (before dedup);
- * any output pointer may be NULL. */
+ * two or more records among those grouped by sorting (with the default
+ * grouping, only what its partitions did not hold), candidate pairs, verified
+ * pair words (before dedup); any output pointer may be NULL. */
 XTN_API int xtn_plan_stats(xtn_plan* plan, int64_t* records, int64_t* groups, int64_t* candidates,
                    int64_t* survivors, xtn_stream_t stream);
 XTN_API int xtn_plan_free(xtn_plan* plan);
@@ -369,8 +380,9 @@ XTN_API int xtn_tcrdist_filter_noalloc(const uint8_t* seqs, const int64_t* offse
  *                           of every pass, 1 = expand counts the first pass
  *                           and each sort pass counts the next
  *   XTN_TUNE_GROUPING     : how a search groups its records: 0 = expanded into
- *                           fingerprint partitions, whose repeated keys a
- *                           filter finds in shared memory (default); 1 =
+ *                           fingerprint partitions (in two steps past 655 M
+ *                           records), whose repeated keys a filter finds in
+ *                           shared memory (default); 1 =
  *                           global radix passes on every bit, then a flag
  *                           pass; 2 = global radix passes on the top bits,
  *                           then one shared-memory pass per block of buckets

@@ -13,8 +13,8 @@
 //        the second bitmap -- all members of groups of two or more, plus the
 //        few lone records that another key's bits kept.
 //     The bitmaps hold about 20 bits per record in the block's shared
-//     memory, so one block covers tens of thousands of records and no second
-//     partitioning pass is needed.
+//     memory, so one block covers tens of thousands of records and a second
+//     partitioning pass is only needed past 655 M of them.
 //   k_group_kept    : one block per list chains its records by a hash of
 //     their key and lets each one walk the rest of its chain, writing a
 //     candidate word (min id << id_bits | max id) for every record there with

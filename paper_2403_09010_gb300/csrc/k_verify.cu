@@ -532,8 +532,10 @@ void launch_small_rows(const uint64_t* cand, uint64_t n, uint32_t j_bits, const 
 // mostly latency, about 10 us a launch whatever the size.  Sort and dedup
 // before, and now: 10,000 queries (230,000 candidates) 63 + 14 and 12 + 21
 // us, 200,000 sequences (720,000) 68 + 14 and 12 + 29, overlap of 500,000
-// (1.9 M) 94 + 14 and 14 + 27.  A group with more distinct words than a block
-// holds sets DERR_CAPACITY (the caller sorts).
+// (1.9 M) 94 + 14 and 14 + 27.  A group of more than 2,048 rows (300,000 to
+// 500,000 sequences of one repertoire) takes the sort of four words a thread:
+// 78 to 98 + 14 to 22 and 13 to 16 + 82 to 86.  A group with more distinct
+// words than a block holds sets DERR_CAPACITY (the caller sorts).
 __global__ void __launch_bounds__(SR_THREADS)
     k_bucket_rows(const uint64_t* __restrict__ words, const uint64_t* __restrict__ n_words,
                   const uint64_t* __restrict__ starts, uint32_t pair_bits, uint32_t j_bits,
